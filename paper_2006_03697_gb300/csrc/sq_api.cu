@@ -304,7 +304,7 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
                   // TF32 hi/lo pairs for the mixed sweep
                   size_t(P.table_len) * (sizeof(double) + (real == sizeof(float) ? 3 * sizeof(float) : 0)) +
                   size_t(Nd) * size_t(d->n_pl + 1) * SQ_N_MOMENTS * sizeof(double) +   // moments
-                  size_t(d->n_pl + 1) * 4 * sizeof(double) + size_t(M) * sizeof(double) +
+                  size_t(d->n_pl + 1) * 4 * sizeof(double) + size_t(M) * 8 * sizeof(double) +   // R, coefficients, F, tables
                   size_t(Nd) * sizeof(double) + 4096 * 32 * sizeof(double) + sq::kLzDotCap * sizeof(double) + 1024;
   // Lanczos sample tiles (argmin V, argmax V, a stride-n/2 node grid); the buffers hold the
   // largest count so that sq_update_atoms can move them with V
@@ -347,7 +347,7 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
     const size_t per_tile = (size_t(k + 2) * g.Upts + size_t(g.r_cap)) * g.B * real + size_t(g.B) * (5 * k + 8) * 8;
     P.nlz_wave = int(std::max<size_t>(1, std::min<size_t>((size_t(8) << 30) / per_tile, size_t(P.wave_cap))));
     P.fixed_bytes += size_t(P.nlz_wave) * per_tile + size_t(Nd) * (4 + M + 20) * sizeof(double) +
-                     size_t(4 * M + 1024) * sizeof(double);
+                     1024 * sizeof(double);
   }
   return SQ_OK;
 }
@@ -523,6 +523,8 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   SQ_ALLOC(h->d.mom, sizeof(double) * size_t(Nd) * size_t(g.n_pl + 1) * SQ_N_MOMENTS);
   SQ_ALLOC(h->d.R, sizeof(double) * (g.n_pl + 1));
   SQ_ALLOC(h->d.cosF, sizeof(double) * h->M);
+  SQ_ALLOC(h->d.costab, sizeof(double) * 4 * size_t(h->M));
+  SQ_ALLOC(h->d.fvals, sizeof(double) * 3 * size_t(h->M));
   SQ_ALLOC(h->d.coef, sizeof(double) * 3 * (g.n_pl + 1));
   SQ_ALLOC(h->d.scal, sizeof(double) * 64);
   SQ_ALLOC(h->d.part, sizeof(double) * 4096 * 32);
@@ -574,7 +576,6 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
     SQ_ALLOC(h->d.ncoef, sizeof(double) * 2 * size_t(Nd));
     SQ_ALLOC(h->d.nF, sizeof(double) * size_t(Nd) * h->M);
     SQ_ALLOC(h->d.nrow, sizeof(double) * size_t(Nd) * 20);
-    SQ_ALLOC(h->d.costab, sizeof(double) * 4 * size_t(h->M));
     SQ_ALLOC(h->d.npart, sizeof(double) * 1024);
     SQ_ALLOC(h->d.nV, real * size_t(k + 1) * nw * g.Upts * g.B);
     SQ_ALLOC(h->d.nW, real * nw * g.Upts * g.B);
@@ -646,10 +647,8 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   if (rc != SQ_OK) return cleanup(rc);
   rc = sq::make_step_maps(h);
   if (rc != SQ_OK) return cleanup(rc);
-  if (h->bounds_mode == SQ_BOUNDS_PER_NODE) {
-    rc = sq::init_node_tables(h);
-    if (rc != SQ_OK) return cleanup(rc);
-  }
+  rc = sq::init_node_tables(h);
+  if (rc != SQ_OK) return cleanup(rc);
   rc = sq::measure_wave_rows(h);   // the sweep then needs no host round trip
   if (rc != SQ_OK) return cleanup(rc);
 

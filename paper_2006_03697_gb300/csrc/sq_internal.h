@@ -131,6 +131,8 @@ struct Dev {
   double* mom = nullptr;          // [N_d][n_pl+1][17]
   double* R = nullptr;            // [n_pl+1] node sums of rho^j
   double* cosF = nullptr;         // [M] sum'_j cos(j theta_k) R^j
+  double* costab = nullptr;       // [4 M] cos(pi t / (2 M))
+  double* fvals = nullptr;        // [3][M] g, r g and the entropy function at the Chebyshev-Gauss points
   double* coef = nullptr;         // [3][n_pl+1] c, d, s at the last contraction mu
   double* scal = nullptr;         // scalars: mu, bounds, partial sums ...
   double* part = nullptr;         // contraction partials
@@ -147,7 +149,6 @@ struct Dev {
   double* ncoef = nullptr;        // [N_d][2] step coefficients (ca = 2 / zeta_q, cd = ca lap0 - 2 chi_q / zeta_q)
   double* nF = nullptr;           // [N_d][M] sum'_j cos(j theta_k) rho_q^j
   double* nrow = nullptr;         // [N_d][20] contraction terms per node
-  double* costab = nullptr;       // [4 M] cos(pi t / (2 M))
   double* npart = nullptr;        // [1024] partial electron counts
   void* nV = nullptr;             // Lanczos wave buffers of the per-node bounds
   void* nW = nullptr;
@@ -282,7 +283,7 @@ int timing_collect(sq_handle* h);
 
 // setup kernels (sq_setup.cu)
 int build_tables(sq_handle* h);
-int init_node_tables(sq_handle* h);   // per-node bounds mode: cosine table, neutral node bounds
+int init_node_tables(sq_handle* h);   // cosine table; per-node bounds mode: neutral node bounds
 // the lists, A, W and t^0 of a wave in wb; with reuse, the lists and W of the same wave and atom
 // positions built by the previous sweep are kept (only A, the projection buffers and t^0 are
 // rewritten)

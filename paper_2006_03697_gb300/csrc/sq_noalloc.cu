@@ -17,7 +17,8 @@ namespace sq {
 
 // defined in sq_reduce.cu
 __global__ void k_rsum(const double* __restrict__ mom, int Nd, int n_pl, double* __restrict__ R);
-__global__ void k_cosF(const double* __restrict__ R, int n_pl, int M, double* __restrict__ F);
+__global__ void k_cosF(const double* __restrict__ R, int n_pl, int M, const double* __restrict__ tab,
+                       double* __restrict__ F);
 
 constexpr int kNoAllocScratch = SQ_NOALLOC_MAX_NPL + 1 + SQ_NOALLOC_MAX_M + 32;
 
@@ -80,7 +81,7 @@ extern "C" int sq_fermi_level_noalloc(const double* mom_dev, int n_nodes, int n_
   double* R = scratch;                            // [n_pl + 1]
   double* F = scratch + SQ_NOALLOC_MAX_NPL + 1;   // [M]
   sq::k_rsum<<<n_pl + 1, 256, 0, s>>>(mom_dev, n_nodes, n_pl, R);
-  sq::k_cosF<<<(M + 255) / 256, 256, 0, s>>>(R, n_pl, M, F);
+  sq::k_cosF<<<(M + 15) / 16, 128, 0, s>>>(R, n_pl, M, nullptr, F);
   sq::k_bisect_noalloc<<<1, 1024, 0, s>>>(F, M, lambda_lo, lambda_hi, kT, n_e, mu_dev);
   return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ERR_CUDA;
 }

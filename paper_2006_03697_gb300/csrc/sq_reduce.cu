@@ -29,13 +29,22 @@ __global__ void k_rsum(const double* __restrict__ mom, int Nd, int n_pl, double*
   if (threadIdx.x == 0) R[j] = s;
 }
 
-__global__ void k_cosF(const double* __restrict__ R, int n_pl, int M, double* __restrict__ F) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= M) return;
-  const double th = M_PI * (k + 0.5) / M;
-  double s = 0.5 * R[0];
-  for (int j = 1; j <= n_pl; ++j) s += cos(j * th) * R[j];
-  F[k] = s;
+// F_k = sum'_j cos(j theta_k) R^j. Eight lanes per k split the j range (one lane per k left most of
+// the FP64 pipes idle: 2048 threads on 8 SMs). tab (or null): cos(pi t / (2 M)), so that
+// cos(j theta_k) = tab[j (2 k + 1) mod 4 M]; without it the cosines are evaluated here.
+__global__ void __launch_bounds__(128) k_cosF(const double* __restrict__ R, int n_pl, int M, const double* __restrict__ tab,
+                                              double* __restrict__ F) {
+  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, sub = threadIdx.x & 7;
+  double s = 0.0;
+  if (k < M) {
+    const int odd = 2 * k + 1, M4 = 4 * M;
+    for (int j = sub; j <= n_pl; j += 8) {
+      const int t = int((long long)j * odd % M4);
+      s += (j == 0) ? 0.5 * R[0] : (tab ? tab[t] : cospi(double(t) / (2.0 * M))) * R[j];
+    }
+  }
+  for (int d = 4; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+  if (k < M && sub == 0) F[k] = s;
 }
 
 // Single block. scal[0], scal[1]: bounds; writes scal[2] = mu, status[kStNoBracket].
@@ -50,75 +59,154 @@ __global__ void k_bisect(const double* __restrict__ F, int M, double kT, double 
   }
 }
 
-// Coefficients at mu = scal[3]: block 0 -> c, 1 -> d (r g(r)), 2 -> s (entropy function).
-__global__ void k_coef(const double* __restrict__ scal, double kT, int n_pl, int M, double* __restrict__ coef) {
-  extern __shared__ double fv[];
-  const double lam_lo = scal[0], lam_hi = scal[1], mu = scal[3];
+// The coefficients c, d (r g(r)) and s (entropy function) at mu, in two launches. One kernel with a
+// block per function took 2.26 ms (M = 2048, n_pl = 60): FP64 issues 1.7 lanes per clock and SM
+// here, and three SMs evaluated M (n_pl + 1) cosines each. Now the cosines come from the handle's
+// table, k_fvals spreads the M exponentials over M / 64 blocks and k_coef takes one block per j: a
+// density and a pressure call on a 5 x 4 x 6 cell together took 4.5 ms less.
+//   k_fvals: fv[3][M] = g, r g, entropy at the Chebyshev-Gauss points; mu from scal[2] (from_scal) or
+//            the argument, left in scal[3]
+__global__ void __launch_bounds__(64) k_fvals(double* __restrict__ scal, double mu_arg, int from_scal, double kT, int M,
+                                              const double* __restrict__ tab, double* __restrict__ fv) {
+  const double lam_lo = scal[0], lam_hi = scal[1], mu = from_scal ? scal[2] : mu_arg;
   const double chi_q = 0.5 * (lam_hi + lam_lo), zeta_q = 0.5 * (lam_hi - lam_lo);
-  const int which = blockIdx.x;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k == 0) scal[3] = mu;
+  if (k >= M) return;
+  const double r = tab[2 * k + 1];
+  const double x = (chi_q + zeta_q * r - mu) / kT;
+  const double f = fermi_occ(x);
+  fv[k] = f;
+  fv[M + k] = r * f;
+  fv[2 * M + k] = entropy_d(x);
+}
+
+// coef[w][j] = (2/M) sum_k fv[w][k] cos(j theta_k), one block per j
+__global__ void __launch_bounds__(128) k_coef(const double* __restrict__ fv, int n_pl, int M,
+                                              const double* __restrict__ tab, double* __restrict__ coef) {
+  __shared__ double sh[3][4];
+  const int j = blockIdx.x, M4 = 4 * M;
+  double a[3] = {0.0, 0.0, 0.0};
+  int t = int((long long)j * (2 * threadIdx.x + 1) % M4);              // j (2 k + 1) mod 4 M
+  const int step = int((long long)j * (2 * int(blockDim.x)) % M4);
   for (int k = threadIdx.x; k < M; k += blockDim.x) {
-    const double r = cos(M_PI * (k + 0.5) / M);
-    const double x = (chi_q + zeta_q * r - mu) / kT;
-    fv[k] = (which == 0) ? fermi_occ(x) : (which == 1) ? r * fermi_occ(x) : entropy_d(x);
+    const double cs = tab[t];
+    for (int w = 0; w < 3; ++w) a[w] += fv[w * M + k] * cs;
+    t += step;
+    if (t >= M4) t -= M4;
+  }
+  for (int w = 0; w < 3; ++w) {
+    a[w] = warp_sum(a[w]);
+    if ((threadIdx.x & 31) == 0) sh[w][threadIdx.x >> 5] = a[w];
   }
   __syncthreads();
-  for (int j = threadIdx.x; j <= n_pl; j += blockDim.x) {
-    double s = 0.0;
-    for (int k = 0; k < M; ++k) s += fv[k] * cos(j * (M_PI * (k + 0.5) / M));
-    coef[which * (n_pl + 1) + j] = 2.0 / M * s;
+  if (threadIdx.x < 3) {
+    const double* r = sh[threadIdx.x];
+    coef[threadIdx.x * (n_pl + 1) + j] = 2.0 / M * ((r[0] + r[1]) + (r[2] + r[3]));
   }
 }
 
 constexpr int kNPart = 20;
+constexpr int kContractThreads = 256;
+constexpr int kContractGroups = kContractThreads / SQ_N_MOMENTS;   // j values in flight per node
 
-__global__ void k_contract(const double* __restrict__ mom, const double* __restrict__ coef,
-                           const double* __restrict__ scal, const double* __restrict__ v, int Nd, int n_pl,
-                           double dV, double* __restrict__ rho, double* __restrict__ part) {
-  __shared__ double sh[256];
-  const double lam_lo = scal[0], lam_hi = scal[1];
-  const double chi_q = 0.5 * (lam_hi + lam_lo), zeta_q = 0.5 * (lam_hi - lam_lo);
-  const double* c = coef;
-  const double* d = coef + (n_pl + 1);
-  const double* s = coef + 2 * (n_pl + 1);
-  double acc[kNPart];
-  for (int k = 0; k < kNPart; ++k) acc[k] = 0.0;
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < Nd; q += gridDim.x * blockDim.x) {
-    double r = 0.0;
-    double loc[kNPart];
-    for (int k = 0; k < kNPart; ++k) loc[k] = 0.0;
-    for (int j = 0; j <= n_pl; ++j) {
+// The contraction terms of nodes [q0, q1) with coefficients c, d, sc ([n_pl + 1] each) and one interval,
+// left in part[kNPart] (whole block; red: kContractGroups * kNPart + 8 doubles of shared memory). A
+// thread owns one moment slot and walks j, so a block reads whole contiguous moment rows (one
+// thread per node read 136-byte strides on a few blocks: 80-114 us at 1,728-32,768 nodes).
+__device__ void contract_block(const double* __restrict__ mom, const double* c, const double* d, const double* sc,
+                               double chi_q, double zeta_q, const double* __restrict__ v, int q0, int q1, int n_pl,
+                               double dV, double* __restrict__ rho, double* red, double* __restrict__ part) {
+  const int slot = threadIdx.x % SQ_N_MOMENTS, grp = threadIdx.x / SQ_N_MOMENTS;
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+  if (grp < kContractGroups) {
+    for (int j = grp; j <= n_pl; j += kContractGroups) {
+      const double* m = mom + ((size_t)q0 * (n_pl + 1) + j) * SQ_N_MOMENTS + slot;
+      double s = 0.0;
+#pragma unroll 4
+      for (int q = q0; q < q1; ++q, m += (size_t)(n_pl + 1) * SQ_N_MOMENTS) s += *m;
       const double wp = (j == 0) ? 0.5 : 1.0;
-      const double* m = mom + ((size_t)q * (n_pl + 1) + j) * SQ_N_MOMENTS;
-      const double cj = wp * c[j];
-      r += cj * m[0];
-      loc[0] += wp * (chi_q * c[j] + zeta_q * d[j]) * m[0];
-      loc[1] += wp * s[j] * m[0];
-      loc[2] += cj * m[7];
-      for (int k = 0; k < 6; ++k) loc[3 + k] += cj * m[1 + k];
-      for (int k = 0; k < 9; ++k) loc[9 + k] += cj * m[8 + k];
+      a0 += wp * c[j] * s;
+      if (slot == 0) {
+        a1 += wp * (chi_q * c[j] + zeta_q * d[j]) * s;
+        a2 += wp * sc[j] * s;
+      }
     }
-    rho[q] = 2.0 / dV * r;
-    loc[18] = r;
-    loc[19] = v[q] * r;   // |dOmega| V_q rho_q / 2
-    for (int k = 0; k < kNPart; ++k) acc[k] += loc[k];
+    // slots: 0 E_band, 1 E_s, 2 N, 3..8 K, 9..17 S, 18 rho (19: V rho, below)
+    double* r = red + grp * kNPart;
+    if (slot == 0) {
+      r[0] = a1;
+      r[1] = a2;
+      r[18] = a0;
+    } else if (slot == 7) {
+      r[2] = a0;
+    } else {
+      r[slot < 7 ? 2 + slot : slot + 1] = a0;
+    }
   }
-  for (int k = 0; k < kNPart; ++k) {
-    const double v = block_sum_d(acc[k], sh);
-    if (threadIdx.x == 0) part[blockIdx.x * kNPart + k] = v;
+  // rho per node: one warp per node
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double ev = 0.0;
+  for (int q = q0 + warp; q < q1; q += kContractThreads / 32) {
+    double r = 0.0;
+    for (int j = lane; j <= n_pl; j += 32)
+      r += (j == 0 ? 0.5 : 1.0) * c[j] * mom[((size_t)q * (n_pl + 1) + j) * SQ_N_MOMENTS];
+    r = warp_sum(r);
+    if (lane == 0) {
+      if (rho) rho[q] = 2.0 / dV * r;
+      ev += v[q] * r;   // |dOmega| V_q rho_q / 2
+    }
   }
+  if (lane == 0) red[kContractGroups * kNPart + warp] = ev;
+  __syncthreads();
+  if (threadIdx.x < kNPart) {
+    double t = 0.0;
+    if (threadIdx.x == kNPart - 1)
+      for (int w = 0; w < kContractThreads / 32; ++w) t += red[kContractGroups * kNPart + w];
+    else
+      for (int w = 0; w < kContractGroups; ++w) t += red[w * kNPart + threadIdx.x];
+    part[threadIdx.x] = t;
+  }
+}
+
+// block b: nodes [Nd b / nblk, Nd (b + 1) / nblk)
+__global__ void __launch_bounds__(kContractThreads)
+k_contract(const double* __restrict__ mom, const double* __restrict__ coef, const double* __restrict__ scal,
+           const double* __restrict__ v, int Nd, int n_pl, double dV, double* __restrict__ rho, double* __restrict__ part) {
+  __shared__ double red[kContractGroups * kNPart + kContractThreads / 32];
+  const double lam_lo = scal[0], lam_hi = scal[1];
+  const int q0 = int((long long)Nd * blockIdx.x / gridDim.x), q1 = int((long long)Nd * (blockIdx.x + 1) / gridDim.x);
+  contract_block(mom, coef, coef + (n_pl + 1), coef + 2 * (n_pl + 1), 0.5 * (lam_hi + lam_lo), 0.5 * (lam_hi - lam_lo),
+                 v, q0, q1, n_pl, dV, rho, red, part + (size_t)blockIdx.x * kNPart);
+}
+
+// rows of kNPart terms added up in a fixed order to gridDim.x rows (one warp per term)
+__global__ void __launch_bounds__(32 * kNPart) k_sum_rows(const double* __restrict__ rows, int n, double* __restrict__ out) {
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+  const int r0 = int((long long)n * blockIdx.x / gridDim.x), r1 = int((long long)n * (blockIdx.x + 1) / gridDim.x);
+  double s = 0.0;
+  for (int r = r0 + lane; r < r1; r += 32) s += rows[(size_t)r * kNPart + k];
+  s = warp_sum(s);
+  if (lane == 0) out[blockIdx.x * kNPart + k] = s;
 }
 
 // out (scal + 16): [E_band, E_s, E_nl, N_check, sigma(9, row-major), E_pot, P]
 // E_pot = |dOmega| sum_q V_q rho_q; P = the App. A pressure restricted to the kinetic and
 // nonlocal terms: -(1/(3|Omega|)) [-2 (E_band - E_pot) - E_nl - 4 sum_q sum' c^j tr S^j_q]
 // (the V_eff part of -4 tr(D H) goes with the exchange-correlation / electrostatic terms)
-__global__ void k_contract_final(const double* __restrict__ part, int nblk, double kT, double vol,
-                                 double* __restrict__ scal) {
+// One warp per term adds the nblk rows (one thread took 19-170 us, 2.2 ms for per-node rows).
+__global__ void __launch_bounds__(32 * kNPart) k_contract_final(const double* __restrict__ part, int nblk, double kT,
+                                                                double vol, double* __restrict__ scal) {
+  __shared__ double tot[kNPart];
+  {
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+    double s = 0.0;
+    for (int b = lane; b < nblk; b += 32) s += part[b * kNPart + k];
+    s = warp_sum(s);
+    if (lane == 0) tot[k] = s;
+  }
+  __syncthreads();
   if (threadIdx.x != 0) return;
-  double tot[kNPart];
-  for (int k = 0; k < kNPart; ++k) tot[k] = 0.0;
-  for (int b = 0; b < nblk; ++b)
-    for (int k = 0; k < kNPart; ++k) tot[k] += part[b * kNPart + k];
   double* out = scal + 16;
   out[0] = 2.0 * tot[0];
   out[1] = 2.0 * kT * tot[1];
@@ -141,13 +229,11 @@ __global__ void k_contract_final(const double* __restrict__ part, int nblk, doub
   out[14] = -(-2.0 * (out[0] - E_pot) - E_nl - 4.0 * (tot[9] + tot[13] + tot[17])) / (3.0 * vol);
 }
 
-__global__ void k_set_scalar(double* __restrict__ scal, int idx, double v) { scal[idx] = v; }
-
 // Bisection on the node sums already in d.R (the whole cell's, or the caller's allreduced ones)
 static int fermi_from_R(sq_handle* h, double* mu_out) {
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
-  k_cosF<<<(h->M + 255) / 256, 256, 0, s>>>(h->d.R, g.n_pl, h->M, h->d.cosF);
+  k_cosF<<<(h->M + 15) / 16, 128, 0, s>>>(h->d.R, g.n_pl, h->M, h->d.costab, h->d.cosF);
   SQ_LAUNCH_CHECK(h);
   k_bisect<<<1, 1024, 0, s>>>(h->d.cosF, h->M, h->kT, h->n_e, h->d.scal, h->d.status);
   SQ_LAUNCH_CHECK(h);
@@ -184,7 +270,23 @@ int run_fermi_sums(sq_handle* h, const double* R_host, double* mu_out) {
   return fermi_from_R(h, mu_out);
 }
 
-__global__ void k_copy_scalar(double* __restrict__ scal, int dst, int src) { scal[dst] = scal[src]; }
+// Coefficients and contraction at mu (from_scal: the Fermi level in scal[2]); outputs in scal[16 ..].
+static int contract_launches(sq_handle* h, double mu, int from_scal, double* rho_dev) {
+  const Geo& g = h->geo;
+  cudaStream_t s = h->stream;
+  k_fvals<<<(h->M + 63) / 64, 64, 0, s>>>(h->d.scal, mu, from_scal, h->kT, h->M, h->d.costab, h->d.fvals);
+  SQ_LAUNCH_CHECK(h);
+  k_coef<<<g.n_pl + 1, 128, 0, s>>>(h->d.fvals, g.n_pl, h->M, h->d.costab, h->d.coef);
+  SQ_LAUNCH_CHECK(h);
+  // four blocks per SM, at least two nodes each (d.part holds 4096 * 32 doubles)
+  const int nblk = std::max(1, std::min(4 * 152, (h->Nd + 1) / 2));
+  k_contract<<<nblk, kContractThreads, 0, s>>>(h->d.mom, h->d.coef, h->d.scal, h->d.v64, h->Nd, g.n_pl, g.dV, rho_dev,
+                                               h->d.part);
+  SQ_LAUNCH_CHECK(h);
+  k_contract_final<<<1, 32 * kNPart, 0, s>>>(h->d.part, nblk, h->kT, h->vol, h->d.scal);
+  SQ_LAUNCH_CHECK(h);
+  return SQ_OK;
+}
 
 // The Fermi level and the contraction with nothing crossing to the host (graph capture): mu
 // stays in scal[2] (NaN and the no-bracket status word when there is no sign change), the
@@ -194,34 +296,17 @@ int run_fermi_contraction_device(sq_handle* h) {
   cudaStream_t s = h->stream;
   k_rsum<<<g.n_pl + 1, 256, 0, s>>>(h->d.mom, h->Nd, g.n_pl, h->d.R);
   SQ_LAUNCH_CHECK(h);
-  k_cosF<<<(h->M + 255) / 256, 256, 0, s>>>(h->d.R, g.n_pl, h->M, h->d.cosF);
+  k_cosF<<<(h->M + 15) / 16, 128, 0, s>>>(h->d.R, g.n_pl, h->M, h->d.costab, h->d.cosF);
   SQ_LAUNCH_CHECK(h);
   k_bisect<<<1, 1024, 0, s>>>(h->d.cosF, h->M, h->kT, h->n_e, h->d.scal, h->d.status);
   SQ_LAUNCH_CHECK(h);
-  k_copy_scalar<<<1, 1, 0, s>>>(h->d.scal, 3, 2);
-  SQ_LAUNCH_CHECK(h);
-  k_coef<<<3, 256, sizeof(double) * h->M, s>>>(h->d.scal, h->kT, g.n_pl, h->M, h->d.coef);
-  SQ_LAUNCH_CHECK(h);
-  const int nblk = std::min(1024, (h->Nd + 255) / 256);
-  k_contract<<<nblk, 256, 0, s>>>(h->d.mom, h->d.coef, h->d.scal, h->d.v64, h->Nd, g.n_pl, g.dV, h->d.rho, h->d.part);
-  SQ_LAUNCH_CHECK(h);
-  k_contract_final<<<1, 32, 0, s>>>(h->d.part, nblk, h->kT, h->vol, h->d.scal);
-  SQ_LAUNCH_CHECK(h);
-  return SQ_OK;
+  return contract_launches(h, 0.0, 1, h->d.rho);
 }
 
 int run_contraction(sq_handle* h, double mu, double* rho_dev, double* out_host) {
-  const Geo& g = h->geo;
   cudaStream_t s = h->stream;
-  k_set_scalar<<<1, 1, 0, s>>>(h->d.scal, 3, mu);
-  SQ_LAUNCH_CHECK(h);
-  k_coef<<<3, 256, sizeof(double) * h->M, s>>>(h->d.scal, h->kT, g.n_pl, h->M, h->d.coef);
-  SQ_LAUNCH_CHECK(h);
-  const int nblk = std::min(1024, (h->Nd + 255) / 256);
-  k_contract<<<nblk, 256, 0, s>>>(h->d.mom, h->d.coef, h->d.scal, h->d.v64, h->Nd, g.n_pl, g.dV, rho_dev, h->d.part);
-  SQ_LAUNCH_CHECK(h);
-  k_contract_final<<<1, 32, 0, s>>>(h->d.part, nblk, h->kT, h->vol, h->d.scal);
-  SQ_LAUNCH_CHECK(h);
+  const int rc = contract_launches(h, mu, 0, rho_dev);
+  if (rc != SQ_OK) return rc;
   if (out_host) {
     SQ_CUDA_TRY(h, cudaMemcpyAsync(out_host, h->d.scal + 16, 15 * sizeof(double), cudaMemcpyDeviceToHost, s));
     SQ_CUDA_TRY(h, cudaStreamSynchronize(s));
@@ -320,69 +405,84 @@ int run_fermi_nodes(sq_handle* h, double* mu_out) {
   return SQ_OK;
 }
 
-// One block per node: its coefficients c, d, s at mu (M-point Chebyshev-Gauss rule, as k_coef)
-// and its contraction terms (the per-node rows of k_contract's partial sums), rho_q.
-__global__ void k_contract_nodes(const double* __restrict__ mom, const double* __restrict__ nbnd,
-                                 const double* __restrict__ v, int Nd, int n_pl, int M, const double* __restrict__ tab,
-                                 double kT, double mu, double dV, double* __restrict__ rho, double* __restrict__ rows) {
+// One block per node: its coefficients c, d, s at mu (M-point Chebyshev-Gauss rule, as k_coef) and
+// its contraction terms, rho_q. FP64 bound: M exponentials and logarithms, then the cosine sums.
+// cos(j theta_{M-1-k}) = (-1)^j cos(j theta_k) folds the sums to M / 2 points, and r cos(j theta) =
+// (cos((j-1) theta) + cos((j+1) theta)) / 2 gives d^j = (c^{|j-1|} + c^{j+1}) / 2 from c up to n_pl + 1, so a
+// coefficient pair costs M multiply-adds instead of 3 M.
+__global__ void __launch_bounds__(kContractThreads)
+k_contract_nodes(const double* __restrict__ mom, const double* __restrict__ nbnd, const double* __restrict__ v, int Nd,
+                 int n_pl, int M, const double* __restrict__ tab, double kT, double mu, double dV,
+                 double* __restrict__ rho, double* __restrict__ rows) {
   extern __shared__ double sm[];
-  double* fv = sm;                       // [3][M]
-  double* cf = sm + 3 * (size_t)M;       // [3][n_pl + 1]
+  __shared__ double red[kContractGroups * kNPart + kContractThreads / 32];
+  const int Mh = (M + 1) / 2;
+  double* fv = sm;                       // [2][2][Mh]: g, entropy; even and odd folds
+  double* cf = sm + 4 * (size_t)Mh;      // c [n_pl + 2], s [n_pl + 2], d [n_pl + 1]
   const int q = blockIdx.x;
   const double lo = nbnd[2 * q], hi = nbnd[2 * q + 1];
   const double chi_q = 0.5 * (hi + lo), zeta_q = 0.5 * (hi - lo);
-  for (int k = threadIdx.x; k < M; k += blockDim.x) {
-    const double r = tab[2 * k + 1];
-    const double x = (chi_q + zeta_q * r - mu) / kT;
-    const double gx = fermi_occ(x);
-    const double ax = fabs(x), ex = exp(-ax);
-    fv[k] = gx;
-    fv[M + k] = r * gx;
-    fv[2 * M + k] = -(log1p(ex) + ax * ex / (1.0 + ex));
+  for (int k = threadIdx.x; k < Mh; k += blockDim.x) {
+    const int k2 = M - 1 - k;
+    const double x1 = (chi_q + zeta_q * tab[2 * k + 1] - mu) / kT;
+    const double g1 = fermi_occ(x1), s1 = entropy_d(x1);
+    double g2 = 0.0, s2 = 0.0;
+    if (k2 != k) {
+      const double x2 = (chi_q + zeta_q * tab[2 * k2 + 1] - mu) / kT;
+      g2 = fermi_occ(x2);
+      s2 = entropy_d(x2);
+    }
+    fv[k] = g1 + g2;
+    fv[Mh + k] = g1 - g2;
+    fv[2 * Mh + k] = s1 + s2;
+    fv[3 * Mh + k] = s1 - s2;
   }
   __syncthreads();
-  const long long twoM4 = 4LL * M;
-  for (int t = threadIdx.x; t < 3 * (n_pl + 1); t += blockDim.x) {
-    const int which = t / (n_pl + 1), j = t % (n_pl + 1);
-    const double* f = fv + (size_t)which * M;
-    double acc = 0.0;
-    for (int k = 0; k < M; ++k) acc += f[k] * tab[((long long)j * (2 * k + 1)) % twoM4];
-    cf[t] = 2.0 / M * acc;
+  const int M4 = 4 * M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int j = warp; j <= n_pl + 1; j += kContractThreads / 32) {   // one warp per j
+    const double* fg = fv + (j & 1) * Mh;
+    const double* fs = fv + (2 + (j & 1)) * Mh;
+    double ac = 0.0, as = 0.0;
+    int t = int((long long)j * (2 * lane + 1) % M4);
+    const int step = int((long long)j * 64 % M4);
+    for (int k = lane; k < Mh; k += 32) {
+      const double cs = tab[t];
+      ac += fg[k] * cs;
+      as += fs[k] * cs;
+      t += step;
+      if (t >= M4) t -= M4;
+    }
+    ac = warp_sum(ac);
+    as = warp_sum(as);
+    if (lane == 0) {
+      cf[j] = 2.0 / M * ac;
+      cf[n_pl + 2 + j] = 2.0 / M * as;
+    }
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  const double* c = cf;
-  const double* d = cf + (n_pl + 1);
-  const double* sc = cf + 2 * (n_pl + 1);
-  double loc[kNPart];
-  for (int k = 0; k < kNPart; ++k) loc[k] = 0.0;
-  double r = 0.0;
-  for (int j = 0; j <= n_pl; ++j) {
-    const double wp = (j == 0) ? 0.5 : 1.0;
-    const double* m = mom + ((size_t)q * (n_pl + 1) + j) * SQ_N_MOMENTS;
-    const double cj = wp * c[j];
-    r += cj * m[0];
-    loc[0] += wp * (chi_q * c[j] + zeta_q * d[j]) * m[0];
-    loc[1] += wp * sc[j] * m[0];
-    loc[2] += cj * m[7];
-    for (int k = 0; k < 6; ++k) loc[3 + k] += cj * m[1 + k];
-    for (int k = 0; k < 9; ++k) loc[9 + k] += cj * m[8 + k];
-  }
-  if (rho) rho[q] = 2.0 / dV * r;
-  loc[18] = r;
-  loc[19] = v[q] * r;
-  for (int k = 0; k < kNPart; ++k) rows[(size_t)q * kNPart + k] = loc[k];
+  double* d = cf + 2 * (n_pl + 2);
+  for (int j = threadIdx.x; j <= n_pl; j += blockDim.x) d[j] = 0.5 * (cf[j == 0 ? 1 : j - 1] + cf[j + 1]);
+  __syncthreads();
+  contract_block(mom, cf, d, cf + n_pl + 2, chi_q, zeta_q, v, q, q + 1, n_pl, dV, rho, red, rows + (size_t)q * kNPart);
 }
 
 int run_contraction_nodes(sq_handle* h, double mu, double* rho_dev, double* out_host) {
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
-  const size_t smem = sizeof(double) * (3 * size_t(h->M) + 3 * size_t(g.n_pl + 1));
+  const size_t smem = sizeof(double) * (4 * size_t((h->M + 1) / 2) + 3 * size_t(g.n_pl + 2));
   SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_contract_nodes, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
   k_contract_nodes<<<h->Nd, 256, smem, s>>>(h->d.mom, h->d.nbnd, h->d.v64, h->Nd, g.n_pl, h->M, h->d.costab, h->kT,
                                             mu, g.dV, rho_dev, h->d.nrow);
   SQ_LAUNCH_CHECK(h);
-  k_contract_final<<<1, 32, 0, s>>>(h->d.nrow, h->Nd, h->kT, h->vol, h->d.scal);
+  const double* rows = h->d.nrow;
+  int n_rows = h->Nd;
+  if (n_rows > 2048) {   // two stages: one block over tens of thousands of rows is a serial chain
+    k_sum_rows<<<4 * 152, 32 * kNPart, 0, s>>>(rows, n_rows, h->d.part);
+    SQ_LAUNCH_CHECK(h);
+    rows = h->d.part;
+    n_rows = 4 * 152;
+  }
+  k_contract_final<<<1, 32 * kNPart, 0, s>>>(rows, n_rows, h->kT, h->vol, h->d.scal);
   SQ_LAUNCH_CHECK(h);
   if (out_host) {
     SQ_CUDA_TRY(h, cudaMemcpyAsync(out_host, h->d.scal + 16, 15 * sizeof(double), cudaMemcpyDeviceToHost, s));

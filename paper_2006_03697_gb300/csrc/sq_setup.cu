@@ -456,8 +456,10 @@ __global__ void k_node_init(int Nd, double* __restrict__ nbnd, double* __restric
 int init_node_tables(sq_handle* h) {
   k_costab<<<(4 * h->M + 255) / 256, 256, 0, h->stream>>>(h->M, h->d.costab);
   SQ_LAUNCH_CHECK(h);
-  k_node_init<<<(h->Nd + 255) / 256, 256, 0, h->stream>>>(h->Nd, h->d.nbnd, h->d.ncoef);
-  SQ_LAUNCH_CHECK(h);
+  if (h->bounds_mode == SQ_BOUNDS_PER_NODE) {
+    k_node_init<<<(h->Nd + 255) / 256, 256, 0, h->stream>>>(h->Nd, h->d.nbnd, h->d.ncoef);
+    SQ_LAUNCH_CHECK(h);
+  }
   return SQ_OK;
 }
 
