@@ -1,6 +1,8 @@
 // Device-side helpers shared by the SQ kernels.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "sq_internal.h"
 
 namespace sq {
@@ -122,36 +124,116 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
   return r;
 }
 
+// Root finder of the Fermi level: keeps a bracket N(lo) < N_e <= N(hi) and ends when it is
+// < 1e-13 max(1, |mu|) wide or after 200 evaluations, mu = the final midpoint (the bisection rule of
+// the API). ln N is concave where the electrons are dilute, so Newton steps on ln N approach the
+// root in a few evaluations (plain bisection took 52, each M exponentials); a step that leaves
+// the bracket, a non-positive N or slope, or 64 evaluations without an end fall back to the midpoint.
+// Once a step is below 2 % of the tolerance the next point is taken just across the root (27 ulp of
+// mu), which closes the bracket.
+struct FermiRoot {
+  double lo, hi, n_e, mu;
+  int it;
+  __host__ __device__ void init(double a, double b, double ne) {
+    lo = a;
+    hi = b;
+    n_e = ne;
+    mu = 0.5 * (a + b);
+    it = 0;
+  }
+  // n, dn: N and dN/dmu at mu; true when done (mu is then the result)
+  __host__ __device__ bool update(double n, double dn) {
+    ++it;
+    const bool below = n < n_e;
+    if (below) lo = mu;
+    else hi = mu;
+    const double am = fabs(mu), tol = 1e-13 * (am > 1.0 ? am : 1.0);
+    if (hi - lo < tol || it >= 200) {
+      mu = 0.5 * (lo + hi);
+      return true;
+    }
+    double next = lo;   // outside the open bracket: midpoint
+    if (it < 64 && n > 0.0 && dn > 0.0) {
+      next = mu + log(n_e / n) * n / dn;
+      if (fabs(next - mu) < 0.02 * tol) next = below ? mu + 0.06 * tol : mu - 0.06 * tol;
+    }
+    mu = (next > lo && next < hi) ? next : 0.5 * (lo + hi);
+    return false;
+  }
+};
+
 // N(mu) = 2 sum'_j c^j(mu) R^j = (4/M) sum_k g((chi + zeta cos theta_k - mu) / kT) F_k with
 // F_k = sum'_j cos(j theta_k) R^j, theta_k = pi (k + 1/2) / M (the M-point Chebyshev-Gauss rule
-// for the coefficient integral of Sec. 4). Whole block; same value in every thread.
-__device__ __forceinline__ double electron_count_F(const double* F, int M, double chi_q, double zeta_q, double kT,
-                                                  double mu, double* sh) {
-  double s = 0.0;
-  for (int k = threadIdx.x; k < M; k += blockDim.x)
-    s += fermi_occ((chi_q + zeta_q * cos(M_PI * (k + 0.5) / M) - mu) / kT) * F[k];
-  return 4.0 / M * block_sum_d(s, sh);
-}
+// for the coefficient integral of Sec. 4), and its root N(mu) = N_e on
+// [lam_lo - 40 kT, lam_hi + 40 kT]. One cluster of kFermiCluster blocks: M FP64 exponentials per
+// evaluation are bound by the 1.7 FP64 lanes per clock of an SM (one block: 43 us at M = 2048), so the
+// points are spread over 8 SMs and the blocks' sums meet in distributed shared memory, two barriers'
+// worth of slots so that one cluster barrier per evaluation suffices. Every thread adds the same
+// numbers in the same order, so all blocks take the same steps. Returns false (and leaves *mu alone)
+// when N(mu) - N_e has no sign change on the bracket.
+constexpr int kFermiCluster = 8, kFermiThreads = 256;
 
-// The Fermi-level rule of the library: bisection on N(mu) = N_e over
-// [lam_lo - 40 kT, lam_hi + 40 kT] until the bracket is < 1e-13 max(1, |mu|) or 200 steps, mu =
-// the final midpoint. Returns false (and leaves *mu alone) when N(mu) - N_e has no sign change
-// on the bracket. Whole block (sh: blockDim.x doubles); every thread gets the same result.
-__device__ __forceinline__ bool fermi_bisect_rule(const double* F, int M, double lam_lo, double lam_hi, double kT,
-                                                  double n_e, double* sh, double* mu) {
+__device__ __forceinline__ bool fermi_cluster_search(const double* __restrict__ F, int M, double lam_lo, double lam_hi,
+                                                    double kT, double n_e, double* mu) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cl = cg::this_cluster();
+  const int rank = int(cl.block_rank());
   const double chi_q = 0.5 * (lam_hi + lam_lo), zeta_q = 0.5 * (lam_hi - lam_lo);
-  double lo = lam_lo - 40.0 * kT, hi = lam_hi + 40.0 * kT;
-  const double nlo = electron_count_F(F, M, chi_q, zeta_q, kT, lo, sh);
-  const double nhi = electron_count_F(F, M, chi_q, zeta_q, kT, hi, sh);
-  if (!(nlo < n_e && n_e < nhi)) return false;
-  for (int it = 0; it < 200; ++it) {
-    const double mid = 0.5 * (lo + hi);
-    if (electron_count_F(F, M, chi_q, zeta_q, kT, mid, sh) < n_e) lo = mid;
-    else hi = mid;
-    if (hi - lo < 1e-13 * fmax(1.0, fabs(mid))) break;
+  constexpr int kWarps = kFermiThreads / 32;
+  constexpr int kPts = SQ_NOALLOC_MAX_M / (kFermiCluster * kFermiThreads);   // most points per thread
+  __shared__ double sums[2][2][kWarps];   // [slot][N, dN][warp]
+  double lam[kPts], f[kPts];
+  int np = 0;
+#pragma unroll
+  for (int i = 0; i < kPts; ++i) {
+    const int k = (i * kFermiCluster + rank) * kFermiThreads + threadIdx.x;
+    lam[i] = f[i] = 0.0;
+    if (k < M) {
+      lam[i] = chi_q + zeta_q * cospi((k + 0.5) / M);
+      f[i] = F[k];
+      np = i + 1;
+    }
   }
-  *mu = 0.5 * (lo + hi);
-  return true;
+  int slot = 0;
+  auto count = [&](double x, double& n, double& dn) {
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int i = 0; i < kPts; ++i)
+      if (i < np) {
+        const double g = fermi_occ((lam[i] - x) / kT), gf = g * f[i];
+        s0 += gf;
+        s1 += gf * (1.0 - g);
+      }
+    s0 = warp_sum(s0);
+    s1 = warp_sum(s1);
+    if ((threadIdx.x & 31) == 0) {
+      sums[slot][0][threadIdx.x >> 5] = s0;
+      sums[slot][1][threadIdx.x >> 5] = s1;
+    }
+    cl.sync();
+    n = dn = 0.0;
+    const int lane = threadIdx.x & 31;   // lanes: 8 blocks x 4 warps each, then the other 4 warps
+    static_assert(kFermiCluster == 8 && kWarps == 8, "one lane per block and half of its warps");
+    const double* r = cl.map_shared_rank(&sums[slot][0][0], lane >> 2);
+    const int w = lane & 3;
+    n = 4.0 / M * warp_sum(r[w] + r[w + 4]);
+    dn = 4.0 / M / kT * warp_sum(r[kWarps + w] + r[kWarps + w + 4]);
+    slot ^= 1;
+  };
+  const double lo = lam_lo - 40.0 * kT, hi = lam_hi + 40.0 * kT;
+  double n0, n1, dn;
+  count(lo, n0, dn);
+  count(hi, n1, dn);
+  bool ok = n0 < n_e && n_e < n1;
+  if (ok) {
+    FermiRoot r;
+    r.init(lo, hi, n_e);
+    do count(r.mu, n0, dn);
+    while (!r.update(n0, dn));
+    *mu = r.mu;
+  }
+  cl.sync();   // no block leaves while another still reads its sums
+  return ok;
 }
 
 }  // namespace sq

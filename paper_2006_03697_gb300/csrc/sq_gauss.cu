@@ -5,7 +5,7 @@
 // implicit QL with Wilkinson shifts, rotating only the first row of the eigenvector matrix);
 // then [f(H_q)]_qq ~ sum_i w_qi f(theta_qi), exact for polynomials of degree <= 2k - 1.
 // rho_q = (2 / |dOmega|) sum_i w_qi g(theta_qi), the Fermi level solves
-// 2 sum_q sum_i w_qi g(theta_qi) = N_e (bisection, the rule of the Clenshaw-Curtis path) and
+// 2 sum_q sum_i w_qi g(theta_qi) = N_e (the root search of the Clenshaw-Curtis path) and
 // E_band = 2 sum_q sum_i w_qi theta_qi g(theta_qi).
 #include <algorithm>
 #include <cmath>
@@ -89,23 +89,26 @@ __global__ void k_gauss_eig(int ncols, int k, const double* __restrict__ alpha, 
   }
 }
 
-// part[block] = sum over the block's columns of 2 sum_i w g((theta - mu) / kT) (fixed order)
-__global__ void k_gauss_count(int ncols, int k, const double* __restrict__ theta, const double* __restrict__ wgt,
-                              double mu, double kT, double* __restrict__ part) {
+// part[2 block], part[2 block + 1] = the block's share of N(mu) = 2 sum w g((theta - mu) / kT) and of
+// dN/dmu, over all (column, node) pairs (a thread per column walked its k nodes with a stride: 90 us)
+__global__ void __launch_bounds__(256) k_gauss_count(long long n, const double* __restrict__ theta,
+                                                     const double* __restrict__ wgt, double mu, double kT,
+                                                     double* __restrict__ part) {
   __shared__ double sh[256];
-  double acc = 0.0;
-  for (int col = blockIdx.x * blockDim.x + threadIdx.x; col < ncols; col += gridDim.x * blockDim.x)
-    for (int i = 0; i < k; ++i) {
-      const double w = wgt[(size_t)col * k + i];
-      if (w != 0.0) acc += 2.0 * w * fermi_occ((theta[(size_t)col * k + i] - mu) / kT);
-    }
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
+  double a0 = 0.0, a1 = 0.0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double w = wgt[i];
+    if (w == 0.0) continue;
+    const double g = fermi_occ((theta[i] - mu) / kT);
+    a0 += 2.0 * w * g;
+    a1 += 2.0 * w * g * (1.0 - g);
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+  a0 = block_sum_d(a0, sh);
+  a1 = block_sum_d(a1, sh);
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = a0;
+    part[2 * blockIdx.x + 1] = a1 / kT;
+  }
 }
 
 // Smallest and largest Gauss node with a non-zero weight: per block, then (k_gauss_minmax_final)
@@ -146,12 +149,15 @@ __global__ void k_gauss_minmax_final(const double* __restrict__ part, int nblk, 
   out[1] = hi;
 }
 
-// out[0] = sum of part[0..n) in order (one thread)
-__global__ void k_gauss_sum(const double* __restrict__ part, int n, double* __restrict__ out) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  double t = 0.0;
-  for (int i = 0; i < n; ++i) t += part[i];
-  out[0] = t;
+// out[c] = sum over i of part[i * nc + c], c < nc, fixed order (one block of 256)
+__global__ void __launch_bounds__(256) k_gauss_sum(const double* __restrict__ part, int n, int nc, double* __restrict__ out) {
+  __shared__ double sh[256];
+  for (int c = 0; c < nc; ++c) {
+    double t = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) t += part[i * nc + c];
+    t = block_sum_d(t, sh);
+    if (threadIdx.x == 0) out[c] = t;
+  }
 }
 
 // rho at every valid node and the band-energy partial sums per block
@@ -249,7 +255,7 @@ static int gauss_t(sq_handle* h, int k, double* mu_out, double* rho_host, double
                                                 wgt + (size_t)t0 * g.B * k, h->d.status);
     if (cudaGetLastError() != cudaSuccess) rc = fail(h, SQ_ERR_CUDA, "k_gauss_eig launch failed");
   }
-  // Fermi level: bisection with the Clenshaw-Curtis path's rule; the bracket from the extreme
+  // Fermi level: the Clenshaw-Curtis path's root finder; the bracket from the extreme
   // weighted Gauss nodes (device reduction, two doubles to the host)
   double tmin = 0.0, tmax = 0.0;
   if (rc == SQ_OK) {
@@ -268,39 +274,38 @@ static int gauss_t(sq_handle* h, int k, double* mu_out, double* rho_host, double
       tmax = ext[1];
     }
   }
+  const int cblk = nblk / 2;   // part holds nblk doubles: a pair per block
   auto count = [&](double mu, double* out) -> int {
-    k_gauss_count<<<nblk, 256, 0, s>>>(ncols_all, k, theta, wgt, mu, h->kT, part);
-    k_gauss_sum<<<1, 32, 0, s>>>(part, nblk, sum);
+    k_gauss_count<<<cblk, 256, 0, s>>>((long long)ncols_all * k, theta, wgt, mu, h->kT, part);
+    k_gauss_sum<<<1, 256, 0, s>>>(part, cblk, 2, sum);
     if (cudaGetLastError() != cudaSuccess) return SQ_ERR_CUDA;
-    if (cudaMemcpyAsync(out, sum, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SQ_ERR_CUDA;
+    if (cudaMemcpyAsync(out, sum, 2 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SQ_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return SQ_ERR_CUDA;
     return SQ_OK;
   };
   double mu = 0.0;
   if (rc == SQ_OK) {
-    double lo = tmin - 40.0 * h->kT, hi = tmax + 40.0 * h->kT, nlo = 0.0, nhi = 0.0;
-    if (count(lo, &nlo) != SQ_OK || count(hi, &nhi) != SQ_OK) {
+    const double lo = tmin - 40.0 * h->kT, hi = tmax + 40.0 * h->kT;
+    double nlo[2], nhi[2], nm[2];
+    if (count(lo, nlo) != SQ_OK || count(hi, nhi) != SQ_OK) {
       rc = fail(h, SQ_ERR_CUDA, "electron count failed");
-    } else if (!(nlo < h->n_e && h->n_e < nhi)) {
+    } else if (!(nlo[0] < h->n_e && h->n_e < nhi[0])) {
       rc = fail(h, SQ_ERR_NO_BRACKET, "N(mu) - N_e has no sign change on the bisection bracket");
     } else {
-      for (int it = 0; it < 200; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        double nm = 0.0;
-        if (count(mid, &nm) != SQ_OK) {
+      FermiRoot r;
+      r.init(lo, hi, h->n_e);
+      do {
+        if (count(r.mu, nm) != SQ_OK) {
           rc = fail(h, SQ_ERR_CUDA, "electron count failed");
           break;
         }
-        if (nm < h->n_e) lo = mid;
-        else hi = mid;
-        if (hi - lo < 1e-13 * std::max(1.0, std::fabs(mid))) break;
-      }
-      mu = 0.5 * (lo + hi);
+      } while (!r.update(nm[0], nm[1]));
+      mu = r.mu;
     }
   }
   if (rc == SQ_OK) {
     k_gauss_rho<<<nblk, 256, 0, s>>>(g, g.n_tiles, k, theta, wgt, mu, h->kT, rho, part);
-    k_gauss_sum<<<1, 32, 0, s>>>(part, nblk, sum);
+    k_gauss_sum<<<1, 256, 0, s>>>(part, nblk, 1, sum);
     double eb = 0.0;
     int st[kStCount];
     if (cudaGetLastError() != cudaSuccess ||

@@ -29,15 +29,15 @@ namespace {
 std::mutex g_mu;
 double* g_scratch_ptr[256] = {nullptr};   // last looked-up device address of the scratch, per device ordinal
 
-// The library's bisection rule (fermi_bisect_rule, shared with sq_fermi_level), with the
-// bounds passed by value and mu written to the caller's device pointer (NaN when
-// N(mu) - N_e has no sign change on the bracket).
-__global__ void k_bisect_noalloc(const double* __restrict__ F, int M, double lam_lo, double lam_hi, double kT,
-                                 double n_e, double* __restrict__ mu_out) {
-  __shared__ double sh[1024];
+// The library's Fermi search (fermi_cluster_search, shared with sq_fermi_level), with the bounds
+// passed by value and mu written to the caller's device pointer (NaN when N(mu) - N_e has no
+// sign change on the bracket).
+__global__ void __cluster_dims__(kFermiCluster, 1, 1) __launch_bounds__(kFermiThreads)
+k_fermi_noalloc(const double* __restrict__ F, int M, double lam_lo, double lam_hi, double kT, double n_e,
+                double* __restrict__ mu_out) {
   double mu = 0.0;
-  const bool ok = fermi_bisect_rule(F, M, lam_lo, lam_hi, kT, n_e, sh, &mu);
-  if (threadIdx.x == 0) *mu_out = ok ? mu : NAN;
+  const bool ok = fermi_cluster_search(F, M, lam_lo, lam_hi, kT, n_e, &mu);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *mu_out = ok ? mu : NAN;
 }
 
 }  // namespace
@@ -82,6 +82,6 @@ extern "C" int sq_fermi_level_noalloc(const double* mom_dev, int n_nodes, int n_
   double* F = scratch + SQ_NOALLOC_MAX_NPL + 1;   // [M]
   sq::k_rsum<<<n_pl + 1, 256, 0, s>>>(mom_dev, n_nodes, n_pl, R);
   sq::k_cosF<<<(M + 15) / 16, 128, 0, s>>>(R, n_pl, M, nullptr, F);
-  sq::k_bisect_noalloc<<<1, 1024, 0, s>>>(F, M, lambda_lo, lambda_hi, kT, n_e, mu_dev);
+  sq::k_fermi_noalloc<<<sq::kFermiCluster, sq::kFermiThreads, 0, s>>>(F, M, lambda_lo, lambda_hi, kT, n_e, mu_dev);
   return cudaGetLastError() == cudaSuccess ? SQ_OK : SQ_ERR_CUDA;
 }

@@ -4,7 +4,7 @@
 //   F_k      = sum'_j cos(j theta_k) R^j,  theta_k = pi (k + 1/2) / M
 //   N(mu)    = 2 sum'_j c^j(mu) R^j = (4/M) sum_k g((chi + zeta cos theta_k - mu)/kT) F_k
 // because c^j = (2/M) sum_k g(cos theta_k) cos(j theta_k) is the M-point Chebyshev-Gauss
-// rule for the Clenshaw-Curtis coefficient integral of Sec. 4; bisection on N(mu) = N_e.
+// rule for the Clenshaw-Curtis coefficient integral of Sec. 4; safeguarded root of N(mu) = N_e.
 // The contraction evaluates c^j, d^j (coefficients of r g(r), App. A) and s^j (entropy
 // function) at mu and forms rho_q, E_band, E_s, E_nl and sigma (Sec. 4 stress sums).
 #include <algorithm>
@@ -47,13 +47,12 @@ __global__ void __launch_bounds__(128) k_cosF(const double* __restrict__ R, int 
   if (k < M && sub == 0) F[k] = s;
 }
 
-// Single block. scal[0], scal[1]: bounds; writes scal[2] = mu, status[kStNoBracket].
-__global__ void k_bisect(const double* __restrict__ F, int M, double kT, double n_e, double* __restrict__ scal,
-                         int* __restrict__ status) {
-  __shared__ double sh[1024];
+// scal[0], scal[1]: bounds; writes scal[2] = mu, status[kStNoBracket].
+__global__ void __cluster_dims__(kFermiCluster, 1, 1) __launch_bounds__(kFermiThreads)
+k_fermi(const double* __restrict__ F, int M, double kT, double n_e, double* __restrict__ scal, int* __restrict__ status) {
   double mu = 0.0;
-  const bool ok = fermi_bisect_rule(F, M, scal[0], scal[1], kT, n_e, sh, &mu);
-  if (threadIdx.x == 0) {
+  const bool ok = fermi_cluster_search(F, M, scal[0], scal[1], kT, n_e, &mu);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     scal[2] = ok ? mu : NAN;
     status[kStNoBracket] = ok ? 0 : 1;
   }
@@ -229,13 +228,13 @@ __global__ void __launch_bounds__(32 * kNPart) k_contract_final(const double* __
   out[14] = -(-2.0 * (out[0] - E_pot) - E_nl - 4.0 * (tot[9] + tot[13] + tot[17])) / (3.0 * vol);
 }
 
-// Bisection on the node sums already in d.R (the whole cell's, or the caller's allreduced ones)
+// Fermi search on the node sums already in d.R (the whole cell's, or the caller's allreduced ones)
 static int fermi_from_R(sq_handle* h, double* mu_out) {
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
   k_cosF<<<(h->M + 15) / 16, 128, 0, s>>>(h->d.R, g.n_pl, h->M, h->d.costab, h->d.cosF);
   SQ_LAUNCH_CHECK(h);
-  k_bisect<<<1, 1024, 0, s>>>(h->d.cosF, h->M, h->kT, h->n_e, h->d.scal, h->d.status);
+  k_fermi<<<kFermiCluster, kFermiThreads, 0, s>>>(h->d.cosF, h->M, h->kT, h->n_e, h->d.scal, h->d.status);
   SQ_LAUNCH_CHECK(h);
   double mu = 0.0;
   int st[kStCount];
@@ -298,7 +297,7 @@ int run_fermi_contraction_device(sq_handle* h) {
   SQ_LAUNCH_CHECK(h);
   k_cosF<<<(h->M + 15) / 16, 128, 0, s>>>(h->d.R, g.n_pl, h->M, h->d.costab, h->d.cosF);
   SQ_LAUNCH_CHECK(h);
-  k_bisect<<<1, 1024, 0, s>>>(h->d.cosF, h->M, h->kT, h->n_e, h->d.scal, h->d.status);
+  k_fermi<<<kFermiCluster, kFermiThreads, 0, s>>>(h->d.cosF, h->M, h->kT, h->n_e, h->d.scal, h->d.status);
   SQ_LAUNCH_CHECK(h);
   return contract_launches(h, 0.0, 1, h->d.rho);
 }
@@ -322,86 +321,124 @@ int run_contraction(sq_handle* h, double mu, double* rho_dev, double* out_host) 
 //   F_q(k) = sum'_j cos(j theta_k) rho_q^j      (one table of N_d x M, formed once per search).
 // tab[t] = cos(pi t / (2 M)), so cos(j theta_k) = tab[j (2 k + 1) mod 4 M].
 
-__global__ void k_cosF_nodes(const double* __restrict__ mom, int Nd, int n_pl, int M, const double* __restrict__ tab,
-                             double* __restrict__ F) {
+// F_q(k) for k and M - 1 - k together: cos(j theta_{M-1-k}) = (-1)^j cos(j theta_k), so the even and the odd
+// part are summed once (half the FP64 multiply-adds).
+__global__ void __launch_bounds__(256) k_cosF_nodes(const double* __restrict__ mom, int Nd, int n_pl, int M,
+                                                    const double* __restrict__ tab, double* __restrict__ F) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
-  if (k >= M || q >= Nd) return;
+  if (k >= (M + 1) / 2 || q >= Nd) return;
   const double* m = mom + (size_t)q * (n_pl + 1) * SQ_N_MOMENTS;
-  const long long twoM4 = 4LL * M, odd = 2LL * k + 1;
-  double s = 0.5 * m[0];
-  for (int j = 1; j <= n_pl; ++j) s += tab[(j * odd) % twoM4] * m[(size_t)j * SQ_N_MOMENTS];
-  F[(size_t)q * M + k] = s;
+  const int M4 = 4 * M, odd = 2 * k + 1;
+  double s[2] = {0.5 * m[0], 0.0};
+  int t = 0;
+  for (int j = 1; j <= n_pl; j += 2) {
+    t += odd;
+    if (t >= M4) t -= M4;
+    s[1] += tab[t] * m[(size_t)j * SQ_N_MOMENTS];
+    if (j == n_pl) break;
+    t += odd;
+    if (t >= M4) t -= M4;
+    s[0] += tab[t] * m[(size_t)(j + 1) * SQ_N_MOMENTS];
+  }
+  F[(size_t)q * M + k] = s[0] + s[1];
+  F[(size_t)q * M + M - 1 - k] = s[0] - s[1];   // k = M - 1 - k: the odd part is zero there
 }
 
-// part[block] = (4/M) sum over the block's nodes and all k of g((chi_q + zeta_q cos theta_k - mu)/kT) F_q(k)
-__global__ void k_count_nodes(const double* __restrict__ F, const double* __restrict__ nbnd, int Nd, int M,
-                              const double* __restrict__ tab, double kT, double mu, double* __restrict__ part) {
+// part[2 block], part[2 block + 1] = N and dN/dmu of the block's nodes:
+// (4/M) sum_q sum_k g((chi_q + zeta_q cos theta_k - mu)/kT) F_q(k), and g (1 - g) / kT in place of g
+__global__ void __launch_bounds__(256) k_count_nodes(const double* __restrict__ F, const double* __restrict__ nbnd, int Nd,
+                                                     int M, const double* __restrict__ tab, double kT, double mu,
+                                                     double* __restrict__ part) {
   __shared__ double sh[256];
-  double acc = 0.0;
+  double a0 = 0.0, a1 = 0.0;
   for (int q = blockIdx.x; q < Nd; q += gridDim.x) {
     const double lo = nbnd[2 * q], hi = nbnd[2 * q + 1];
     const double chi_q = 0.5 * (hi + lo), zeta_q = 0.5 * (hi - lo);
     const double* Fq = F + (size_t)q * M;
-    for (int k = threadIdx.x; k < M; k += blockDim.x)
-      acc += fermi_occ((chi_q + zeta_q * tab[2 * k + 1] - mu) / kT) * Fq[k];
-  }
-  const double t = block_sum_d(acc, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = 4.0 / M * t;
-}
-
-// out[0] = sum of part[0..n) in order; with ext: out[1] = min lo_q, out[2] = max hi_q
-__global__ void k_sum_parts(const double* __restrict__ part, int n, const double* __restrict__ nbnd, int Nd,
-                            double* __restrict__ out) {
-  if (threadIdx.x != 0) return;
-  double t = 0.0;
-  for (int i = 0; i < n; ++i) t += part[i];
-  out[0] = t;
-  if (nbnd) {
-    double lo = INFINITY, hi = -INFINITY;
-    for (int q = 0; q < Nd; ++q) {
-      lo = fmin(lo, nbnd[2 * q]);
-      hi = fmax(hi, nbnd[2 * q + 1]);
+    for (int k = threadIdx.x; k < M; k += blockDim.x) {
+      const double g = fermi_occ((chi_q + zeta_q * tab[2 * k + 1] - mu) / kT), gf = g * Fq[k];
+      a0 += gf;
+      a1 += gf * (1.0 - g);
     }
-    out[1] = lo;
-    out[2] = hi;
+  }
+  a0 = block_sum_d(a0, sh);
+  a1 = block_sum_d(a1, sh);
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = 4.0 / M * a0;
+    part[2 * blockIdx.x + 1] = 4.0 / M / kT * a1;
   }
 }
 
-constexpr int kCountBlocks = 1024;
+// out[0], out[1] = sums of the (N, dN/dmu) pairs, fixed order; with nbnd: out[2] = min lo_q,
+// out[3] = max hi_q. One block of 256.
+__global__ void __launch_bounds__(256) k_sum_parts(const double* __restrict__ part, int n, const double* __restrict__ nbnd,
+                                                   int Nd, double* __restrict__ out) {
+  __shared__ double sh[256], slo[256], shi[256];
+  double a0 = 0.0, a1 = 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    a0 += part[2 * i];
+    a1 += part[2 * i + 1];
+  }
+  a0 = block_sum_d(a0, sh);
+  a1 = block_sum_d(a1, sh);
+  if (threadIdx.x == 0) {
+    out[0] = a0;
+    out[1] = a1;
+  }
+  if (!nbnd) return;
+  double lo = INFINITY, hi = -INFINITY;
+  for (int q = threadIdx.x; q < Nd; q += blockDim.x) {
+    lo = fmin(lo, nbnd[2 * q]);
+    hi = fmax(hi, nbnd[2 * q + 1]);
+  }
+  slo[threadIdx.x] = lo;
+  shi[threadIdx.x] = hi;
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if (threadIdx.x < w) {
+      slo[threadIdx.x] = fmin(slo[threadIdx.x], slo[threadIdx.x + w]);
+      shi[threadIdx.x] = fmax(shi[threadIdx.x], shi[threadIdx.x + w]);
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    out[2] = slo[0];
+    out[3] = shi[0];
+  }
+}
+
+constexpr int kCountBlocks = 512;   // d.npart holds 1024 doubles: a pair per block
 
 int run_fermi_nodes(sq_handle* h, double* mu_out) {
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
   const int M = h->M;
-  k_cosF_nodes<<<dim3((M + 255) / 256, h->Nd), 256, 0, s>>>(h->d.mom, h->Nd, g.n_pl, M, h->d.costab, h->d.nF);
+  k_cosF_nodes<<<dim3(((M + 1) / 2 + 255) / 256, h->Nd), 256, 0, s>>>(h->d.mom, h->Nd, g.n_pl, M, h->d.costab, h->d.nF);
   SQ_LAUNCH_CHECK(h);
-  double* out = h->d.scal + 40;   // [count, min lo, max hi]
+  double* out = h->d.scal + 40;   // [N, dN/dmu, min lo, max hi]
   auto count = [&](double mu, double* res, bool ext) -> int {
     k_count_nodes<<<kCountBlocks, 256, 0, s>>>(h->d.nF, h->d.nbnd, h->Nd, M, h->d.costab, h->kT, mu, h->d.npart);
     SQ_LAUNCH_CHECK(h);
-    k_sum_parts<<<1, 32, 0, s>>>(h->d.npart, kCountBlocks, ext ? h->d.nbnd : nullptr, h->Nd, out);
+    k_sum_parts<<<1, 256, 0, s>>>(h->d.npart, kCountBlocks, ext ? h->d.nbnd : nullptr, h->Nd, out);
     SQ_LAUNCH_CHECK(h);
-    SQ_CUDA_TRY(h, cudaMemcpyAsync(res, out, (ext ? 3 : 1) * sizeof(double), cudaMemcpyDeviceToHost, s));
+    SQ_CUDA_TRY(h, cudaMemcpyAsync(res, out, (ext ? 4 : 2) * sizeof(double), cudaMemcpyDeviceToHost, s));
     SQ_CUDA_TRY(h, cudaStreamSynchronize(s));
     return SQ_OK;
   };
   // the shared mode's rule on [min lo_q - 40 kT, max hi_q + 40 kT]
-  double e[3];
+  double e[4], nlo[2], nhi[2];
   int rc = count(0.0, e, true);
   if (rc != SQ_OK) return rc;
-  double lo = e[1] - 40.0 * h->kT, hi = e[2] + 40.0 * h->kT, nlo = 0.0, nhi = 0.0;
-  if ((rc = count(lo, &nlo, false)) != SQ_OK || (rc = count(hi, &nhi, false)) != SQ_OK) return rc;
-  if (!(nlo < h->n_e && h->n_e < nhi))
+  const double lo = e[2] - 40.0 * h->kT, hi = e[3] + 40.0 * h->kT;
+  if ((rc = count(lo, nlo, false)) != SQ_OK || (rc = count(hi, nhi, false)) != SQ_OK) return rc;
+  if (!(nlo[0] < h->n_e && h->n_e < nhi[0]))
     return fail(h, SQ_ERR_NO_BRACKET, "N(mu) - N_e has no sign change on the bisection bracket");
-  for (int it = 0; it < 200; ++it) {
-    const double mid = 0.5 * (lo + hi);
-    double nm = 0.0;
-    if ((rc = count(mid, &nm, false)) != SQ_OK) return rc;
-    if (nm < h->n_e) lo = mid;
-    else hi = mid;
-    if (hi - lo < 1e-13 * std::max(1.0, std::fabs(mid))) break;
-  }
-  if (mu_out) *mu_out = 0.5 * (lo + hi);
+  FermiRoot r;
+  r.init(lo, hi, h->n_e);
+  do {
+    if ((rc = count(r.mu, e, false)) != SQ_OK) return rc;
+  } while (!r.update(e[0], e[1]));
+  if (mu_out) *mu_out = r.mu;
   return SQ_OK;
 }
 
