@@ -205,76 +205,144 @@ __global__ void k_lz_mark_empty(int ncols, const double* __restrict__ nrm, int l
   if (col < ncols) keff[col] = (nrm[(size_t)col * ld] > 0.0) ? -1 : 0;
 }
 
-// Sturm count of eigenvalues of the tridiagonal (a, b) below x.
-__device__ int sturm_count(const double* a, const double* b, int n, double x) {
+constexpr int kMaxLanczos = 128;
+constexpr int kRitzWarps = 4;   // columns per block of the Ritz kernels
+
+struct RitzBuf {
+  double a[kMaxLanczos], b[kMaxLanczos], b2[kMaxLanczos];
+  double y[2][kMaxLanczos], inv[2][kMaxLanczos];
+};
+
+// Number of eigenvalues of the tridiagonal (a, b) below x: the sign changes of the Sturm polynomials
+// p_i = (a_i - x) p_{i-1} - b_{i-1}^2 p_{i-2}, rescaled by powers of two (three FP64 instructions a step;
+// the ratio form needs a division, about 20).
+__device__ __forceinline__ int sturm_count(const RitzBuf& r, int n, double x) {
   int cnt = 0;
-  double d = 1.0;
-  for (int i = 0; i < n; ++i) {
-    d = a[i] - x - (i > 0 ? b[i - 1] * b[i - 1] / d : 0.0);
-    if (d == 0.0) d = -1e-300;
-    if (d < 0.0) ++cnt;
+  double p0 = 1.0, p1 = r.a[0] - x;
+  if (p1 == 0.0) p1 = -1e-300;
+  bool neg = p1 < 0.0;   // sign of p_i relative to p_{i-1}: a change is an eigenvalue below x
+  cnt += neg;
+  for (int i = 1; i < n; ++i) {
+    double p2 = (r.a[i] - x) * p1 - r.b2[i - 1] * p0;
+    if (p2 == 0.0) p2 = (p1 > 0.0) ? -1e-300 : 1e-300;   // a zero counts as a change, as in the ratio form
+    cnt += (p2 < 0.0) != (p1 < 0.0);
+    p0 = p1;
+    p1 = p2;
+    if ((i & 7) == 7) {
+      const double m = fmax(fabs(p0), fabs(p1));
+      if (m > 1e120) {
+        p0 *= 0x1p-400;
+        p1 *= 0x1p-400;
+      } else if (m < 1e-120) {
+        p0 *= 0x1p400;
+        p1 *= 0x1p400;
+      }
+    }
   }
   return cnt;
 }
 
-// |last component| of the unit eigenvector for the extreme eigenvalue theta, by two steps
-// of inverse iteration with the shift just outside the spectrum (definite, so the
-// unpivoted tridiagonal solve is stable).
-__device__ double last_component(const double* a, const double* b, int n, double shift, double* y, double* dd) {
-  for (int i = 0; i < n; ++i) y[i] = 1.0;
-  for (int it = 0; it < 3; ++it) {
-    // LDL^T of (T - shift I), then solve
-    dd[0] = a[0] - shift;
-    for (int i = 1; i < n; ++i) dd[i] = a[i] - shift - b[i - 1] * b[i - 1] / dd[i - 1];
-    for (int i = 1; i < n; ++i) y[i] -= b[i - 1] / dd[i - 1] * y[i - 1];
-    y[n - 1] /= dd[n - 1];
-    for (int i = n - 2; i >= 0; --i) y[i] = (y[i] - b[i] * y[i + 1]) / dd[i];
-    double nr = 0.0;
-    for (int i = 0; i < n; ++i) nr += y[i] * y[i];
-    nr = sqrt(nr);
-    for (int i = 0; i < n; ++i) y[i] /= nr;
+// Extreme Ritz values of the tridiagonal of one column, widened by their residual norms
+// |beta_last| |last component of the unit eigenvector|. One warp per column: lanes 0..15 bracket the
+// smallest and lanes 16..31 the largest eigenvalue, 16 Sturm counts a round (a bisection by one
+// thread, with a division per Sturm step, took 2.6 ms); then lanes 0 and 16 run three steps of inverse
+// iteration with the shift just outside the spectrum (definite, so the unpivoted solve is stable).
+__device__ void ritz_interval(RitzBuf& r, const double* __restrict__ a, const double* __restrict__ b, int n, double& lo,
+                              double& hi) {
+  const int lane = threadIdx.x & 31, half = lane >> 4, sub = lane & 15;
+  const unsigned full = 0xffffffffu;
+  __syncwarp();
+  for (int i = lane; i < n; i += 32) {
+    r.a[i] = a[i];
+    r.b[i] = b[i];
+    r.b2[i] = b[i] * b[i];
   }
-  return fabs(y[n - 1]);
+  __syncwarp();
+  double gl = INFINITY, gu = -INFINITY;   // Gershgorin interval
+  for (int i = lane; i < n; i += 32) {
+    const double w = (i > 0 ? fabs(r.b[i - 1]) : 0.0) + (i < n - 1 ? fabs(r.b[i]) : 0.0);
+    gl = fmin(gl, r.a[i] - w);
+    gu = fmax(gu, r.a[i] + w);
+  }
+  for (int d = 16; d > 0; d >>= 1) {
+    gl = fmin(gl, __shfl_xor_sync(full, gl, d));
+    gu = fmax(gu, __shfl_xor_sync(full, gu, d));
+  }
+  // a half's bracket (l, u]: the count at l is below the target, at u it is not
+  const int target = half ? n : 1;
+  double l = gl, u = gu;
+  for (int it = 0; it < 64; ++it) {
+    const double w = u - l;
+    const bool open = w > 1e-15 * fmax(1.0, fmax(fabs(l), fabs(u)));
+    if (!__any_sync(full, open)) break;
+    const double x = l + w * (sub + 1) / 17.0;
+    const unsigned m = (__ballot_sync(full, sturm_count(r, n, x) >= target) >> (16 * half)) & 0xffffu;
+    const int first = m ? __ffs(m) - 1 : 16;   // first point of the half at or past the eigenvalue
+    const double xu = __shfl_sync(full, x, 16 * half + min(first, 15));
+    const double xl = __shfl_sync(full, x, 16 * half + max(first - 1, 0));
+    if (open) {
+      if (first < 16) u = xu;
+      if (first > 0) l = xl;
+    }
+  }
+  const double theta = 0.5 * (l + u);
+  double res = fabs(r.b[n - 1]);
+  if (n > 1 && sub == 0) {
+    const double shift = half ? theta + 1e-10 * fmax(gu - gl, 1e-300) : theta - 1e-10 * fmax(gu - gl, 1e-300);
+    double* y = r.y[half];
+    double* inv = r.inv[half];
+    inv[0] = 1.0 / (r.a[0] - shift);   // LDL^T of (T - shift I)
+    y[0] = 1.0;
+    for (int i = 1; i < n; ++i) {
+      inv[i] = 1.0 / (r.a[i] - shift - r.b2[i - 1] * inv[i - 1]);
+      y[i] = 1.0;
+    }
+    for (int it = 0; it < 3; ++it) {
+      double t = y[0];
+      for (int i = 1; i < n; ++i) {
+        t = y[i] - r.b[i - 1] * inv[i - 1] * t;
+        y[i] = t;
+      }
+      t = 0.0;
+      double nr = 0.0;
+      for (int i = n - 1; i >= 0; --i) {
+        t = (i == n - 1) ? y[i] * inv[i] : (y[i] - r.b[i] * t) * inv[i];
+        y[i] = t;
+        nr += t * t;
+      }
+      nr = 1.0 / sqrt(nr);
+      for (int i = 0; i < n; ++i) y[i] *= nr;
+    }
+    res *= fabs(y[n - 1]);
+  }
+  lo = __shfl_sync(full, theta, 0) - __shfl_sync(full, res, 0);
+  hi = __shfl_sync(full, theta, 16) + __shfl_sync(full, res, 16);
 }
 
-constexpr int kMaxLanczos = 128;
+// colb[2 col], colb[2 col + 1] = each column's widened Ritz extremes (an empty column: +inf, -inf)
+__global__ void __launch_bounds__(32 * kRitzWarps)
+k_lz_bounds(int ncols, int k, const double* __restrict__ alpha, const double* __restrict__ beta,
+            const int* __restrict__ keff, double* __restrict__ colb) {
+  __shared__ RitzBuf buf[kRitzWarps];
+  const int col = blockIdx.x * kRitzWarps + (threadIdx.x >> 5);
+  if (col >= ncols) return;
+  double lo = INFINITY, hi = -INFINITY;
+  if (keff[col] > 0)
+    ritz_interval(buf[threadIdx.x >> 5], alpha + (size_t)col * k, beta + (size_t)col * k, keff[col], lo, hi);
+  if ((threadIdx.x & 31) == 0) {
+    colb[2 * col] = lo;
+    colb[2 * col + 1] = hi;
+  }
+}
 
-// One block: Ritz extremes with residual bounds per column, min / max over columns,
-// widening by 1 % of the width; writes scal[8] = lo, scal[9] = hi.
-__global__ void k_lz_bounds(int ncols, int k, const double* __restrict__ alpha, const double* __restrict__ beta,
-                            const int* __restrict__ keff, double* __restrict__ scal) {
+// min / max over the columns, widened by 1 % of the width; writes scal[8] = lo, scal[9] = hi.
+__global__ void __launch_bounds__(256) k_lz_bounds_final(int ncols, const double* __restrict__ colb,
+                                                         double* __restrict__ scal) {
   __shared__ double slo[256], shi[256];
   double lo = INFINITY, hi = -INFINITY;
-  double y[kMaxLanczos], dd[kMaxLanczos];
   for (int col = threadIdx.x; col < ncols; col += blockDim.x) {
-    const int n = keff[col];
-    if (n <= 0) continue;
-    const double* a = alpha + (size_t)col * k;
-    const double* b = beta + (size_t)col * k;
-    double gl = INFINITY, gu = -INFINITY;
-    for (int i = 0; i < n; ++i) {
-      const double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i < n - 1 ? fabs(b[i]) : 0.0);
-      gl = fmin(gl, a[i] - r);
-      gu = fmax(gu, a[i] + r);
-    }
-    double l = gl, u = gu;                      // smallest eigenvalue: count(x) >= 1
-    for (int it = 0; it < 200 && u - l > 1e-15 * fmax(1.0, fmax(fabs(l), fabs(u))); ++it) {
-      const double mid = 0.5 * (l + u);
-      if (sturm_count(a, b, n, mid) >= 1) u = mid; else l = mid;
-    }
-    const double tmin = 0.5 * (l + u);
-    l = gl; u = gu;                             // largest eigenvalue: count(x) == n
-    for (int it = 0; it < 200 && u - l > 1e-15 * fmax(1.0, fmax(fabs(l), fabs(u))); ++it) {
-      const double mid = 0.5 * (l + u);
-      if (sturm_count(a, b, n, mid) >= n) u = mid; else l = mid;
-    }
-    const double tmax = 0.5 * (l + u);
-    const double bl = fabs(b[n - 1]);
-    const double del = 1e-10 * fmax(gu - gl, 1e-300);
-    const double rmin = (n > 1) ? bl * last_component(a, b, n, tmin - del, y, dd) : bl;
-    const double rmax = (n > 1) ? bl * last_component(a, b, n, tmax + del, y, dd) : bl;
-    lo = fmin(lo, tmin - rmin);
-    hi = fmax(hi, tmax + rmax);
+    lo = fmin(lo, colb[2 * col]);
+    hi = fmax(hi, colb[2 * col + 1]);
   }
   slo[threadIdx.x] = lo;
   shi[threadIdx.x] = hi;
@@ -298,10 +366,12 @@ __global__ void k_lz_bounds(int ncols, int k, const double* __restrict__ alpha, 
 // columns) and the step coefficients the recurrence of that node uses, with the scaling rules
 // of set_bounds (SQ_MIXED: FP32-exact 2 / zeta and -2 chi / zeta; the diagonal coefficient
 // rounded once; the stencil's constant-mode offset and that rounding folded into the centre).
-__global__ void k_lz_node_bounds(Geo g, Wave w, int k, const double* __restrict__ alpha, const double* __restrict__ beta,
-                                 const int* __restrict__ keff, int mixed, double lap_offset, double* __restrict__ nbnd,
-                                 double* __restrict__ ncoef) {
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32 * kRitzWarps)
+k_lz_node_bounds(Geo g, Wave w, int k, const double* __restrict__ alpha, const double* __restrict__ beta,
+                 const int* __restrict__ keff, int mixed, double lap_offset, double* __restrict__ nbnd,
+                 double* __restrict__ ncoef) {
+  __shared__ RitzBuf buf[kRitzWarps];
+  const int col = blockIdx.x * kRitzWarps + (threadIdx.x >> 5);
   if (col >= w.ntiles * g.B) return;
   int o[3], qo[3];
   tile_origin(g, wave_tile(w, col / g.B), o);
@@ -310,33 +380,9 @@ __global__ void k_lz_node_bounds(Geo g, Wave w, int k, const double* __restrict_
   const int node = (o[0] + qo[0]) + g.n[0] * ((o[1] + qo[1]) + g.n[1] * (o[2] + qo[2]));
   const int n = keff[col];
   if (n <= 0) return;
-  double y[kMaxLanczos], dd[kMaxLanczos];
-  const double* a = alpha + (size_t)col * k;
-  const double* b = beta + (size_t)col * k;
-  double gl = INFINITY, gu = -INFINITY;
-  for (int i = 0; i < n; ++i) {
-    const double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i < n - 1 ? fabs(b[i]) : 0.0);
-    gl = fmin(gl, a[i] - r);
-    gu = fmax(gu, a[i] + r);
-  }
-  double l = gl, u = gu;
-  for (int it = 0; it < 200 && u - l > 1e-15 * fmax(1.0, fmax(fabs(l), fabs(u))); ++it) {
-    const double mid = 0.5 * (l + u);
-    if (sturm_count(a, b, n, mid) >= 1) u = mid; else l = mid;
-  }
-  const double tmin = 0.5 * (l + u);
-  l = gl;
-  u = gu;
-  for (int it = 0; it < 200 && u - l > 1e-15 * fmax(1.0, fmax(fabs(l), fabs(u))); ++it) {
-    const double mid = 0.5 * (l + u);
-    if (sturm_count(a, b, n, mid) >= n) u = mid; else l = mid;
-  }
-  const double tmax = 0.5 * (l + u);
-  const double bl = fabs(b[n - 1]);
-  const double del = 1e-10 * fmax(gu - gl, 1e-300);
-  const double rmin = (n > 1) ? bl * last_component(a, b, n, tmin - del, y, dd) : bl;
-  const double rmax = (n > 1) ? bl * last_component(a, b, n, tmax + del, y, dd) : bl;
-  double lo = tmin - rmin, hi = tmax + rmax;
+  double lo, hi;
+  ritz_interval(buf[threadIdx.x >> 5], alpha + (size_t)col * k, beta + (size_t)col * k, n, lo, hi);
+  if ((threadIdx.x & 31) != 0) return;
   const double wdt = hi - lo;
   lo -= 0.01 * wdt;
   hi += 0.01 * wdt;
@@ -444,7 +490,10 @@ static int run_lanczos_t(sq_handle* h) {
   const double* beta = alpha + (size_t)ncols * k;
   const int* keff = (const int*)(beta + (size_t)ncols * k);
   cudaStream_t s = h->stream;
-  k_lz_bounds<<<1, 256, 0, s>>>(ncols, k, alpha, beta, keff, h->d.scal);
+  double* colb = h->d.lzC + (size_t)2 * ncols * (k + 1);   // the norms' slots, free after the last step
+  k_lz_bounds<<<(ncols + kRitzWarps - 1) / kRitzWarps, 32 * kRitzWarps, 0, s>>>(ncols, k, alpha, beta, keff, colb);
+  SQ_LAUNCH_CHECK(h);
+  k_lz_bounds_final<<<1, 256, 0, s>>>(ncols, colb, h->d.scal);
   SQ_LAUNCH_CHECK(h);
   return set_bounds_device(h);   // no host round trip: the whole evaluation can be graph-captured
 }
@@ -501,7 +550,7 @@ static int run_lanczos_nodes_t(sq_handle* h) {
     const double* alpha = h->d.nC + (size_t)3 * ncols * (k + 1);
     const double* beta = alpha + (size_t)ncols * k;
     const int* keff = (const int*)(beta + (size_t)ncols * k);
-    k_lz_node_bounds<<<(ncols + 63) / 64, 64, 0, h->stream>>>(g, w, k, alpha, beta, keff, h->precision == SQ_MIXED,
+    k_lz_node_bounds<<<(ncols + kRitzWarps - 1) / kRitzWarps, 32 * kRitzWarps, 0, h->stream>>>(g, w, k, alpha, beta, keff, h->precision == SQ_MIXED,
                                                                h->lap_offset, h->d.nbnd, h->d.ncoef);
     SQ_LAUNCH_CHECK(h);
   }
