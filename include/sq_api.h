@@ -384,8 +384,8 @@ void sq_server_destroy(sq_server* s);
  * the region dimension). Host outputs: mu_out, rho_out [N_d] (x fastest), e_band_out, each may
  * be NULL. Allocates and frees its own device scratch, not counted by sq_footprint_bytes: Krylov
  * waves of at most 16 GiB (and at most 80 % of the free device memory; fewer tiles per wave when
- * less is free) plus 2 N_d k + N_d doubles for the Gauss nodes, weights and density; synchronises
- * the stream.
+ * less is free) plus 2 N_d k + N_d doubles for the Gauss nodes, weights and density and about
+ * 20,000 (k + 1) doubles of partial products; synchronises the stream.
  * Errors: SQ_ERR_INVALID_ARG (k), SQ_ERR_OOM, SQ_ERR_NO_BRACKET, SQ_ERR_CUDA. */
 int sq_gauss_density(sq_handle* h, int k, double* mu_out, double* rho_out, double* e_band_out);
 

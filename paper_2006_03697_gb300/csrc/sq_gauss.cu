@@ -209,7 +209,7 @@ static int gauss_t(sq_handle* h, int k, double* mu_out, double* rho_host, double
     cudaGetLastError();
     free_b = size_t(16) << 30;
   }
-  const size_t fixed = 2 * sizeof(double) * (size_t)g.n_tiles * g.B * k + sizeof(double) * (size_t)h->Nd;
+  const size_t fixed = 2 * sizeof(double) * (size_t)g.n_tiles * g.B * k + sizeof(double) * ((size_t)h->Nd + lz_dots_len(k));
   const size_t wave_budget = std::min<size_t>(size_t(16) << 30, free_b > fixed ? (free_b - fixed) / 10 * 8 : 0);
   const int wt = int(std::max<size_t>(1, std::min<size_t>(wave_budget / per_tile, (size_t)h->wave_cap)));
   const int ncols_all = g.n_tiles * g.B;
@@ -227,12 +227,13 @@ static int gauss_t(sq_handle* h, int k, double* mu_out, double* rho_host, double
     bufs.clear();
   };
   Real *V = nullptr, *W = nullptr, *P = nullptr;
-  double *C = nullptr, *theta = nullptr, *wgt = nullptr, *part = nullptr, *sum = nullptr, *rho = nullptr;
+  double *C = nullptr, *dots = nullptr, *theta = nullptr, *wgt = nullptr, *part = nullptr, *sum = nullptr, *rho = nullptr;
   const int nblk = 1024;
   if (!alloc((void**)&V, sizeof(Real) * (size_t)(k + 1) * wt * g.Upts * g.B) ||
       !alloc((void**)&W, sizeof(Real) * (size_t)wt * g.Upts * g.B) ||
       !alloc((void**)&P, sizeof(Real) * (size_t)wt * g.r_cap * g.B) ||
       !alloc((void**)&C, sizeof(double) * (size_t)wt * g.B * (5 * k + 8)) ||
+      !alloc((void**)&dots, sizeof(double) * lz_dots_len(k)) ||
       !alloc((void**)&theta, sizeof(double) * (size_t)ncols_all * k) ||
       !alloc((void**)&wgt, sizeof(double) * (size_t)ncols_all * k) ||
       !alloc((void**)&part, sizeof(double) * nblk) || !alloc((void**)&sum, 2 * sizeof(double)) ||
@@ -245,7 +246,7 @@ static int gauss_t(sq_handle* h, int k, double* mu_out, double* rho_host, double
     rc = fail(h, SQ_ERR_CUDA, "status reset failed");
   for (int t0 = 0; t0 < g.n_tiles && rc == SQ_OK; t0 += wt) {
     const Wave w{t0, std::min(wt, g.n_tiles - t0), nullptr};
-    rc = lanczos_columns<Real>(h, w, 1, k, V, W, P, C, &h->wb);
+    rc = lanczos_columns<Real>(h, w, 1, k, V, W, P, C, dots, &h->wb);
     if (rc != SQ_OK) break;
     const int ncols = w.ntiles * g.B;
     const double* alpha = C + (size_t)3 * ncols * (k + 1);

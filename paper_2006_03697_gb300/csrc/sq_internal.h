@@ -34,7 +34,10 @@ constexpr int kBrick = 4;        // brick side in points
 constexpr int kMaxCh = 8;        // projector channels per atom
 constexpr int kThreads = 256;    // block size of the tile kernels
 constexpr int kMaxU = 2 * 64 + 8; // largest union-window extent (m <= 64, b = 2, x padded to 4)
-constexpr size_t kLzDotCap = 8192;   // doubles of the Lanczos dot-product chunk partials
+constexpr int kMaxLanczos = 128;         // most Lanczos steps
+constexpr int kLzChunkTiles = 8 * 152;   // most (chunk, tile) blocks of a Lanczos wave split into chunks
+// doubles of their partial products: two sets of up to k + 1 products of 8 nodes, and the norms
+inline size_t lz_dots_len(int k) { return size_t(kLzChunkTiles) * 8 * (2 * size_t(k + 1) + 1); }
 
 struct AtomTab {
   int lo[3];        // support box corner (absolute lattice coordinates of the base image)
@@ -143,7 +146,7 @@ struct Dev {
   double* lzP = nullptr;          // projections of the Lanczos vector [nst][r_cap][B]
   double* lzC = nullptr;          // Gram-Schmidt coefficients / alpha, beta [cols][...]
   int* lz_tiles = nullptr;        // sample tile ids [nst]
-  double* lzdot = nullptr;        // chunk partials of the Lanczos dot products of small waves [kLzDotCap]
+  double* lzdot = nullptr;        // chunk partials of the Lanczos products [lz_dots_len(lanczos_k)]
   // per-node bounds mode (SQ_BOUNDS_PER_NODE)
   double* nbnd = nullptr;         // [N_d][2] effective (lo, hi) of every node
   double* ncoef = nullptr;        // [N_d][2] step coefficients (ca = 2 / zeta_q, cd = ca lap0 - 2 chi_q / zeta_q)
@@ -304,7 +307,7 @@ int run_lanczos(sq_handle* h);
 // k-step Lanczos of every node column of a wave (start 0: hash vector, 1: e_q); see sq_lanczos.cu
 template <typename Real>
 int lanczos_columns(sq_handle* h, const Wave& w, int start, int k, Real* V, Real* W, Real* P, double* C,
-                    WaveBufs* b);
+                    double* dots, WaveBufs* b);
 int run_fermi(sq_handle* h, double* mu_out);
 // per-node bounds mode (sq_lanczos.cu, sq_reduce.cu)
 int run_lanczos_nodes(sq_handle* h);

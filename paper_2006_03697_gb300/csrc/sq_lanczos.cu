@@ -20,7 +20,6 @@ namespace sq {
 
 constexpr int kTileLz = 8;              // nodes per tile (columns per tile)
 constexpr int kMaxLanczosVecs = 136;    // Krylov vectors held (k + 1, k <= 128 + 7)
-constexpr int kLzDotChunks = 32;        // most chunks a dot product of a small wave is split into
 
 // Start vector of the column of node q: 1 + (hash(i, node) mod 1009) / 1009 on the window
 // (i = window-local index, C order z, y, x), zero elsewhere; normalised afterwards.
@@ -67,145 +66,223 @@ __global__ void k_lz_init_unit(Geo g, Wave w, Real* __restrict__ V0) {
   }
 }
 
-// out[col * ld + i] = <V_i, x>_col for i < nvec (one block per (i, tile); fixed-order sums:
-// per thread in the vectors' precision, across threads in FP64)
+// ---- Gram-Schmidt on the Krylov vectors of a wave.
+// One block per (chunk of a tile's points, tile), in rounds of 256 groups of four nodes. Update: a thread
+// owns one group and walks the vectors. Products: the round's x sits in shared memory and the eight warps
+// share out the vectors V_i, each taking all groups of its vectors, so x is read from memory once, a
+// V chunk read by the update is still in cache for the products, and no product crosses warps. The
+// four products of a lane are added over the warp by a reduce-scatter (5 exchanges in place of 16).
+// Cross-thread sums keep FP64's accuracy: FP64 vectors add doubles, FP32 vectors add pairs of floats
+// (two-sum; FP64 adds issue at 1.7 lanes per clock here and cost more than the products).
+constexpr int kLzThreads = 256, kLzWarps = kLzThreads / 32;
+
+template <typename Real> struct LzV4;
+template <> struct LzV4<float> { using T = float4; };
+template <> struct LzV4<double> { using T = double4_32a; };
+
+struct FloatPair { float h, l; };
+
+__device__ __forceinline__ FloatPair lz_add(FloatPair a, FloatPair b) {   // Knuth's two-sum, tails added
+  const float s = __fadd_rn(a.h, b.h), z = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, z)), __fsub_rn(b.h, z));
+  const float t = __fadd_rn(e, __fadd_rn(a.l, b.l)), h = __fadd_rn(s, t);
+  return {h, __fsub_rn(t, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ double lz_add(double a, double b) { return a + b; }
+__device__ __forceinline__ FloatPair lz_shfl(FloatPair a, int m) {
+  return {__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
+}
+__device__ __forceinline__ double lz_shfl(double a, int m) { return __shfl_xor_sync(0xffffffffu, a, m); }
+__device__ __forceinline__ double lz_double(FloatPair a) { return double(a.h) + double(a.l); }
+__device__ __forceinline__ double lz_double(double a) { return a; }
+template <typename Real> struct LzAcc;
+template <> struct LzAcc<float> {
+  using T = FloatPair;
+  static __device__ __forceinline__ T make(float x) { return {x, 0.f}; }
+};
+template <> struct LzAcc<double> {
+  using T = double;
+  static __device__ __forceinline__ T make(double x) { return x; }
+};
+
+// the four products of a lane (nodes 4 (lane & 1) ..), added over the warp's 16 lanes of that parity into
+// acc[8] (lanes 0 .. 7 add one node each; one warp per acc)
 template <typename Real>
-__global__ void k_lz_dots(Geo g, Wave w, const Real* __restrict__ V, int nvec, size_t vstride,
-                          const Real* __restrict__ x, double* __restrict__ out, int ld) {
-  const int i = blockIdx.x, tl = blockIdx.y;
-  const size_t base = (size_t)tl * g.Upts * g.B;
-  const Real* Vi = V + (size_t)i * vstride + base;
-  const Real* xt = x + base;
-  const int q = threadIdx.x % g.B;
-  Real s = Real(0);
-  for (int e = threadIdx.x; e < g.Upts * g.B; e += blockDim.x) s += Vi[e] * xt[e];
-  __shared__ double red[kThreads];
-  red[threadIdx.x] = double(s);
+__device__ __forceinline__ void lz_warp_add(const Real d[4], typename LzAcc<Real>::T* acc) {
+  using A = typename LzAcc<Real>::T;
+  const int lane = threadIdx.x & 31, s0 = (lane >> 1) & 1, s1 = (lane >> 2) & 1;
+  const A v0 = LzAcc<Real>::make(d[0]), v1 = LzAcc<Real>::make(d[1]), v2 = LzAcc<Real>::make(d[2]), v3 = LzAcc<Real>::make(d[3]);
+  const A k0 = lz_add(s0 ? v2 : v0, lz_shfl(s0 ? v0 : v2, 2));
+  const A k1 = lz_add(s0 ? v3 : v1, lz_shfl(s0 ? v1 : v3, 2));
+  A k = lz_add(s1 ? k1 : k0, lz_shfl(s1 ? k0 : k1, 4));
+  k = lz_add(k, lz_shfl(k, 8));
+  k = lz_add(k, lz_shfl(k, 16));
+  if (lane < 8) {
+    A* slot = acc + 4 * (lane & 1) + 2 * s0 + s1;
+    *slot = lz_add(*slot, k);
+  }
+}
+
+enum LzMode { kLzDots = 0, kLzUpdateDots = 1, kLzUpdateNorm = 2, kLzNorm = 3 };
+
+// in, out[((tile nch + chunk) ld + i) 8 + node]: the chunk's share of <V_i, x>; norms, <x, x>, are packed
+// (ld = 1, i = 0).
+//   kLzDots        out = V^T x
+//   kLzUpdateDots  x -= V (sum over chunks of in), then out = V^T x
+//   kLzUpdateNorm  x -= V (sum over chunks of in), then out = x^T x
+//   kLzNorm        out = x^T x
+// The coefficient of the last vector goes to (kLzUpdateDots) or is added to (kLzUpdateNorm)
+// alpha[col k + nvec - 1].
+template <typename Real, int MODE>
+__global__ void __launch_bounds__(kLzThreads)
+k_lz_ortho(Geo g, const Real* __restrict__ V, int nvec, size_t vstride, Real* __restrict__ x,
+           const double* __restrict__ in, double* __restrict__ out, int ld, int k, double* __restrict__ alpha) {
+  using V4 = typename LzV4<Real>::T;
+  using A = typename LzAcc<Real>::T;
+  extern __shared__ __align__(16) unsigned char lz_smem[];
+  constexpr bool kNorm = MODE == kLzUpdateNorm || MODE == kLzNorm;
+  constexpr bool kUpdate = MODE == kLzUpdateDots || MODE == kLzUpdateNorm;
+  const int nch = gridDim.x, c = blockIdx.x, tl = blockIdx.y, warp = threadIdx.x >> 5;
+  V4* xs = reinterpret_cast<V4*>(lz_smem);                             // [kLzThreads] the round's x
+  A* acc = reinterpret_cast<A*>(xs + kLzThreads);                      // products [nvec][8], norms [kLzWarps][8]
+  Real* cf = reinterpret_cast<Real*>(acc + (kNorm ? kLzWarps : nvec) * kTileLz);   // [nvec][8]
+  for (int i = threadIdx.x; i < (kNorm ? kLzWarps : nvec) * kTileLz; i += kLzThreads) acc[i] = LzAcc<Real>::make(Real(0));
+  if constexpr (kUpdate) {
+    for (int i = threadIdx.x; i < nvec * kTileLz; i += kLzThreads) {
+      const double* p = in + (size_t)tl * nch * ld * kTileLz + i;
+      double s = 0.0;
+#pragma unroll 4
+      for (int cc = 0; cc < nch; ++cc) s += p[(size_t)cc * ld * kTileLz];
+      cf[i] = Real(s);
+      if (c == 0 && i / kTileLz == nvec - 1) {
+        double* al = alpha + (size_t)(tl * kTileLz + i % kTileLz) * k + nvec - 1;
+        *al = (MODE == kLzUpdateDots) ? s : *al + s;
+      }
+    }
+  }
   __syncthreads();
-  if (threadIdx.x < g.B) {
-    double t = 0.0;
-    for (int th = q; th < kThreads; th += g.B) t += red[th];
-    out[((size_t)tl * g.B + q) * ld + i] = t;
+  const size_t n = (size_t)g.Upts * 2;                  // groups of four nodes of the tile
+  const size_t g0 = (size_t)g.Upts * c / nch * 2, g1 = (size_t)g.Upts * (c + 1) / nch * 2;
+  const V4* Vt = reinterpret_cast<const V4*>(V) + (size_t)tl * n;
+  V4* xt = reinterpret_cast<V4*>(x) + (size_t)tl * n;
+  const size_t vs = vstride / 4;
+  const int lane = threadIdx.x & 31;
+  for (size_t r0 = g0; r0 < g1; r0 += kLzThreads) {
+    const size_t p = r0 + threadIdx.x;
+    V4 xv;
+    xv.x = xv.y = xv.z = xv.w = Real(0);
+    if (p < g1) {
+      xv = xt[p];
+      if constexpr (kUpdate) {
+        const Real* ci = cf + 4 * (threadIdx.x & 1);
+        Real u[4] = {Real(0), Real(0), Real(0), Real(0)};
+#pragma unroll 4
+        for (int i = 0; i < nvec; ++i, ci += kTileLz) {
+          const V4 t = Vt[i * vs + p];
+          u[0] += ci[0] * t.x; u[1] += ci[1] * t.y; u[2] += ci[2] * t.z; u[3] += ci[3] * t.w;
+        }
+        xv.x -= u[0]; xv.y -= u[1]; xv.z -= u[2]; xv.w -= u[3];
+        xt[p] = xv;
+      }
+    }
+    if constexpr (kNorm) {
+      if (r0 + 32 * warp < g1) {
+        const Real d[4] = {xv.x * xv.x, xv.y * xv.y, xv.z * xv.z, xv.w * xv.w};
+        lz_warp_add<Real>(d, acc + warp * kTileLz);
+      }
+    } else {
+      xs[threadIdx.x] = xv;
+      __syncthreads();
+      const int ng = int(min((size_t)kLzThreads, g1 - r0));
+      for (int i = warp; i < nvec; i += kLzWarps) {
+        const V4* Vi = Vt + i * vs + r0;
+        Real d[4] = {Real(0), Real(0), Real(0), Real(0)};
+#pragma unroll
+        for (int e = 0; e < kLzThreads; e += 32)
+          if (e + lane < ng) {
+            const V4 t = Vi[e + lane], xx = xs[e + lane];
+            d[0] += xx.x * t.x; d[1] += xx.y * t.y; d[2] += xx.z * t.z; d[3] += xx.w * t.w;
+          }
+        lz_warp_add<Real>(d, acc + i * kTileLz);
+      }
+      __syncthreads();
+    }
   }
-}
-
-// The same products for waves of few tiles (the Lanczos sample tiles): block (i, tile, c) sums
-// chunk c of the tile's vector pair into part[((tile * nvec + i) * nch + c) * B + node], and
-// k_lz_dots_sum adds the nch chunks of every (tile, node, i) in order, so a product spreads over
-// nch times more blocks and the result does not depend on scheduling.
-template <typename Real>
-__global__ void k_lz_dots_part(Geo g, Wave w, const Real* __restrict__ V, int nvec, size_t vstride,
-                               const Real* __restrict__ x, double* __restrict__ part, int nch) {
-  const int i = blockIdx.x, tl = blockIdx.y, c = blockIdx.z;
-  const size_t n = (size_t)g.Upts * g.B;
-  const size_t len = ((n + nch - 1) / nch + g.B - 1) / g.B * g.B;   // chunks start at a node-0 slot
-  const size_t e0 = (size_t)c * len, e1 = min(n, e0 + len);
-  const size_t base = (size_t)tl * n;
-  const Real* Vi = V + (size_t)i * vstride + base;
-  const Real* xt = x + base;
-  const int q = threadIdx.x % g.B;
-  Real s = Real(0);
-  for (size_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) s += Vi[e] * xt[e];
-  __shared__ double red[kThreads];
-  red[threadIdx.x] = double(s);
   __syncthreads();
-  if (threadIdx.x < g.B) {
-    double t = 0.0;
-    for (int th = q; th < kThreads; th += g.B) t += red[th];
-    part[(((size_t)tl * nvec + i) * nch + c) * g.B + q] = t;
+  for (int i = threadIdx.x; i < (kNorm ? 1 : nvec) * kTileLz; i += kLzThreads) {
+    double s = lz_double(acc[i]);
+    if constexpr (kNorm)
+      for (int w = 1; w < kLzWarps; ++w) s += lz_double(acc[w * kTileLz + i]);
+    out[((size_t)tl * nch + c) * (kNorm ? 1 : ld) * kTileLz + i] = s;
   }
 }
 
-__global__ void k_lz_dots_sum(const double* __restrict__ part, int ntiles, int nvec, int nch, int B,
-                              double* __restrict__ out, int ld) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= ntiles * nvec * B) return;
-  const int q = k % B, i = (k / B) % nvec, tl = k / (B * nvec);
-  double t = 0.0;
-  for (int c = 0; c < nch; ++c) t += part[(((size_t)tl * nvec + i) * nch + c) * B + q];
-  out[((size_t)tl * B + q) * ld + i] = t;
-}
-
-// out[(tile node) * ld + i] = V_i . x per node column, one launch (or two for few tiles)
+// End of step i: beta_i = ||x||; a column whose beta falls below 1e-12 max(1, |alpha_i|) or that took all
+// kk steps stops with k_eff = i + 1 (keff < 0 while running). V_next = x / beta for running columns, zero
+// otherwise (Vn null: no next vector). i < 0: normalises the start vector; a zero one marks an empty
+// column (keff = 0). The blocks of a tile all form the same decision; the first one records it (a
+// block that already reads the recorded keff comes to the same decision).
 template <typename Real>
-static int lz_dots(sq_handle* h, const Wave& w, const Real* V, int nvec, size_t vstride, const Real* x, double* out,
-                   int ld) {
-  const Geo& g = h->geo;
-  cudaStream_t s = h->stream;
-  const int blocks = nvec * w.ntiles;
-  const int nch = std::max(1, std::min(kLzDotChunks, (2 * 152 + blocks - 1) / std::max(1, blocks)));
-  if (blocks >= 2 * 152 || !h->d.lzdot || size_t(blocks) * nch * g.B > kLzDotCap) {
-    k_lz_dots<Real><<<dim3(nvec, w.ntiles), kThreads, 0, s>>>(g, w, V, nvec, vstride, x, out, ld);
-    SQ_LAUNCH_CHECK(h);
-    return SQ_OK;
-  }
-  k_lz_dots_part<Real><<<dim3(nvec, w.ntiles, nch), kThreads, 0, s>>>(g, w, V, nvec, vstride, x, h->d.lzdot, nch);
-  SQ_LAUNCH_CHECK(h);
-  const int nk = w.ntiles * nvec * g.B;
-  k_lz_dots_sum<<<(nk + 255) / 256, 256, 0, s>>>(h->d.lzdot, w.ntiles, nvec, nch, g.B, out, ld);
-  SQ_LAUNCH_CHECK(h);
-  return SQ_OK;
-}
-
-// x -= sum_i coef[col * ld + i] V_i; grid (blocks per tile, tiles): a block's coefficients
-// (8 columns x nvec) are converted to the vectors' precision once, in shared memory
-template <typename Real>
-__global__ void k_lz_update(Geo g, Wave w, const Real* __restrict__ V, int nvec, size_t vstride,
-                            const double* __restrict__ coef, int ld, Real* __restrict__ x) {
-  __shared__ Real cf[kTileLz][kMaxLanczosVecs];
+__global__ void __launch_bounds__(256)
+k_lz_scale(Geo g, const Real* x, const double* __restrict__ nrm, int nch, int i, int kk, int k,
+           const double* __restrict__ alpha, double* __restrict__ beta, int* keff, Real* Vn) {
+  using V4 = typename LzV4<Real>::T;
+  __shared__ Real bb_s[kTileLz], inv_s[kTileLz], low_s[kTileLz];   // beta, 1 / beta and its rounding error
   const int tl = blockIdx.y;
-  for (int k2 = threadIdx.x; k2 < g.B * nvec; k2 += blockDim.x) {
-    const int q = k2 / nvec, i = k2 % nvec;
-    cf[q][i] = Real(coef[((size_t)tl * g.B + q) * ld + i]);
+  if (threadIdx.x < kTileLz) {
+    const size_t col = (size_t)tl * kTileLz + threadIdx.x;
+    double s = 0.0;
+    for (int c = 0; c < nch; ++c) s += nrm[((size_t)tl * nch + c) * kTileLz + threadIdx.x];
+    const double b = sqrt(s);
+    bool run;
+    if (i < 0) {
+      run = b > 0.0;
+      if (blockIdx.x == 0) keff[col] = run ? -1 : 0;
+    } else {
+      const bool live = keff[col] < 0;
+      const double a = alpha[col * k + i];
+      const bool stop = i == kk - 1 || b <= 1e-12 * fmax(1.0, fabs(a));
+      run = live && !stop;
+      if (blockIdx.x == 0 && live) {
+        beta[col * k + i] = b;
+        if (stop) keff[col] = i + 1;
+      }
+    }
+    const double r = run ? 1.0 / b : 0.0;
+    bb_s[threadIdx.x] = run ? Real(b) : Real(0);
+    inv_s[threadIdx.x] = Real(r);
+    low_s[threadIdx.x] = Real(r - double(Real(r)));
   }
   __syncthreads();
-  const size_t per_tile = (size_t)g.Upts * g.B;
-  const size_t base = per_tile * tl;
-  for (size_t r = blockIdx.x * (size_t)blockDim.x + threadIdx.x; r < per_tile; r += (size_t)gridDim.x * blockDim.x) {
-    const int q = int(r % g.B);
-    Real acc = Real(0);
-    for (int i = 0; i < nvec; ++i) acc += cf[q][i] * V[(size_t)i * vstride + base + r];
-    x[base + r] -= acc;
+  if (!Vn) return;
+  const size_t n = (size_t)g.Upts * 2;
+  const V4* xt = reinterpret_cast<const V4*>(x) + (size_t)tl * n;
+  V4* vt = reinterpret_cast<V4*>(Vn) + (size_t)tl * n;
+  const int h = 4 * (threadIdx.x & 1);
+  Real bb[4], inv[4], low[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    bb[q] = bb_s[h + q];
+    inv[q] = inv_s[h + q];
+    low[q] = low_s[h + q];
+  }
+  // x / beta rounded once, without a division per element: FP64 corrects x (1 / beta) by its remainder,
+  // FP32 takes 1 / beta as a pair of floats
+  auto div = [&](Real v, int q) -> Real {
+    if constexpr (sizeof(Real) == 8) {
+      const Real t = v * inv[q];
+      return fma(fma(-bb[q], t, v), inv[q], t);
+    } else {
+      return fmaf(v, inv[q], v * low[q]);
+    }
+  };
+  for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x) {
+    V4 t = xt[p];
+    t.x = div(t.x, 0); t.y = div(t.y, 1); t.z = div(t.z, 2); t.w = div(t.w, 3);
+    vt[p] = t;
   }
 }
 
-// Per column: alpha_i = cA_i + cB_i, beta_i = ||w||; a column whose beta falls below
-// 1e-12 max(1, |alpha_i|) stops with k_eff = i + 1 (keff < 0 while running).
-__global__ void k_lz_step(int ncols, int i, int kk, int k, const double* __restrict__ cA, const double* __restrict__ cB,
-                          int ld, const double* __restrict__ nrm, double* __restrict__ alpha, double* __restrict__ beta,
-                          int* __restrict__ keff) {
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= ncols || keff[col] >= 0) return;
-  const double a = cA[(size_t)col * ld + i] + cB[(size_t)col * ld + i];
-  const double b = sqrt(nrm[(size_t)col * ld]);
-  alpha[(size_t)col * k + i] = a;
-  beta[(size_t)col * k + i] = b;
-  if (i == kk - 1 || b <= 1e-12 * fmax(1.0, fabs(a))) keff[col] = i + 1;
-}
-
-// V_next = x / beta for running columns (zero otherwise). With first != 0: normalise the
-// start vector in place (beta = sqrt(nrm)); a zero start vector marks an empty column.
-template <typename Real>
-__global__ void k_lz_scale(Geo g, Wave w, const Real* __restrict__ x, const double* __restrict__ nrm, int ld,
-                           int* __restrict__ keff, Real* __restrict__ Vn, int first) {
-  const size_t per_tile = (size_t)g.Upts * g.B;
-  const size_t total = per_tile * w.ntiles;
-  for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total; idx += (size_t)gridDim.x * blockDim.x) {
-    const int tl = int(idx / per_tile);
-    const int q = int(idx % per_tile) % g.B;
-    const size_t col = (size_t)tl * g.B + q;
-    const double b = sqrt(nrm[col * ld]);
-    const bool run = first ? (b > 0.0) : (keff[col] < 0);
-    Vn[idx] = run ? Real(double(x[idx]) / b) : Real(0);
-  }
-}
-
-__global__ void k_lz_mark_empty(int ncols, const double* __restrict__ nrm, int ld, int* __restrict__ keff) {
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  if (col < ncols) keff[col] = (nrm[(size_t)col * ld] > 0.0) ? -1 : 0;
-}
-
-constexpr int kMaxLanczos = 128;
 constexpr int kRitzWarps = 4;   // columns per block of the Ritz kernels
 
 struct RitzBuf {
@@ -408,10 +485,10 @@ k_lz_node_bounds(Geo g, Wave w, int k, const double* __restrict__ alpha, const d
 // k-step Lanczos (CGS2 reorthogonalisation) of every node column of the wave's tiles, from the
 // hash start vector (start = 0, the spectral bounds) or from e_q (start = 1, Gauss SQ). V holds
 // k + 1 vectors of the wave, W one, P the projections; C is (5 k + 8) doubles per column:
-// cA, cB, nrm [ncols][k + 1], alpha, beta [ncols][k], keff (ints) - see lz_alpha etc.
+// cA, cB, nrm [ncols][k + 1], alpha, beta [ncols][k], keff (ints).
 template <typename Real>
 int lanczos_columns(sq_handle* h, const Wave& w, int start, int k, Real* V, Real* W, Real* P, double* C,
-                    WaveBufs* b) {
+                    double* dots, WaveBufs* b) {
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
   const int nst = w.ntiles;
@@ -421,15 +498,21 @@ int lanczos_columns(sq_handle* h, const Wave& w, int start, int k, Real* V, Real
   const int ncols = nst * g.B;
   const int ld = k + 1;
   const size_t vstride = (size_t)nst * g.Upts * g.B;
-  double* cA = C;
-  double* cB = cA + (size_t)ncols * ld;
-  double* nrm = cB + (size_t)ncols * ld;
-  double* alpha = nrm + (size_t)ncols * ld;
+  // chunks per tile: about eight blocks per SM, of at least 64 points, at most 32 (every block of a
+  // tile adds the chunks' products for its coefficients). dots holds the partial products of two passes
+  // and the norms; a wave of more tiles than it holds has one chunk per tile, in C.
+  const int nch = std::max(1, std::min({kLzChunkTiles / std::max(1, nst), 32, (g.Upts + 63) / 64}));
+  const bool small = nch * nst <= kLzChunkTiles;
+  const size_t set = (size_t)(small ? kLzChunkTiles : nst) * ld * kTileLz;
+  double* cA = small ? dots : C;
+  double* cB = cA + set;
+  double* nrm = cB + set;
+  double* alpha = C + (size_t)3 * ncols * ld;
   double* beta = alpha + (size_t)ncols * k;
   int* keff = (int*)(beta + (size_t)ncols * k);
   const int eb = 1024;
-  const int ub = int(std::min<size_t>(64, ((size_t)g.Upts * g.B + 255) / 256));   // update blocks per tile
-  const int cb = (ncols + 127) / 128;
+  const dim3 og(nch, nst);
+  const dim3 sg(std::max(1, std::min((2 * g.Upts + 255) / 256, 8 * 152 / std::max(1, nst) + 1)), nst);
   // the sample tiles' lists (their own buffers) only change with the atoms; a graph capture
   // records the build
   int rc = SQ_OK;
@@ -443,38 +526,32 @@ int lanczos_columns(sq_handle* h, const Wave& w, int start, int k, Real* V, Real
   if (start == 0) k_lz_init<Real><<<eb, 256, 0, s>>>(g, w, V);
   else k_lz_init_unit<Real><<<eb, 256, 0, s>>>(g, w, V);
   SQ_LAUNCH_CHECK(h);
-  rc = lz_dots<Real>(h, w, V, 1, vstride, V, nrm, ld);
-  if (rc != SQ_OK) return rc;
-  k_lz_mark_empty<<<cb, 128, 0, s>>>(ncols, nrm, ld, keff);
+  const size_t xsb = 4 * sizeof(Real) * kLzThreads, acc1 = sizeof(double) * kTileLz;   // x of a round, sums per product
+  k_lz_ortho<Real, kLzNorm><<<og, kLzThreads, xsb + acc1 * kLzWarps, s>>>(g, V, 0, vstride, V, nullptr, nrm, ld, k, nullptr);
   SQ_LAUNCH_CHECK(h);
-  k_lz_scale<Real><<<eb, 256, 0, s>>>(g, w, V, nrm, ld, keff, V, 1);
+  k_lz_scale<Real><<<sg, 256, 0, s>>>(g, V, nrm, nch, -1, kk, k, alpha, beta, keff, V);
   SQ_LAUNCH_CHECK(h);
   for (int i = 0; i < kk; ++i) {
     Real* Vi = V + (size_t)i * vstride;
+    const int nv = i + 1;
+    const size_t cfb = sizeof(Real) * nv * kTileLz;
     rc = launch_apply_h(h, w, Vi, W, P, *b);
     if (rc != SQ_OK) return rc;
-    rc = lz_dots<Real>(h, w, V, i + 1, vstride, W, cA, ld);
-    if (rc != SQ_OK) return rc;
-    k_lz_update<Real><<<dim3(ub, nst), 256, 0, s>>>(g, w, V, i + 1, vstride, cA, ld, W);
+    k_lz_ortho<Real, kLzDots><<<og, kLzThreads, xsb + acc1 * nv, s>>>(g, V, nv, vstride, W, nullptr, cA, ld, k, nullptr);
     SQ_LAUNCH_CHECK(h);
-    rc = lz_dots<Real>(h, w, V, i + 1, vstride, W, cB, ld);
-    if (rc != SQ_OK) return rc;
-    k_lz_update<Real><<<dim3(ub, nst), 256, 0, s>>>(g, w, V, i + 1, vstride, cB, ld, W);
+    k_lz_ortho<Real, kLzUpdateDots><<<og, kLzThreads, xsb + acc1 * nv + cfb, s>>>(g, V, nv, vstride, W, cA, cB, ld, k, alpha);
     SQ_LAUNCH_CHECK(h);
-    rc = lz_dots<Real>(h, w, W, 1, vstride, W, nrm, ld);
-    if (rc != SQ_OK) return rc;
-    k_lz_step<<<cb, 128, 0, s>>>(ncols, i, kk, k, cA, cB, ld, nrm, alpha, beta, keff);
+    k_lz_ortho<Real, kLzUpdateNorm><<<og, kLzThreads, xsb + acc1 * kLzWarps + cfb, s>>>(g, V, nv, vstride, W, cB, nrm, ld, k, alpha);
     SQ_LAUNCH_CHECK(h);
-    if (i < kk - 1) {
-      k_lz_scale<Real><<<eb, 256, 0, s>>>(g, w, W, nrm, ld, keff, V + (size_t)(i + 1) * vstride, 0);
-      SQ_LAUNCH_CHECK(h);
-    }
+    k_lz_scale<Real><<<sg, 256, 0, s>>>(g, W, nrm, nch, i, kk, k, alpha, beta, keff,
+                                        i < kk - 1 ? V + (size_t)(i + 1) * vstride : (Real*)nullptr);
+    SQ_LAUNCH_CHECK(h);
   }
   return SQ_OK;
 }
 
-template int lanczos_columns<float>(sq_handle*, const Wave&, int, int, float*, float*, float*, double*, WaveBufs*);
-template int lanczos_columns<double>(sq_handle*, const Wave&, int, int, double*, double*, double*, double*, WaveBufs*);
+template int lanczos_columns<float>(sq_handle*, const Wave&, int, int, float*, float*, float*, double*, double*, WaveBufs*);
+template int lanczos_columns<double>(sq_handle*, const Wave&, int, int, double*, double*, double*, double*, double*, WaveBufs*);
 
 template <typename Real>
 static int run_lanczos_t(sq_handle* h) {
@@ -484,7 +561,7 @@ static int run_lanczos_t(sq_handle* h) {
   const Wave w{0, nst, h->d.lz_tiles};
   // the sample tiles' lists go to their own buffers, so the sweep's lists (and W) stay valid
   int rc = lanczos_columns<Real>(h, w, 0, k, reinterpret_cast<Real*>(h->d.lzV), reinterpret_cast<Real*>(h->d.lzW),
-                                 reinterpret_cast<Real*>(h->d.lzP), h->d.lzC, &h->lzb);
+                                 reinterpret_cast<Real*>(h->d.lzP), h->d.lzC, h->d.lzdot, &h->lzb);
   if (rc != SQ_OK) return rc;
   const double* alpha = h->d.lzC + (size_t)3 * ncols * (k + 1);
   const double* beta = alpha + (size_t)ncols * k;
@@ -544,7 +621,7 @@ static int run_lanczos_nodes_t(sq_handle* h) {
   for (int t0 = h->tile_begin; t0 < h->tile_end; t0 += h->nlz_wave) {
     const Wave w{t0, std::min(h->nlz_wave, h->tile_end - t0), nullptr};
     int rc = lanczos_columns<Real>(h, w, 0, k, reinterpret_cast<Real*>(h->d.nV), reinterpret_cast<Real*>(h->d.nW),
-                                   reinterpret_cast<Real*>(h->d.nP), h->d.nC, &h->wb);
+                                   reinterpret_cast<Real*>(h->d.nP), h->d.nC, h->d.lzdot, &h->wb);
     if (rc != SQ_OK) return rc;
     const int ncols = w.ntiles * g.B;
     const double* alpha = h->d.nC + (size_t)3 * ncols * (k + 1);
