@@ -28,113 +28,172 @@
 namespace sq {
 
 // ------------------------------------------------------------------------------ Lanczos apply
-// P[row][q] = gamma |dOmega| chi_row^T v (one block per atom image of a tile)
+template <typename Real> struct V4;
+template <> struct V4<float> { using T = float4; };
+template <> struct V4<double> { using T = double4_32a; };
+
 template <typename Real>
-__global__ void __launch_bounds__(kThreads)
+__device__ __forceinline__ void load4(const Real* p, Real out[4]) {
+  const typename V4<Real>::T x = *reinterpret_cast<const typename V4<Real>::T*>(p);
+  out[0] = x.x;
+  out[1] = x.y;
+  out[2] = x.z;
+  out[3] = x.w;
+}
+
+// P[row][q] = gamma |dOmega| chi_row^T v: one block per atom image of a tile (images in a stride of
+// gridDim.x). A thread owns an (x, y) column of the image's box and half of the nodes: one projector load
+// per point serves four nodes, and the column only walks the z-chord of the support sphere (FP32 with a
+// 1e-5 margin; points past it hold zeros). Per thread in the vectors' precision, across threads in FP64,
+// fixed order. One thread per (point, node) with an integer division each took 74 us for the 10
+// sample tiles of a 12^3 cell and 691 us for its 216 tiles.
+constexpr int kProjThreads = 128;
+template <typename Real>
+__global__ void __launch_bounds__(kProjThreads)
 k_project(Geo g, Wave w, const Real* __restrict__ Tn, const Real* __restrict__ chi, const AtomTab* __restrict__ atoms,
-          const double* __restrict__ chs, const TileEntry* __restrict__ entries, const int* __restrict__ n_entries,
-          Real* __restrict__ P) {
-  const int eidx = blockIdx.x, tl = blockIdx.y, t = wave_tile(w, tl);
-  if (eidx >= n_entries[tl]) return;
+          const double* __restrict__ rcmax, const double* __restrict__ chs, const TileEntry* __restrict__ entries,
+          const int* __restrict__ n_entries, Real* __restrict__ P) {
+  const int tl = blockIdx.y, t = wave_tile(w, tl), B = 8;
   int o[3];
   tile_origin(g, t, o);
-  const TileEntry te = entries[(size_t)tl * g.e_cap + eidx];
-  const AtomTab at = atoms[te.atom];
-  const int B = g.B;
-  int lo[3], hi[3];
-  for (int a = 0; a < 3; ++a) {
-    const int blo = at.lo[a] + te.s[a] * g.n[a] - (o[a] - g.m[a]);   // box corner in U-local coords
-    lo[a] = max(0, blo);
-    hi[a] = min(g.U[a], blo + at.dim[a]);
-  }
-  const int nx = max(0, hi[0] - lo[0]), ny = max(0, hi[1] - lo[1]), nzz = max(0, hi[2] - lo[2]);
-  const int nel = nx * ny * nzz * B;
   const Real* T = Tn + (size_t)tl * g.Upts * B;
-  Real acc[kMaxCh];
-#pragma unroll
-  for (int c = 0; c < kMaxCh; ++c) acc[c] = Real(0);
-  for (int i = threadIdx.x; i < nel; i += kThreads) {
-    const int p = i / B, q = i % B;
-    const int lx = lo[0] + p % nx, ly = lo[1] + (p / nx) % ny, lz = lo[2] + p / (nx * ny);
-    const Real tv = T[((size_t)(lz * g.U[1] + ly) * g.U[0] + lx) * B + q];
-    if (tv == Real(0)) continue;
-    const int li = box_index(at, te.s, g.n, o[0] - g.m[0] + lx, o[1] - g.m[1] + ly, o[2] - g.m[2] + lz);
-    const Real* cr = chi_row(chi, at, li);
-#pragma unroll
-    for (int c = 0; c < kMaxCh; ++c)
-      if (c < at.nch) acc[c] += cr[c] * tv;
-  }
-  __shared__ double red[kThreads][kMaxCh];
-#pragma unroll
-  for (int c = 0; c < kMaxCh; ++c) red[threadIdx.x][c] = double(acc[c]);
-  __syncthreads();
   Real* Pt = P + (size_t)tl * g.r_cap * B;
-  for (int k2 = threadIdx.x; k2 < B * at.nch; k2 += kThreads) {
-    const int qq = k2 % B, c = k2 / B;
-    double s = 0.0;
-    for (int th = qq; th < kThreads; th += B) s += red[th][c];
-    Pt[(size_t)(te.row0 + c) * B + qq] = Real(s * chs[6 * (at.ch0 + c)]);
+  const int half = threadIdx.x & 1, lane = threadIdx.x >> 1;
+  __shared__ Real red[16][kProjThreads / 2 * 2 + 1];   // [channel 4 x node 4][thread]
+  for (int eidx = blockIdx.x; eidx < n_entries[tl]; eidx += gridDim.x) {
+    const TileEntry te = entries[(size_t)tl * g.e_cap + eidx];
+    const AtomTab& at = atoms[te.atom];
+    const float rc = float(rcmax[te.atom]), rc2 = rc * rc * (1.f + 1e-5f) + 1e-10f;
+    int lo[3], hi[3], bl[3];
+    for (int a = 0; a < 3; ++a) {
+      bl[a] = at.lo[a] + te.s[a] * g.n[a] - (o[a] - g.m[a]);   // box corner in U-local coords
+      lo[a] = max(0, bl[a]);
+      hi[a] = min(g.U[a], bl[a] + at.dim[a]);
+    }
+    const int nx = max(0, hi[0] - lo[0]), ny = max(0, hi[1] - lo[1]);
+    const float hx = float(g.h[0]), hy = float(g.h[1]), hz = float(g.h[2]);
+    const int dx = at.dim[0], dxy = at.dim[0] * at.dim[1], nchp = at.nchp;
+    for (int c0 = 0; c0 < at.nch; c0 += 4) {
+      Real acc[4][4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        for (int q = 0; q < 4; ++q) acc[c][q] = Real(0);
+      for (int col = lane; col < nx * ny; col += kProjThreads / 2) {
+        const int lx = lo[0] + col % nx, ly = lo[1] + col / nx;
+        const float px = float(lx - bl[0]) * hx + at.dlo[0], py = float(ly - bl[1]) * hy + at.dlo[1];
+        const float r2 = rc2 - px * px - py * py;
+        if (r2 < 0.f) continue;
+        const float zc = sqrtf(r2) * (1.f + 1e-6f);
+        const int z0 = max(lo[2], bl[2] + int(ceilf((-zc - at.dlo[2]) / hz - 1e-3f)));
+        const int z1 = min(hi[2] - 1, bl[2] + int(floorf((zc - at.dlo[2]) / hz + 1e-3f)));
+        const Real* tp = T + ((size_t)(z0 * g.U[1] + ly) * g.U[0] + lx) * B + 4 * half;
+        const Real* cp = chi + at.off + ((long long)(z0 - bl[2]) * dxy + (ly - bl[1]) * dx + (lx - bl[0])) * nchp + c0;
+        const size_t ts = (size_t)g.U[1] * g.U[0] * B, cs = (size_t)dxy * nchp;
+#pragma unroll 4
+        for (int z = z0; z <= z1; ++z, tp += ts, cp += cs) {
+          Real tv[4], cv[4];
+          load4(tp, tv);
+          load4(cp, cv);
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[c][q] += cv[c] * tv[q];
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        for (int q = 0; q < 4; ++q) red[4 * c + q][threadIdx.x] = acc[c][q];
+      __syncthreads();
+      // 32 sums (channel, node) of 64 threads each, four lanes per sum
+      const int k2 = threadIdx.x >> 2, sub = threadIdx.x & 3, c = k2 >> 3, q = k2 & 7;
+      double s = 0.0;
+      for (int th = (q >> 2) + 2 * sub; th < kProjThreads; th += 8) s += double(red[4 * c + (q & 3)][th]);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      if (sub == 0 && c0 + c < at.nch) Pt[(size_t)(te.row0 + c0 + c) * B + q] = Real(s * chs[6 * (at.ch0 + c0 + c)]);
+    }
   }
 }
 
-// out = H_q v on every node window of the wave (zero outside the windows); P from k_project. One
-// block per (brick row: 4 y- and 4 z-planes of the window, all x; tile), so the few sample tiles
-// of the Lanczos bounds still spread over the GPU.
+// out = H_q v on every node window of the wave (zero outside the windows); P from k_project. One block
+// per (4^3 brick of the window, tile): a warp is one z-plane of the brick, a thread one point and four of
+// its nodes, so the brick's image records (table offset, 64-bit sphere mask) are warp-uniform and a
+// projector load serves four nodes. One thread per (point, node) that looked every image of
+// its brick up in the atom tables took 78 us for the 10 sample tiles of a 12^3 cell, 410 us for
+// its 216 tiles.
+constexpr int kApplyThreads = 128;
 template <typename Real>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kApplyThreads)
 k_apply_h(Geo g, Wave w, const Real* __restrict__ Tc, Real* __restrict__ Tn, const Real* __restrict__ P,
-          const Real* __restrict__ chi, const AtomTab* __restrict__ atoms, const TileEntry* __restrict__ entries,
-          const int* __restrict__ blist, const int* __restrict__ bn, const Real* __restrict__ v) {
-  const int row = blockIdx.x, tl = blockIdx.y, t = wave_tile(w, tl);
+          const Real* __restrict__ chi, const int4* __restrict__ brec, const int* __restrict__ bn, const Real* __restrict__ v) {
+  const int br = blockIdx.x, tl = blockIdx.y, t = wave_tile(w, tl), B = 8;
   int o[3];
   tile_origin(g, t, o);
-  const int Ux = g.U[0], Uy = g.U[1], Uz = g.U[2], B = g.B;
+  const int bx = br % g.nbr[0], by = (br / g.nbr[0]) % g.nbr[1], bz = br / (g.nbr[0] * g.nbr[1]);
+  const int half = threadIdx.x & 1, pa = (threadIdx.x >> 1) & 3, pb = (threadIdx.x >> 3) & 3, pc = threadIdx.x >> 5;
+  const int u[3] = {bx * kBrick + pa, by * kBrick + pb, bz * kBrick + pc};
+  const int Ux = g.U[0], Uy = g.U[1], Uz = g.U[2];
+  if (u[1] >= Uy || u[2] >= Uz) return;
   const size_t tbase = (size_t)tl * g.Upts * B;
   const Real* T = Tc + tbase;
-  const Real* Pt = P + (size_t)tl * g.r_cap * B;
-  const TileEntry* ent = entries + (size_t)tl * g.e_cap;
-  const int z0 = (row / g.nbr[1]) * kBrick, nz = min(kBrick, Uz - z0);
-  const int y0 = (row % g.nbr[1]) * kBrick, ny = min(kBrick, Uy - y0);
-  const int nel = Ux * ny * nz * B;
+  const Real* Pt = P + (size_t)tl * g.r_cap * B + 4 * half;
+  const size_t e = (size_t)((u[2] * Uy + u[1]) * Ux + u[0]) * B + 4 * half;
+  bool in[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int qo[3] = {q & 1, q >> 1, half};
+    in[q] = node_valid(g, o, qo) && in_window(g, qo, u[0], u[1], u[2]);
+  }
   const int st[3] = {B, Ux * B, Ux * Uy * B};
   const int Ua[3] = {Ux, Uy, Uz};
-  for (int i = threadIdx.x; i < nel; i += kThreads) {
-    const int p = i / B, q = i % B;
-    int qo[3];
-    node_offset(g, q, qo);
-    const int ux = p % Ux, uy = y0 + (p / Ux) % ny, uz = z0 + p / (Ux * ny);
-    const size_t e = (size_t)((uz * Uy + uy) * Ux + ux) * B + q;
-    if (!node_valid(g, o, qo) || !in_window(g, qo, ux, uy, uz)) {
-      Tn[tbase + e] = Real(0);
-      continue;
-    }
-    const Real tc = T[e];
-    Real y = Real(g.lap0) * tc;
-    const int u[3] = {ux, uy, uz};
-    for (int a = 0; a < 3; ++a)
-      for (int pp = 1; pp <= g.n_o; ++pp) {
-        const Real fp = (u[a] + pp < Ua[a]) ? T[e + (size_t)pp * st[a]] : Real(0);
-        const Real fm = (u[a] - pp >= 0) ? T[e - (size_t)pp * st[a]] : Real(0);
-        y += Real(g.lap[a][pp]) * (fp + fm);
-      }
-    const int ax = o[0] - g.m[0] + ux, ay = o[1] - g.m[1] + uy, az = o[2] - g.m[2] + uz;
-    int wx = ax % g.n[0]; if (wx < 0) wx += g.n[0];
-    int wy = ay % g.n[1]; if (wy < 0) wy += g.n[1];
-    int wz = az % g.n[2]; if (wz < 0) wz += g.n[2];
-    y += v[(wz * g.n[1] + wy) * g.n[0] + wx] * tc;
-    const int br = ((uz / kBrick) * g.nbr[1] + uy / kBrick) * g.nbr[0] + ux / kBrick;
-    const int* lst = blist + ((size_t)tl * g.nbricks + br) * g.br_cap;
-    const int nb = bn[(size_t)tl * g.nbricks + br];
-    for (int k = 0; k < nb; ++k) {
-      const TileEntry te = ent[lst[k]];
-      const AtomTab at = atoms[te.atom];
-      const int li = box_index(at, te.s, g.n, ax, ay, az);
-      if (li < 0) continue;
-      const Real* cr = chi_row(chi, at, li);
-      for (int c = 0; c < at.nch; ++c) y += cr[c] * Pt[(size_t)(te.row0 + c) * B + q];
-    }
-    Tn[tbase + e] = y;
+  Real tc[4], y[4];
+  load4(T + e, tc);
+  int wr[3];
+  for (int a = 0; a < 3; ++a) {
+    wr[a] = (o[a] - g.m[a] + u[a]) % g.n[a];
+    if (wr[a] < 0) wr[a] += g.n[a];
   }
+  const Real diag = Real(g.lap0) + v[(wr[2] * g.n[1] + wr[1]) * g.n[0] + wr[0]];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) y[q] = diag * tc[q];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    for (int pp = 1; pp <= g.n_o; ++pp) {
+      Real fp[4] = {Real(0), Real(0), Real(0), Real(0)}, fm[4] = {Real(0), Real(0), Real(0), Real(0)};
+      if (u[a] + pp < Ua[a]) load4(T + e + (size_t)pp * st[a], fp);
+      if (u[a] - pp >= 0) load4(T + e - (size_t)pp * st[a], fm);
+      const Real wl = Real(g.lap[a][pp]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) y[q] += wl * (fp[q] + fm[q]);
+    }
+  const int4* rb = brec + ((size_t)tl * g.nbricks + br) * g.br_cap * 2;
+  const int nb = bn[(size_t)tl * g.nbricks + br];
+  const int bit = pa + 4 * pb + 16 * (pc & 1);
+  for (int k = 0; k < nb; ++k) {
+    const int4 r0 = rb[2 * k], r1 = rb[2 * k + 1];
+    if (!((unsigned(pc < 2 ? r1.z : r1.w) >> bit) & 1u)) continue;
+    const int nch = r0.w & 0xff, nchp = (r0.w >> 8) & 0xff;
+    const Real* cp = chi + r0.x + ((pc * r1.y + pb) * r1.x + pa) * nchp;
+    for (int c0 = 0; c0 < nch; c0 += 4) {
+      Real cv[4];
+      load4(cp + c0, cv);
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c0 + c < nch) {
+          Real pv[4];
+          load4(Pt + (size_t)(r0.y + c0 + c) * B, pv);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) y[q] += cv[c] * pv[q];
+        }
+    }
+  }
+  typename V4<Real>::T out;
+  out.x = in[0] ? y[0] : Real(0);
+  out.y = in[1] ? y[1] : Real(0);
+  out.z = in[2] ? y[2] : Real(0);
+  out.w = in[3] ? y[3] : Real(0);
+  *reinterpret_cast<typename V4<Real>::T*>(Tn + tbase + e) = out;
 }
 
 // ------------------------------------------------------------------------------ sweep step
@@ -150,19 +209,6 @@ template <> struct Coef<double> {
   static __device__ __forceinline__ double lap(const Geo& g, int a, int p) { return g.lap[a][p]; }
   static __device__ __forceinline__ double grd(const Geo& g, int a, int p) { return g.grd[a][p]; }
 };
-
-template <typename Real> struct V4;
-template <> struct V4<float> { using T = float4; };
-template <> struct V4<double> { using T = double4_32a; };
-
-template <typename Real>
-__device__ __forceinline__ void load4(const Real* p, Real out[4]) {
-  const typename V4<Real>::T x = *reinterpret_cast<const typename V4<Real>::T*>(p);
-  out[0] = x.x;
-  out[1] = x.y;
-  out[2] = x.z;
-  out[3] = x.w;
-}
 
 constexpr int kTileB = 8;   // nodes per tile (2 x 2 x 2); one warp = 4 points x 8 nodes
 
@@ -951,11 +997,10 @@ static int apply_h_t(sq_handle* h, const Wave& w, const Real* v, Real* out, Real
                      const WaveBufs& b) {
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
-  k_project<Real><<<dim3(g.e_cap, w.ntiles), kThreads, 0, s>>>(g, w, v, chi, h->d.atoms, h->d.gdv, b.entries,
-                                                               b.n_entries, P);
+  k_project<Real><<<dim3(std::min(g.e_cap, 256), w.ntiles), kProjThreads, 0, s>>>(
+      g, w, v, chi, h->d.atoms, h->d.rcmax, h->d.gdv, b.entries, b.n_entries, P);
   SQ_LAUNCH_CHECK(h);
-  k_apply_h<Real><<<dim3(g.nbr[2] * g.nbr[1], w.ntiles), kThreads, 0, s>>>(g, w, v, out, P, chi, h->d.atoms, b.entries,
-                                                               b.brick_list, b.brick_n, vpot);
+  k_apply_h<Real><<<dim3(g.nbricks, w.ntiles), kApplyThreads, 0, s>>>(g, w, v, out, P, chi, b.brick_rec, b.brick_n, vpot);
   SQ_LAUNCH_CHECK(h);
   return SQ_OK;
 }
