@@ -138,6 +138,7 @@ struct Plan {
   int tile_begin = 0, tile_end = 0;   // the tiles this handle sweeps (the node partition)
   int lz_cap = 0;                     // most Lanczos sample tiles any V_eff can select
   int nlz_wave = 0;                   // tiles per Lanczos wave of the per-node bounds
+  size_t part_floats = 0, table_cap = 0, head_cap = 0;   // partial projections and brick tables of the split mixed step
 };
 
 // Sample nodes of the Lanczos bounds: argmin V, argmax V and a stride-n/2 node grid; their
@@ -269,7 +270,7 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
     // capacity bounds: images of this atom that can meet a window of extent W on axis a
     long long nimg_u = 1, nimg_b = 1;
     for (int a = 0; a < 3; ++a) {
-      nimg_u *= floor_div(g.U[a] + dmax[a] - 2, g.n[a]) + 1;
+      nimg_u *= floor_div(sq::kBrick * g.nbr[a] + dmax[a] - 2, g.n[a]) + 1;   // whole bricks of the window
       nimg_b *= floor_div(sq::kBrick + dmax[a] - 2, g.n[a]) + 1;
     }
     if (at.nch == 0) { nimg_u = nimg_b = 0; }
@@ -294,8 +295,12 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
                      3 * size_t(g.Upts) * tileB * real +        // W
                      2 * size_t(g.r_cap) * tileB * real +       // A, P
                      2 * size_t(g.r_cap) * tileB * sizeof(double) +   // Pg ping-pong (FP64)
-                     size_t(g.nslab) * tileB * 9 * sizeof(double) +
+                     size_t(std::max(g.nslab, sq::stencil_chunks(g))) * tileB * 9 * sizeof(double) +
                      size_t(g.nslab) * (size_t(g.r_cap) + 1) * sizeof(int);   // slab row maps
+  int max_nch = 1;
+  for (const sq::AtomTab& at : P.atoms) max_nch = std::max(max_nch, at.nch);
+  const bool split = d->precision == SQ_MIXED && max_nch <= 4;   // the split mixed step
+  if (split) P.per_tile_bytes += (size_t(g.e_cap) + 1 + size_t(g.nbricks) * g.br_cap) * sizeof(int);   // image -> brick index
   long long Nd = (long long)g.n[0] * g.n[1] * g.n[2];
   int M = d->cheb_quad_M > 0 ? d->cheb_quad_M : 2048;
   P.fixed_bytes = size_t(Nd) * (sizeof(double) + sizeof(float)) +                       // V
@@ -342,6 +347,25 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
   const long long nwaves = (ntl + wc - 1) / wc;
   P.wave_cap = int((ntl + nwaves - 1) / nwaves);
   P.wave_cap = std::max<int>(P.wave_cap, P.lz_cap);
+  if (split) {
+    // partial projections of the whole wave, at most 4 GiB (the sweep then takes the tiles in chunks), at least
+    // one tile of the fullest bricks possible, and brick tables; sized for 2.5 times the mean number of
+    // images whose sphere meets a brick (Steiner's formula for the sphere and the box) plus 16, which
+    // uniform and clustered atoms stay below (fuller bricks take k_step)
+    double mean = 0.0;
+    const double a = sq::kBrick * g.h[0], b = sq::kBrick * g.h[1], c = sq::kBrick * g.h[2];
+    for (double r : P.rcmax)
+      mean += (a * b * c + 2.0 * (a * b + b * c + c * a) * r + M_PI * (a + b + c) * r * r + 4.0 / 3.0 * M_PI * r * r * r) /
+              (d->L[0] * d->L[1] * d->L[2]);
+    const int imgs = int(std::min<double>(g.br_cap, std::ceil(2.5 * mean) + 16.0));
+    const size_t rows = size_t(sq::nl_rows_padded(imgs, max_nch)), rows_top = size_t(sq::nl_rows_padded(g.br_cap, max_nch));
+    P.part_floats = std::max(std::min(size_t(P.wave_cap) * g.nbricks * rows * tileB, size_t(1) << 30),
+                             size_t(g.nbricks) * rows_top * tileB);
+    const size_t bricks = sq::nl_bricks_max(g, P.wave_cap);
+    P.table_cap = bricks * rows * 64 * sizeof(float2);
+    P.head_cap = bricks * (2 + size_t(g.br_cap));
+    P.fixed_bytes += P.part_floats * sizeof(float) + size_t(ch) * sizeof(float2) + P.table_cap + P.head_cap * sizeof(int);
+  }
   if (d->bounds_mode == SQ_BOUNDS_PER_NODE) {
     // every node's own Lanczos: waves of tiles with k + 2 Krylov vectors each under 8 GiB, the
     // per-node interval and step coefficients, the Fermi-search cosine sums and contraction rows
@@ -469,6 +493,10 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   h->nlz_wave = P.nlz_wave;
   h->proj4 = true;
   for (const sq::AtomTab& at : P.atoms) h->proj4 = h->proj4 && at.nchp <= 4;
+  for (const sq::AtomTab& at : P.atoms) h->max_nch = std::max(h->max_nch, at.nch);
+  h->part_floats = P.part_floats;
+  h->table_cap = P.table_cap;
+  h->head_cap = P.head_cap;
   h->table_len = P.table_len;
   h->n_ch_total = int(P.ch_l.size());
   h->wave_cap = P.wave_cap;
@@ -483,6 +511,7 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   if (const char* env = std::getenv("SQ_STEP_SMEM_ROWS")) {
     const long v = std::strtol(env, nullptr, 10);
     if (v >= 0 && v < h->step_rows_cap) h->step_rows_cap = int(v);
+    h->step_rows_env = true;
   }
   // SQ_STEP_KERNEL=staged selects the TMA-staged step for a mixed sweep (sq_step_tma.cu; slower than
   // the default step kernel on the workloads measured, kept for comparison), SQ_STAGE_RECS its
@@ -550,7 +579,15 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   SQ_ALLOC(h->wb.P, real * size_t(wt) * g.r_cap * g.B);
   SQ_ALLOC(h->wb.Pg[0], sizeof(double) * size_t(wt) * g.r_cap * g.B);   // projections: FP64 sums
   SQ_ALLOC(h->wb.Pg[1], sizeof(double) * size_t(wt) * g.r_cap * g.B);
-  SQ_ALLOC(h->wb.Spart, sizeof(double) * size_t(wt) * g.nslab * g.B * 9);
+  SQ_ALLOC(h->wb.Spart, sizeof(double) * size_t(wt) * std::max(g.nslab, sq::stencil_chunks(g)) * g.B * 9);
+  if (h->part_floats > 0) {
+    SQ_ALLOC(h->wb.proj_start, sizeof(int) * size_t(wt) * (size_t(g.e_cap) + 1));
+    SQ_ALLOC(h->wb.proj_idx, sizeof(unsigned) * size_t(wt) * g.nbricks * g.br_cap);
+    SQ_ALLOC(h->wb.Part, sizeof(float) * h->part_floats);
+    SQ_ALLOC(h->wb.nl_X, h->table_cap);
+    SQ_ALLOC(h->wb.nl_head, sizeof(int) * h->head_cap);
+    SQ_ALLOC(h->d.gdvp, sizeof(float2) * std::max(1, h->n_ch_total));
+  }
   if (!h->lanczos_tiles.empty()) {
     const size_t nst = size_t(P.lz_cap);
     const int k = h->lanczos_k;
@@ -619,6 +656,9 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   SQ_H2D(h->d.gdv64, g64.data(), sizeof(double) * g64.size());
   if (!P.rcmax.empty()) SQ_H2D(h->d.rcmax, P.rcmax.data(), sizeof(double) * P.rcmax.size());
   SQ_H2D(h->d.gdv32, g32.data(), sizeof(float) * g32.size());
+  std::vector<float2> gp(g32.size(), make_float2(0.f, 0.f));
+  for (int c = 0; c < h->n_ch_total; ++c) gp[c] = make_float2(g32[c], float(g64[c] - double(g32[c])));
+  if (h->d.gdvp) SQ_H2D(h->d.gdvp, gp.data(), sizeof(float2) * gp.size());
   if (!h->lanczos_tiles.empty())
     SQ_H2D(h->d.lz_tiles, h->lanczos_tiles.data(), sizeof(int) * h->lanczos_tiles.size());
   double sc[64];

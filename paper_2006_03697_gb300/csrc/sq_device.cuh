@@ -37,11 +37,14 @@ __device__ __forceinline__ bool in_window(const Geo& g, const int qo[3], int ux,
          (unsigned)(uz - qo[2]) <= (unsigned)(2 * g.m[2]);
 }
 
-// x = hi + lo with hi, lo TF32 values (11 significant bits each, held in FP32 registers)
+// x = hi + lo with hi, lo TF32 values (11 significant bits each, held in FP32 registers): hi by Dekker's
+// split (x rounded to 24 - 13 bits), lo, exact in 12 bits and a sign, rounded to 11 by half an ulp and a mask.
+// Six cheap instructions; cvt.rna.tf32 expands to about a dozen integer ones on this part and made the
+// splits the largest share of the projector kernels' instructions. A NaN stays one through hi.
 __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(x));
-  const float r = x - __uint_as_float(hi);
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(r));
+  const float t = __fmul_rn(x, 8193.f), h = __fsub_rn(t, __fsub_rn(t, x));
+  hi = __float_as_uint(h);
+  lo = (__float_as_uint(__fsub_rn(x, h)) + 0x1000u) & 0xffffe000u;
 }
 
 // d (16 x 8, FP32) += a (16 x 8, TF32, row) * b (8 x 8, TF32, col); fragment of lane (g, t),

@@ -117,7 +117,12 @@ struct WaveBufs {
   void* A = nullptr;              // Real [wt][r_cap][B]  chi_row(x_q)
   void* P = nullptr;              // Real [wt][r_cap][B]  gamma |dOmega| chi^T t (Lanczos apply)
   void* Pg[2] = {nullptr, nullptr};   // double [wt][r_cap][B]  gamma |dOmega| chi^T t^j, ping-pong
-  double* Spart = nullptr;        // [wt][nslab][B][9]
+  double* Spart = nullptr;        // [wt][slabs or stencil row chunks][B][9]
+  int* proj_start = nullptr;      // [wt][e_cap + 1] split mixed step: an image's entries of proj_idx
+  unsigned* proj_idx = nullptr;   // [wt][nbricks * br_cap] brick << 16 | first projector row in the brick
+  int* nl_head = nullptr;         // per absolute brick: images, rows, rows of the images (k_nl_table)
+  float2* nl_X = nullptr;         // per absolute brick: [rows][64 points] projector values, TF32 (hi, lo)
+  float* Part = nullptr;          // partial projections of a chunk of tiles [tiles][nbricks][rows][B]
 };
 
 struct Dev {
@@ -128,6 +133,7 @@ struct Dev {
   double* gdv64 = nullptr;        // gamma * dV per channel
   double* rcmax = nullptr;        // per atom: largest projector radius
   float* gdv32 = nullptr;
+  float2* gdvp = nullptr;         // gamma * dV per channel as a pair of floats
   double* chi64 = nullptr;        // projector tables
   float* chi32 = nullptr;
   float* chi32s = nullptr;        // mixed: each FP32 table value as a TF32 (hi, lo) pair
@@ -205,8 +211,7 @@ struct sq_handle {
   long long lz_lists_epoch = -1;    // atom epoch of the Lanczos sample tiles' lists in lzb
   std::vector<int> lanczos_tiles;
   long long launches = 0;
-  // step-kernel launches by variant: [0] projections staged in shared memory, tensor-core
-  // projector phases; [1] shared memory, scalar phases; [2] projections in global memory;
+  // step-kernel launches by variant: [0] the split mixed step; [1] shared memory, scalar phases; [2] projections in global memory;
   // [3] the TMA-staged step (sq_step_tma.cu)
   long long step_variant[4] = {0, 0, 0, 0};
   // tensor maps of the TMA-staged step: t buffers (x, y, z sticks, brick), W, projector tables
@@ -218,6 +223,10 @@ struct sq_handle {
   int stage_recs_cap = 16;          // SQ_STAGE_RECS: atom images per stage of the staged step
   bool stage_wait_test = false;     // SQ_STAGE_WAIT_TEST=1: the staged step's copy wait runs out (tests)
   int step_rows_cap = 0;            // most projector rows a step block stages in shared memory
+  bool step_rows_env = false;       // SQ_STEP_SMEM_ROWS was given
+  size_t part_floats = 0;           // floats of wb.Part
+  size_t table_cap = 0, head_cap = 0;   // bytes of wb.nl_X, ints of wb.nl_head
+  int max_nch = 1;                  // most projector channels of an atom
   int step_warps = 0;               // warps per step block (0: the brick-count rule; set by the tuner)
   // optional event timing of the sweep kernels
   bool timing = false;
@@ -258,6 +267,22 @@ int make_step_maps(sq_handle* h);
 size_t step_tma_smem_bytes(int rows, int cap_rec);
 int launch_step_tma(sq_handle* h, const Wave& w, dim3 grid, int ic, int ip, float* Tn, const double* Pg, double* Pgn,
                     int mode, int rows, int cap_rec);
+// the split FP32 step (sq_step_mixed.cu): rows of a tile per stencil block and blocks per tile, the brick
+// tables of a wave, the step on t buffers (P^j in wb.Pg), and the projections of a new column
+// (TF32 planes in wb.Pg[1], float pairs in wb.Pg[0])
+int stencil_rows(const Geo& g);
+int stencil_chunks(const Geo& g);
+int build_nl_tables(sq_handle* h, size_t wi);
+int launch_step_mixed(sq_handle* h, size_t wi, const float* Tc, const float* Tp, float* Tn, int mode);
+int launch_project_mixed(sq_handle* h, size_t wi, const float* T);
+// table rows of a brick of imgs images: whole MMA tiles and 16 rows of zeros
+inline int nl_rows_padded(int imgs, int max_nch) { return (imgs * max_nch + 15) / 16 * 16 + 16; }
+size_t nl_bricks_max(const Geo& g, int wave_cap);
+// floats from the hi to the lo plane of the split projections in wb.Pg[1]
+inline size_t nl_plane(const sq_handle* h) { return size_t(h->wave_cap) * h->geo.r_cap * 8; }
+bool nl_fits(const sq_handle* h, size_t wi);   // do the wave's tables fit their buffers?
+// does the split step run wave wi?
+bool use_split(const sq_handle* h, size_t wi);
 // one recurrence step launch (mode 1) of wave 0 with the handle's current settings, timed with
 // CUDA events on its stream (sq_sweep.cu; the autotuner's measurement)
 int time_step_launch(sq_handle* h, int reps, double* ms_out);
@@ -287,10 +312,10 @@ int timing_collect(sq_handle* h);
 // setup kernels (sq_setup.cu)
 int build_tables(sq_handle* h);
 int init_node_tables(sq_handle* h);   // cosine table; per-node bounds mode: neutral node bounds
-// the lists, A, W and t^0 of a wave in wb; with reuse, the lists and W of the same wave and atom
+// the lists, A, W and t^0 of wave wi in wb; with reuse, the lists and W of the same wave and atom
 // positions built by the previous sweep are kept (only A, the projection buffers and t^0 are
 // rewritten)
-int build_wave_lists(sq_handle* h, const Wave& w, bool reuse);
+int build_wave_lists(sq_handle* h, size_t wi, bool reuse);
 
 // sweep (sq_sweep.cu)
 int run_sweep(sq_handle* h);

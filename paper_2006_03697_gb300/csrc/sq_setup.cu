@@ -56,7 +56,7 @@ __global__ void k_tile_entries(Geo g, Wave w, const AtomTab* __restrict__ atoms,
   int ulo[3], uhi[3];
   for (int a = 0; a < 3; ++a) {
     ulo[a] = o[a] - g.m[a];
-    uhi[a] = ulo[a] + g.U[a] - 1;
+    uhi[a] = ulo[a] + kBrick * g.nbr[a] - 1;   // whole bricks: tiles that share a brick list the same images
   }
   TileEntry* out = entries + (size_t)tl * g.e_cap;
   int base_e = 0, base_r = 0;
@@ -141,12 +141,12 @@ __global__ void k_brick_lists(Geo g, Wave w, const AtomTab* __restrict__ atoms, 
   tile_origin(g, t, o);
   const int bx = br % g.nbr[0], by = (br / g.nbr[0]) % g.nbr[1], bz = br / (g.nbr[0] * g.nbr[1]);
   const int bl[3] = {o[0] - g.m[0] + bx * kBrick, o[1] - g.m[1] + by * kBrick, o[2] - g.m[2] + bz * kBrick};
-  const int bhi[3] = {o[0] - g.m[0] + min(g.U[0], (bx + 1) * kBrick) - 1,
-                      o[1] - g.m[1] + min(g.U[1], (by + 1) * kBrick) - 1,
-                      o[2] - g.m[2] + min(g.U[2], (bz + 1) * kBrick) - 1};
+  // whole bricks, also past the window's edge (points outside it hold zero columns), so that the tiles that
+  // share a brick of absolute lattice points have the same records for it
+  const int bhi[3] = {bl[0] + kBrick - 1, bl[1] + kBrick - 1, bl[2] + kBrick - 1};
   // the slab: all of U in x and z, the brick's planes in y
   const int sl[3] = {o[0] - g.m[0], bl[1], o[2] - g.m[2]};
-  const int shi[3] = {o[0] - g.m[0] + g.U[0] - 1, bhi[1], o[2] - g.m[2] + g.U[2] - 1};
+  const int shi[3] = {sl[0] + kBrick * g.nbr[0] - 1, bhi[1], sl[2] + kBrick * g.nbr[2] - 1};
   const bool slab_writer = (bx == 0 && bz == 0);
   int* smap = slab_map + ((size_t)tl * g.nslab + by) * g.r_cap;
   const int ne = n_entries[tl];
@@ -201,7 +201,7 @@ __global__ void k_brick_lists(Geo g, Wave w, const AtomTab* __restrict__ atoms, 
         float r2 = 0.f;
         for (int a = 0; a < 3; ++a) {
           const int l = l0[a] + pl[a];
-          in = in && (bl[a] + pl[a] <= bhi[a]) && l >= 0 && l < ats.dim[a];
+          in = in && l >= 0 && l < ats.dim[a];
           const float d = float(l) * float(g.h[a]) + ats.dlo[a];   // (lo + l) h - R, box-relative
           r2 += d * d;
         }
@@ -234,12 +234,14 @@ __global__ void k_brick_lists(Geo g, Wave w, const AtomTab* __restrict__ atoms, 
 }
 
 // A[row][q] = chi_row(x_q) (w_q^T V_nl,q = sum_rows gamma |dOmega| A chi_row^T), the
-// projections of t^0 = w_q, Pg0 = gamma |dOmega| A, and a zeroed accumulator Pg1.
+// projections of t^0 = w_q, Pg0 = gamma |dOmega| A, and a zeroed accumulator Pg1. The split mixed step
+// (lo_plane != 0) keeps the projections as a pair of floats in Pg0's slots and, rounded to FP32, as TF32
+// hi and lo planes in Pg1's buffer.
 template <typename Real>
 __global__ void k_atable(Geo g, Wave w, const AtomTab* __restrict__ atoms, const double* __restrict__ chs,
                          const Real* __restrict__ chi, const TileEntry* __restrict__ entries,
                          const int* __restrict__ n_entries, Real* __restrict__ A, double* __restrict__ Pg0_,
-                         double* __restrict__ Pg1_) {
+                         double* __restrict__ Pg1_, size_t lo_plane) {
   const int tl = blockIdx.x, t = wave_tile(w, tl);
   int o[3];
   tile_origin(g, t, o);
@@ -260,8 +262,20 @@ __global__ void k_atable(Geo g, Wave w, const AtomTab* __restrict__ atoms, const
     for (int c = 0; c < at.nch; ++c) {
       const double x = (li >= 0) ? double(chi_row(chi, at, li)[c]) : 0.0;
       At[(size_t)(te.row0 + c) * g.B + q] = Real(x);
-      Pg0[(size_t)(te.row0 + c) * g.B + q] = chs[6 * (at.ch0 + c)] * x;   // gamma |dOmega| chi^T t^0
-      Pg1[(size_t)(te.row0 + c) * g.B + q] = 0.0;
+      const size_t k = (size_t)(te.row0 + c) * g.B + q;
+      const double p = chs[6 * (at.ch0 + c)] * x;   // gamma |dOmega| chi^T t^0
+      if (lo_plane) {
+        const float r = float(p);
+        uint32_t hi, lo;
+        split_tf32(r, hi, lo);
+        reinterpret_cast<float2*>(Pg0)[k] = make_float2(r, float(p - double(r)));
+        float* Pf = reinterpret_cast<float*>(Pg1_) + (size_t)tl * g.r_cap * g.B + k;
+        Pf[0] = __uint_as_float(hi);
+        Pf[lo_plane] = __uint_as_float(lo);
+      } else {
+        Pg0[k] = p;
+        Pg1[k] = 0.0;
+      }
     }
   }
 }
@@ -383,8 +397,9 @@ __global__ void k_init_t0(Geo g, Wave w, Real* __restrict__ T0) {
 }
 
 template <typename Real>
-static int wave_lists_t(sq_handle* h, const Wave& w, bool reuse, const Real* chi, const Real* gdvR, Real* A, Real* W,
+static int wave_lists_t(sq_handle* h, size_t wi, bool reuse, const Real* chi, const Real* gdvR, Real* A, Real* W,
                         Real* T0) {
+  const Wave& w = h->waves[wi];
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
   const sq_handle::ListsKey& key = h->lists_key;
@@ -392,10 +407,12 @@ static int wave_lists_t(sq_handle* h, const Wave& w, bool reuse, const Real* chi
                     key.epoch == h->atoms_epoch;
   if (!same) {
     int rc = build_wave_entries(h, w);
+    if (rc == SQ_OK && use_split(h, wi)) rc = build_nl_tables(h, wi);
     if (rc != SQ_OK) return rc;
   }
   k_atable<Real><<<w.ntiles, 256, 0, s>>>(g, w, h->d.atoms, h->d.gdv, chi, h->wb.entries, h->wb.n_entries, A,
-                                          (double*)h->wb.Pg[0], (double*)h->wb.Pg[1]);
+                                          (double*)h->wb.Pg[0], (double*)h->wb.Pg[1],
+                                          use_split(h, wi) ? nl_plane(h) : 0);
   SQ_LAUNCH_CHECK(h);
   if (!same) {
     k_wtable<Real><<<dim3(g.nbr[2], w.ntiles), 224, 0, s>>>(g, w, h->d.atoms, gdvR, chi, h->wb.entries,
@@ -463,11 +480,11 @@ int init_node_tables(sq_handle* h) {
   return SQ_OK;
 }
 
-int build_wave_lists(sq_handle* h, const Wave& w, bool reuse) {
+int build_wave_lists(sq_handle* h, size_t wi, bool reuse) {
   if (h->precision == SQ_FP64)
-    return wave_lists_t<double>(h, w, reuse, h->d.chi64, h->d.gdv64, (double*)h->wb.A, (double*)h->wb.W,
+    return wave_lists_t<double>(h, wi, reuse, h->d.chi64, h->d.gdv64, (double*)h->wb.A, (double*)h->wb.W,
                                 (double*)h->wb.T[0]);
-  return wave_lists_t<float>(h, w, reuse, h->d.chi32, h->d.gdv32, (float*)h->wb.A, (float*)h->wb.W,
+  return wave_lists_t<float>(h, wi, reuse, h->d.chi32, h->d.gdv32, (float*)h->wb.A, (float*)h->wb.W,
                              (float*)h->wb.T[0]);
 }
 

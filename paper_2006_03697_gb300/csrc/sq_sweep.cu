@@ -4,22 +4,21 @@
 // and the per-node moments rho^j, K^j_ab, N^j, S^j_ab of each column.
 //
 // Kernels (Real = double for SQ_FP64, float for SQ_MIXED; node sums always FP64):
-//   k_step      one block per (z-slab of 4 planes, tile), 4..8 warps; each warp walks whole
-//               4^3 bricks, so the atom-image records of a brick (table offset, 64-bit mask of
-//               the points inside the support sphere) are warp-uniform. Per brick:
-//               A  the nonlocal apply sum_rows chi_row(u) Pg^j (Pg^j staged in shared memory);
-//                  SQ_MIXED: a TF32 tensor-core product over the brick (3-term hi/lo split,
-//                  tables stored pre-split), SQ_FP64: scalar and record-major;
+//   k_step      SQ_FP64, and SQ_MIXED with more than 4 projector channels per atom (SQ_MIXED otherwise
+//               takes the split step of sq_step_mixed.cu). One block per (y-row of bricks, tile), 4..8
+//               warps; each warp walks whole 4^3 bricks, so the atom-image records of a brick (table
+//               offset, 64-bit mask of the points inside the support sphere) are warp-uniform. Per brick:
+//               A  the nonlocal apply sum_rows chi_row(u) Pg^j (Pg^j staged in shared memory),
+//                  record-major;
 //               B  Laplacian + V + the apply, the window mask, the recurrence update and the
 //                  nonlocal-stress partial sum_u W_b (grad_a t^j) (the gradient taps reuse the
-//                  Laplacian loads); SQ_MIXED: two nodes per lane (8-byte loads);
-//               C  fused, the projections gamma |dOmega| chi^T t^{j+1} of the new column
-//                  (SQ_MIXED: the transposed tensor-core product; SQ_FP64: register sums and a
-//                  reduce-scatter over the point lanes), one shared-memory FP64 add per
+//                  Laplacian loads);
+//               C  fused, the projections gamma |dOmega| chi^T t^{j+1} of the new column (register
+//                  sums and a reduce-scatter over the point lanes), one shared-memory FP64 add per
 //                  (image, channel, node), one global add per row and node per slab.
 //   k_moments   one block per tile: rho^j, K^j (restricted grad_a grad_b at the node),
 //               N^j = sum_rows chi(x_q) Pg^j, S^j = sum of the slab partials; FP64 table
-//               row; then clears Pg^j, which accumulates the projections of step j + 1.
+//               row; then (k_step) clears Pg^j, which accumulates the projections of step j + 1.
 //   k_apply_h / k_project   plain H_q v for the Lanczos bounds (sweep precision).
 #include <algorithm>
 
@@ -212,17 +211,6 @@ template <> struct Coef<double> {
 
 constexpr int kTileB = 8;   // nodes per tile (2 x 2 x 2); one warp = 4 points x 8 nodes
 
-// ---- warp-level TF32 tensor-core products for the FP32 projector phases.
-// x = hi + lo with hi, lo TF32 (11 significant bits each); a product is taken as
-// hi*hi + hi*lo + lo*hi with FP32 accumulation (the lo*lo term, ~2^-22 relative, is dropped).
-
-// (mma_tf32: the warp-level m16n8k8 TF32 product, sq_device.cuh)
-
-__device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
-
-// the brick's t values in the per-warp shared array: point p = a + 4 b + 16 c, node q
-__device__ __forceinline__ int tn_index(int p, int q) { return (p >> 2) * 32 + (p & 3) * kTileB + q; }
-
 // mode 0: t^1 = Hhat t^0;  mode 1: t^{j+1} = 2 Hhat t^j - t^{j-1};  mode 2: moments only.
 // Each warp walks whole 4^3 bricks of the slab: iteration it covers brick points
 // (a, b, c) = (lane >> 3, it & 3, it >> 2) for node q = lane & 7, so the 4 x-points of an
@@ -245,11 +233,11 @@ static int step_warps(int bricks_per_slab) {
   return best;
 }
 
-template <typename Real, int NO, bool kSmemP, bool kMMA>
+template <typename Real, int NO, bool kSmemP>
 __global__ void __launch_bounds__(kStepThreads, sizeof(Real) == 4 ? 4 : 2)
 k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, Real* __restrict__ Tn,
        const double* __restrict__ Pg, double* __restrict__ Pg_next, const Real* __restrict__ Wt,
-       const Real* __restrict__ chi, const float* __restrict__ chis, const Real* __restrict__ gdv,
+       const Real* __restrict__ chi, const Real* __restrict__ gdv,
        const int4* __restrict__ brec, const int* __restrict__ slab_n, const int* __restrict__ slab_map, const int* __restrict__ bn,
        const Real* __restrict__ v, const double* __restrict__ scal, int mode, double* __restrict__ Spart,
        int rows_smem, const double* __restrict__ ncoef, int* __restrict__ status) {
@@ -313,48 +301,20 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
   qo[1] = (q >> 1) & 1;
   qo[2] = q >> 2;
   const bool valid = node_valid(g, o, qo);
-  // step coefficients of the lane's node(s): the block's (shared bounds) or each node's own
-  // (per-node bounds; paired phase: nodes 2 np2 and 2 np2 + 1, scalar phase: node q)
-  Real caA = ca, cdA = cd, caB = ca, cdB = cd;
-  if (ncoef) {
-    auto own = [&](int qx, int qy, int qz, Real& c_a, Real& c_d) {
-      const int qq[3] = {qx, qy, qz};
-      if (!node_valid(g, o, qq)) return;
-      const int node = (o[0] + qx) + g.n[0] * ((o[1] + qy) + g.n[1] * (o[2] + qz));
-      c_a = Real(f * ncoef[2 * node]);
-      c_d = Real(f * ncoef[2 * node + 1]);
-    };
-    if constexpr (kMMA) {
-      const int p2 = lane & 3;
-      own(0, p2 & 1, p2 >> 1, caA, cdA);
-      own(1, p2 & 1, p2 >> 1, caB, cdB);
-    } else {
-      own(qo[0], qo[1], qo[2], caA, cdA);
-    }
+  // step coefficients of the lane's node: the block's (shared bounds) or the node's own
+  // (per-node bounds)
+  Real caA = ca, cdA = cd;
+  if (ncoef && valid) {
+    const int node = (o[0] + qo[0]) + g.n[0] * ((o[1] + qo[1]) + g.n[1] * (o[2] + qo[2]));
+    caA = Real(f * ncoef[2 * node]);
+    cdA = Real(f * ncoef[2 * node + 1]);
   }
   const Real* Wq = Wt + (size_t)tl * 3 * g.Upts * kTileB;
   const size_t wstr = (size_t)g.Upts * kTileB;
-  // S partial sums: per lane across bricks (scalar path); the paired phase B reduces them per
-  // brick over its point lanes into a per-warp FP32 array (red, read as floats), so no S
-  // registers stay live through the projector phases
+  // S partial sums, per lane across bricks
   Real sacc[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) sacc[k] = Real(0);
-  float* red32 = reinterpret_cast<float*>(red) + warp * kTileB * 9;
-  if constexpr (kMMA) {
-    for (int k = lane; k < kTileB * 9; k += 32) red32[k] = 0.f;
-    __syncwarp();
-  }
-  // paired phase B: lane = node pair np2 (nodes 2 np2, 2 np2 + 1: x offsets 0 and 1), x-point xa2,
-  // y parity yb2
-  const int np2 = lane & 3, xa2 = (lane >> 2) & 3, yb2 = lane >> 4;
-  const int qo2[3] = {0, np2 & 1, np2 >> 1};
-  bool valid2[2];
-  {
-    int qa[3] = {0, qo2[1], qo2[2]}, qb[3] = {1, qo2[1], qo2[2]};
-    valid2[0] = node_valid(g, o, qa);
-    valid2[1] = node_valid(g, o, qb);
-  }
   const int nbx = g.nbr[0], nby = g.nbr[1], nbz = g.nbr[2];
 
   for (int bi = warp; bi < nbx * nbz; bi += nw) {
@@ -363,56 +323,7 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
     const int4* rb = brec + ((size_t)tl * g.nbricks + br) * g.br_cap * 2;
     const int nb = bn[(size_t)tl * g.nbricks + br];
     Real* tnv = tn_sm + warp * 16 * 32 + lane;   // per lane and brick point: V_nl t^j, then t^{j+1}
-    if constexpr (kMMA) {
-      // phase A on tensor cores: Y[64 points][8 nodes] = X[64 points][4 nb rows] Pg^j[4 nb rows][8],
-      // X = the brick's projector values (zero outside each image's sphere). M = brick points
-      // (m-tile = one z-plane), N = the 8 nodes, K = 2 images x 4 channels per k-step, ordered so
-      // that each lane's A and B elements are two adjacent channels of one image:
-      // K = t -> (image k2 + t / 2, channel 2 (t % 2)), K = t + 4 -> the next channel.
-      const int g8 = lane >> 2, t4 = lane & 3, ch = 2 * (t4 & 1);
-      const int pa0 = g8 & 3, pb0 = g8 >> 2;         // lane's rows: points (pa0, pb0, c), (pa0, pb0 + 2, c)
-      float acc[4][4];
-#pragma unroll
-      for (int mt = 0; mt < 4; ++mt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[mt][i] = 0.f;
-      for (int k2 = 0; k2 < nb; k2 += 2) {
-        const int kr = k2 + (t4 >> 1);
-        int4 r0 = make_int4(0, 0, 0, 0), r1 = make_int4(0, 0, 0, 0);
-        if (kr < nb) {
-          r0 = rb[2 * kr];
-          r1 = rb[2 * kr + 1];
-        }
-        const int nch = r0.w & 0xff, prow = int(unsigned(r0.w) >> 16);
-        const float p0 = (ch < nch) ? float(Pstage[(prow + ch) * kTileB + g8]) : 0.f;
-        const float p1 = (ch + 1 < nch) ? float(Pstage[(prow + ch + 1) * kTileB + g8]) : 0.f;
-        uint32_t bh[2], bl[2];
-        split_tf32(p0, bh[0], bl[0]);
-        split_tf32(p1, bh[1], bl[1]);
-        const int dx = r1.x, plane = r1.x * r1.y * 4;
-        // (hi, lo) pairs of channels ch, ch + 1 at point (pa0, pb0, 0): one 16-byte load per point
-        // (FP32 values split in the kernel instead halve these bytes but measured 3.5 % slower)
-        const float* xb = chis + 2 * (r0.x + (pb0 * dx + pa0) * 4 + ch);
-        const unsigned mlo = unsigned(r1.z) >> g8, mhi = unsigned(r1.w) >> g8;
-#pragma unroll
-        for (int mt = 0; mt < 4; ++mt) {
-          const unsigned mw = (mt < 2) ? mlo : mhi;
-          const int sh = 16 * (mt & 1);
-          uint4 x0 = make_uint4(0u, 0u, 0u, 0u), x1 = make_uint4(0u, 0u, 0u, 0u);
-          if ((mw >> sh) & 1u) x0 = *reinterpret_cast<const uint4*>(xb + 2 * mt * plane);
-          if ((mw >> (sh + 8)) & 1u) x1 = *reinterpret_cast<const uint4*>(xb + 2 * (mt * plane + 8 * dx));
-          const uint32_t ah[4] = {x0.x, x1.x, x0.z, x1.z}, al[4] = {x0.y, x1.y, x0.w, x1.w};
-          mma_tf32(acc[mt], al, bh);   // small terms first
-          mma_tf32(acc[mt], ah, bl);
-          mma_tf32(acc[mt], ah, bh);
-        }
-      }
-      Real* tw = tn_sm + warp * 16 * 32;
-#pragma unroll
-      for (int mt = 0; mt < 4; ++mt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) tw[tn_index(16 * mt + g8 + 8 * (i >> 1), 2 * t4 + (i & 1))] = Real(acc[mt][i]);
-    } else {
+    {
       // phase A: nonlocal apply, record-major: sum_rows chi_row(u) Pg^j[row][q] for the lane's
       // 16 points; the table loads of one record are independent of each other
 #pragma unroll 1
@@ -446,81 +357,7 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
       }
     }
     __syncwarp();
-    if constexpr (kMMA) {
-      // phase B with two nodes per lane: lane = (node pair np, x-point xa, y parity yb); iteration
-      // it covers brick points (xa, 2 (it % 2) + yb, it / 2) for nodes 2 np and 2 np + 1, so every
-      // t / W load is an 8-byte pair and a brick takes 8 iterations (half the load round trips)
-      Real* tw = tn_sm + warp * 16 * 32;
-      float sb[18];   // S partials of nodes 2 np2 and 2 np2 + 1 over this brick
-#pragma unroll
-      for (int k = 0; k < 18; ++k) sb[k] = 0.f;
-#pragma unroll 1
-      for (int it = 0; it < 8; ++it) {
-        const int pb = 2 * (it & 1) + yb2, pc = it >> 1;
-        const int ux = bx * kBrick + xa2, uy = by * kBrick + pb, uz = bz * kBrick + pc;
-        const int p = xa2 + 4 * pb + 16 * pc;
-        const bool inU = (uy < Uy) && (uz < Uz);
-        const size_t e = (size_t)((uz * Uy + uy) * Ux + ux) * kTileB + 2 * np2;
-        const bool inyz = inU && (unsigned)(uy - qo2[1]) <= (unsigned)(2 * g.m[1]) &&
-                          (unsigned)(uz - qo2[2]) <= (unsigned)(2 * g.m[2]);
-        const bool in0 = inyz && valid2[0] && (unsigned)ux <= (unsigned)(2 * g.m[0]);
-        const bool in1 = inyz && valid2[1] && (unsigned)(ux - 1) <= (unsigned)(2 * g.m[0]);
-        float2 tn = make_float2(0.f, 0.f);
-        if (in0 || in1) {
-          const float2 w0 = ld2(Wq + e), w1 = ld2(Wq + wstr + e), w2 = ld2(Wq + 2 * wstr + e);
-          const float2 tp = (mode == 1) ? ld2(Tp + tbase + e) : make_float2(0.f, 0.f);
-          const float2 tc = ld2(T + e);
-          float2 y = make_float2(0.f, 0.f);           // off-diagonal part of H t^j
-          float2 gr[3];
-          const int u[3] = {ux, uy, uz};
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            gr[a] = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int pp = 1; pp <= NO; ++pp) {
-              const float2 fp = (u[a] + pp < Ua[a]) ? ld2(T + e + (size_t)pp * st[a]) : make_float2(0.f, 0.f);
-              const float2 fm = (u[a] - pp >= 0) ? ld2(T + e - (size_t)pp * st[a]) : make_float2(0.f, 0.f);
-              const float wl = Coef<float>::lap(g, a, pp), wg = Coef<float>::grd(g, a, pp);
-              y.x += wl * (fp.x + fm.x);
-              y.y += wl * (fp.y + fm.y);
-              gr[a].x += wg * (fp.x - fm.x);
-              gr[a].y += wg * (fp.y - fm.y);
-            }
-          }
-          const float vloc = float(v[wrz[uz] + wry[pb] + wrx[ux]]);
-          const float2 ynl = *reinterpret_cast<const float2*>(tw + tn_index(p, 2 * np2));   // phase A
-          y.x += ynl.x;
-          y.y += ynl.y;
-          if (mode != 2) {
-            const float dgA = float(cdA) + float(caA) * vloc, dgB = float(cdB) + float(caB) * vloc;
-            if (in0) tn.x = float(caA) * y.x + dgA * tc.x - float(cc) * tp.x;
-            if (in1) tn.y = float(caB) * y.y + dgB * tc.y - float(cc) * tp.y;
-            *reinterpret_cast<float2*>(Tn + tbase + e) = tn;
-          }
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {   // W is zero outside each node's window
-            sb[3 * a + 0] += gr[a].x * w0.x;
-            sb[3 * a + 1] += gr[a].x * w1.x;
-            sb[3 * a + 2] += gr[a].x * w2.x;
-            sb[9 + 3 * a + 0] += gr[a].y * w0.y;
-            sb[9 + 3 * a + 1] += gr[a].y * w1.y;
-            sb[9 + 3 * a + 2] += gr[a].y * w2.y;
-          }
-        } else if (inU && mode != 2) {
-          *reinterpret_cast<float2*>(Tn + tbase + e) = tn;
-        }
-        *reinterpret_cast<float2*>(tw + tn_index(p, 2 * np2)) = tn;
-      }
-      // the brick's S partials: sum over the 8 point lanes of each node pair, lanes 0..3 add
-#pragma unroll
-      for (int k = 0; k < 18; ++k) {
-        float sv = sb[k];
-        sv += __shfl_xor_sync(0xffffffffu, sv, 4);
-        sv += __shfl_xor_sync(0xffffffffu, sv, 8);
-        sv += __shfl_xor_sync(0xffffffffu, sv, 16);
-        if (lane < 4) red32[(2 * lane + k / 9) * 9 + k % 9] += sv;
-      }
-    } else {
+    {
 #pragma unroll 1
       for (int it = 0; it < 16; ++it) {
         const int pb = it & 3, pc = it >> 2;
@@ -571,54 +408,7 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
     // reduce-scatter over the 4 x-point lanes (xor 8, then xor 16) leaves lane (pa, q) with the
     // brick sum of channel c0 + pa for node q, so one FP64 conversion and one shared add per
     // lane cover 4 channels x 8 nodes (FP64 instructions are narrow on this part)
-    if constexpr (kMMA) {
-      if (project) {
-        // phase C on tensor cores: Pg^{j+1}[4 nb rows][8] += X^T[4 nb rows][64 points] t^{j+1}[64][8].
-        // M = 4 images x 4 channels per m-tile, ordered so each lane's A elements are two adjacent
-        // channels of one image (row g -> image m4 + g / 2, channel 2 (g % 2); row g + 8 -> the
-        // next channel), K = 8 brick points per k-step, N = the 8 nodes.
-        const int g8 = lane >> 2, t4 = lane & 3, ch = 2 * (g8 & 1);
-        const Real* tw = tn_sm + warp * 16 * 32;
-        // one m-tile (4 images) per pass; separate accumulators for the three split terms
-        // measured slower (more registers live across the gather loads), so one chain
-        for (int m4 = 0; m4 < nb; m4 += 4) {
-          const int kr = m4 + (g8 >> 1);
-          int4 r0 = make_int4(0, 0, 0, 0), r1 = make_int4(0, 0, 0, 0);
-          if (kr < nb) {
-            r0 = rb[2 * kr];
-            r1 = rb[2 * kr + 1];
-          }
-          const int dx = r1.x, dy = r1.y;
-          const float* xb = chis + 2 * (r0.x + t4 * 4 + ch);   // (hi, lo) pairs at point (t4, 0, 0)
-          const unsigned mlo = unsigned(r1.z) >> t4, mhi = unsigned(r1.w) >> t4;
-          float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-          for (int ks = 0; ks < 8; ++ks) {
-            // points p0 = 8 ks + t4 = (t4, 2 (ks % 2), ks / 2) and p1 = p0 + 4 (one row further in b)
-            const unsigned mw = (ks < 4) ? mlo : mhi;
-            const int sh = 8 * (ks & 3);
-            const float* xp = xb + 2 * ((ks >> 1) * dy + 2 * (ks & 1)) * dx * 4;
-            uint4 x0 = make_uint4(0u, 0u, 0u, 0u), x1 = make_uint4(0u, 0u, 0u, 0u);
-            if ((mw >> sh) & 1u) x0 = *reinterpret_cast<const uint4*>(xp);
-            if ((mw >> (sh + 4)) & 1u) x1 = *reinterpret_cast<const uint4*>(xp + 2 * dx * 4);
-            const uint32_t ah[4] = {x0.x, x0.z, x1.x, x1.z}, al[4] = {x0.y, x0.w, x1.y, x1.w};
-            uint32_t bh[2], bl[2];
-            split_tf32(float(tw[tn_index(8 * ks + t4, g8)]), bh[0], bl[0]);
-            split_tf32(float(tw[tn_index(8 * ks + t4 + 4, g8)]), bh[1], bl[1]);
-            mma_tf32(d, al, bh);
-            mma_tf32(d, ah, bl);
-            mma_tf32(d, ah, bh);
-          }
-          const int nch = r0.w & 0xff, prow = int(unsigned(r0.w) >> 16);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int cc = ch + (i >> 1);
-            if (cc < nch && d[i] != 0.f)
-              atomicAdd(&Ps[(prow + cc) * kTileB + 2 * t4 + (i & 1)], double(d[i] * float(gdv[r0.z + cc])));
-          }
-        }
-      }
-    } else {
+    {
       if (project) {
         const bool b0 = (pa & 1) != 0, b1 = (pa & 2) != 0;
         for (int k = 0; k < nb; ++k) {
@@ -655,22 +445,18 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
     }
   }
   // S partials: fixed-order reduction per node (the point lanes by shuffles, then warps)
-  if constexpr (!kMMA) {
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      double sv = double(sacc[k]);
-      sv += __shfl_xor_sync(0xffffffffu, sv, 8);
-      sv += __shfl_xor_sync(0xffffffffu, sv, 16);
-      if (lane < kTileB) red[(warp * kTileB + lane) * 9 + k] = sv;
-    }
+  for (int k = 0; k < 9; ++k) {
+    double sv = double(sacc[k]);
+    sv += __shfl_xor_sync(0xffffffffu, sv, 8);
+    sv += __shfl_xor_sync(0xffffffffu, sv, 16);
+    if (lane < kTileB) red[(warp * kTileB + lane) * 9 + k] = sv;
   }
   __syncthreads();
   for (int k2 = threadIdx.x; k2 < kTileB * 9; k2 += blockDim.x) {
     const int qq = k2 / 9, k = k2 % 9;
     double sv = 0.0;
-    for (int wv = 0; wv < nw; ++wv)
-      sv += kMMA ? double(reinterpret_cast<const float*>(red)[(wv * kTileB + qq) * 9 + k])
-                 : red[(wv * kTileB + qq) * 9 + k];
+    for (int wv = 0; wv < nw; ++wv) sv += red[(wv * kTileB + qq) * 9 + k];
     Spart[(((size_t)tl * g.nslab + slab) * kTileB + qq) * 9 + k] = sv;
   }
   if (kSmemP && project) {
@@ -683,11 +469,13 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
 
 __constant__ int c_kpairs[6][2] = {{0, 0}, {1, 1}, {2, 2}, {1, 2}, {0, 2}, {0, 1}};
 
-// Moments of t^j per node (one warp per node), then Pg^j := 0 (the accumulator of step j + 1).
-template <typename Real>
+// Moments of t^j per node (one warp per node), then Pg^j := 0 (the accumulator of step j + 1). kPair: the
+// split mixed step, which keeps the projections as pairs of floats and rewrites them each step.
+// nslab: S^j partials per tile.
+template <typename Real, bool kPair>
 __global__ void __launch_bounds__(kThreads)
 k_moments(Geo g, Wave w, int j, const Real* __restrict__ Tj, const Real* __restrict__ A, double* __restrict__ Pg,
-          const int* __restrict__ n_rows, const double* __restrict__ Spart, double* __restrict__ mom) {
+          const int* __restrict__ n_rows, const double* __restrict__ Spart, int nslab, double* __restrict__ mom) {
   const int tl = blockIdx.x, t = wave_tile(w, tl);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int o[3];
@@ -735,11 +523,21 @@ k_moments(Geo g, Wave w, int j, const Real* __restrict__ Tj, const Real* __restr
     }
     // N^j = w_q^T V_nl,q t^j = sum_rows chi_row(x_q) (gamma |dOmega| chi_row^T t^j)
     double nacc = 0.0;
-    for (int r = lane; r < nr; r += 32) nacc += double(At[(size_t)r * B + q]) * double(Pt[(size_t)r * B + q]);
+    for (int r = lane; r < nr; r += 32) {
+      const size_t k = (size_t)r * B + q;
+      double p;
+      if constexpr (kPair) {
+        const float2 x = reinterpret_cast<const float2*>(Pt)[k];
+        p = double(x.x) + double(x.y);
+      } else {
+        p = Pt[k];
+      }
+      nacc += double(At[k]) * p;
+    }
     out[7] = warp_sum(nacc);
     double sv = 0.0;
     if (lane < 9)
-      for (int sl = 0; sl < g.nslab; ++sl) sv += Spart[(((size_t)tl * g.nslab + sl) * B + q) * 9 + lane];
+      for (int sl = 0; sl < nslab; ++sl) sv += Spart[(((size_t)tl * nslab + sl) * B + q) * 9 + lane];
     for (int k = 0; k < 9; ++k) out[8 + k] = __shfl_sync(0xffffffffu, sv, k);
     if (lane < SQ_N_MOMENTS) {
       double val = 0.0;
@@ -749,8 +547,10 @@ k_moments(Geo g, Wave w, int j, const Real* __restrict__ Tj, const Real* __restr
       mom[((size_t)node * (g.n_pl + 1) + j) * SQ_N_MOMENTS + lane] = val;
     }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < nr * B; i += kThreads) Pt[i] = 0.0;
+  if constexpr (!kPair) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < nr * B; i += kThreads) Pt[i] = 0.0;
+  }
 }
 
 // dynamic shared memory of k_step: staged projections (at most kStepRowsSmemMax, else they stay
@@ -776,29 +576,20 @@ static int launch_step(sq_handle* h, const Wave& w, dim3 grid, size_t smem, cons
   // dynamic size this kernel uses)
   if (rows_smem <= h->step_rows_cap) {
     smem += smem_warps;
-    if (sizeof(Real) == 4 && h->proj4) {
-      h->step_variant[0]++;
-      SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_step<Real, NO, true, sizeof(Real) == 4>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, kStepSmemMax));
-      k_step<Real, NO, true, sizeof(Real) == 4><<<grid, nthr, smem, h->stream>>>(
-          h->geo, w, Tc, Tp, Tn, Pg, Pgn, W, chi, h->d.chi32s, gdv, h->wb.brick_rec, h->wb.slab_n, h->wb.slab_map,
-          h->wb.brick_n, v, h->d.scal, mode, h->wb.Spart, rows_smem, ncoef, h->d.status);
-      SQ_LAUNCH_CHECK(h);
-      return SQ_OK;
-    }
     h->step_variant[1]++;
-    SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_step<Real, NO, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_step<Real, NO, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         kStepSmemMax));
-    k_step<Real, NO, true, false><<<grid, nthr, smem, h->stream>>>(h->geo, w, Tc, Tp, Tn, Pg, Pgn, W, chi, nullptr, gdv,
-                                                                h->wb.brick_rec, h->wb.slab_n, h->wb.slab_map, h->wb.brick_n, v,
-                                                                h->d.scal, mode, h->wb.Spart, rows_smem, ncoef, h->d.status);
+    k_step<Real, NO, true><<<grid, nthr, smem, h->stream>>>(h->geo, w, Tc, Tp, Tn, Pg, Pgn, W, chi, gdv, h->wb.brick_rec,
+                                                            h->wb.slab_n, h->wb.slab_map, h->wb.brick_n, v, h->d.scal,
+                                                            mode, h->wb.Spart, rows_smem, ncoef, h->d.status);
   } else {
     h->step_variant[2]++;
-    SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_step<Real, NO, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_step<Real, NO, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         kStepSmemMax));
-    k_step<Real, NO, false, false><<<grid, nthr, smem_warps, h->stream>>>(h->geo, w, Tc, Tp, Tn, Pg, Pgn, W, chi, nullptr, gdv,
-                                                              h->wb.brick_rec, h->wb.slab_n, h->wb.slab_map, h->wb.brick_n, v,
-                                                              h->d.scal, mode, h->wb.Spart, 0, ncoef, h->d.status);
+    k_step<Real, NO, false><<<grid, nthr, smem_warps, h->stream>>>(h->geo, w, Tc, Tp, Tn, Pg, Pgn, W, chi, gdv,
+                                                                   h->wb.brick_rec, h->wb.slab_n, h->wb.slab_map,
+                                                                   h->wb.brick_n, v, h->d.scal, mode, h->wb.Spart, 0,
+                                                                   ncoef, h->d.status);
   }
   SQ_LAUNCH_CHECK(h);
   return SQ_OK;
@@ -834,6 +625,13 @@ static bool use_tma(const sq_handle* h, size_t wi) {
   return step_tma_smem_bytes(rows, stage_recs(h, wi)) <= kStepTmaSmemMax;
 }
 
+// The split mixed step: SQ_MIXED with at most 4 channels per atom, unless the staged step was asked for, or
+// SQ_STEP_SMEM_ROWS asks for the global-memory projections of k_step.
+bool use_split(const sq_handle* h, size_t wi) {
+  if (h->precision != SQ_MIXED || !h->proj4 || !h->wb.Part || use_tma(h, wi) || !nl_fits(h, wi)) return false;
+  return !(h->step_rows_env && wi < h->wave_rows.size() && std::max(1, h->wave_rows[wi]) > h->step_rows_cap);
+}
+
 template <typename Real>
 static int sweep_t(sq_handle* h, const Real* chi, const Real* v, const Real* gdv) {
   const Geo& g = h->geo;
@@ -854,7 +652,8 @@ static int sweep_t(sq_handle* h, const Real* chi, const Real* v, const Real* gdv
     NvtxRange nvtx("sweep wave");
     const Wave& w = h->waves[wi];
     // a captured graph must rebuild the lists itself (the atoms may move before it runs again)
-    int rc = build_wave_lists(h, w, !capturing);
+    int rc = build_wave_lists(h, wi, !capturing);
+    const bool split = use_split(h, wi);
     if (rc != SQ_OK) return rc;
     // largest slab projector-row count of the wave (measured once per layout) sizes the
     // per-slab shared accumulator
@@ -878,7 +677,9 @@ static int sweep_t(sq_handle* h, const Real* chi, const Real* v, const Real* gdv
       const int mode = (j == g.n_pl) ? 2 : (j == 0 ? 0 : 1);
       const double vecs = (mode == 0) ? 2.0 : (mode == 1) ? 3.0 : 1.0;   // reads t^j (t^{j-1}), writes t^{j+1}
       cudaEvent_t ev = capturing ? nullptr : timing_begin(h, SQ_K_STENCIL, vecs * col_bytes);
-      if (sizeof(Real) == 4 && use_tma(h, wi))
+      if (split)
+        rc = launch_step_mixed(h, wi, (const float*)Tc, (const float*)Tp, (float*)Tn, mode);
+      else if (sizeof(Real) == 4 && use_tma(h, wi))
         rc = launch_step_tma(h, w, gstencil, j % 3, (j + 2) % 3, (float*)Tn, Pg[j % 2], Pg[(j + 1) % 2], mode,
                              std::max(1, rmax), stage_recs(h, wi));
       else
@@ -886,9 +687,20 @@ static int sweep_t(sq_handle* h, const Real* chi, const Real* v, const Real* gdv
       if (rc != SQ_OK) return rc;
       timing_end(h, ev);
       ev = capturing ? nullptr : timing_begin(h, SQ_K_MOMENTS, 0.0);
-      k_moments<Real><<<w.ntiles, kThreads, 0, s>>>(g, w, j, Tc, A, Pg[j % 2], h->wb.n_rows, h->wb.Spart, h->d.mom);
+      if (split)
+        k_moments<Real, true><<<w.ntiles, kThreads, 0, s>>>(g, w, j, Tc, A, Pg[0], h->wb.n_rows, h->wb.Spart,
+                                                            stencil_chunks(g), h->d.mom);
+      else
+        k_moments<Real, false><<<w.ntiles, kThreads, 0, s>>>(g, w, j, Tc, A, Pg[j % 2], h->wb.n_rows, h->wb.Spart,
+                                                             g.nslab, h->d.mom);
       timing_end(h, ev);
       SQ_LAUNCH_CHECK(h);
+      if (split && mode != 2) {
+        ev = capturing ? nullptr : timing_begin(h, SQ_K_PROJECT, 0.0);
+        rc = launch_project_mixed(h, wi, (const float*)Tn);
+        if (rc != SQ_OK) return rc;
+        timing_end(h, ev);
+      }
     }
   }
   if (capturing) return SQ_OK;   // the status words are read after the graph runs
@@ -925,7 +737,7 @@ static int time_step_t(sq_handle* h, int reps, double* ms_out, const Real* chi, 
   // that cost, spread over the sweep's n_pl + 1 steps, belongs to the step time the tuner compares
   const bool rebuilt = h->waves.size() > 1 || !h->keep_lists;
   cudaEventRecord(e0, s);
-  int rc = build_wave_lists(h, w, !rebuilt);
+  int rc = build_wave_lists(h, 0, !rebuilt);
   cudaEventRecord(e1, s);
   float ms_lists = 0.f;
   if (rc == SQ_OK && rebuilt && cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms_lists, e0, e1);
@@ -938,22 +750,25 @@ static int time_step_t(sq_handle* h, int reps, double* ms_out, const Real* chi, 
   double* Pg[2] = {(double*)h->wb.Pg[0], (double*)h->wb.Pg[1]};
   const size_t smem = std::max<size_t>(1, size_t(h->wave_rows[0])) * kTileB * (sizeof(double) + sizeof(Real));
   const dim3 grid(g.nslab, w.ntiles);
-  const bool tma = sizeof(Real) == 4 && use_tma(h, 0);
+  const bool tma = sizeof(Real) == 4 && use_tma(h, 0), split = use_split(h, 0);
   const int rows = std::max(1, h->wave_rows[0]), recs = stage_recs(h, 0);
+  auto step = [&](int c, int p, int n, int mode) -> int {
+    if (split) {
+      const int r = launch_step_mixed(h, 0, (const float*)T[c], (const float*)T[p], (float*)T[n], mode);
+      return r != SQ_OK ? r : launch_project_mixed(h, 0, (const float*)T[n]);
+    }
+    if (tma) return launch_step_tma(h, w, grid, c, p, (float*)T[n], Pg[c], Pg[1 - c], mode, rows, recs);
+    return dispatch_step<Real>(h, w, grid, smem, T[c], T[p], T[n], Pg[c], Pg[1 - c], (Real*)h->wb.W, chi, gdv, v, mode);
+  };
   // the first launch (mode 0) forms t^1 from t^0, so the timed launches read defined values
-  if (tma)
-    rc = launch_step_tma(h, w, grid, 0, 2, (float*)T[1], Pg[0], Pg[1], 0, rows, recs);
-  else
-    rc = dispatch_step<Real>(h, w, grid, smem, T[0], T[2], T[1], Pg[0], Pg[1], (Real*)h->wb.W, chi, gdv, v, 0);
+  rc = step(0, 2, 1, 0);
   if (rc != SQ_OK) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     return rc;
   }
   cudaEventRecord(e0, s);
-  for (int r = 0; r < reps && rc == SQ_OK; ++r)
-    rc = tma ? launch_step_tma(h, w, grid, 1, 0, (float*)T[2], Pg[1], Pg[0], 1, rows, recs)
-             : dispatch_step<Real>(h, w, grid, smem, T[1], T[0], T[2], Pg[1], Pg[0], (Real*)h->wb.W, chi, gdv, v, 1);
+  for (int r = 0; r < reps && rc == SQ_OK; ++r) rc = step(1, 0, 2, 1);
   cudaEventRecord(e1, s);
   float ms = 0.f;
   const cudaError_t e = cudaEventSynchronize(e1);
