@@ -145,14 +145,12 @@ def peaks():
 
 
 def step_kernel_hash() -> str:
-    """sha1 of the step kernel's source text (its device helpers and the kernel, through its
-    end, plus sq_device.cuh): the committed traffic figure is valid for that text only."""
+    """sha1 of the mixed step's source text (sq_step_mixed.cu and sq_device.cuh): the committed
+    traffic figure is valid for that text only."""
     csrc = os.path.join(ROOT, "paper_2006_03697_gb300", "csrc")
-    src = open(os.path.join(csrc, "sq_sweep.cu")).read()
-    start = src.index("template <typename Real> struct Coef;")
-    end = src.index("__constant__ int c_kpairs", start)
+    src = open(os.path.join(csrc, "sq_step_mixed.cu")).read()
     dev = open(os.path.join(csrc, "sq_device.cuh")).read()
-    return hashlib.sha1((src[start:end] + dev).encode()).hexdigest()
+    return hashlib.sha1((src + dev).encode()).hexdigest()
 
 
 def stencil_traffic(sweep_hash: str, tiles_per_launch: float):

@@ -221,6 +221,16 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
       }
     g.lap0 = double(float(-side));
   }
+  for (int a = 0; a < 3; ++a)
+    for (int dd = 0; dd <= 2 * d->n_o; ++dd) {
+      double sum = 0.0;   // over p + q = dd, 0 < |p| <= min(n_o, m) (the midpoint lies in the window), 0 < |q| <= n_o
+      for (int p = -d->n_o; p <= d->n_o; ++p) {
+        const int q = dd - p;
+        if (p == 0 || q == 0 || std::abs(p) > g.m[a] || std::abs(q) > d->n_o) continue;
+        sum += (p > 0 ? 1.0 : -1.0) * g.grd[a][std::abs(p)] * (q > 0 ? 1.0 : -1.0) * g.grd[a][std::abs(q)];
+      }
+      g.grd2[a][dd] = sum;
+    }
   g.lap0f = float(g.lap0);
   for (int a = 0; a < 3; ++a)
     for (int p = 0; p <= sq::kMaxNo; ++p) {

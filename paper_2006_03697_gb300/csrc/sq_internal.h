@@ -84,6 +84,7 @@ struct Geo {
   double lap0;                    // -1/2 sum_a w0 / h_a^2
   double lap[3][kMaxNo + 1];      // -1/2 w_p / h_a^2
   double grd[3][kMaxNo + 1];      // g_p / h_a
+  double grd2[3][2 * kMaxNo + 1]; // [grad_a grad_a]_{c, c + d} at a window's centre c, d = 0 .. 2 n_o (both factors restricted)
   float lap0f;                    // float copies used by the FP32 sweep (constant-bank operands)
   float lapf[3][kMaxNo + 1];
   float grdf[3][kMaxNo + 1];

@@ -131,7 +131,7 @@ __device__ __forceinline__ bool image_meets_box(const Geo& g, const TileEntry& t
 // slab's bounding box contains each brick's) are numbered slab-locally in entry order; the
 // record carries that number (bits 16..31 of r0.w) and the first brick of the slab writes the
 // slab's row map (slab row -> tile row) and count.
-__global__ void k_brick_lists(Geo g, Wave w, const AtomTab* __restrict__ atoms, const double* __restrict__ rcmax,
+__global__ void k_brick_lists(Geo g, Wave w, int whole, const AtomTab* __restrict__ atoms, const double* __restrict__ rcmax,
                               const TileEntry* __restrict__ entries, const int* __restrict__ n_entries,
                               int* __restrict__ blist, int* __restrict__ bn, int4* __restrict__ rec,
                               float4* __restrict__ d0, int4* __restrict__ tma, int* __restrict__ slab_n,
@@ -141,9 +141,11 @@ __global__ void k_brick_lists(Geo g, Wave w, const AtomTab* __restrict__ atoms, 
   tile_origin(g, t, o);
   const int bx = br % g.nbr[0], by = (br / g.nbr[0]) % g.nbr[1], bz = br / (g.nbr[0] * g.nbr[1]);
   const int bl[3] = {o[0] - g.m[0] + bx * kBrick, o[1] - g.m[1] + by * kBrick, o[2] - g.m[2] + bz * kBrick};
-  // whole bricks, also past the window's edge (points outside it hold zero columns), so that the tiles that
-  // share a brick of absolute lattice points have the same records for it
-  const int bhi[3] = {bl[0] + kBrick - 1, bl[1] + kBrick - 1, bl[2] + kBrick - 1};
+  // the brick's part of the window; for the split mixed step whole bricks, also past the window's edge
+  // (points outside it hold zero columns), so that the tiles that share a brick of absolute lattice points
+  // have the same records for it
+  int bhi[3];
+  for (int a = 0; a < 3; ++a) bhi[a] = whole ? bl[a] + kBrick - 1 : min(bl[a] + kBrick, o[a] - g.m[a] + g.U[a]) - 1;
   // the slab: all of U in x and z, the brick's planes in y
   const int sl[3] = {o[0] - g.m[0], bl[1], o[2] - g.m[2]};
   const int shi[3] = {sl[0] + kBrick * g.nbr[0] - 1, bhi[1], sl[2] + kBrick * g.nbr[2] - 1};
@@ -201,7 +203,7 @@ __global__ void k_brick_lists(Geo g, Wave w, const AtomTab* __restrict__ atoms, 
         float r2 = 0.f;
         for (int a = 0; a < 3; ++a) {
           const int l = l0[a] + pl[a];
-          in = in && l >= 0 && l < ats.dim[a];
+          in = in && bl[a] + pl[a] <= bhi[a] && l >= 0 && l < ats.dim[a];
           const float d = float(l) * float(g.h[a]) + ats.dlo[a];   // (lo + l) h - R, box-relative
           r2 += d * d;
         }
@@ -434,7 +436,7 @@ int build_wave_entries(sq_handle* h, const Wave& w, WaveBufs* b) {
   if (b == &h->wb) h->lists_key = {w.tile0, w.ntiles, w.ids, h->atoms_epoch, false};
   k_tile_entries<<<w.ntiles, 256, 0, s>>>(g, w, h->d.atoms, b->entries, b->n_entries, b->n_rows, h->d.status);
   SQ_LAUNCH_CHECK(h);
-  k_brick_lists<<<dim3(g.nbricks, w.ntiles), 32, 0, s>>>(g, w, h->d.atoms, h->d.rcmax, b->entries, b->n_entries,
+  k_brick_lists<<<dim3(g.nbricks, w.ntiles), 32, 0, s>>>(g, w, h->wb.Part ? 1 : 0, h->d.atoms, h->d.rcmax, b->entries, b->n_entries,
                                                           b->brick_list, b->brick_n, b->brick_rec, b->brick_d0,
                                                           b->brick_tma, b->slab_n, b->slab_map, h->d.status);
   SQ_LAUNCH_CHECK(h);

@@ -467,8 +467,6 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
   }
 }
 
-__constant__ int c_kpairs[6][2] = {{0, 0}, {1, 1}, {2, 2}, {1, 2}, {0, 2}, {0, 1}};
-
 // Moments of t^j per node (one warp per node), then Pg^j := 0 (the accumulator of step j + 1). kPair: the
 // split mixed step, which keeps the projections as pairs of floats and rewrites them each step.
 // nslab: S^j partials per tile.
@@ -497,54 +495,69 @@ k_moments(Geo g, Wave w, int j, const Real* __restrict__ Tj, const Real* __restr
       if ((unsigned)x >= (unsigned)g.U[0] || (unsigned)y >= (unsigned)g.U[1] || (unsigned)z >= (unsigned)g.U[2]) return 0.0;
       return double(T[((size_t)(z * g.U[1] + y) * g.U[0] + x) * B + q]);
     };
-    double out[SQ_N_MOMENTS];
-    out[0] = tval(c[0], c[1], c[2]);
-    // K^j_ab = [grad_a,q grad_b,q t^j]_q with both factors restricted to the window
-    for (int pr = 0; pr < 6; ++pr) {
-      const int a = c_kpairs[pr][0], b = c_kpairs[pr][1];
-      double term = 0.0;
-      if (lane < 2 * g.n_o) {
-        const int pp = lane / 2 + 1;
-        const int sg = (lane % 2 == 0) ? 1 : -1;
-        if (pp <= g.m[a]) {
-          int k[3] = {c[0], c[1], c[2]};
-          k[a] += sg * pp;
-          double gb = 0.0;
-          for (int p2 = 1; p2 <= g.n_o; ++p2) {
-            int kp[3] = {k[0], k[1], k[2]}, km[3] = {k[0], k[1], k[2]};
-            kp[b] += p2;
-            km[b] -= p2;
-            gb += g.grd[b][p2] * (tval(kp[0], kp[1], kp[2]) - tval(km[0], km[1], km[2]));
-          }
-          term = sg * g.grd[a][pp] * gb;
-        }
+    // K^j_ab = [grad_a,q grad_b,q t^j]_q with both factors restricted to the window (columns are zero outside
+    // it). FP64 issues 1.7 lanes per clock and SM, so the sums are arranged for few FP64 instructions: the
+    // diagonal pairs are one 4 n_o + 1 point stencil, the others the quadruples t(i,j) - t(-i,j) - t(i,-j) +
+    // t(-i,-j), and the seven totals share one reduce-scatter (200 -> 60 instructions per node at n_o = 6).
+    double val[8];
+    val[7] = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int d = lane - 2 * g.n_o;
+      val[a] = (lane <= 4 * g.n_o)
+                   ? g.grd2[a][abs(d)] * tval(c[0] + (a == 0 ? d : 0), c[1] + (a == 1 ? d : 0), c[2] + (a == 2 ? d : 0)) : 0.0;
+    }
+#pragma unroll
+    for (int pr = 3; pr < 6; ++pr) {
+      const int a = (pr == 3) ? 1 : 0, b = (pr == 5) ? 1 : 2;   // yz, xz, xy
+      double s = 0.0;
+      for (int e = lane; e < g.n_o * g.n_o; e += 32) {
+        const int i = e / g.n_o + 1, j = e - (i - 1) * g.n_o + 1;
+        auto at = [&](int si, int sj) {
+          return tval(c[0] + (a == 0 ? si : 0), c[1] + (a == 1 ? si : b == 1 ? sj : 0), c[2] + (b == 2 ? sj : 0));
+        };
+        s += g.grd[a][i] * g.grd[b][j] * ((at(i, j) - at(-i, j)) - (at(i, -j) - at(-i, -j)));
       }
-      out[1 + pr] = warp_sum(term);
+      val[pr] = s;
     }
     // N^j = w_q^T V_nl,q t^j = sum_rows chi_row(x_q) (gamma |dOmega| chi_row^T t^j)
-    double nacc = 0.0;
-    for (int r = lane; r < nr; r += 32) {
-      const size_t k = (size_t)r * B + q;
-      double p;
-      if constexpr (kPair) {
+    if constexpr (kPair) {   // float pairs: products and sums with their rounding errors (FP64's accuracy at FP32 rates)
+      float nh = 0.f, nl = 0.f;
+      for (int r = lane; r < nr; r += 32) {
+        const size_t k = (size_t)r * B + q;
         const float2 x = reinterpret_cast<const float2*>(Pt)[k];
-        p = double(x.x) + double(x.y);
-      } else {
-        p = Pt[k];
+        const float ak = At[k], p = __fmul_rn(ak, x.x), pe = fmaf(ak, x.x, -p) + ak * x.y;
+        const float sm = __fadd_rn(nh, p), z = __fsub_rn(sm, nh);
+        nl = __fadd_rn(nl, __fadd_rn(__fadd_rn(__fsub_rn(nh, __fsub_rn(sm, z)), __fsub_rn(p, z)), pe));
+        nh = sm;
       }
-      nacc += double(At[k]) * p;
+      val[6] = double(nh) + double(nl);
+    } else {
+      double nacc = 0.0;
+      for (int r = lane; r < nr; r += 32) nacc += double(At[(size_t)r * B + q]) * Pt[(size_t)r * B + q];
+      val[6] = nacc;
     }
-    out[7] = warp_sum(nacc);
-    double sv = 0.0;
-    if (lane < 9)
-      for (int sl = 0; sl < nslab; ++sl) sv += Spart[(((size_t)tl * nslab + sl) * B + q) * 9 + lane];
-    for (int k = 0; k < 9; ++k) out[8 + k] = __shfl_sync(0xffffffffu, sv, k);
-    if (lane < SQ_N_MOMENTS) {
-      double val = 0.0;
+    auto halve = [&](int n, int d) {   // keep n of 2 n values, hand the others to the partner lane
+      const bool up = (lane & d) != 0;
 #pragma unroll
-      for (int k = 0; k < SQ_N_MOMENTS; ++k)
-        if (k == lane) val = out[k];
-      mom[((size_t)node * (g.n_pl + 1) + j) * SQ_N_MOMENTS + lane] = val;
+      for (int k = 0; k < n; ++k) {
+        const double give = up ? val[k] : val[k + n], keep = up ? val[k + n] : val[k];
+        val[k] = keep + __shfl_xor_sync(0xffffffffu, give, d);
+      }
+    };
+    halve(4, 16);
+    halve(2, 8);
+    halve(1, 4);
+    val[0] += __shfl_xor_sync(0xffffffffu, val[0], 2);
+    val[0] += __shfl_xor_sync(0xffffffffu, val[0], 1);
+    double* row = mom + ((size_t)node * (g.n_pl + 1) + j) * SQ_N_MOMENTS;
+    const int slot = 1 + (lane >> 4) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+    if ((lane & 3) == 0 && slot < 8) row[slot] = val[0];
+    if (lane == 1) row[0] = tval(c[0], c[1], c[2]);
+    if (lane < 9) {
+      double sv = 0.0;
+      for (int sl = 0; sl < nslab; ++sl) sv += Spart[(((size_t)tl * nslab + sl) * B + q) * 9 + lane];
+      row[8 + lane] = sv;
     }
   }
   if constexpr (!kPair) {
