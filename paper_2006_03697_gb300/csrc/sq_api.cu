@@ -302,7 +302,7 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
                      size_t(g.nbricks) * (size_t(g.br_cap) + 1) * sizeof(int) +
                      size_t(g.nbricks) * size_t(g.br_cap) * 4 * sizeof(int4) +   // records, corner offsets, TMA boxes
                      3 * size_t(g.Upts) * tileB * real +        // T ring
-                     3 * size_t(g.Upts) * tileB * real +        // W
+                     size_t(d->precision == SQ_FP64 ? 9 : 3) * g.Upts * tileB * real +   // W (G)
                      2 * size_t(g.r_cap) * tileB * real +       // A, P
                      2 * size_t(g.r_cap) * tileB * sizeof(double) +   // Pg ping-pong (FP64)
                      size_t(std::max(g.nslab, sq::stencil_chunks(g))) * tileB * 9 * sizeof(double) +
@@ -584,7 +584,7 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   SQ_ALLOC(h->wb.slab_n, sizeof(int) * size_t(wt) * g.nslab);
   SQ_ALLOC(h->wb.slab_map, sizeof(int) * size_t(wt) * g.nslab * g.r_cap);
   for (int i = 0; i < 3; ++i) SQ_ALLOC(h->wb.T[i], real * size_t(wt) * g.Upts * g.B);
-  SQ_ALLOC(h->wb.W, real * size_t(wt) * 3 * g.Upts * g.B);
+  SQ_ALLOC(h->wb.W, real * size_t(wt) * (f64 ? 9 : 3) * g.Upts * g.B);
   SQ_ALLOC(h->wb.A, real * size_t(wt) * g.r_cap * g.B);
   SQ_ALLOC(h->wb.P, real * size_t(wt) * g.r_cap * g.B);
   SQ_ALLOC(h->wb.Pg[0], sizeof(double) * size_t(wt) * g.r_cap * g.B);   // projections: FP64 sums

@@ -114,7 +114,7 @@ struct WaveBufs {
   int* slab_n = nullptr;          // [wt][nslab] projector rows meeting each slab (y-row of bricks)
   int* slab_map = nullptr;        // [wt][nslab][r_cap] slab row -> tile row
   void* T[3] = {nullptr, nullptr, nullptr};   // Real [wt][Upts][B]
-  void* W = nullptr;              // Real [wt][3][Upts][B]
+  void* W = nullptr;              // FP32: W_b [wt][3][Upts][B]; FP64: G_ab = -grad_a W_b [wt][9][Upts][B]
   void* A = nullptr;              // Real [wt][r_cap][B]  chi_row(x_q)
   void* P = nullptr;              // Real [wt][r_cap][B]  gamma |dOmega| chi^T t (Lanczos apply)
   void* Pg[2] = {nullptr, nullptr};   // double [wt][r_cap][B]  gamma |dOmega| chi^T t^j, ping-pong

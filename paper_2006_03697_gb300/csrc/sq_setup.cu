@@ -294,15 +294,15 @@ __global__ void __launch_bounds__(224, sizeof(Real) == 4 ? 4 : 1) k_wtable(Geo g
                                                 const TileEntry* __restrict__ entries, const int* __restrict__ blist,
                                                 const int4* __restrict__ brec, const float4* __restrict__ bd0,
                                                 const int* __restrict__ bn, const Real* __restrict__ A,
-                                                Real* __restrict__ W) {
+                                                Real* __restrict__ W0, Real* __restrict__ W1, Real* __restrict__ W2,
+                                                size_t tile_stride) {
   const int slab = blockIdx.x, tl = blockIdx.y, t = wave_tile(w, tl);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int o[3];
   tile_origin(g, t, o);
   const TileEntry* ent = entries + (size_t)tl * g.e_cap;
   const Real* At = A + (size_t)tl * g.r_cap * g.B;
-  Real* Wt = W + (size_t)tl * 3 * g.Upts * g.B;
-  const size_t wstr = (size_t)g.Upts * g.B;
+  Real* const Wt[3] = {W0 + tl * tile_stride, W1 + tl * tile_stride, W2 + tl * tile_stride};
   const int q = lane & 7, pa = lane >> 3;
   int qo[3];
   node_offset(g, q, qo);
@@ -378,9 +378,35 @@ __global__ void __launch_bounds__(224, sizeof(Real) == 4 ? 4 : 1) k_wtable(Geo g
         const bool inw = valid && in_window(g, qo, ux, uy, uz);
         const size_t e = ((size_t)(uz * g.U[1] + uy) * g.U[0] + ux) * g.B + q;
 #pragma unroll
-        for (int b = 0; b < 3; ++b) Wt[b * wstr + e] = inw ? acc[i][b] : Real(0);
+        for (int b = 0; b < 3; ++b) Wt[b][e] = inw ? acc[i][b] : Real(0);
       }
     }
+  }
+}
+
+// FP64 sweeps contract S^j_ab = sum_u W_b (grad_a t^j) as -sum_u (grad_a W_b) t^j (the restricted grad_a is
+// antisymmetric): G_ab = -grad_a W_b, formed once per sweep, makes S^j nine multiply-adds per point and step in
+// place of 6 n_o + 9 (FP64 issues 1.7 lanes per clock and SM; the nine fields' 72 bytes a point are cheap
+// next to that). One thread per (point, node); columns are zero outside each node's window.
+__global__ void __launch_bounds__(256) k_gtable(Geo g, const double* __restrict__ W0, const double* __restrict__ W1,
+                                                const double* __restrict__ W2, double* __restrict__ G) {
+  const size_t n = (size_t)g.Upts * g.B;
+  const double* Wb[3] = {W0 + blockIdx.y * n, W1 + blockIdx.y * n, W2 + blockIdx.y * n};
+  double* Gt = G + blockIdx.y * 9 * n;
+  const int st[3] = {g.B, g.U[0] * g.B, g.U[0] * g.U[1] * g.B};
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    const int p = int(e) / g.B;
+    const int u[3] = {p % g.U[0], p / g.U[0] % g.U[1], p / (g.U[0] * g.U[1])};
+    for (int a = 0; a < 3; ++a)
+      for (int b = 0; b < 3; ++b) {
+        double s = 0.0;
+        for (int pp = 1; pp <= g.n_o; ++pp) {
+          const double up = (u[a] + pp < g.U[a]) ? Wb[b][e + (size_t)pp * st[a]] : 0.0;
+          const double dn = (u[a] - pp >= 0) ? Wb[b][e - (size_t)pp * st[a]] : 0.0;
+          s += g.grd[a][pp] * (dn - up);
+        }
+        Gt[(3 * a + b) * n + e] = s;
+      }
   }
 }
 
@@ -417,10 +443,20 @@ static int wave_lists_t(sq_handle* h, size_t wi, bool reuse, const Real* chi, co
                                           use_split(h, wi) ? nl_plane(h) : 0);
   SQ_LAUNCH_CHECK(h);
   if (!same) {
+    // FP32: W itself, [tile][3][points]; FP64: W in the three column buffers (t^0 is written below), then G
+    const size_t n = (size_t)g.Upts * g.B;
+    const bool f64 = sizeof(Real) == 8;
+    Real* Wp[3];
+    for (int b = 0; b < 3; ++b) Wp[b] = f64 ? (Real*)h->wb.T[b] : W + b * n;
     k_wtable<Real><<<dim3(g.nbr[2], w.ntiles), 224, 0, s>>>(g, w, h->d.atoms, gdvR, chi, h->wb.entries,
                                                             h->wb.brick_list, h->wb.brick_rec, h->wb.brick_d0,
-                                                            h->wb.brick_n, A, W);
+                                                            h->wb.brick_n, A, Wp[0], Wp[1], Wp[2], f64 ? n : 3 * n);
     SQ_LAUNCH_CHECK(h);
+    if (f64) {
+      k_gtable<<<dim3(unsigned((n + 255) / 256), w.ntiles), 256, 0, s>>>(g, (const double*)Wp[0], (const double*)Wp[1],
+                                                                         (const double*)Wp[2], (double*)W);
+      SQ_LAUNCH_CHECK(h);
+    }
     h->lists_key.full = true;
   }
   SQ_CUDA_TRY(h, cudaMemsetAsync(T0, 0, sizeof(Real) * (size_t)w.ntiles * g.Upts * g.B, s));

@@ -233,7 +233,8 @@ static int step_warps(int bricks_per_slab) {
   return best;
 }
 
-template <typename Real, int NO, bool kSmemP>
+// NCH: every atom has one channel (1: a table value per point in place of a padded group of four) or any number (4)
+template <typename Real, int NO, bool kSmemP, int NCH>
 __global__ void __launch_bounds__(kStepThreads, sizeof(Real) == 4 ? 4 : 2)
 k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, Real* __restrict__ Tn,
        const double* __restrict__ Pg, double* __restrict__ Pg_next, const Real* __restrict__ Wt,
@@ -309,7 +310,8 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
     caA = Real(f * ncoef[2 * node]);
     cdA = Real(f * ncoef[2 * node + 1]);
   }
-  const Real* Wq = Wt + (size_t)tl * 3 * g.Upts * kTileB;
+  constexpr bool kG = sizeof(Real) == 8;   // S^j from G_ab t^j (k_gtable) in place of W_b grad_a t^j
+  const Real* Wq = Wt + (size_t)tl * (kG ? 9 : 3) * g.Upts * kTileB;
   const size_t wstr = (size_t)g.Upts * kTileB;
   // S partial sums, per lane across bricks
   Real sacc[9];
@@ -337,6 +339,16 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
           const int prow = kSmemP ? (int(unsigned(r0.w) >> 16)) : r0.y;
           const unsigned mk = unsigned(half ? r1.w : r1.z) >> pa;   // bits pa + 4 i of this half
           if (!(mk & 0x11111111u)) continue;
+          if constexpr (NCH == 1) {
+            const Real pv = pg(prow * kTileB + q);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if ((mk >> (4 * i)) & 1u) {
+                const int it = 8 * half + i;
+                ynl[i] += chi[r0.x + (((it >> 2) * r1.y + (it & 3)) * r1.x + pa) * nchp] * pv;
+              }
+            continue;
+          }
           for (int c0 = 0; c0 < nch; c0 += 4) {
             Real pv[4];
 #pragma unroll
@@ -368,21 +380,22 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
         Real tn = Real(0);
         if (inwin) {
           // loads that do not depend on the stencil, issued first
-          const Real w0 = Wq[e], w1 = Wq[wstr + e], w2 = Wq[2 * wstr + e];
+          Real wv[kG ? 9 : 3];
+#pragma unroll
+          for (int k = 0; k < (kG ? 9 : 3); ++k) wv[k] = Wq[k * wstr + e];
           const Real tp = (mode == 1) ? Tp[tbase + e] : Real(0);
           const Real tc = T[e];
           Real y = Real(0);                           // off-diagonal part of H t^j
-          Real gr[3];
+          Real gr[3] = {Real(0), Real(0), Real(0)};
           const int u[3] = {ux, uy, uz};
 #pragma unroll
           for (int a = 0; a < 3; ++a) {
-            gr[a] = Real(0);
 #pragma unroll
             for (int pp = 1; pp <= NO; ++pp) {
               const Real fp = (u[a] + pp < Ua[a]) ? T[e + (size_t)pp * st[a]] : Real(0);
               const Real fm = (u[a] - pp >= 0) ? T[e - (size_t)pp * st[a]] : Real(0);
               y += Coef<Real>::lap(g, a, pp) * (fp + fm);
-              gr[a] += Coef<Real>::grd(g, a, pp) * (fp - fm);
+              if constexpr (!kG) gr[a] += Coef<Real>::grd(g, a, pp) * (fp - fm);
             }
           }
           const Real vloc = v[wrz[uz] + wry[pb] + wrx[ux]];   // V_eff at the wrapped node
@@ -393,9 +406,8 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
           }
 #pragma unroll
           for (int a = 0; a < 3; ++a) {
-            sacc[3 * a + 0] += gr[a] * w0;
-            sacc[3 * a + 1] += gr[a] * w1;
-            sacc[3 * a + 2] += gr[a] * w2;
+#pragma unroll
+            for (int b = 0; b < 3; ++b) sacc[3 * a + b] += kG ? wv[kG ? 3 * a + b : 0] * tc : gr[a] * wv[b];
           }
         } else if (inU && mode != 2) {
           Tn[tbase + e] = Real(0);
@@ -416,6 +428,17 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
           const int nch = r0.w & 0xff, nchp = (r0.w >> 8) & 0xff;
           const int prow = kSmemP ? (int(unsigned(r0.w) >> 16)) : r0.y;
           const unsigned mlo = unsigned(r1.z) >> pa, mhi = unsigned(r1.w) >> pa;
+          if constexpr (NCH == 1) {
+            Real acc = Real(0);
+#pragma unroll 8
+            for (int it = 0; it < 16; ++it)
+              if (((it < 8 ? mlo : mhi) >> (4 * (it & 7))) & 1u)
+                acc += chi[r0.x + (((it >> 2) * r1.y + (it & 3)) * r1.x + pa) * nchp] * tnv[it * 32];
+            acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+            acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+            if (pa == 0 && acc != Real(0)) atomicAdd(&Ps[prow * kTileB + q], double(acc * gdv[r0.z]));
+            continue;
+          }
           for (int c0 = 0; c0 < nch; c0 += 4) {
             Real acc[4] = {Real(0), Real(0), Real(0), Real(0)};
 #pragma unroll 4
@@ -587,23 +610,20 @@ static int launch_step(sq_handle* h, const Wave& w, dim3 grid, size_t smem, cons
   // The dynamic-size attribute belongs to the function, not the launch, and handles on other
   // host threads launch the same kernel, so every caller sets the same value (the largest
   // dynamic size this kernel uses)
-  if (rows_smem <= h->step_rows_cap) {
-    smem += smem_warps;
-    h->step_variant[1]++;
-    SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_step<Real, NO, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        kStepSmemMax));
-    k_step<Real, NO, true><<<grid, nthr, smem, h->stream>>>(h->geo, w, Tc, Tp, Tn, Pg, Pgn, W, chi, gdv, h->wb.brick_rec,
-                                                            h->wb.slab_n, h->wb.slab_map, h->wb.brick_n, v, h->d.scal,
-                                                            mode, h->wb.Spart, rows_smem, ncoef, h->d.status);
-  } else {
-    h->step_variant[2]++;
-    SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_step<Real, NO, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        kStepSmemMax));
-    k_step<Real, NO, false><<<grid, nthr, smem_warps, h->stream>>>(h->geo, w, Tc, Tp, Tn, Pg, Pgn, W, chi, gdv,
-                                                                   h->wb.brick_rec, h->wb.slab_n, h->wb.slab_map,
-                                                                   h->wb.brick_n, v, h->d.scal, mode, h->wb.Spart, 0,
-                                                                   ncoef, h->d.status);
-  }
+  const bool staged = rows_smem <= h->step_rows_cap, one = h->max_nch == 1;
+  h->step_variant[staged ? 1 : 2]++;
+  auto go = [&](auto kernel, size_t bytes, int rows) -> int {
+    SQ_CUDA_TRY(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStepSmemMax));
+    kernel<<<grid, nthr, bytes, h->stream>>>(h->geo, w, Tc, Tp, Tn, Pg, Pgn, W, chi, gdv, h->wb.brick_rec, h->wb.slab_n,
+                                             h->wb.slab_map, h->wb.brick_n, v, h->d.scal, mode, h->wb.Spart, rows, ncoef,
+                                             h->d.status);
+    return SQ_OK;
+  };
+  int rc;
+  if (staged) rc = one ? go(k_step<Real, NO, true, 1>, smem + smem_warps, rows_smem)
+                       : go(k_step<Real, NO, true, 4>, smem + smem_warps, rows_smem);
+  else rc = one ? go(k_step<Real, NO, false, 1>, smem_warps, 0) : go(k_step<Real, NO, false, 4>, smem_warps, 0);
+  if (rc != SQ_OK) return rc;
   SQ_LAUNCH_CHECK(h);
   return SQ_OK;
 }
