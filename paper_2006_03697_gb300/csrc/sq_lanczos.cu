@@ -80,47 +80,12 @@ template <typename Real> struct LzV4;
 template <> struct LzV4<float> { using T = float4; };
 template <> struct LzV4<double> { using T = double4_32a; };
 
-struct FloatPair { float h, l; };
-
-__device__ __forceinline__ FloatPair lz_add(FloatPair a, FloatPair b) {   // Knuth's two-sum, tails added
-  const float s = __fadd_rn(a.h, b.h), z = __fsub_rn(s, a.h);
-  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, z)), __fsub_rn(b.h, z));
-  const float t = __fadd_rn(e, __fadd_rn(a.l, b.l)), h = __fadd_rn(s, t);
-  return {h, __fsub_rn(t, __fsub_rn(h, s))};
-}
-__device__ __forceinline__ double lz_add(double a, double b) { return a + b; }
-__device__ __forceinline__ FloatPair lz_shfl(FloatPair a, int m) {
-  return {__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
-}
-__device__ __forceinline__ double lz_shfl(double a, int m) { return __shfl_xor_sync(0xffffffffu, a, m); }
-__device__ __forceinline__ double lz_double(FloatPair a) { return double(a.h) + double(a.l); }
-__device__ __forceinline__ double lz_double(double a) { return a; }
-template <typename Real> struct LzAcc;
-template <> struct LzAcc<float> {
-  using T = FloatPair;
-  static __device__ __forceinline__ T make(float x) { return {x, 0.f}; }
-};
-template <> struct LzAcc<double> {
-  using T = double;
-  static __device__ __forceinline__ T make(double x) { return x; }
-};
-
-// the four products of a lane (nodes 4 (lane & 1) ..), added over the warp's 16 lanes of that parity into
-// acc[8] (lanes 0 .. 7 add one node each; one warp per acc)
+// the four products of a lane (nodes 4 (lane & 1) ..), added over the warp into acc[8] (one warp per acc)
 template <typename Real>
 __device__ __forceinline__ void lz_warp_add(const Real d[4], typename LzAcc<Real>::T* acc) {
-  using A = typename LzAcc<Real>::T;
-  const int lane = threadIdx.x & 31, s0 = (lane >> 1) & 1, s1 = (lane >> 2) & 1;
-  const A v0 = LzAcc<Real>::make(d[0]), v1 = LzAcc<Real>::make(d[1]), v2 = LzAcc<Real>::make(d[2]), v3 = LzAcc<Real>::make(d[3]);
-  const A k0 = lz_add(s0 ? v2 : v0, lz_shfl(s0 ? v0 : v2, 2));
-  const A k1 = lz_add(s0 ? v3 : v1, lz_shfl(s0 ? v1 : v3, 2));
-  A k = lz_add(s1 ? k1 : k0, lz_shfl(s1 ? k0 : k1, 4));
-  k = lz_add(k, lz_shfl(k, 8));
-  k = lz_add(k, lz_shfl(k, 16));
-  if (lane < 8) {
-    A* slot = acc + 4 * (lane & 1) + 2 * s0 + s1;
-    *slot = lz_add(*slot, k);
-  }
+  int node;
+  const auto s = lz_warp_sum<Real>(d, &node);
+  if ((threadIdx.x & 31) < 8) acc[node] = lz_add(acc[node], s);
 }
 
 enum LzMode { kLzDots = 0, kLzUpdateDots = 1, kLzUpdateNorm = 2, kLzNorm = 3 };

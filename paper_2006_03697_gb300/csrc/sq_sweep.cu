@@ -43,11 +43,10 @@ __device__ __forceinline__ void load4(const Real* p, Real out[4]) {
 // P[row][q] = gamma |dOmega| chi_row^T v: one block per atom image of a tile (images in a stride of
 // gridDim.x). A thread owns an (x, y) column of the image's box and half of the nodes: one projector load
 // per point serves four nodes, and the column only walks the z-chord of the support sphere (FP32 with a
-// 1e-5 margin; points past it hold zeros). Per thread in the vectors' precision, across threads in FP64,
-// fixed order. One thread per (point, node) with an integer division each took 74 us for the 10
-// sample tiles of a 12^3 cell and 691 us for its 216 tiles.
-constexpr int kProjThreads = 128;
-template <typename Real>
+// 1e-5 margin; points past it hold zeros). Per thread in the vectors' precision, across threads as
+// doubles (FP64) or float pairs, fixed order. NCH as in k_step.
+constexpr int kProjThreads = 128, kProjWarps = kProjThreads / 32;
+template <typename Real, int NCH>
 __global__ void __launch_bounds__(kProjThreads)
 k_project(Geo g, Wave w, const Real* __restrict__ Tn, const Real* __restrict__ chi, const AtomTab* __restrict__ atoms,
           const double* __restrict__ rcmax, const double* __restrict__ chs, const TileEntry* __restrict__ entries,
@@ -58,7 +57,7 @@ k_project(Geo g, Wave w, const Real* __restrict__ Tn, const Real* __restrict__ c
   const Real* T = Tn + (size_t)tl * g.Upts * B;
   Real* Pt = P + (size_t)tl * g.r_cap * B;
   const int half = threadIdx.x & 1, lane = threadIdx.x >> 1;
-  __shared__ Real red[16][kProjThreads / 2 * 2 + 1];   // [channel 4 x node 4][thread]
+  __shared__ typename LzAcc<Real>::T red[kProjWarps][NCH * 8];   // [warp][channel][node]
   for (int eidx = blockIdx.x; eidx < n_entries[tl]; eidx += gridDim.x) {
     const TileEntry te = entries[(size_t)tl * g.e_cap + eidx];
     const AtomTab& at = atoms[te.atom];
@@ -72,10 +71,10 @@ k_project(Geo g, Wave w, const Real* __restrict__ Tn, const Real* __restrict__ c
     const int nx = max(0, hi[0] - lo[0]), ny = max(0, hi[1] - lo[1]);
     const float hx = float(g.h[0]), hy = float(g.h[1]), hz = float(g.h[2]);
     const int dx = at.dim[0], dxy = at.dim[0] * at.dim[1], nchp = at.nchp;
-    for (int c0 = 0; c0 < at.nch; c0 += 4) {
-      Real acc[4][4];
+    for (int c0 = 0; c0 < at.nch; c0 += NCH) {
+      Real acc[NCH][4];
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+      for (int c = 0; c < NCH; ++c)
         for (int q = 0; q < 4; ++q) acc[c][q] = Real(0);
       for (int col = lane; col < nx * ny; col += kProjThreads / 2) {
         const int lx = lo[0] + col % nx, ly = lo[1] + col / nx;
@@ -90,27 +89,30 @@ k_project(Geo g, Wave w, const Real* __restrict__ Tn, const Real* __restrict__ c
         const size_t ts = (size_t)g.U[1] * g.U[0] * B, cs = (size_t)dxy * nchp;
 #pragma unroll 4
         for (int z = z0; z <= z1; ++z, tp += ts, cp += cs) {
-          Real tv[4], cv[4];
+          Real tv[4], cv[NCH];
           load4(tp, tv);
-          load4(cp, cv);
+          if constexpr (NCH == 1) cv[0] = *cp;
+          else load4(cp, cv);
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
+          for (int c = 0; c < NCH; ++c)
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc[c][q] += cv[c] * tv[q];
         }
       }
-      __syncthreads();
+      __syncthreads();   // red free
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
-        for (int q = 0; q < 4; ++q) red[4 * c + q][threadIdx.x] = acc[c][q];
+      for (int c = 0; c < NCH; ++c) {
+        int node;
+        const auto s = lz_warp_sum<Real>(acc[c], &node);
+        if ((threadIdx.x & 31) < 8) red[threadIdx.x >> 5][8 * c + node] = s;
+      }
       __syncthreads();
-      // 32 sums (channel, node) of 64 threads each, four lanes per sum
-      const int k2 = threadIdx.x >> 2, sub = threadIdx.x & 3, c = k2 >> 3, q = k2 & 7;
-      double s = 0.0;
-      for (int th = (q >> 2) + 2 * sub; th < kProjThreads; th += 8) s += double(red[4 * c + (q & 3)][th]);
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      s += __shfl_xor_sync(0xffffffffu, s, 2);
-      if (sub == 0 && c0 + c < at.nch) Pt[(size_t)(te.row0 + c0 + c) * B + q] = Real(s * chs[6 * (at.ch0 + c0 + c)]);
+      if (threadIdx.x < NCH * 8 && c0 + int(threadIdx.x >> 3) < at.nch) {
+        const int c = c0 + (threadIdx.x >> 3);
+        double s = lz_double(red[0][threadIdx.x]);
+        for (int i = 1; i < kProjWarps; ++i) s += lz_double(red[i][threadIdx.x]);
+        Pt[(size_t)(te.row0 + c) * B + (threadIdx.x & 7)] = Real(s * chs[6 * (at.ch0 + c)]);
+      }
     }
   }
 }
@@ -122,7 +124,7 @@ k_project(Geo g, Wave w, const Real* __restrict__ Tn, const Real* __restrict__ c
 // its brick up in the atom tables took 78 us for the 10 sample tiles of a 12^3 cell, 410 us for
 // its 216 tiles.
 constexpr int kApplyThreads = 128;
-template <typename Real>
+template <typename Real, int NCH>
 __global__ void __launch_bounds__(kApplyThreads)
 k_apply_h(Geo g, Wave w, const Real* __restrict__ Tc, Real* __restrict__ Tn, const Real* __restrict__ P,
           const Real* __restrict__ chi, const int4* __restrict__ brec, const int* __restrict__ bn, const Real* __restrict__ v) {
@@ -169,22 +171,36 @@ k_apply_h(Geo g, Wave w, const Real* __restrict__ Tc, Real* __restrict__ Tn, con
   const int4* rb = brec + ((size_t)tl * g.nbricks + br) * g.br_cap * 2;
   const int nb = bn[(size_t)tl * g.nbricks + br];
   const int bit = pa + 4 * pb + 16 * (pc & 1);
-  for (int k = 0; k < nb; ++k) {
-    const int4 r0 = rb[2 * k], r1 = rb[2 * k + 1];
-    if (!((unsigned(pc < 2 ? r1.z : r1.w) >> bit) & 1u)) continue;
-    const int nch = r0.w & 0xff, nchp = (r0.w >> 8) & 0xff;
-    const Real* cp = chi + r0.x + ((pc * r1.y + pb) * r1.x + pa) * nchp;
-    for (int c0 = 0; c0 < nch; c0 += 4) {
-      Real cv[4];
-      load4(cp + c0, cv);
+  if constexpr (NCH == 1) {
+#pragma unroll 4
+    for (int k = 0; k < nb; ++k) {
+      const int4 r0 = rb[2 * k], r1 = rb[2 * k + 1];
+      Real pv[4];
+      load4(Pt + (size_t)r0.y * B, pv);
+      if ((unsigned(pc < 2 ? r1.z : r1.w) >> bit) & 1u) {
+        const Real cv = chi[r0.x + ((pc * r1.y + pb) * r1.x + pa) * ((r0.w >> 8) & 0xff)];
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (c0 + c < nch) {
-          Real pv[4];
-          load4(Pt + (size_t)(r0.y + c0 + c) * B, pv);
+        for (int q = 0; q < 4; ++q) y[q] += cv * pv[q];
+      }
+    }
+  } else {
+    for (int k = 0; k < nb; ++k) {
+      const int4 r0 = rb[2 * k], r1 = rb[2 * k + 1];
+      if (!((unsigned(pc < 2 ? r1.z : r1.w) >> bit) & 1u)) continue;
+      const int nch = r0.w & 0xff, nchp = (r0.w >> 8) & 0xff;
+      const Real* cp = chi + r0.x + ((pc * r1.y + pb) * r1.x + pa) * nchp;
+      for (int c0 = 0; c0 < nch; c0 += 4) {
+        Real cv[4];
+        load4(cp + c0, cv);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) y[q] += cv[c] * pv[q];
-        }
+        for (int c = 0; c < 4; ++c)
+          if (c0 + c < nch) {
+            Real pv[4];
+            load4(Pt + (size_t)(r0.y + c0 + c) * B, pv);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) y[q] += cv[c] * pv[q];
+          }
+      }
     }
   }
   typename V4<Real>::T out;
@@ -845,10 +861,12 @@ static int apply_h_t(sq_handle* h, const Wave& w, const Real* v, Real* out, Real
                      const WaveBufs& b) {
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
-  k_project<Real><<<dim3(std::min(g.e_cap, 256), w.ntiles), kProjThreads, 0, s>>>(
+  const bool one = h->max_nch == 1;
+  (one ? k_project<Real, 1> : k_project<Real, 4>)<<<dim3(std::min(g.e_cap, 256), w.ntiles), kProjThreads, 0, s>>>(
       g, w, v, chi, h->d.atoms, h->d.rcmax, h->d.gdv, b.entries, b.n_entries, P);
   SQ_LAUNCH_CHECK(h);
-  k_apply_h<Real><<<dim3(g.nbricks, w.ntiles), kApplyThreads, 0, s>>>(g, w, v, out, P, chi, b.brick_rec, b.brick_n, vpot);
+  (one ? k_apply_h<Real, 1> : k_apply_h<Real, 4>)<<<dim3(g.nbricks, w.ntiles), kApplyThreads, 0, s>>>(
+      g, w, v, out, P, chi, b.brick_rec, b.brick_n, vpot);
   SQ_LAUNCH_CHECK(h);
   return SQ_OK;
 }
