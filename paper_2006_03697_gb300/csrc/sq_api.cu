@@ -313,7 +313,7 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
   if (split) P.per_tile_bytes += (size_t(g.e_cap) + 1 + size_t(g.nbricks) * g.br_cap) * sizeof(int);   // image -> brick index
   long long Nd = (long long)g.n[0] * g.n[1] * g.n[2];
   int M = d->cheb_quad_M > 0 ? d->cheb_quad_M : 2048;
-  P.fixed_bytes = size_t(Nd) * (sizeof(double) + sizeof(float)) +                       // V
+  P.fixed_bytes = size_t(sq::kStepFill) * g.B * 9 * sizeof(double) + size_t(Nd) * (sizeof(double) + sizeof(float)) +                       // V
                   P.atoms.size() * sizeof(sq::AtomTab) + size_t(ch) * 6 * sizeof(double) +
                   // projector tables: FP64 (always; the Lanczos apply and the FP64 sweep), FP32 and
                   // TF32 hi/lo pairs for the mixed sweep
@@ -589,7 +589,7 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   SQ_ALLOC(h->wb.P, real * size_t(wt) * g.r_cap * g.B);
   SQ_ALLOC(h->wb.Pg[0], sizeof(double) * size_t(wt) * g.r_cap * g.B);   // projections: FP64 sums
   SQ_ALLOC(h->wb.Pg[1], sizeof(double) * size_t(wt) * g.r_cap * g.B);
-  SQ_ALLOC(h->wb.Spart, sizeof(double) * size_t(wt) * std::max(g.nslab, sq::stencil_chunks(g)) * g.B * 9);
+  SQ_ALLOC(h->wb.Spart, sizeof(double) * std::max(size_t(wt) * std::max(g.nslab, sq::stencil_chunks(g)), size_t(sq::kStepFill)) * g.B * 9);
   if (h->part_floats > 0) {
     SQ_ALLOC(h->wb.proj_start, sizeof(int) * size_t(wt) * (size_t(g.e_cap) + 1));
     SQ_ALLOC(h->wb.proj_idx, sizeof(unsigned) * size_t(wt) * g.nbricks * g.br_cap);

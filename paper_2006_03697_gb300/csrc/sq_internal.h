@@ -118,7 +118,7 @@ struct WaveBufs {
   void* A = nullptr;              // Real [wt][r_cap][B]  chi_row(x_q)
   void* P = nullptr;              // Real [wt][r_cap][B]  gamma |dOmega| chi^T t (Lanczos apply)
   void* Pg[2] = {nullptr, nullptr};   // double [wt][r_cap][B]  gamma |dOmega| chi^T t^j, ping-pong
-  double* Spart = nullptr;        // [wt][slabs or stencil row chunks][B][9]
+  double* Spart = nullptr;        // [wt][slabs, their bricks or stencil row chunks][B][9]
   int* proj_start = nullptr;      // [wt][e_cap + 1] split mixed step: an image's entries of proj_idx
   unsigned* proj_idx = nullptr;   // [wt][nbricks * br_cap] brick << 16 | first projector row in the brick
   int* nl_head = nullptr;         // per absolute brick: images, rows, rows of the images (k_nl_table)
@@ -273,6 +273,7 @@ int launch_step_tma(sq_handle* h, const Wave& w, dim3 grid, int ic, int ip, floa
 // (TF32 planes in wb.Pg[1], float pairs in wb.Pg[0])
 int stencil_rows(const Geo& g);
 int stencil_chunks(const Geo& g);
+constexpr int kStepFill = 4 * 152;   // bricks of a wave up to which the FP64 step spreads each over four warps
 int build_nl_tables(sq_handle* h, size_t wi);
 int launch_step_mixed(sq_handle* h, size_t wi, const float* Tc, const float* Tp, float* Tn, int mode);
 int launch_project_mixed(sq_handle* h, size_t wi, const float* T);

@@ -249,6 +249,16 @@ static int step_warps(int bricks_per_slab) {
   return best;
 }
 
+// FP64 sweeps with at most one brick per SM quarter (of small cells, or a short last wave) give each brick a
+// block of its own and each of its four z-planes a warp: the FP64 unit of a quarter takes one warp
+// instruction in 75 clocks, so a brick's time is its longest warp's, and one warp per brick leaves most quarters
+// idle. 18 tiles of a 5 x 4 x 6 cell, 144 bricks: 210 -> 68 us a step (a block per brick with
+// one warp: 232 us). Returns the blocks per slab; 1: whole bricks per warp, all of the slab's in one block.
+int step_parts(const Geo& g, int ntiles, bool fp64) {
+  const int bricks = g.nbr[0] * g.nbr[2];
+  return fp64 && (long long)bricks * g.nslab * ntiles <= kStepFill ? bricks : 1;
+}
+
 // NCH: every atom has one channel (1: a table value per point in place of a padded group of four) or any number (4)
 template <typename Real, int NO, bool kSmemP, int NCH>
 __global__ void __launch_bounds__(kStepThreads, sizeof(Real) == 4 ? 4 : 2)
@@ -335,7 +345,12 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
   for (int k = 0; k < 9; ++k) sacc[k] = Real(0);
   const int nbx = g.nbr[0], nby = g.nbr[1], nbz = g.nbr[2];
 
-  for (int bi = warp; bi < nbx * nbz; bi += nw) {
+  // a warp's units of work: whole bricks, or one z-plane of a brick (step_parts); FP64 takes a plane's four
+  // points per lane at a time, FP32 two planes'
+  constexpr int kGrp = kG ? 1 : 2;   // planes per group
+  const int bps = nbx * nbz, sub = gridDim.z > 1 ? 4 : 1;
+  for (int un = blockIdx.z + gridDim.z * warp; un < bps * sub; un += gridDim.z * nw) {
+    const int bi = un % bps, pl0 = un / bps, pl1 = sub > 1 ? pl0 + 1 : 4;   // planes [pl0, pl1)
     const int bx = bi % nbx, bz = bi / nbx, by = slab;
     const int br = (bz * nby + by) * nbx + bx;
     const int4* rb = brec + ((size_t)tl * g.nbricks + br) * g.br_cap * 2;
@@ -343,24 +358,24 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
     Real* tnv = tn_sm + warp * 16 * 32 + lane;   // per lane and brick point: V_nl t^j, then t^{j+1}
     {
       // phase A: nonlocal apply, record-major: sum_rows chi_row(u) Pg^j[row][q] for the lane's
-      // 16 points; the table loads of one record are independent of each other
+      // points; the table loads of one record are independent of each other
 #pragma unroll 1
-      for (int half = 0; half < 2; ++half) {        // 8 points at a time keeps the accumulators in registers
-        Real ynl[8];
+      for (int pl = pl0; pl < pl1; pl += kGrp) {   // a few points at a time keep the accumulators in registers
+        Real ynl[4 * kGrp];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) ynl[i] = Real(0);
+        for (int i = 0; i < 4 * kGrp; ++i) ynl[i] = Real(0);
         for (int k = 0; k < nb; ++k) {
           const int4 r0 = rb[2 * k], r1 = rb[2 * k + 1];
           const int nch = r0.w & 0xff, nchp = (r0.w >> 8) & 0xff;
           const int prow = kSmemP ? (int(unsigned(r0.w) >> 16)) : r0.y;
-          const unsigned mk = unsigned(half ? r1.w : r1.z) >> pa;   // bits pa + 4 i of this half
-          if (!(mk & 0x11111111u)) continue;
+          const unsigned mk = unsigned(pl < 2 ? r1.z : r1.w) >> (pa + 16 * (pl & 1));   // bits 4 i of this group
+          if (!(mk & (kGrp == 1 ? 0x1111u : 0x11111111u))) continue;
           if constexpr (NCH == 1) {
             const Real pv = pg(prow * kTileB + q);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < 4 * kGrp; ++i)
               if ((mk >> (4 * i)) & 1u) {
-                const int it = 8 * half + i;
+                const int it = 4 * pl + i;
                 ynl[i] += chi[r0.x + (((it >> 2) * r1.y + (it & 3)) * r1.x + pa) * nchp] * pv;
               }
             continue;
@@ -370,9 +385,9 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
 #pragma unroll
             for (int c = 0; c < 4; ++c) pv[c] = (c0 + c < nch) ? pg((prow + c0 + c) * kTileB + q) : Real(0);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < 4 * kGrp; ++i) {
               if ((mk >> (4 * i)) & 1u) {
-                const int it = 8 * half + i;
+                const int it = 4 * pl + i;
                 Real cv[4];
                 load4(chi + r0.x + (((it >> 2) * r1.y + (it & 3)) * r1.x + pa) * nchp + c0, cv);
                 ynl[i] += cv[0] * pv[0] + cv[1] * pv[1] + cv[2] * pv[2] + cv[3] * pv[3];
@@ -381,13 +396,13 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
           }
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) tnv[(8 * half + i) * 32] = ynl[i];
+        for (int i = 0; i < 4 * kGrp; ++i) tnv[(4 * pl + i) * 32] = ynl[i];
       }
     }
     __syncwarp();
     {
 #pragma unroll 1
-      for (int it = 0; it < 16; ++it) {
+      for (int it = 4 * pl0; it < 4 * pl1; ++it) {
         const int pb = it & 3, pc = it >> 2;
         const int ux = bx * kBrick + pa, uy = by * kBrick + pb, uz = bz * kBrick + pc;
         const bool inU = (uy < Uy) && (uz < Uz);
@@ -444,10 +459,11 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
           const int nch = r0.w & 0xff, nchp = (r0.w >> 8) & 0xff;
           const int prow = kSmemP ? (int(unsigned(r0.w) >> 16)) : r0.y;
           const unsigned mlo = unsigned(r1.z) >> pa, mhi = unsigned(r1.w) >> pa;
+          if (sub > 1 && !((unsigned(pl0 < 2 ? r1.z : r1.w) >> (16 * (pl0 & 1))) & 0xffffu)) continue;
           if constexpr (NCH == 1) {
             Real acc = Real(0);
 #pragma unroll 8
-            for (int it = 0; it < 16; ++it)
+            for (int it = 4 * pl0; it < 4 * pl1; ++it)
               if (((it < 8 ? mlo : mhi) >> (4 * (it & 7))) & 1u)
                 acc += chi[r0.x + (((it >> 2) * r1.y + (it & 3)) * r1.x + pa) * nchp] * tnv[it * 32];
             acc += __shfl_xor_sync(0xffffffffu, acc, 8);
@@ -458,7 +474,7 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
           for (int c0 = 0; c0 < nch; c0 += 4) {
             Real acc[4] = {Real(0), Real(0), Real(0), Real(0)};
 #pragma unroll 4
-            for (int it = 0; it < 16; ++it) {
+            for (int it = 4 * pl0; it < 4 * pl1; ++it) {
               const unsigned bit = ((it < 8 ? mlo : mhi) >> (4 * (it & 7))) & 1u;
               if (bit) {
                 const Real tv = tnv[it * 32];
@@ -496,7 +512,7 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
     const int qq = k2 / 9, k = k2 % 9;
     double sv = 0.0;
     for (int wv = 0; wv < nw; ++wv) sv += red[(wv * kTileB + qq) * 9 + k];
-    Spart[(((size_t)tl * g.nslab + slab) * kTileB + qq) * 9 + k] = sv;
+    Spart[((((size_t)tl * g.nslab + slab) * gridDim.z + blockIdx.z) * kTileB + qq) * 9 + k] = sv;
   }
   if (kSmemP && project) {
     for (int i = threadIdx.x; i < nsr * kTileB; i += blockDim.x) {
@@ -621,7 +637,9 @@ static int launch_step(sq_handle* h, const Wave& w, dim3 grid, size_t smem, cons
                        int mode) {
   const int rows_smem = int(smem / (kTileB * (sizeof(double) + sizeof(Real))));
   const double* ncoef = (h->bounds_mode == SQ_BOUNDS_PER_NODE) ? h->d.ncoef : nullptr;
-  const int nw = h->step_warps > 0 ? h->step_warps : step_warps(h->geo.nbr[0] * h->geo.nbr[2]), nthr = 32 * nw;
+  grid.z = step_parts(h->geo, w.ntiles, sizeof(Real) == 8);
+  const int nw = h->step_warps > 0 ? h->step_warps : grid.z > 1 ? 4 : step_warps(h->geo.nbr[0] * h->geo.nbr[2]);
+  const int nthr = 32 * nw;
   const size_t smem_warps = size_t(nw) * (kTileB * 9 * sizeof(double) + 16 * 32 * sizeof(Real));
   // The dynamic-size attribute belongs to the function, not the launch, and handles on other
   // host threads launch the same kernel, so every caller sets the same value (the largest
@@ -710,6 +728,7 @@ static int sweep_t(sq_handle* h, const Real* chi, const Real* v, const Real* gdv
     const size_t smem = std::max<size_t>(1, size_t(rmax)) * kTileB * (sizeof(double) + sizeof(Real));
 
     const dim3 gstencil(g.nslab, w.ntiles);
+    const int parts = step_parts(g, w.ntiles, sizeof(Real) == 8);   // k_step's blocks per slab
     // algorithmic bytes of one stencil launch: node columns x region points x vectors moved
     long long nodes = 0;
     for (int tl = 0; tl < w.ntiles; ++tl) {
@@ -741,7 +760,7 @@ static int sweep_t(sq_handle* h, const Real* chi, const Real* v, const Real* gdv
                                                             stencil_chunks(g), h->d.mom);
       else
         k_moments<Real, false><<<w.ntiles, kThreads, 0, s>>>(g, w, j, Tc, A, Pg[j % 2], h->wb.n_rows, h->wb.Spart,
-                                                             g.nslab, h->d.mom);
+                                                             g.nslab * parts, h->d.mom);
       timing_end(h, ev);
       SQ_LAUNCH_CHECK(h);
       if (split && mode != 2) {
