@@ -6,7 +6,7 @@ stencil (n_o = 6), Gaussian V_eff and s+p Kleinman-Bylander projectors, kT = 3.1
 R_cut = 4 bohr (27^3 region per node), n_pl = 60 (seeded synthetic input).
 
 One step = one stress evaluation: Lanczos spectral bounds, the per-wave setup (atom-image
-lists, projector weights), the Chebyshev sweep with all moments, the Fermi-level bisection
+lists, projector weights), the Chebyshev sweep with all moments, the Fermi-level search
 and the contraction into rho, energies and sigma - every row of the hot path.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--precision mixed|fp64]

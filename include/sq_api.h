@@ -231,9 +231,10 @@ size_t sq_footprint_bytes(const sq_instance_desc* desc);
 long long sq_kernel_launches(const sq_handle* h);
 
 /* Launches of the Chebyshev step kernel since sq_setup, by variant, into counts[4] (host):
- *   counts[0]  projections of the block's atom images staged in shared memory, projector
- *              phases on tensor cores (SQ_MIXED, at most 4 channels per atom)
- *   counts[1]  staged in shared memory, scalar projector phases (SQ_FP64, or > 4 channels)
+ *   counts[0]  the split mixed step (SQ_MIXED, at most 4 channels per atom): projector apply and
+ *              projections on tensor cores and the stencil, each a kernel of its own
+ *   counts[1]  one kernel, projections of the block's atom images staged in shared memory, scalar
+ *              projector phases (SQ_FP64, > 4 channels, or bricks fuller than the split step's tables)
  *   counts[2]  projections read and accumulated in global memory (a block meets more
  *              projector rows than shared memory holds: dense atoms, large R_cut)
  *   counts[3]  the TMA-staged step (SQ_MIXED, at most 4 channels per atom, one projector
@@ -241,7 +242,7 @@ long long sq_kernel_launches(const sq_handle* h);
  *              (t^j with its stencil halo, W, t^{j-1}, the projector values of the images meeting
  *              it) copied into shared memory by the tensor memory accelerator
  * The environment variables, read by sq_setup: SQ_STEP_SMEM_ROWS lowers the row count above
- * which a block uses global memory (tuning and tests); SQ_STEP_KERNEL=staged puts a mixed handle
+ * which a block uses global memory, also in place of the split mixed step (tuning and tests); SQ_STEP_KERNEL=staged puts a mixed handle
  * on the TMA-staged step where its shared memory fits, SQ_STAGE_RECS (1..64, default 16) sets
  * the atom images per stage. Errors: SQ_ERR_INVALID_ARG. */
 int sq_step_launch_counts(const sq_handle* h, long long* counts);

@@ -12,7 +12,7 @@
 //                  record-major;
 //               B  Laplacian + V + the apply, the window mask, the recurrence update and the
 //                  nonlocal-stress partial sum_u W_b (grad_a t^j) (the gradient taps reuse the
-//                  Laplacian loads);
+//                  Laplacian loads; SQ_FP64: sum_u G_ab t^j, G = -grad_a W_b formed once per sweep);
 //               C  fused, the projections gamma |dOmega| chi^T t^{j+1} of the new column (register
 //                  sums and a reduce-scatter over the point lanes), one shared-memory FP64 add per
 //                  (image, channel, node), one global add per row and node per slab.
@@ -44,7 +44,9 @@ __device__ __forceinline__ void load4(const Real* p, Real out[4]) {
 // gridDim.x). A thread owns an (x, y) column of the image's box and half of the nodes: one projector load
 // per point serves four nodes, and the column only walks the z-chord of the support sphere (FP32 with a
 // 1e-5 margin; points past it hold zeros). Per thread in the vectors' precision, across threads as
-// doubles (FP64) or float pairs, fixed order. NCH as in k_step.
+// doubles (FP64) or float pairs, fixed order. NCH as in k_step. Bound by load latency (FP32) and the FP64
+// units (FP64). 216 tiles of a 12^3 cell, one channel: 278 us with the block's partial products summed in FP64 through
+// shared memory and channels padded to four -> 85 us; its 10 sample tiles 21 -> 12 us.
 constexpr int kProjThreads = 128, kProjWarps = kProjThreads / 32;
 template <typename Real, int NCH>
 __global__ void __launch_bounds__(kProjThreads)
@@ -120,9 +122,9 @@ k_project(Geo g, Wave w, const Real* __restrict__ Tn, const Real* __restrict__ c
 // out = H_q v on every node window of the wave (zero outside the windows); P from k_project. One block
 // per (4^3 brick of the window, tile): a warp is one z-plane of the brick, a thread one point and four of
 // its nodes, so the brick's image records (table offset, 64-bit sphere mask) are warp-uniform and a
-// projector load serves four nodes. One thread per (point, node) that looked every image of
-// its brick up in the atom tables took 78 us for the 10 sample tiles of a 12^3 cell, 410 us for
-// its 216 tiles.
+// projector load serves four nodes. Bound by load latency: with one channel per atom four images are read
+// at once (105 -> 73 us for the 216 tiles of a 12^3 cell, 15 -> 12 us for its 10 sample tiles). One thread per
+// (point, node) that looked every image of its brick up in the atom tables took 410 and 78 us.
 constexpr int kApplyThreads = 128;
 template <typename Real, int NCH>
 __global__ void __launch_bounds__(kApplyThreads)
