@@ -512,7 +512,11 @@ int run_contraction_nodes(sq_handle* h, double mu, double* rho_dev, double* out_
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
   const size_t smem = sizeof(double) * (4 * size_t((h->M + 1) / 2) + 3 * size_t(g.n_pl + 2));
-  SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_contract_nodes, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+  // the attribute belongs to the function and handles on other host threads launch it too: every caller sets the
+  // size of the largest M and n_pl sq_setup accepts (192 KB), never its own
+  constexpr int kMaxM = 6144, kMaxNpl = 4096;
+  constexpr int smem_max = int(sizeof(double)) * (4 * (kMaxM / 2) + 3 * (kMaxNpl + 2));
+  SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_contract_nodes, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
   k_contract_nodes<<<h->Nd, 256, smem, s>>>(h->d.mom, h->d.nbnd, h->d.v64, h->Nd, g.n_pl, h->M, h->d.costab, h->kT,
                                             mu, g.dV, rho_dev, h->d.nrow);
   SQ_LAUNCH_CHECK(h);
