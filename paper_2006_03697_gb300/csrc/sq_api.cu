@@ -138,7 +138,8 @@ struct Plan {
   int tile_begin = 0, tile_end = 0;   // the tiles this handle sweeps (the node partition)
   int lz_cap = 0;                     // most Lanczos sample tiles any V_eff can select
   int nlz_wave = 0;                   // tiles per Lanczos wave of the per-node bounds
-  size_t part_floats = 0, table_cap = 0, head_cap = 0;   // partial projections and brick tables of the split mixed step
+  bool split_able = false;            // the split mixed step can run
+  size_t nl_bricks = 0;               // most bricks of its tables
 };
 
 // Sample nodes of the Lanczos bounds: argmin V, argmax V and a stride-n/2 node grid; their
@@ -173,6 +174,33 @@ int lanczos_sample_cap(const sq::Geo& g) {
     grid *= (g.n[a] + st - 1) / st;
   }
   return std::min(2 + grid, g.n_tiles);
+}
+
+// Bricks that a sphere of radius rc can meet: the most over 4^3 positions of its centre in a brick (a brick's points
+// span 3 h), and a twentieth more.
+double bricks_met(const sq::Geo& g, double rc) {
+  constexpr int kPos = 4;
+  std::vector<double> d2[3][kPos];   // squared distance along an axis from the centre to each brick
+  for (int a = 0; a < 3; ++a)
+    for (int p = 0; p < kPos; ++p) {
+      const double c = sq::kBrick * g.h[a] * p / kPos;   // centre, past the first point of brick 0
+      const int reach = int(rc / (sq::kBrick * g.h[a])) + 2;
+      for (int b = -reach; b <= reach; ++b) {
+        const double lo = sq::kBrick * g.h[a] * b, hi = lo + (sq::kBrick - 1) * g.h[a];
+        const double x = c < lo ? lo - c : c > hi ? c - hi : 0.0;
+        if (x <= rc) d2[a][p].push_back(x * x);
+      }
+    }
+  for (int p = 0; p < kPos; ++p) std::sort(d2[2][p].begin(), d2[2][p].end());
+  long long most = 0;
+  for (int p = 0; p < kPos * kPos * kPos; ++p) {
+    const std::vector<double>&dx = d2[0][p % kPos], &dy = d2[1][p / kPos % kPos], &dz = d2[2][p / (kPos * kPos)];
+    long long n = 0;
+    for (double x : dx)
+      for (double y : dy) n += std::upper_bound(dz.begin(), dz.end(), rc * rc - x - y) - dz.begin();
+    most = std::max(most, n);
+  }
+  return 1.05 * double(most) + 2.0;
 }
 
 int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
@@ -309,8 +337,24 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
                      size_t(g.nslab) * (size_t(g.r_cap) + 1) * sizeof(int);   // slab row maps
   int max_nch = 1;
   for (const sq::AtomTab& at : P.atoms) max_nch = std::max(max_nch, at.nch);
-  const bool split = d->precision == SQ_MIXED && max_nch <= 4;   // the split mixed step
-  if (split) P.per_tile_bytes += (size_t(g.e_cap) + 1 + size_t(g.nbricks) * g.br_cap) * sizeof(int);   // image -> brick index
+  P.split_able = d->precision == SQ_MIXED && max_nch <= 4;
+  // its image -> brick index and the bricks' rows (nl_*: what each atom's images bring, bricks_met)
+  double nl_tile_rows = 0.0, nl_tile_imgs = 0.0;
+  std::vector<double> met(P.atoms.size(), 0.0);
+  if (P.split_able) {
+    double mult = 1.0;
+    for (int a = 0; a < 3; ++a) mult *= (sq::kBrick * g.nbr[a] + g.n[a] - 1) / g.n[a];
+    for (size_t J = 0; J < P.atoms.size(); ++J) {
+      size_t I = 0;
+      while (P.rcmax[I] != P.rcmax[J]) ++I;   // atoms of one radius share the count
+      met[J] = I < J ? met[I] : bricks_met(g, P.rcmax[J]);
+      if (P.atoms[J].nch == 0) continue;
+      const double in_tile = std::min(mult * met[J], double(g.nbricks) * mult);
+      nl_tile_imgs += in_tile;
+      nl_tile_rows += in_tile * P.atoms[J].nch;
+    }
+    P.per_tile_bytes += (size_t(g.e_cap) + 1 + size_t(nl_tile_imgs) + g.nbricks) * sizeof(int);
+  }
   long long Nd = (long long)g.n[0] * g.n[1] * g.n[2];
   int M = d->cheb_quad_M > 0 ? d->cheb_quad_M : 2048;
   P.fixed_bytes = size_t(sq::kStepFill) * g.B * 9 * sizeof(double) + size_t(Nd) * (sizeof(double) + sizeof(float)) +                       // V
@@ -357,24 +401,31 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
   const long long nwaves = (ntl + wc - 1) / wc;
   P.wave_cap = int((ntl + nwaves - 1) / nwaves);
   P.wave_cap = std::max<int>(P.wave_cap, P.lz_cap);
-  if (split) {
-    // partial projections of the whole wave, at most 4 GiB (the sweep then takes the tiles in chunks), at least
-    // one tile of the fullest bricks possible, and brick tables; sized for 2.5 times the mean number of
-    // images whose sphere meets a brick (Steiner's formula for the sphere and the box) plus 16, which
-    // uniform and clustered atoms stay below (fuller bricks take k_step)
-    double mean = 0.0;
-    const double a = sq::kBrick * g.h[0], b = sq::kBrick * g.h[1], c = sq::kBrick * g.h[2];
-    for (double r : P.rcmax)
-      mean += (a * b * c + 2.0 * (a * b + b * c + c * a) * r + M_PI * (a + b + c) * r * r + 4.0 / 3.0 * M_PI * r * r * r) /
-              (d->L[0] * d->L[1] * d->L[2]);
-    const int imgs = int(std::min<double>(g.br_cap, std::ceil(2.5 * mean) + 16.0));
-    const size_t rows = size_t(sq::nl_rows_padded(imgs, max_nch)), rows_top = size_t(sq::nl_rows_padded(g.br_cap, max_nch));
-    P.part_floats = std::max(std::min(size_t(P.wave_cap) * g.nbricks * rows * tileB, size_t(1) << 30),
-                             size_t(g.nbricks) * rows_top * tileB);
-    const size_t bricks = sq::nl_bricks_max(g, P.wave_cap);
-    P.table_cap = bricks * rows * 64 * sizeof(float2);
-    P.head_cap = bricks * (2 + size_t(g.br_cap));
-    P.fixed_bytes += P.part_floats * sizeof(float) + size_t(ch) * sizeof(float2) + P.table_cap + P.head_cap * sizeof(int);
+  if (P.split_able) {
+    // brick tables and partial projections (sized by ensure_nl_buffers from what the atoms' positions need; here:
+    // every periodic image that reaches a brick of the wave meets as many bricks as it can)
+    P.nl_bricks = sq::nl_bricks_max(g, P.wave_cap);
+    const long long n01 = (long long)g.tiles[0] * g.tiles[1];
+    const long long tz = std::min<long long>(g.tiles[2], (P.wave_cap + n01 - 1) / n01 + 1);
+    double mult = 0.0, rows = 0.0, imgs = 0.0;
+    for (int cls = 0; cls < 8; ++cls) {
+      const long long t[3] = {g.tiles[0], g.tiles[1], tz};
+      double m = 1.0;
+      for (int a = 0; a < 3; ++a) {
+        const long long cnt = (t[a] + (a < 2 && ((cls >> a) & 1) ? 0 : 1)) / 2;
+        m *= cnt > 0 ? double((sq::kBrick * (cnt + g.nbr[a] - 1) + g.n[a] - 1) / g.n[a]) : 0.0;
+      }
+      mult += m;
+    }
+    bool mixed_nch = false;
+    for (size_t J = 0; J < P.atoms.size(); ++J) {
+      imgs += mult * met[J] * (P.atoms[J].nch > 0);
+      rows += mult * met[J] * P.atoms[J].nch;
+      mixed_nch = mixed_nch || P.atoms[J].nch != P.atoms[0].nch;
+    }
+    const double part = std::min<double>(sq::kNlPartFloats * sizeof(float), 1.0625 * P.wave_cap * nl_tile_rows * tileB * sizeof(float));
+    P.fixed_bytes += size_t(rows * 64 * sizeof(float2)) + (mixed_nch ? size_t(imgs) * sizeof(int) : 0) + size_t(part) +
+                     P.nl_bricks * sizeof(int4) + size_t(ch) * sizeof(float2);
   }
   if (d->bounds_mode == SQ_BOUNDS_PER_NODE) {
     // every node's own Lanczos: waves of tiles with k + 2 Krylov vectors each under 8 GiB, the
@@ -443,6 +494,13 @@ int timing_collect(sq_handle* h) {
   return SQ_OK;
 }
 
+void dev_free(sq_handle* h, void* p, size_t bytes) {
+  if (!p) return;
+  cudaFree(p);
+  h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), p));
+  h->bytes -= bytes;
+}
+
 int dev_alloc(sq_handle* h, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
@@ -504,9 +562,7 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   h->proj4 = true;
   for (const sq::AtomTab& at : P.atoms) h->proj4 = h->proj4 && at.nchp <= 4;
   for (const sq::AtomTab& at : P.atoms) h->max_nch = std::max(h->max_nch, at.nch);
-  h->part_floats = P.part_floats;
-  h->table_cap = P.table_cap;
-  h->head_cap = P.head_cap;
+  h->split_able = P.split_able;
   h->table_len = P.table_len;
   h->n_ch_total = int(P.ch_l.size());
   h->wave_cap = P.wave_cap;
@@ -590,12 +646,11 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   SQ_ALLOC(h->wb.Pg[0], sizeof(double) * size_t(wt) * g.r_cap * g.B);   // projections: FP64 sums
   SQ_ALLOC(h->wb.Pg[1], sizeof(double) * size_t(wt) * g.r_cap * g.B);
   SQ_ALLOC(h->wb.Spart, sizeof(double) * std::max(size_t(wt) * std::max(g.nslab, sq::stencil_chunks(g)), size_t(sq::kStepFill)) * g.B * 9);
-  if (h->part_floats > 0) {
+  SQ_ALLOC(h->wb.nl_cnt, sizeof(int) * 8);
+  if (h->split_able) {   // (nl_X, nl_img, proj_idx and Part: ensure_nl_buffers)
     SQ_ALLOC(h->wb.proj_start, sizeof(int) * size_t(wt) * (size_t(g.e_cap) + 1));
-    SQ_ALLOC(h->wb.proj_idx, sizeof(unsigned) * size_t(wt) * g.nbricks * g.br_cap);
-    SQ_ALLOC(h->wb.Part, sizeof(float) * h->part_floats);
-    SQ_ALLOC(h->wb.nl_X, h->table_cap);
-    SQ_ALLOC(h->wb.nl_head, sizeof(int) * h->head_cap);
+    SQ_ALLOC(h->wb.proj_off, sizeof(int) * size_t(wt) * g.nbricks);
+    SQ_ALLOC(h->wb.nl_head, sizeof(int4) * P.nl_bricks);
     SQ_ALLOC(h->d.gdvp, sizeof(float2) * std::max(1, h->n_ch_total));
   }
   if (!h->lanczos_tiles.empty()) {

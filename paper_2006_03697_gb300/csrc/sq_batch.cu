@@ -61,6 +61,8 @@ struct sq_batch {
   int chains = 0;                       // parallel branches of the graph (members round-robin)
   std::vector<std::vector<int>> rows;   // wave layouts the graph was captured with
   std::vector<std::vector<int>> recs;   // and the brick image counts (staged step)
+  std::vector<std::vector<int>> nl;     // and the split step's rows per tile (-1: another step runs the wave)
+  std::vector<long long> nl_epoch;      // and its buffers
   cudaStream_t s0 = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -75,6 +77,21 @@ void drop_graph(sq_batch* b) {
   if (b->graph) cudaGraphDestroy(b->graph);
   b->exec = nullptr;
   b->graph = nullptr;
+}
+
+// what a capture bakes in of the split mixed step: whether it runs a wave, and the Part rows per tile
+std::vector<int> split_layout(const sq_handle* h) {
+  std::vector<int> r;
+  for (size_t w = 0; w < h->waves.size(); ++w)
+    r.push_back(sq::use_split(h, w) ? (w < h->wave_nl.size() ? h->wave_nl[w].tile_rows : 0) : -1);
+  return r;
+}
+
+bool split_stale(const std::vector<int>& old, const std::vector<int>& now) {
+  if (old.size() != now.size()) return true;
+  for (size_t w = 0; w < now.size(); ++w)
+    if (now[w] > old[w] || (now[w] < 0) != (old[w] < 0)) return true;
+  return false;
 }
 
 // one handle's evaluation with nothing crossing to the host
@@ -140,9 +157,13 @@ int capture(sq_batch* b) {
   }
   b->rows.clear();
   b->recs.clear();
+  b->nl.clear();
+  b->nl_epoch.clear();
   for (sq_handle* h : b->hs) {
     b->rows.push_back(h->wave_rows);
     b->recs.push_back(h->wave_recs);
+    b->nl.push_back(split_layout(h));
+    b->nl_epoch.push_back(h->nl_epoch);
   }
   return SQ_OK;
 }
@@ -185,7 +206,9 @@ int sq_batch_run(sq_batch* b, double* mu_out, sq_energies* e_out, double* sigma_
   sq::NvtxRange nvtx("sq_batch_run");
   const int n = int(b->hs.size());
   bool stale = !b->exec;
-  for (int i = 0; i < n; ++i)
+  for (int i = 0; i < n && !stale; ++i)
+    stale = b->nl_epoch[i] != b->hs[i]->nl_epoch || split_stale(b->nl[i], split_layout(b->hs[i]));
+  for (int i = 0; i < n && !stale; ++i)
     for (size_t w = 0; w < b->hs[i]->wave_rows.size(); ++w)
       if (b->rows[i].size() != b->hs[i]->wave_rows.size() || b->hs[i]->wave_rows[w] > b->rows[i][w] ||
           b->recs[i].size() != b->hs[i]->wave_recs.size() || b->hs[i]->wave_recs[w] > b->recs[i][w])

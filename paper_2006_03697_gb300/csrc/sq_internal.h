@@ -119,11 +119,21 @@ struct WaveBufs {
   void* P = nullptr;              // Real [wt][r_cap][B]  gamma |dOmega| chi^T t (Lanczos apply)
   void* Pg[2] = {nullptr, nullptr};   // double [wt][r_cap][B]  gamma |dOmega| chi^T t^j, ping-pong
   double* Spart = nullptr;        // [wt][slabs, their bricks or stencil row chunks][B][9]
-  int* proj_start = nullptr;      // [wt][e_cap + 1] split mixed step: an image's entries of proj_idx
-  unsigned* proj_idx = nullptr;   // [wt][nbricks * br_cap] brick << 16 | first projector row in the brick
-  int* nl_head = nullptr;         // per absolute brick: images, rows, rows of the images (k_nl_table)
-  float2* nl_X = nullptr;         // per absolute brick: [rows][64 points] projector values, TF32 (hi, lo)
-  float* Part = nullptr;          // partial projections of a chunk of tiles [tiles][nbricks][rows][B]
+  // the split mixed step (sq_step_mixed.cu)
+  int* proj_start = nullptr;      // [wt][e_cap + 1] an image's entries of proj_idx
+  int* proj_idx = nullptr;        // [wt][idx_cap] first Part row of an image in a brick it meets
+  int* proj_off = nullptr;        // [wt][nbricks] a brick's first Part row among its tile's
+  int* nl_cnt = nullptr;          // counters of the table builds, results of measure_wave_rows
+  int4* nl_head = nullptr;        // per absolute brick (k_nl_table)
+  int* nl_img = nullptr;          // image lists of bricks whose images differ in their channels
+  float2* nl_X = nullptr;         // [rows][64 points] projector values of the bricks, TF32 (hi, lo)
+  float* Part = nullptr;          // partial projections of a chunk of tiles [tiles][rows of a tile][B]
+};
+
+// what the split mixed step's tables of a wave need: rows of nl_X, entries of nl_img, and most Part rows and
+// proj_idx entries of a tile
+struct NlNeed {
+  int x_rows = 0, imgs = 0, tile_rows = 0, tile_imgs = 0;
 };
 
 struct Dev {
@@ -194,6 +204,8 @@ struct sq_handle {
   std::vector<sq::Wave> waves;
   std::vector<int> wave_rows;       // per wave: most projector rows of a slab (shared-memory size)
   std::vector<int> wave_recs;       // per wave: most atom images meeting one brick (staged step)
+  std::vector<sq::NlNeed> wave_nl;  // per wave: sizes of the split mixed step's tables
+  long long nl_epoch = 0;           // bumped whenever one of their buffers is reallocated
   int tile_begin = 0, tile_end = 0;   // tiles this handle sweeps (node partition)
   int wave_cap = 0;
   sq::Dev d;
@@ -225,8 +237,9 @@ struct sq_handle {
   bool stage_wait_test = false;     // SQ_STAGE_WAIT_TEST=1: the staged step's copy wait runs out (tests)
   int step_rows_cap = 0;            // most projector rows a step block stages in shared memory
   bool step_rows_env = false;       // SQ_STEP_SMEM_ROWS was given
+  bool split_able = false;          // SQ_MIXED and at most 4 channels per atom: the split step can run
   size_t part_floats = 0;           // floats of wb.Part
-  size_t table_cap = 0, head_cap = 0;   // bytes of wb.nl_X, ints of wb.nl_head
+  size_t x_rows_cap = 0, img_cap = 0, idx_cap = 0;   // rows of wb.nl_X, entries of wb.nl_img, of wb.proj_idx per tile
   int max_nch = 1;                  // most projector channels of an atom
   int step_warps = 0;               // warps per step block (0: the brick-count rule; set by the tuner)
   // optional event timing of the sweep kernels
@@ -277,14 +290,17 @@ constexpr int kStepFill = 4 * 152;   // bricks of a wave up to which the FP64 st
 int build_nl_tables(sq_handle* h, size_t wi);
 int launch_step_mixed(sq_handle* h, size_t wi, const float* Tc, const float* Tp, float* Tn, int mode);
 int launch_project_mixed(sq_handle* h, size_t wi, const float* T);
-// table rows of a brick of imgs images: whole MMA tiles and 16 rows of zeros
-inline int nl_rows_padded(int imgs, int max_nch) { return (imgs * max_nch + 15) / 16 * 16 + 16; }
 size_t nl_bricks_max(const Geo& g, int wave_cap);
+constexpr size_t kNlPartFloats = size_t(1) << 29;   // most floats of wb.Part
+int count_nl_tables(sq_handle* h, size_t wi, int* cnt);
+int ensure_nl_buffers(sq_handle* h);
 // floats from the hi to the lo plane of the split projections in wb.Pg[1]
 inline size_t nl_plane(const sq_handle* h) { return size_t(h->wave_cap) * h->geo.r_cap * 8; }
 bool nl_fits(const sq_handle* h, size_t wi);   // do the wave's tables fit their buffers?
-// does the split step run wave wi?
+// may the split step run wave wi, and does it (its tables fit)?
+bool want_split(const sq_handle* h, size_t wi);
 bool use_split(const sq_handle* h, size_t wi);
+void dev_free(sq_handle* h, void* p, size_t bytes);
 // one recurrence step launch (mode 1) of wave 0 with the handle's current settings, timed with
 // CUDA events on its stream (sq_sweep.cu; the autotuner's measurement)
 int time_step_launch(sq_handle* h, int reps, double* ms_out);

@@ -489,7 +489,7 @@ int build_wave_entries(sq_handle* h, const Wave& w, WaveBufs* b) {
   if (b == &h->wb) h->lists_key = {w.tile0, w.ntiles, w.ids, h->atoms_epoch, false};
   k_tile_entries<<<w.ntiles, 256, 0, s>>>(g, w, h->d.atoms, b->entries, b->n_entries, b->n_rows, h->d.status);
   SQ_LAUNCH_CHECK(h);
-  k_brick_lists<<<dim3(g.nbricks, w.ntiles), 32, 0, s>>>(g, w, h->wb.Part ? 1 : 0, h->d.atoms, h->d.rcmax, b->entries, b->n_entries,
+  k_brick_lists<<<dim3(g.nbricks, w.ntiles), 32, 0, s>>>(g, w, h->split_able ? 1 : 0, h->d.atoms, h->d.rcmax, b->entries, b->n_entries,
                                                           b->brick_list, b->brick_n, b->brick_rec, b->brick_d0,
                                                           b->brick_tma, b->slab_n, b->slab_map, h->d.status);
   SQ_LAUNCH_CHECK(h);

@@ -22,9 +22,7 @@ namespace sq {
 constexpr int kNlThreads = 256;   // k_nl_apply: 8 warps
 constexpr int kPrThreads = 256;   // k_nl_project: 8 warps over 1 .. 4 row tiles
 constexpr int kNlRows = 64;       // projector rows of a brick per pass (eight K-steps of 8)
-constexpr int kNlPitch = 68;      // points per row in shared memory (float2; conflict-free fragments)
 constexpr int kNlList = 352;      // (tile, brick) pairs per list
-constexpr int kNlSteps = kNlRows / 8;
 constexpr int kApG = 8;           // tiles per staged group of k_nl_apply (one per warp)
 constexpr int kPrG = 8;           // of k_nl_project
 __device__ __forceinline__ void cp16(unsigned dst, const void* src) {
@@ -39,9 +37,11 @@ __device__ __forceinline__ float2 ld2g(const float* p) { return *reinterpret_cas
 struct NlGrid {
   int tlo[3], thi[3];   // range of the wave's tiles per axis
   int nb[3];            // most bricks of a class per axis
+  int z0, nz;           // brick layers of the launch (those the tiles of a chunk reach)
 };
 
-static NlGrid nl_grid(const Geo& g, const Wave& w) {
+// of a wave, for a launch over its tiles [c0, c0 + cn)
+static NlGrid nl_grid(const Geo& g, const Wave& w, int c0, int cn) {
   NlGrid r;
   const int t1 = w.tile0 + w.ntiles - 1, n01 = g.tiles[0] * g.tiles[1];
   const int lo[3] = {0, 0, w.tile0 / n01}, hi[3] = {g.tiles[0] - 1, g.tiles[1] - 1, t1 / n01};
@@ -54,8 +54,19 @@ static NlGrid nl_grid(const Geo& g, const Wave& w) {
     r.thi[1] = t1 / g.tiles[0] % g.tiles[1];
   }
   for (int a = 0; a < 3; ++a) r.nb[a] = (r.thi[a] - r.tlo[a] + 2) / 2 + g.nbr[a] - 1;
+  const int z0 = (w.tile0 + c0) / n01, z1 = (w.tile0 + c0 + cn - 1) / n01;
+  int f0 = r.nb[2], f1 = 0;
+  for (int k = 0; k < 2; ++k) {   // tile layers of parity k
+    const int base = std::max(0, (r.tlo[2] - k + 1) >> 1), ilo = std::max(0, (z0 - k + 1) >> 1), ihi = (z1 - k) >> 1;
+    if (ihi < ilo) continue;
+    f0 = std::min(f0, ilo - base);
+    f1 = std::max(f1, ihi - base + g.nbr[2]);
+  }
+  r.z0 = f0;
+  r.nz = f1 - f0;
   return r;
 }
+static NlGrid nl_grid(const Geo& g, const Wave& w) { return nl_grid(g, w, 0, w.ntiles); }
 
 size_t nl_bricks_max(const Geo& g, int wave_cap) {   // of any wave of up to wave_cap contiguous tiles
   const long long n01 = (long long)g.tiles[0] * g.tiles[1];
@@ -72,7 +83,7 @@ struct NlBrick {
 };
 
 __device__ __forceinline__ bool nl_brick(const Geo& g, const NlGrid& n, NlBrick& r) {
-  const int f[3] = {int(blockIdx.x), int(blockIdx.y), int(blockIdx.z >> 3)}, cls = blockIdx.z & 7;
+  const int f[3] = {int(blockIdx.x), int(blockIdx.y), int(blockIdx.z >> 3) + n.z0}, cls = blockIdx.z & 7;
   for (int a = 0; a < 3; ++a) {
     r.kap[a] = (cls >> a) & 1;
     const int ilo = max(0, (n.tlo[a] - r.kap[a] + 1) >> 1), ihi = (n.thi[a] - r.kap[a]) >> 1;   // ihi < ilo: no tile
@@ -81,22 +92,43 @@ __device__ __forceinline__ bool nl_brick(const Geo& g, const NlGrid& n, NlBrick&
     r.lo[a] = max(ilo, r.beta[a] - g.nbr[a] + 1);
     r.cnt[a] = min(ihi, r.beta[a]) - r.lo[a] + 1;
   }
-  r.index = (int(blockIdx.z) * n.nb[1] + f[1]) * n.nb[0] + f[0];
+  r.index = ((8 * f[2] + cls) * n.nb[1] + f[1]) * n.nb[0] + f[0];
   return true;
 }
 
+// table entry of brick br of global tile t
+__device__ __forceinline__ int nl_index(const Geo& g, const NlGrid& n, int t, int br) {
+  const int tc[3] = {t % g.tiles[0], t / g.tiles[0] % g.tiles[1], t / (g.tiles[0] * g.tiles[1])};
+  const int b[3] = {br % g.nbr[0], br / g.nbr[0] % g.nbr[1], br / (g.nbr[0] * g.nbr[1])};
+  int f[3], cls = 0;
+  for (int a = 0; a < 3; ++a) {
+    const int k = tc[a] & 1;
+    f[a] = (tc[a] >> 1) + b[a] - max(0, (n.tlo[a] - k + 1) >> 1);
+    cls |= k << a;
+  }
+  return ((8 * f[2] + cls) * n.nb[1] + f[1]) * n.nb[0] + f[0];
+}
+
+// Where the partial projections of a chunk's tiles go: off[tile of the wave][brick] = the brick's first row among
+// the tile's (-1: the tile is left out), rows of Part per tile
+struct NlPart {
+  const int* off;
+  int rows;
+};
+
 struct NlShared {
-  // tile of the chunk, tile * nbricks + brick, first point of the brick in the tile's window, points of the
-  // brick inside the window in y | in z << 4
+  // tile of the chunk, tile * nbricks + brick (apply) or first row in Part (project), first point of the brick in
+  // the tile's window, points of the brick inside the window in y | in z << 4
   int4 list[kNlList];
   int img[32];                   // first row (of the pass) << 4 | channels of the images of the pass
   int n, nb, nrows, nimg, row0;
+  int x0;                        // the brick's first row in X
 };
 
 // the brick's tiles among tiles [c0, c0 + cn) of the wave, entries [i0, i0 + kNlList) of the class box, by
 // threads first, first + 1, ... of the block (between barriers; sh.n starts at 0)
 __device__ __forceinline__ void nl_list(const Geo& g, const Wave& w, int c0, int cn, const NlBrick& b, int i0, int first,
-                                        NlShared& sh) {
+                                        const NlPart& part, NlShared& sh) {
   const int total = b.cnt[0] * b.cnt[1] * b.cnt[2], n = min(kNlList, total - i0);
   for (int i = int(threadIdx.x) - first; i >= 0 && i < n; i += blockDim.x - first) {
     const int f = i0 + i, f1 = f / b.cnt[0], f2 = f1 / b.cnt[1];
@@ -105,37 +137,79 @@ __device__ __forceinline__ void nl_list(const Geo& g, const Wave& w, int c0, int
                    w.tile0 - c0;
     if (tl < 0 || tl >= cn) continue;
     const int bx = b.beta[0] - i3[0], by = b.beta[1] - i3[1], bz = b.beta[2] - i3[2];
-    sh.list[atomicAdd(&sh.n, 1)] = make_int4(tl, tl * g.nbricks + (bz * g.nbr[1] + by) * g.nbr[0] + bx,
-                                             kBrick * ((bz * g.U[1] + by) * g.U[0] + bx),
+    int y = tl * g.nbricks + (bz * g.nbr[1] + by) * g.nbr[0] + bx;
+    if (part.off) {
+      const int o = __ldg(part.off + (size_t)c0 * g.nbricks + y);
+      if (o < 0) continue;
+      y = tl * part.rows + o;
+    }
+    sh.list[atomicAdd(&sh.n, 1)] = make_int4(tl, y, kBrick * ((bz * g.U[1] + by) * g.U[0] + bx),
                                              min(kBrick, g.U[1] - kBrick * by) | min(kBrick, g.U[2] - kBrick * bz) << 4);
   }
 }
 
-// Table of the wave's bricks, built with its lists and read by every step: head [2 + imgs] = images, rows,
-// then first row << 4 | channels per image; X [rows][64 points] = the image's channel at the brick's points
-// as a TF32 (hi, lo) pair, zero outside the support sphere, and 16 rows of zeros after the last one. The
-// records of all tiles that share a brick list the same images in the same order, so any of them will do.
+// Table of the wave's bricks, built with its lists and read by every step. head [brick] = {images, rows, first row
+// in X, c}: c >= 0: every image has c channels, else its image list (first row << 4 | channels) starts at
+// img[-1 - c]; X [rows][64 points] = the image's channel at the brick's points as a TF32 (hi, lo) pair, zero
+// outside the support sphere. The records of all tiles that share a brick list the same images in the same
+// order, so any of them will do. Rows are handed out by a counter, a brick taking what it needs: the sum over the
+// bricks hardly depends on where the atoms are, while the fullest brick of a cluster holds several times the mean
+// (a fixed number of rows per brick had to be 2.5 times the mean and sent clusters to the scalar step: 48 H in a
+// 3.9 bohr sphere of a 16 bohr cell, 257 ms an evaluation with the step before the split one, 506 with the scalar one).
+// cnt [2] = rows, images needed; X null: counts only.
 __global__ void __launch_bounds__(128)
 k_nl_table(Geo g, Wave w, NlGrid grid, const float* __restrict__ chis, const int4* __restrict__ brec,
-           const int* __restrict__ bn, int imgs, int rows_cap, int* __restrict__ head, float2* __restrict__ X,
-           int* __restrict__ status) {
+           const int* __restrict__ bn, long long rows_cap, long long img_cap, int* __restrict__ cnt, int4* __restrict__ head,
+           int* __restrict__ img, float2* __restrict__ X, int* __restrict__ status) {
   __shared__ NlShared sh;
-  __shared__ int row_of[32];
+  __shared__ int row_of[32], wsum[4], wlo[4], whi[4];
+  __shared__ int4 hd_s;
   NlBrick b;
   if (!nl_brick(g, grid, b)) return;
-  int* hd = head + (size_t)b.index * (2 + imgs);
-  float2* Xb = X + (size_t)b.index * rows_cap * 64;
   const int total = b.cnt[0] * b.cnt[1] * b.cnt[2], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i0 = 0; i0 < total; i0 += kNlList) {
     __syncthreads();
     if (threadIdx.x == 0) sh.n = 0;
     __syncthreads();
-    nl_list(g, w, 0, w.ntiles, b, i0, 0, sh);
+    nl_list(g, w, 0, w.ntiles, b, i0, 0, NlPart{nullptr, 0}, sh);
     __syncthreads();
     if (sh.n == 0) continue;
     const size_t tb = sh.list[0].y;
     const int4* rec = brec + tb * g.br_cap * 2;
     const int nb = bn[tb];
+    int sum = 0, lo = kMaxCh, hi = 0;   // rows; fewest and most channels of an image
+    for (int k = threadIdx.x; k < nb; k += blockDim.x) {
+      const int nch = rec[2 * k].w & 0xff;
+      sum += nch;
+      lo = min(lo, nch);
+      hi = max(hi, nch);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+      wsum[warp] = sum;
+      wlo[warp] = lo;
+      whi[warp] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const int rows = wsum[0] + wsum[1] + wsum[2] + wsum[3];
+      const int l = min(min(wlo[0], wlo[1]), min(wlo[2], wlo[3])), h = max(max(whi[0], whi[1]), max(whi[2], whi[3]));
+      const bool list = nb > 0 && l != h;
+      int4 hd = make_int4(nb, rows, atomicAdd(cnt, rows), nb > 0 ? h : 0);
+      if (list) hd.w = -1 - atomicAdd(cnt + 1, nb);
+      if (X && (hd.z + (long long)rows > rows_cap || (list && -1ll - hd.w + nb > img_cap))) {
+        atomicOr(status + kStOverflow, 8);   // a launch sized for another layout (a stale graph): refuse
+        hd = make_int4(0, 0, 0, 0);
+      }
+      hd_s = hd;
+      if (X) head[b.index] = hd;
+    }
+    __syncthreads();
+    const int4 hd = hd_s;
+    if (!X || hd.x == 0) return;
+    float2* Xb = X + (size_t)hd.z * 64;
     int row = 0;
     for (int k0 = 0; k0 < nb; k0 += 32) {
       const int k = k0 + lane, nch = k < nb ? rec[2 * k].w & 0xff : 0;
@@ -147,17 +221,10 @@ k_nl_table(Geo g, Wave w, NlGrid grid, const float* __restrict__ chis, const int
       __syncthreads();
       if (warp == 0) {
         row_of[lane] = row + incl - nch;
-        if (k < nb && k < imgs) hd[2 + k] = (row + incl - nch) << 4 | nch;
+        if (hd.w < 0 && k < nb) img[-1 - hd.w + k] = (row + incl - nch) << 4 | nch;
       }
       row += __shfl_sync(0xffffffffu, incl, 31);
       __syncthreads();
-      if (row > rows_cap - 16 || nb > imgs) {   // a launch sized for another layout (a stale graph): refuse
-        if (threadIdx.x == 0) {
-          atomicOr(status + kStOverflow, 8);
-          hd[0] = hd[1] = 0;
-        }
-        return;
-      }
       for (int i = warp; i < min(32, nb - k0); i += 4) {
         const int4 r0 = rec[2 * (k0 + i)], r1 = rec[2 * (k0 + i) + 1];
         for (int h = 0; h < 2; ++h) {   // points lane and lane + 32
@@ -168,20 +235,17 @@ k_nl_table(Geo g, Wave w, NlGrid grid, const float* __restrict__ chis, const int
         }
       }
     }
-    for (int i = threadIdx.x; i < 16 * 64; i += blockDim.x) Xb[row * 64 + i] = make_float2(0.f, 0.f);
-    if (threadIdx.x == 0) {
-      hd[0] = nb;
-      hd[1] = row;
-    }
     return;
   }
-  if (threadIdx.x == 0) hd[0] = hd[1] = 0;
+  if (threadIdx.x == 0 && X) head[b.index] = make_int4(0, 0, 0, 0);
 }
 
 // The next pass over the brick's images (from image k0 on, as many as fit 32 images, one per lane, and
-// kNlRows rows): sh.nimg, sh.nrows, their rows, and sh.row0, the pass's first row in the table. One warp.
-__device__ __forceinline__ void nl_pass(const int* __restrict__ hd, int k0, NlShared& sh) {
-  const int lane = threadIdx.x & 31, nb = hd[0], k = k0 + lane, x = k < nb ? hd[2 + k] : 0;
+// kNlRows rows): sh.nimg, sh.nrows, their rows, and sh.row0, the pass's first row of the brick. One warp.
+__device__ __forceinline__ void nl_pass(const int4* __restrict__ hd_p, const int* __restrict__ img, int k0, NlShared& sh) {
+  const int4 hd = __ldg(hd_p);
+  const int lane = threadIdx.x & 31, nb = hd.x, k = k0 + lane;
+  const int x = k < nb ? (hd.w >= 0 ? (k * hd.w) << 4 | hd.w : __ldg(img - 1 - hd.w + k)) : 0;
   const int first = __shfl_sync(0xffffffffu, x >> 4, 0), end = (x >> 4) + (x & 15) - first;
   const bool fits = k < nb && end <= kNlRows;
   sh.img[lane] = ((x >> 4) - first) << 4 | (x & 15);
@@ -190,6 +254,7 @@ __device__ __forceinline__ void nl_pass(const int* __restrict__ hd, int k0, NlSh
     sh.nb = nb;
     sh.nimg = __popc(m);
     sh.row0 = first;
+    sh.x0 = hd.z;
     if (!m) sh.nrows = 0;
   }
   if (m && lane == 31 - __clz(m)) sh.nrows = end;
@@ -198,18 +263,19 @@ __device__ __forceinline__ void nl_pass(const int* __restrict__ hd, int k0, NlSh
 // Tiles i0 .. of the brick and the first pass of its images, side by side: warp 0 reads the brick's
 // table entry while the others list its tiles.
 __device__ __forceinline__ void nl_begin(const Geo& g, const Wave& w, int c0, int cn, const NlBrick& b, int i0,
-                                         const int* __restrict__ hd, NlShared& sh) {
+                                         const NlPart& part, const int4* __restrict__ hd, const int* __restrict__ img,
+                                         NlShared& sh) {
   __syncthreads();
   if (threadIdx.x == 0) sh.n = 0;
   __syncthreads();
-  if (threadIdx.x < 32) nl_pass(hd, 0, sh);
-  else nl_list(g, w, c0, cn, b, i0, 32, sh);
+  if (threadIdx.x < 32) nl_pass(hd, img, 0, sh);
+  else nl_list(g, w, c0, cn, b, i0, 32, part, sh);
   __syncthreads();
 }
 
-__device__ __forceinline__ void nl_next(const int* __restrict__ hd, int k0, NlShared& sh) {
+__device__ __forceinline__ void nl_next(const int4* __restrict__ hd, const int* __restrict__ img, int k0, NlShared& sh) {
   __syncthreads();
-  if (threadIdx.x < 32) nl_pass(hd, k0, sh);
+  if (threadIdx.x < 32) nl_pass(hd, img, k0, sh);
   __syncthreads();
 }
 
@@ -223,7 +289,7 @@ __device__ __forceinline__ void nl_apply_pass(const Geo& g, NlShared& sh, float*
                                               const float2* __restrict__ X, const float* __restrict__ P, size_t lo_plane,
                                               const int4* __restrict__ brec, float* __restrict__ Y) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g8 = lane >> 2, t4 = lane & 3;
-  const int mt = warp & 3, p = 16 * mt + g8, n = sh.n, nimg = sh.nimg;
+  const int mt = warp & 3, p = 16 * mt + g8, n = sh.n, nimg = sh.nimg, nrows = sh.nrows;
   constexpr int kPlane = 8 * NKS * 8, kTile = 2 * kPlane;   // floats of one plane, one staged tile
   const unsigned bs = (unsigned)__cvta_generic_to_shared(Bs) + warp * kTile * 4;
   // lane = image: first row << 4 | channels, and its first projector row in the warp's tile of a group
@@ -234,8 +300,11 @@ __device__ __forceinline__ void nl_apply_pass(const Geo& g, NlShared& sh, float*
   uint32_t ah[NKS + 1][4], al[NKS + 1][4];   // (one spare: no zero-size arrays)
 #pragma unroll
   for (int ks = 0; ks < NKS; ++ks) {
-    const float2* xr = X + (8 * ks + t4) * 64 + p;   // zeros follow the last row
-    const float2 x0 = __ldg(xr), x1 = __ldg(xr + 8), x2 = __ldg(xr + 256), x3 = __ldg(xr + 264);
+    const float2* xr = X + (8 * ks + t4) * 64 + p;
+    const bool in0 = 8 * ks + t4 < nrows, in1 = 8 * ks + t4 + 4 < nrows;   // (another pass's or brick's rows follow)
+    const float2 zero = make_float2(0.f, 0.f);
+    const float2 x0 = in0 ? __ldg(xr) : zero, x1 = in0 ? __ldg(xr + 8) : zero;
+    const float2 x2 = in1 ? __ldg(xr + 256) : zero, x3 = in1 ? __ldg(xr + 264) : zero;
     ah[ks][0] = __float_as_uint(x0.x); al[ks][0] = __float_as_uint(x0.y);
     ah[ks][1] = __float_as_uint(x1.x); al[ks][1] = __float_as_uint(x1.y);
     ah[ks][2] = __float_as_uint(x2.x); al[ks][2] = __float_as_uint(x2.y);
@@ -302,22 +371,21 @@ constexpr size_t kApSmem = (sizeof(NlShared) + 15) / 16 * 16 + 2 * kApG * kNlRow
 
 __global__ void __launch_bounds__(kNlThreads, 2)
 k_nl_apply(Geo g, Wave w, NlGrid grid, int max_nch, const float* __restrict__ P, size_t lo_plane,
-           const int* __restrict__ head, int imgs, const float2* __restrict__ X, int rows_cap,
+           const int4* __restrict__ head, const int* __restrict__ img, const float2* __restrict__ X,
            const int4* __restrict__ brec, float* __restrict__ Y) {
   extern __shared__ __align__(16) unsigned char nl_smem[];
   NlShared& sh = *reinterpret_cast<NlShared*>(nl_smem);
   float* Bs = reinterpret_cast<float*>(nl_smem + (sizeof(NlShared) + 15) / 16 * 16);
   NlBrick b;
   if (!nl_brick(g, grid, b)) return;
-  const int* hd = head + (size_t)b.index * (2 + imgs);
-  const float2* Xb = X + (size_t)b.index * rows_cap * 64;
+  const int4* hd = head + b.index;
   const int total = b.cnt[0] * b.cnt[1] * b.cnt[2];
   for (int i0 = 0; i0 < total; i0 += kNlList) {
-    nl_begin(g, w, 0, w.ntiles, b, i0, hd, sh);
+    nl_begin(g, w, 0, w.ntiles, b, i0, NlPart{nullptr, 0}, hd, img, sh);
     if (sh.n == 0) continue;
     int k0 = 0;
     for (;;) {
-      const float2* Xp = Xb + sh.row0 * 64;
+      const float2* Xp = X + (size_t)(sh.x0 + sh.row0) * 64;
       switch ((sh.nrows + 7) / 8) {
         case 0: nl_apply_pass<0>(g, sh, Bs, k0, max_nch, Xp, P, lo_plane, brec, Y); break;
         case 1: nl_apply_pass<1>(g, sh, Bs, k0, max_nch, Xp, P, lo_plane, brec, Y); break;
@@ -331,12 +399,12 @@ k_nl_apply(Geo g, Wave w, NlGrid grid, int max_nch, const float* __restrict__ P,
       }
       k0 += sh.nimg;
       if (k0 >= sh.nb) break;
-      nl_next(hd, k0, sh);
+      nl_next(hd, img, k0, sh);
     }
   }
 }
 
-// Part[(tile brick) rows_cap + row][8 nodes] = X^T[rows][64 points] t[64 points][8] of every tile that holds the
+// Part[tile][off[tile][brick] + row][8 nodes] = X^T[rows][64 points] t[64 points][8] of every tile that holds the
 // brick (rows of the brick in record order). Per group of kPrG tiles t is read once (16 bytes a load, one
 // group ahead), split to TF32 (hi, lo) and staged in shared memory for the brick's row tiles: a warp owns
 // 16 rows (A fragments of the 64 points in registers), 16 shared loads and 24 MMAs per tile. Loading and
@@ -345,15 +413,14 @@ constexpr int kPrTile = 2 * 64 * 8;   // floats of one staged tile: hi and lo pl
 constexpr size_t kPrSmem = (sizeof(NlShared) + 15) / 16 * 16 + 2 * kPrG * kPrTile * sizeof(float);
 
 __global__ void __launch_bounds__(kPrThreads, 2)
-k_nl_project(Geo g, Wave w, NlGrid grid, int c0, int cn, const float* __restrict__ T, const int* __restrict__ head,
-             int imgs, const float2* __restrict__ X, int rows_cap, float* __restrict__ Part) {
+k_nl_project(Geo g, Wave w, NlGrid grid, int c0, int cn, const float* __restrict__ T, const int4* __restrict__ head,
+             const int* __restrict__ img, const float2* __restrict__ X, NlPart part, float* __restrict__ Part) {
   extern __shared__ __align__(16) unsigned char nl_smem[];   // tiles c0 .. c0 + cn - 1 of the wave
   NlShared& sh = *reinterpret_cast<NlShared*>(nl_smem);
   float* Bs = reinterpret_cast<float*>(nl_smem + (sizeof(NlShared) + 15) / 16 * 16);
   NlBrick b;
   if (!nl_brick(g, grid, b)) return;
-  const int* hd = head + (size_t)b.index * (2 + imgs);
-  const float2* Xb = X + (size_t)b.index * rows_cap * 64;
+  const int4* hd = head + b.index;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g8 = lane >> 2, t4 = lane & 3;
   const int total = b.cnt[0] * b.cnt[1] * b.cnt[2];
   const float* Tw = T + (size_t)c0 * g.Upts * 8;
@@ -363,7 +430,7 @@ k_nl_project(Geo g, Wave w, NlGrid grid, int c0, int cn, const float* __restrict
   const int py = (pt >> 2) & 3, pz = pt >> 4;
   const int toff = ((pz * g.U[1] + py) * g.U[0] + (pt & 3)) * 8 + 4 * h4;
   for (int i0 = 0; i0 < total; i0 += kNlList) {
-    nl_begin(g, w, c0, cn, b, i0, hd, sh);
+    nl_begin(g, w, c0, cn, b, i0, part, hd, img, sh);
     const int n = sh.n;
     if (n == 0 || sh.nb == 0) continue;
     for (int k0 = 0;;) {
@@ -372,8 +439,8 @@ k_nl_project(Geo g, Wave w, NlGrid grid, int c0, int cn, const float* __restrict
       const int mt = warp % nmt, str = kPrThreads / 32 / nmt + (mt < (kPrThreads / 32) % nmt), r = 16 * mt + g8;
       uint32_t ah[8][4], al[8][4];
       {
-        const float2 *x0p = Xb + (rbase + r) * 64 + t4, *x1p = x0p + 8 * 64;   // padded with zeros to whole tiles
-        const bool in0 = r < nrows, in1 = r + 8 < nrows;   // (another pass's rows may follow)
+        const float2 *x0p = X + (size_t)(sh.x0 + rbase + r) * 64 + t4, *x1p = x0p + 8 * 64;
+        const bool in0 = r < nrows, in1 = r + 8 < nrows;   // (another pass's or brick's rows follow)
         const float2 zero = make_float2(0.f, 0.f);
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
@@ -431,7 +498,7 @@ k_nl_project(Geo g, Wave w, NlGrid grid, int c0, int cn, const float* __restrict
             mma_tf32(dl, ah[ks], bl);
             mma_tf32(dh, ah[ks], bh);
           }
-          float* o = po + (unsigned long long)(unsigned)cur.y * (unsigned)(rows_cap * 8);
+          float* o = po + (size_t)cur.y * 8;
           if (r < nrows) *reinterpret_cast<float2*>(o) = make_float2(dh[0] + dl[0], dh[1] + dl[1]);
           if (r + 8 < nrows) *reinterpret_cast<float2*>(o + 64) = make_float2(dh[2] + dl[2], dh[3] + dl[3]);
         }
@@ -439,24 +506,37 @@ k_nl_project(Geo g, Wave w, NlGrid grid, int c0, int cn, const float* __restrict
       }
       k0 += sh.nimg;
       if (k0 >= sh.nb) break;
-      nl_next(hd, k0, sh);
+      nl_next(hd, img, k0, sh);
     }
   }
 }
 
-// Per tile and image: the (brick << 16 | first row in the brick) of the bricks it meets, in brick order.
-// One thread per image searches the record lists (ascending image order) of the bricks its box overlaps.
+// Per tile: its bricks' first rows in Part (off, brick order), and per image the rows of its first channel, of the
+// bricks it meets in brick order. One thread per image searches the record lists (ascending image order) of the
+// bricks its box overlaps. A tile with more rows or images than the launch was sized for (a stale graph) is refused:
+// off = -1 and no entries, so nothing reaches past Part or idx.
 __global__ void __launch_bounds__(256)
-k_nl_index(Geo g, Wave w, const AtomTab* __restrict__ atoms, const TileEntry* __restrict__ entries,
-           const int* __restrict__ n_entries, const int* __restrict__ blist, const int4* __restrict__ brec,
-           const int* __restrict__ bn, int* __restrict__ start, unsigned* __restrict__ idx) {
+k_nl_index(Geo g, Wave w, NlGrid grid, const AtomTab* __restrict__ atoms, const TileEntry* __restrict__ entries,
+           const int* __restrict__ n_entries, const int* __restrict__ blist, const int* __restrict__ bn,
+           const int4* __restrict__ head, const int* __restrict__ img, int rows_cap, int idx_cap, int* off_, int* start,
+           int* __restrict__ idx, int* __restrict__ status) {
   const int tl = blockIdx.x, t = wave_tile(w, tl);
   int o[3];
   tile_origin(g, t, o);
   const int ne = n_entries[tl];
   const TileEntry* ent = entries + (size_t)tl * g.e_cap;
   int* st = start + (size_t)tl * (g.e_cap + 1);
-  unsigned* ix = idx + (size_t)tl * g.nbricks * g.br_cap;
+  int* ix = idx + (size_t)tl * idx_cap;
+  int* off = off_ + (size_t)tl * g.nbricks;
+  int rows = 0;
+  for (int b0 = 0; b0 < g.nbricks; b0 += blockDim.x) {
+    const int br = b0 + threadIdx.x;
+    int tot;
+    const int first = block_exclusive_scan(br < g.nbricks ? head[nl_index(g, grid, t, br)].y : 0, &tot);
+    if (br < g.nbricks) off[br] = rows + first;
+    rows += tot;
+  }
+  __syncthreads();
   int base = 0;
   for (int e0 = 0; e0 < ne; e0 += blockDim.x) {
     const int e = e0 + threadIdx.x;
@@ -475,7 +555,7 @@ k_nl_index(Geo g, Wave w, const AtomTab* __restrict__ atoms, const TileEntry* __
       for (int bz = lo[2]; bz <= hi[2]; ++bz)
         for (int by = lo[1]; by <= hi[1]; ++by)
           for (int bx = lo[0]; bx <= hi[0]; ++bx) {
-            const size_t br = (size_t)(bz * g.nbr[1] + by) * g.nbr[0] + bx;
+            const int br = (bz * g.nbr[1] + by) * g.nbr[0] + bx;
             const size_t tb = (size_t)tl * g.nbricks + br;
             const int* l = blist + tb * g.br_cap;
             const int nb = bn[tb];
@@ -486,25 +566,28 @@ k_nl_index(Geo g, Wave w, const AtomTab* __restrict__ atoms, const TileEntry* __
               else c = mid;
             }
             if (a < nb && l[a] == e) {
-              if (fill) {
-                int row = 0;
-                for (int k = 0; k < a; ++k) row += brec[(tb * g.br_cap + k) * 2].w & 0xff;
-                ix[at0 + cnt] = unsigned(br) << 16 | unsigned(row);
-              }
+              const int4 hd = head[nl_index(g, grid, t, br)];
+              if (hd.x == 0) continue;   // a brick without a table (refused): nothing of it is in Part
+              if (fill && at0 + cnt < idx_cap) ix[at0 + cnt] = off[br] + (hd.w >= 0 ? a * hd.w : img[-1 - hd.w + a] >> 4);
               ++cnt;
             }
           }
       return cnt;
     };
     int tot;
-    const int off = block_exclusive_scan(e < ne ? walk(false, 0) : 0, &tot);
+    const int first = block_exclusive_scan(e < ne ? walk(false, 0) : 0, &tot);
     if (e < ne) {
-      st[e] = base + off;
-      walk(true, base + off);
+      st[e] = base + first;
+      walk(true, base + first);
     }
     base += tot;
   }
   if (threadIdx.x == 0) st[ne] = base;
+  if (rows <= rows_cap && base <= idx_cap) return;
+  __syncthreads();
+  for (int e = threadIdx.x; e <= ne; e += blockDim.x) st[e] = 0;
+  for (int br = threadIdx.x; br < g.nbricks; br += blockDim.x) off[br] = -1;
+  if (threadIdx.x == 0) atomicOr(status + kStOverflow, 16);
 }
 
 // P[row][q] = gamma |dOmega| times the sum of the row's partial projections over its bricks, as pairs of floats
@@ -520,12 +603,12 @@ __device__ __forceinline__ void pair_add(float& h, float& l, float vh, float vl)
 __global__ void __launch_bounds__(128)
 k_nl_reduce(Geo g, int tl0, const TileEntry* __restrict__ entries, const int* __restrict__ n_entries,
             const AtomTab* __restrict__ atoms, const float2* __restrict__ gdvp, const int* __restrict__ start,
-            const unsigned* __restrict__ idx, int rows_cap, const float* __restrict__ Part, float* __restrict__ P,
+            const int* __restrict__ idx, int idx_cap, int rows_cap, const float* __restrict__ Part, float* __restrict__ P,
             size_t lo_plane, float2* __restrict__ Pp) {
   const int tc = blockIdx.x, tl = tl0 + tc, lane = threadIdx.x & 31;
   const int* st = start + (size_t)tl * (g.e_cap + 1);
-  const unsigned* ix = idx + (size_t)tl * g.nbricks * g.br_cap;
-  const float4* pt = reinterpret_cast<const float4*>(Part + (size_t)tc * g.nbricks * rows_cap * 8);
+  const int* ix = idx + (size_t)tl * idx_cap;
+  const float4* pt = reinterpret_cast<const float4*>(Part + (size_t)tc * rows_cap * 8);
   const int ne = n_entries[tl];
   for (int e = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5); e < ne; e += gridDim.y * (blockDim.x >> 5)) {
     const TileEntry te = entries[(size_t)tl * g.e_cap + e];
@@ -537,8 +620,7 @@ k_nl_reduce(Geo g, int tl0, const TileEntry* __restrict__ entries, const int* __
     if (v4 < 2 * nch) {
 #pragma unroll 4
       for (int i = i0 + sub; i < i1; i += nsub) {
-        const unsigned x = ix[i];
-        const float4 v = pt[((x >> 16) * rows_cap + (x & 0xffffu)) * 2 + v4];
+        const float4 v = pt[ix[i] * 2 + v4];
         pair_add(h[0], l[0], v.x, 0.f);
         pair_add(h[1], l[1], v.y, 0.f);
         pair_add(h[2], l[2], v.z, 0.f);
@@ -840,19 +922,67 @@ static int stencil_no(sq_handle* h, const Wave& w, const float* Tc, const float*
   return stencil_launch<NO, 544, 1, 1>(h, w, Tc, Tp, Tn, has_y, mode);
 }
 
-// images and rows per brick of the wave's tables
-static int nl_imgs(const sq_handle* h, size_t wi) { return std::max(1, h->wave_recs[wi]); }
-static int nl_rows_cap(const sq_handle* h, size_t wi) { return nl_rows_padded(nl_imgs(h, wi), h->max_nch); }
 static bool nl_any(const sq_handle* h) { return h->geo.n_atoms > 0 && h->table_len > 0; }
-static dim3 nl_dim(const NlGrid& n) { return dim3(n.nb[0], n.nb[1], 8 * n.nb[2]); }
+static dim3 nl_dim(const NlGrid& n) { return dim3(n.nb[0], n.nb[1], 8 * n.nz); }
 
+// Do the wave's tables fit their buffers (ensure_nl_buffers) and its bricks a grid?
 bool nl_fits(const sq_handle* h, size_t wi) {
   if (!nl_any(h)) return true;
-  if (wi >= h->wave_recs.size()) return false;
+  if (wi >= h->wave_nl.size()) return false;
+  const NlNeed& need = h->wave_nl[wi];
   const NlGrid n = nl_grid(h->geo, h->waves[wi]);
-  const size_t bricks = size_t(n.nb[0]) * n.nb[1] * n.nb[2] * 8, rows = nl_rows_cap(h, wi);
-  return bricks * rows * 64 * sizeof(float2) <= h->table_cap && bricks * (2 + size_t(nl_imgs(h, wi))) <= h->head_cap &&
-         size_t(h->geo.nbricks) * rows * 8 <= h->part_floats && n.nb[1] < 65536 && 8 * n.nb[2] < 65536;
+  return size_t(need.x_rows) <= h->x_rows_cap && size_t(need.imgs) <= h->img_cap && size_t(need.tile_imgs) <= h->idx_cap &&
+         size_t(need.tile_rows) * 8 <= h->part_floats && n.nb[1] < 65536 && 8 * n.nb[2] < 65536;
+}
+
+// rows and images the tables of wave wi need, added to cnt[0], cnt[1] (after its lists)
+int count_nl_tables(sq_handle* h, size_t wi, int* cnt) {
+  if (!nl_any(h)) return SQ_OK;
+  const Wave& w = h->waves[wi];
+  const NlGrid n = nl_grid(h->geo, w);
+  if (n.nb[1] >= 65536 || 8 * n.nb[2] >= 65536) return SQ_OK;   // nl_fits is false
+  k_nl_table<<<nl_dim(n), 128, 0, h->stream>>>(h->geo, w, n, h->d.chi32s, h->wb.brick_rec, h->wb.brick_n, 0, 0, cnt,
+                                               nullptr, nullptr, nullptr, nullptr);
+  SQ_LAUNCH_CHECK(h);
+  return SQ_OK;
+}
+
+// Buffers for the largest needs of the layout, a sixteenth larger than needed so that moving atoms seldom outgrow
+// them; they never shrink. Part holds the partial projections of the largest wave, at most kNlPartFloats (the sweep
+// then takes the tiles in chunks). What cannot be allocated is left out: nl_fits sends those waves to k_step.
+int ensure_nl_buffers(sq_handle* h) {
+  if (!nl_any(h)) return SQ_OK;
+  NlNeed top;
+  size_t part = 0;
+  for (size_t wi = 0; wi < h->wave_nl.size(); ++wi) {
+    const NlNeed& n = h->wave_nl[wi];
+    top.x_rows = std::max(top.x_rows, n.x_rows);
+    top.imgs = std::max(top.imgs, n.imgs);
+    top.tile_imgs = std::max(top.tile_imgs, n.tile_imgs);
+    const size_t tile = size_t(n.tile_rows) * 8;
+    part = std::max(part, std::max(tile, std::min(kNlPartFloats, tile * h->waves[wi].ntiles)));
+  }
+  auto grow = [&](void** p, size_t* cap, size_t need, size_t unit, size_t most) -> int {
+    if (need <= *cap && *p) return SQ_OK;
+    const size_t want = std::max(need, std::min(most, need + need / 16 + 64));
+    h->nl_epoch++;   // captured graphs hold the old pointer
+    SQ_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    dev_free(h, *p, *cap * unit);
+    *p = nullptr;
+    *cap = 0;
+    if (dev_alloc(h, p, want * unit) != SQ_OK) {   // no error: the other step runs
+      h->err.clear();
+      return SQ_OK;
+    }
+    *cap = want;
+    return SQ_OK;
+  };
+  const size_t any = SIZE_MAX / 2;
+  int rc = grow((void**)&h->wb.nl_X, &h->x_rows_cap, top.x_rows, 64 * sizeof(float2), any);
+  if (rc == SQ_OK) rc = grow((void**)&h->wb.nl_img, &h->img_cap, top.imgs, sizeof(int), any);
+  if (rc == SQ_OK) rc = grow((void**)&h->wb.proj_idx, &h->idx_cap, top.tile_imgs, sizeof(int) * size_t(h->wave_cap), any);
+  if (rc == SQ_OK) rc = grow((void**)&h->wb.Part, &h->part_floats, part, sizeof(float), std::max(part, kNlPartFloats));
+  return rc;
 }
 
 // the wave's brick tables and the image -> brick index, after its lists
@@ -860,11 +990,14 @@ int build_nl_tables(sq_handle* h, size_t wi) {
   if (!nl_any(h)) return SQ_OK;
   const Wave& w = h->waves[wi];
   const NlGrid n = nl_grid(h->geo, w);
-  k_nl_index<<<w.ntiles, 256, 0, h->stream>>>(h->geo, w, h->d.atoms, h->wb.entries, h->wb.n_entries, h->wb.brick_list,
-                                              h->wb.brick_rec, h->wb.brick_n, h->wb.proj_start, h->wb.proj_idx);
+  SQ_CUDA_TRY(h, cudaMemsetAsync(h->wb.nl_cnt, 0, 2 * sizeof(int), h->stream));
+  k_nl_table<<<nl_dim(n), 128, 0, h->stream>>>(h->geo, w, n, h->d.chi32s, h->wb.brick_rec, h->wb.brick_n,
+                                               (long long)h->x_rows_cap, (long long)h->img_cap, h->wb.nl_cnt, h->wb.nl_head,
+                                               h->wb.nl_img, h->wb.nl_X, h->d.status);
   SQ_LAUNCH_CHECK(h);
-  k_nl_table<<<nl_dim(n), 128, 0, h->stream>>>(h->geo, w, n, h->d.chi32s, h->wb.brick_rec, h->wb.brick_n, nl_imgs(h, wi),
-                                               nl_rows_cap(h, wi), h->wb.nl_head, h->wb.nl_X, h->d.status);
+  k_nl_index<<<w.ntiles, 256, 0, h->stream>>>(h->geo, w, n, h->d.atoms, h->wb.entries, h->wb.n_entries, h->wb.brick_list,
+                                              h->wb.brick_n, h->wb.nl_head, h->wb.nl_img, h->wave_nl[wi].tile_rows,
+                                              int(h->idx_cap), h->wb.proj_off, h->wb.proj_start, h->wb.proj_idx, h->d.status);
   SQ_LAUNCH_CHECK(h);
   return SQ_OK;
 }
@@ -874,18 +1007,19 @@ int launch_project_mixed(sq_handle* h, size_t wi, const float* T) {
   if (!nl_any(h)) return SQ_OK;
   const Geo& g = h->geo;
   const Wave& w = h->waves[wi];
-  const NlGrid n = nl_grid(g, w);
-  const int rows_cap = nl_rows_cap(h, wi);
-  const size_t per_tile = size_t(g.nbricks) * rows_cap * 8;
+  const int rows = h->wave_nl[wi].tile_rows;
+  const size_t per_tile = size_t(std::max(1, rows)) * 8;
   SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_nl_project, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kPrSmem)));
-  const int ct = int(std::max<size_t>(1, std::min<size_t>(size_t(w.ntiles), h->part_floats / per_tile)));
+  const int most = int(std::max<size_t>(1, std::min<size_t>(size_t(w.ntiles), h->part_floats / per_tile)));
+  const int nchunk = (w.ntiles + most - 1) / most, ct = (w.ntiles + nchunk - 1) / nchunk;   // equal chunks
   for (int c0 = 0; c0 < w.ntiles; c0 += ct) {
     const int cn = std::min(ct, w.ntiles - c0);
-    k_nl_project<<<nl_dim(n), kPrThreads, kPrSmem, h->stream>>>(g, w, n, c0, cn, T, h->wb.nl_head, nl_imgs(h, wi),
-                                                                h->wb.nl_X, rows_cap, h->wb.Part);
+    const NlGrid n = nl_grid(g, w, c0, cn);
+    k_nl_project<<<nl_dim(n), kPrThreads, kPrSmem, h->stream>>>(g, w, n, c0, cn, T, h->wb.nl_head, h->wb.nl_img, h->wb.nl_X,
+                                                                NlPart{h->wb.proj_off, rows}, h->wb.Part);
     SQ_LAUNCH_CHECK(h);
     k_nl_reduce<<<dim3(cn, 8), 128, 0, h->stream>>>(g, c0, h->wb.entries, h->wb.n_entries, h->d.atoms, h->d.gdvp,
-                                           h->wb.proj_start, h->wb.proj_idx, rows_cap, h->wb.Part,
+                                           h->wb.proj_start, h->wb.proj_idx, int(h->idx_cap), rows, h->wb.Part,
                                            (float*)h->wb.Pg[1], nl_plane(h), (float2*)h->wb.Pg[0]);
     SQ_LAUNCH_CHECK(h);
   }
@@ -900,8 +1034,8 @@ int launch_step_mixed(sq_handle* h, size_t wi, const float* Tc, const float* Tp,
     const NlGrid n = nl_grid(g, w);
     SQ_CUDA_TRY(h, cudaFuncSetAttribute(k_nl_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kApSmem)));
     k_nl_apply<<<nl_dim(n), kNlThreads, kApSmem, h->stream>>>(g, w, n, h->max_nch, (const float*)h->wb.Pg[1],
-                                                              nl_plane(h), h->wb.nl_head, nl_imgs(h, wi), h->wb.nl_X,
-                                                              nl_rows_cap(h, wi), h->wb.brick_rec, Tn);
+                                                              nl_plane(h), h->wb.nl_head, h->wb.nl_img, h->wb.nl_X,
+                                                              h->wb.brick_rec, Tn);
     SQ_LAUNCH_CHECK(h);
   }
   h->step_variant[0]++;

@@ -696,10 +696,11 @@ static bool use_tma(const sq_handle* h, size_t wi) {
 
 // The split mixed step: SQ_MIXED with at most 4 channels per atom, unless the staged step was asked for, or
 // SQ_STEP_SMEM_ROWS asks for the global-memory projections of k_step.
-bool use_split(const sq_handle* h, size_t wi) {
-  if (h->precision != SQ_MIXED || !h->proj4 || !h->wb.Part || use_tma(h, wi) || !nl_fits(h, wi)) return false;
+bool want_split(const sq_handle* h, size_t wi) {
+  if (!h->split_able || use_tma(h, wi)) return false;
   return !(h->step_rows_env && wi < h->wave_rows.size() && std::max(1, h->wave_rows[wi]) > h->step_rows_cap);
 }
+bool use_split(const sq_handle* h, size_t wi) { return want_split(h, wi) && nl_fits(h, wi); }
 
 template <typename Real>
 static int sweep_t(sq_handle* h, const Real* chi, const Real* v, const Real* gdv) {
@@ -856,25 +857,65 @@ int time_step_launch(sq_handle* h, int reps, double* ms_out) {
   return time_step_t<float>(h, reps, ms_out, h->d.chi32, h->d.v32, h->d.gdv32);
 }
 
+// out[0]: most projector rows of a slab, [1]: most images of a brick, [2], [3]: most (brick, row) and (brick, image)
+// pairs of a tile. One block per tile of the wave.
+__global__ void __launch_bounds__(kThreads)
+k_wave_measure(Geo g, const int* __restrict__ slab_n, const int* __restrict__ bn, const int4* __restrict__ brec,
+               int* __restrict__ out) {
+  const int tl = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int slab = 0, most = 0, rows = 0, imgs = 0;
+  for (int i = threadIdx.x; i < g.nslab; i += kThreads) slab = max(slab, slab_n[(size_t)tl * g.nslab + i]);
+  for (int br = warp; br < g.nbricks; br += kThreads / 32) {
+    const size_t tb = (size_t)tl * g.nbricks + br;
+    const int nb = bn[tb];
+    for (int k = lane; k < nb; k += 32) rows += brec[(tb * g.br_cap + k) * 2].w & 0xff;
+    most = max(most, nb);
+    if (lane == 0) imgs += nb;
+  }
+  int tot_rows, tot_imgs;
+  block_exclusive_scan(rows, &tot_rows);
+  block_exclusive_scan(imgs, &tot_imgs);
+  slab = __reduce_max_sync(0xffffffffu, slab);
+  if (lane == 0) {
+    atomicMax(out, slab);
+    atomicMax(out + 1, most);
+  }
+  if (threadIdx.x == 0) {
+    atomicMax(out + 2, tot_rows);
+    atomicMax(out + 3, tot_imgs);
+  }
+}
+
 int measure_wave_rows(sq_handle* h) {
   const Geo& g = h->geo;
   cudaStream_t s = h->stream;
-  std::vector<int> nrows, nrecs;
   h->wave_rows.assign(h->waves.size(), 0);
   h->wave_recs.assign(h->waves.size(), 0);
+  h->wave_nl.assign(h->waves.size(), NlNeed());
   for (size_t wi = 0; wi < h->waves.size(); ++wi) {
     const Wave& w = h->waves[wi];
     int rc = build_wave_entries(h, w);
     if (rc != SQ_OK) return rc;
-    nrows.resize(size_t(w.ntiles) * g.nslab);
-    nrecs.resize(size_t(w.ntiles) * g.nbricks);
-    SQ_CUDA_TRY(h, cudaMemcpyAsync(nrows.data(), h->wb.slab_n, sizeof(int) * nrows.size(), cudaMemcpyDeviceToHost, s));
-    SQ_CUDA_TRY(h, cudaMemcpyAsync(nrecs.data(), h->wb.brick_n, sizeof(int) * nrecs.size(), cudaMemcpyDeviceToHost, s));
+    int* out = h->wb.nl_cnt + 2;   // slab rows, brick images, tile rows, tile images; table rows, images
+    SQ_CUDA_TRY(h, cudaMemsetAsync(out, 0, 6 * sizeof(int), s));
+    k_wave_measure<<<w.ntiles, kThreads, 0, s>>>(g, h->wb.slab_n, h->wb.brick_n, h->wb.brick_rec, out);
+    SQ_LAUNCH_CHECK(h);
+    if (h->split_able) rc = count_nl_tables(h, wi, out + 4);
+    if (rc != SQ_OK) return rc;
+    int r[6];
+    SQ_CUDA_TRY(h, cudaMemcpyAsync(r, out, sizeof(r), cudaMemcpyDeviceToHost, s));
     SQ_CUDA_TRY(h, cudaStreamSynchronize(s));
-    h->wave_rows[wi] = nrows.empty() ? 0 : *std::max_element(nrows.begin(), nrows.end());
-    h->wave_recs[wi] = nrecs.empty() ? 0 : *std::max_element(nrecs.begin(), nrecs.end());
+    h->wave_rows[wi] = r[0];
+    h->wave_recs[wi] = r[1];
+    NlNeed& n = h->wave_nl[wi];
+    n.tile_rows = r[2];
+    n.tile_imgs = r[3];
+    n.x_rows = r[4];
+    n.imgs = r[5];
   }
-  return SQ_OK;
+  bool split = false;
+  for (size_t wi = 0; wi < h->waves.size(); ++wi) split = split || want_split(h, wi);
+  return split ? ensure_nl_buffers(h) : SQ_OK;
 }
 
 template <typename Real>
