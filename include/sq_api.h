@@ -167,7 +167,7 @@ int sq_update_atoms(sq_handle* h, const double* pos, const double* v_eff);
  * bounds for the lists of their sample tiles), instead of rebuilding them in every call. They
  * depend on the positions only: sq_update_atoms with moved atoms discards them, with the same
  * positions and a new V_eff it keeps them. Kept only when the handle's tiles form one wave
- * (sq_footprint_bytes up to about 64 GiB of per-tile buffers). Off by default, where every
+ * (sq_footprint_bytes up to about 56 GiB, SQ_FP64: 24 GiB). Off by default, where every
  * sq_moments rebuilds them as a new snapshot needs. Results are identical either way.
  * Errors: SQ_ERR_INVALID_ARG. */
 int sq_keep_lists(sq_handle* h, int enable);
@@ -224,7 +224,8 @@ int sq_node_bounds(sq_handle* h, double* lo_out, double* hi_out);
 /* Copies the moment table [N_d][n_pl + 1][SQ_N_MOMENTS] (FP64, host) for inspection. */
 int sq_moments_copy(sq_handle* h, double* host_out);
 
-/* Device bytes sq_setup would allocate for desc (0 if desc is invalid); used for admission. */
+/* Device bytes sq_setup would allocate for desc (0 if desc is invalid); used for admission. An upper bound: the
+ * tables of the mixed step are allocated for what the atoms' positions need. */
 size_t sq_footprint_bytes(const sq_instance_desc* desc);
 
 /* Number of CUDA kernels the handle launched since sq_setup (all calls). */
@@ -336,7 +337,8 @@ void sq_batch_destroy(sq_batch* b);
  * those in flight and fewer than max_inflight run; each admitted request runs setup, moments,
  * Fermi level and contraction on its own stream and host thread and is destroyed afterwards
  * (see sq_server_submit_traj for requests that keep their state on the device).
- * A request larger than the whole budget completes with status SQ_ERR_OOM. */
+ * A request whose footprint exceeds the whole budget is set up in smaller waves of tiles (the
+ * same results); one that does not fit even so completes with status SQ_ERR_OOM. */
 typedef struct sq_server sq_server;
 typedef struct {
   long long tag;         /* the caller's tag from sq_server_submit           */

@@ -203,7 +203,20 @@ double bricks_met(const sq::Geo& g, double rc) {
   return 1.05 * double(most) + 2.0;
 }
 
-int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
+// Is the TMA-staged step asked for? (its handles hold the table boxes of the brick records)
+bool staged_requested() {
+  const char* env = std::getenv("SQ_STEP_KERNEL");
+  return env && std::string(env) == "staged";
+}
+
+// The corner offsets of the brick records (16 bytes each) are only read while a wave's W table is built, when the
+// second column buffer is free: they lie in it where it holds them.
+bool d0_in_ring(const sq::Geo& g) {
+  return size_t(g.nbricks) * g.br_cap * sizeof(float4) <= size_t(g.Upts) * g.B * sizeof(float);
+}
+
+// limit > 0: waves as small as it takes to stay within limit bytes (more when one tile does not)
+int make_plan(const sq_instance_desc* d, Plan& P, std::string& why, size_t limit = 0) {
   sq::Geo& g = P.geo;
   std::memset(&g, 0, sizeof(g));
   g.b = 2;
@@ -328,13 +341,15 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
   size_t tileB = size_t(g.B);
   P.per_tile_bytes = size_t(g.e_cap) * sizeof(sq::TileEntry) + 2 * sizeof(int) +
                      size_t(g.nbricks) * (size_t(g.br_cap) + 1) * sizeof(int) +
-                     size_t(g.nbricks) * size_t(g.br_cap) * 4 * sizeof(int4) +   // records, corner offsets, TMA boxes
+                     size_t(g.nbricks) * size_t(g.br_cap) * 2 * sizeof(int4) +   // records
                      3 * size_t(g.Upts) * tileB * real +        // T ring
                      size_t(d->precision == SQ_FP64 ? 9 : 3) * g.Upts * tileB * real +   // W (G)
-                     2 * size_t(g.r_cap) * tileB * real +       // A, P
+                     size_t(g.r_cap) * tileB * real +           // A
                      2 * size_t(g.r_cap) * tileB * sizeof(double) +   // Pg ping-pong (FP64)
                      size_t(std::max(g.nslab, sq::stencil_chunks(g))) * tileB * 9 * sizeof(double) +
                      size_t(g.nslab) * (size_t(g.r_cap) + 1) * sizeof(int);   // slab row maps
+  if (d->precision == SQ_MIXED && !d0_in_ring(g)) P.per_tile_bytes += size_t(g.nbricks) * g.br_cap * sizeof(float4);
+  if (d->precision == SQ_MIXED && staged_requested()) P.per_tile_bytes += size_t(g.nbricks) * g.br_cap * sizeof(int4);
   int max_nch = 1;
   for (const sq::AtomTab& at : P.atoms) max_nch = std::max(max_nch, at.nch);
   P.split_able = d->precision == SQ_MIXED && max_nch <= 4;
@@ -357,15 +372,14 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
   }
   long long Nd = (long long)g.n[0] * g.n[1] * g.n[2];
   int M = d->cheb_quad_M > 0 ? d->cheb_quad_M : 2048;
-  P.fixed_bytes = size_t(sq::kStepFill) * g.B * 9 * sizeof(double) + size_t(Nd) * (sizeof(double) + sizeof(float)) +                       // V
+  P.fixed_bytes = size_t(Nd) * (sizeof(double) + sizeof(float)) +                       // V
                   P.atoms.size() * sizeof(sq::AtomTab) + size_t(ch) * 6 * sizeof(double) +
-                  // projector tables: FP64 (always; the Lanczos apply and the FP64 sweep), FP32 and
-                  // TF32 hi/lo pairs for the mixed sweep
-                  size_t(P.table_len) * (sizeof(double) + (real == sizeof(float) ? 3 * sizeof(float) : 0)) +
+                  // projector tables: FP64, or FP32 and TF32 hi/lo pairs for the mixed sweep
+                  size_t(P.table_len) * (real == sizeof(double) ? sizeof(double) : 3 * sizeof(float)) +
                   size_t(Nd) * size_t(d->n_pl + 1) * SQ_N_MOMENTS * sizeof(double) +   // moments
                   size_t(d->n_pl + 1) * 4 * sizeof(double) + size_t(M) * 8 * sizeof(double) +   // R, coefficients, F, tables
                   size_t(Nd) * sizeof(double) + 4096 * 32 * sizeof(double) + 1024;
-  if (d->bounds_mode != SQ_BOUNDS_GIVEN)
+  if (d->bounds_mode == SQ_BOUNDS_PER_NODE)
     P.fixed_bytes += sizeof(double) * sq::lz_dots_len(d->lanczos_k > 0 ? d->lanczos_k : 40);
   // Lanczos sample tiles (argmin V, argmax V, a stride-n/2 node grid); the buffers hold the
   // largest count so that sq_update_atoms can move them with V
@@ -375,12 +389,13 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
     P.lz_cap = lanczos_sample_cap(g);
     const int k = d->lanczos_k > 0 ? d->lanczos_k : 40;
     const size_t nst = size_t(P.lz_cap);
-    P.fixed_bytes += sizeof(double) * (size_t(k + 2) * nst * g.Upts * g.B + nst * size_t(g.r_cap) * g.B +
-                                       nst * g.B * size_t(5 * k + 8)) + sizeof(int) * nst;
+    P.fixed_bytes += sizeof(double) * sq::lz_dots_len(k, sq::lz_sample_blocks(P.lz_cap, g.Upts));
+    P.fixed_bytes += real * (size_t(k + 2) * nst * g.Upts * g.B + nst * size_t(g.r_cap) * g.B) +
+                     sizeof(double) * nst * g.B * size_t(5 * k + 8) + sizeof(int) * nst;
     // the sample tiles' own entry and brick lists
     P.fixed_bytes += nst * (size_t(g.e_cap) * sizeof(sq::TileEntry) + 2 * sizeof(int) +
                             size_t(g.nbricks) * (size_t(g.br_cap) + 1) * sizeof(int) +
-                            size_t(g.nbricks) * size_t(g.br_cap) * 4 * sizeof(int4) +
+                            size_t(g.nbricks) * size_t(g.br_cap) * 2 * sizeof(int4) +
                             size_t(g.nslab) * (size_t(g.r_cap) + 1) * sizeof(int));
   }
   // the node partition: part part_rank of part_count equal contiguous tile ranges
@@ -391,22 +406,15 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
     P.tile_end = int((long long)g.n_tiles * (d->part_rank + 1) / d->part_count);
   }
   const long long ntl = std::max(1, P.tile_end - P.tile_begin);
-  // tiles per wave: one wave when the whole working set fits in 64 GiB (its lists and W table are
-  // then built once and kept across evaluations), else waves of at most 24 GiB (fewer, larger
-  // launches: less per-wave setup and a smaller tail), with the tiles spread evenly over the waves
-  size_t budget = size_t(24) << 30;
-  if (size_t(ntl) * P.per_tile_bytes <= (size_t(64) << 30)) budget = size_t(ntl) * P.per_tile_bytes;
-  long long wc = std::max<long long>(1, (long long)(budget / std::max<size_t>(P.per_tile_bytes, 1)));
-  wc = std::min<long long>(std::min<long long>(wc, ntl), 32768);
-  const long long nwaves = (ntl + wc - 1) / wc;
-  P.wave_cap = int((ntl + nwaves - 1) / nwaves);
-  P.wave_cap = std::max<int>(P.wave_cap, P.lz_cap);
-  if (P.split_able) {
-    // brick tables and partial projections (sized by ensure_nl_buffers from what the atoms' positions need; here:
-    // every periodic image that reaches a brick of the wave meets as many bricks as it can)
-    P.nl_bricks = sq::nl_bricks_max(g, P.wave_cap);
+  // the split mixed step's brick tables and partial projections for waves of wc tiles (sized by ensure_nl_buffers
+  // from what the atoms' positions need; here: every periodic image that reaches a brick of the wave meets as many
+  // bricks as it can)
+  bool mixed_nch = false;
+  for (const sq::AtomTab& at : P.atoms) mixed_nch = mixed_nch || at.nch != P.atoms[0].nch;
+  auto nl_bytes = [&](long long wc) -> size_t {
+    if (!P.split_able) return 0;
     const long long n01 = (long long)g.tiles[0] * g.tiles[1];
-    const long long tz = std::min<long long>(g.tiles[2], (P.wave_cap + n01 - 1) / n01 + 1);
+    const long long tz = std::min<long long>(g.tiles[2], (wc + n01 - 1) / n01 + 1);
     double mult = 0.0, rows = 0.0, imgs = 0.0;
     for (int cls = 0; cls < 8; ++cls) {
       const long long t[3] = {g.tiles[0], g.tiles[1], tz};
@@ -417,25 +425,64 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why) {
       }
       mult += m;
     }
-    bool mixed_nch = false;
     for (size_t J = 0; J < P.atoms.size(); ++J) {
       imgs += mult * met[J] * (P.atoms[J].nch > 0);
       rows += mult * met[J] * P.atoms[J].nch;
-      mixed_nch = mixed_nch || P.atoms[J].nch != P.atoms[0].nch;
     }
-    const double part = std::min<double>(sq::kNlPartFloats * sizeof(float), 1.0625 * P.wave_cap * nl_tile_rows * tileB * sizeof(float));
-    P.fixed_bytes += size_t(rows * 64 * sizeof(float2)) + (mixed_nch ? size_t(imgs) * sizeof(int) : 0) + size_t(part) +
-                     P.nl_bricks * sizeof(int4) + size_t(ch) * sizeof(float2);
+    const double part = std::min<double>(sq::kNlPartFloats * sizeof(float), 1.0625 * double(wc) * nl_tile_rows * tileB * sizeof(float));
+    return size_t(rows * 64 * sizeof(float2)) + (mixed_nch ? size_t(imgs) * sizeof(int) : 0) + size_t(part) +
+           sq::nl_bricks_max(g, int(wc)) * sizeof(int4);
+  };
+  // tiles per wave: one wave when the whole working set fits in 56 GiB (its lists and W table can then be kept across
+  // evaluations, sq_keep_lists), else waves of at most 24 GiB (fewer, larger launches: less per-wave setup and a
+  // smaller tail), with the tiles spread evenly over the waves. FP64 holds nine G fields where W has three, twice
+  // the bytes of a tile: above 24 GiB it takes two waves at least.
+  const long long most = std::min<long long>(ntl, 32768);
+  const size_t spart_rows = std::max(g.nslab, sq::stencil_chunks(g));   // of S partials per tile; kStepFill bricks at least
+  auto wave_bytes = [&](long long wc) {
+    const size_t bricks = std::min(size_t(sq::kStepFill), size_t(wc) * g.nbricks), rows = size_t(wc) * spart_rows;
+    return size_t(wc) * P.per_tile_bytes + nl_bytes(wc) + (bricks > rows ? (bricks - rows) * tileB * 9 * sizeof(double) : 0);
+  };
+  const size_t one_wave = size_t(d->precision == SQ_FP64 ? 24 : 56) << 30;
+  long long wc = most;
+  if (most < ntl || wave_bytes(ntl) > one_wave) {
+    const size_t budget = d->precision == SQ_FP64 ? std::min(size_t(24) << 30, size_t((ntl + 1) / 2) * P.per_tile_bytes)
+                                                  : size_t(24) << 30;
+    long long lo = 1, hi = most;   // the largest wave within the budget (or one tile)
+    while (lo < hi) {
+      const long long mid = (lo + hi + 1) / 2;
+      if (wave_bytes(mid) <= budget) lo = mid;
+      else hi = mid - 1;
+    }
+    wc = lo;
   }
-  if (d->bounds_mode == SQ_BOUNDS_PER_NODE) {
-    // every node's own Lanczos: waves of tiles with k + 2 Krylov vectors each under 8 GiB, the
-    // per-node interval and step coefficients, the Fermi-search cosine sums and contraction rows
-    const int k = d->lanczos_k > 0 ? d->lanczos_k : 40;
-    const size_t per_tile = (size_t(k + 2) * g.Upts + size_t(g.r_cap)) * g.B * real + size_t(g.B) * (5 * k + 8) * 8;
-    P.nlz_wave = int(std::max<size_t>(1, std::min<size_t>((size_t(8) << 30) / per_tile, size_t(P.wave_cap))));
-    P.fixed_bytes += size_t(P.nlz_wave) * per_tile + size_t(Nd) * (4 + M + 20) * sizeof(double) +
-                     1024 * sizeof(double);
+  const long long nwaves = (ntl + wc - 1) / wc;
+  // per-node bounds: every node's own Lanczos, waves of tiles with k + 2 Krylov vectors each under 8 GiB, the
+  // per-node interval and step coefficients, the Fermi-search cosine sums and contraction rows
+  const size_t lz_tile = (size_t((d->lanczos_k > 0 ? d->lanczos_k : 40) + 2) * g.Upts + size_t(g.r_cap)) * g.B * real +
+                         size_t(g.B) * (5 * (d->lanczos_k > 0 ? d->lanczos_k : 40) + 8) * 8;
+  auto nlz_wave = [&](long long wc) {
+    return d->bounds_mode == SQ_BOUNDS_PER_NODE ? std::max<size_t>(1, std::min<size_t>((size_t(8) << 30) / lz_tile, size_t(wc))) : size_t(0);
+  };
+  if (d->bounds_mode == SQ_BOUNDS_PER_NODE)
+    P.fixed_bytes += size_t(Nd) * (4 + M + 20) * sizeof(double) + 1024 * sizeof(double);
+  if (P.split_able) P.fixed_bytes += size_t(ch) * sizeof(float2);
+  wc = std::max<long long>((ntl + nwaves - 1) / nwaves, P.lz_cap);
+  auto total = [&](long long wc) { return P.fixed_bytes + wave_bytes(wc) + nlz_wave(wc) * lz_tile; };
+  if (limit > 0 && total(wc) > limit) {   // the largest wave within the caller's limit
+    long long lo = 1, hi = std::min(wc, ntl);
+    while (lo < hi) {
+      const long long mid = (lo + hi + 1) / 2;
+      if (total(mid) <= limit) lo = mid;
+      else hi = mid - 1;
+    }
+    const long long n = (ntl + lo - 1) / lo;
+    wc = (ntl + n - 1) / n;
   }
+  P.wave_cap = int(wc);
+  P.nlz_wave = int(nlz_wave(wc));
+  if (P.split_able) P.nl_bricks = sq::nl_bricks_max(g, P.wave_cap);
+  P.fixed_bytes = total(wc) - size_t(wc) * P.per_tile_bytes;
   return SQ_OK;
 }
 }  // namespace
@@ -519,15 +566,23 @@ int dev_alloc(sq_handle* h, void** p, size_t bytes) {
 
 extern "C" {
 
-size_t sq_footprint_bytes(const sq_instance_desc* desc) {
+size_t sq_footprint_bytes(const sq_instance_desc* desc) { return sq::footprint_within(desc, 0); }
+
+int sq_setup(const sq_instance_desc* desc, sq_handle** out) { return sq::setup_within(desc, 0, out); }
+
+}  // extern "C"
+
+namespace sq {
+
+size_t footprint_within(const sq_instance_desc* desc, size_t limit) {
   std::string why;
   if (validate(desc, why) != SQ_OK) return 0;
   Plan P;
-  if (make_plan(desc, P, why) != SQ_OK) return 0;
+  if (make_plan(desc, P, why, limit) != SQ_OK) return 0;
   return P.fixed_bytes + size_t(P.wave_cap) * P.per_tile_bytes;
 }
 
-int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
+int setup_within(const sq_instance_desc* desc, size_t limit, sq_handle** out) {
   sq::NvtxRange nvtx("sq_setup");
   if (!out) { g_setup_err = "out is NULL"; return SQ_ERR_INVALID_ARG; }
   *out = nullptr;
@@ -535,7 +590,7 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   int rc = validate(desc, why);
   if (rc != SQ_OK) { g_setup_err = why; return rc; }
   Plan P;
-  rc = make_plan(desc, P, why);
+  rc = make_plan(desc, P, why, limit);
   if (rc != SQ_OK) { g_setup_err = why; return rc; }
 
   sq_handle* h = new sq_handle();
@@ -582,7 +637,7 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   // SQ_STEP_KERNEL=staged selects the TMA-staged step for a mixed sweep (sq_step_tma.cu; slower than
   // the default step kernel on the workloads measured, kept for comparison), SQ_STAGE_RECS its
   // images per stage
-  if (const char* env = std::getenv("SQ_STEP_KERNEL")) h->step_staged = std::string(env) == "staged";
+  h->step_staged = staged_requested();
   // SQ_STAGE_WAIT_TEST=1: every stage of the staged step waits for 16 bytes that never come, so
   // its bounded wait runs out (the test of SQ_ERR_TIMEOUT; the copies themselves complete)
   if (const char* env = std::getenv("SQ_STAGE_WAIT_TEST")) h->stage_wait_test = std::string(env) == "1";
@@ -614,7 +669,7 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   SQ_ALLOC(h->d.gdv64, sizeof(double) * std::max(1, h->n_ch_total));
   SQ_ALLOC(h->d.rcmax, sizeof(double) * std::max<size_t>(1, P.rcmax.size()));
   SQ_ALLOC(h->d.gdv32, sizeof(float) * std::max(1, h->n_ch_total));
-  SQ_ALLOC(h->d.chi64, sizeof(double) * std::max<long long>(1, P.table_len));
+  if (f64) SQ_ALLOC(h->d.chi64, sizeof(double) * std::max<long long>(1, P.table_len));
   if (!f64) SQ_ALLOC(h->d.chi32, sizeof(float) * std::max<long long>(1, P.table_len));
   if (!f64) SQ_ALLOC(h->d.chi32s, 2 * sizeof(float) * std::max<long long>(1, P.table_len));
   SQ_ALLOC(h->d.mom, sizeof(double) * size_t(Nd) * size_t(g.n_pl + 1) * SQ_N_MOMENTS);
@@ -627,7 +682,9 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   SQ_ALLOC(h->d.part, sizeof(double) * 4096 * 32);
   SQ_ALLOC(h->d.rho, sizeof(double) * Nd);
   SQ_ALLOC(h->d.status, sizeof(int) * sq::kStCount);
-  if (h->bounds_mode != SQ_BOUNDS_GIVEN) SQ_ALLOC(h->d.lzdot, sizeof(double) * sq::lz_dots_len(h->lanczos_k));
+  if (h->bounds_mode == SQ_BOUNDS_PER_NODE) SQ_ALLOC(h->d.lzdot, sizeof(double) * sq::lz_dots_len(h->lanczos_k));
+  if (!h->lanczos_tiles.empty())
+    SQ_ALLOC(h->d.lzdot, sizeof(double) * sq::lz_dots_len(h->lanczos_k, sq::lz_sample_blocks(P.lz_cap, g.Upts)));
   const int wt = h->wave_cap;
   SQ_ALLOC(h->wb.entries, sizeof(sq::TileEntry) * size_t(wt) * g.e_cap);
   SQ_ALLOC(h->wb.n_entries, sizeof(int) * wt);
@@ -635,17 +692,17 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   SQ_ALLOC(h->wb.brick_list, sizeof(int) * size_t(wt) * g.nbricks * g.br_cap);
   SQ_ALLOC(h->wb.brick_n, sizeof(int) * size_t(wt) * g.nbricks);
   SQ_ALLOC(h->wb.brick_rec, sizeof(int4) * 2 * size_t(wt) * g.nbricks * g.br_cap);
-  SQ_ALLOC(h->wb.brick_d0, sizeof(float4) * size_t(wt) * g.nbricks * g.br_cap);
-  SQ_ALLOC(h->wb.brick_tma, sizeof(int4) * size_t(wt) * g.nbricks * g.br_cap);
+  if (!f64 && !d0_in_ring(g)) SQ_ALLOC(h->wb.brick_d0, sizeof(float4) * size_t(wt) * g.nbricks * g.br_cap);
+  if (!f64 && h->step_staged) SQ_ALLOC(h->wb.brick_tma, sizeof(int4) * size_t(wt) * g.nbricks * g.br_cap);
   SQ_ALLOC(h->wb.slab_n, sizeof(int) * size_t(wt) * g.nslab);
   SQ_ALLOC(h->wb.slab_map, sizeof(int) * size_t(wt) * g.nslab * g.r_cap);
   for (int i = 0; i < 3; ++i) SQ_ALLOC(h->wb.T[i], real * size_t(wt) * g.Upts * g.B);
+  if (!f64 && !h->wb.brick_d0) h->wb.brick_d0 = (float4*)h->wb.T[1];
   SQ_ALLOC(h->wb.W, real * size_t(wt) * (f64 ? 9 : 3) * g.Upts * g.B);
   SQ_ALLOC(h->wb.A, real * size_t(wt) * g.r_cap * g.B);
-  SQ_ALLOC(h->wb.P, real * size_t(wt) * g.r_cap * g.B);
   SQ_ALLOC(h->wb.Pg[0], sizeof(double) * size_t(wt) * g.r_cap * g.B);   // projections: FP64 sums
   SQ_ALLOC(h->wb.Pg[1], sizeof(double) * size_t(wt) * g.r_cap * g.B);
-  SQ_ALLOC(h->wb.Spart, sizeof(double) * std::max(size_t(wt) * std::max(g.nslab, sq::stencil_chunks(g)), size_t(sq::kStepFill)) * g.B * 9);
+  SQ_ALLOC(h->wb.Spart, sizeof(double) * std::max(size_t(wt) * std::max(g.nslab, sq::stencil_chunks(g)), std::min(size_t(sq::kStepFill), size_t(wt) * g.nbricks)) * g.B * 9);
   SQ_ALLOC(h->wb.nl_cnt, sizeof(int) * 8);
   if (h->split_able) {   // (nl_X, nl_img, proj_idx and Part: ensure_nl_buffers)
     SQ_ALLOC(h->wb.proj_start, sizeof(int) * size_t(wt) * (size_t(g.e_cap) + 1));
@@ -656,9 +713,9 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   if (!h->lanczos_tiles.empty()) {
     const size_t nst = size_t(P.lz_cap);
     const int k = h->lanczos_k;
-    SQ_ALLOC(h->d.lzV, sizeof(double) * size_t(k + 1) * nst * g.Upts * g.B);
-    SQ_ALLOC(h->d.lzW, sizeof(double) * nst * g.Upts * g.B);
-    SQ_ALLOC(h->d.lzP, sizeof(double) * nst * size_t(g.r_cap) * g.B);
+    SQ_ALLOC(h->d.lzV, real * size_t(k + 1) * nst * g.Upts * g.B);
+    SQ_ALLOC(h->d.lzW, real * nst * g.Upts * g.B);
+    SQ_ALLOC(h->d.lzP, real * nst * size_t(g.r_cap) * g.B);
     SQ_ALLOC(h->d.lzC, sizeof(double) * nst * g.B * size_t(5 * k + 8));
     SQ_ALLOC(h->d.lz_tiles, sizeof(int) * nst);
     // list buffers of the sample tiles (the sweep's wave lists stay untouched by the bounds)
@@ -668,8 +725,6 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
     SQ_ALLOC(h->lzb.brick_list, sizeof(int) * nst * g.nbricks * g.br_cap);
     SQ_ALLOC(h->lzb.brick_n, sizeof(int) * nst * g.nbricks);
     SQ_ALLOC(h->lzb.brick_rec, sizeof(int4) * 2 * nst * g.nbricks * g.br_cap);
-    SQ_ALLOC(h->lzb.brick_d0, sizeof(float4) * nst * g.nbricks * g.br_cap);
-    SQ_ALLOC(h->lzb.brick_tma, sizeof(int4) * nst * g.nbricks * g.br_cap);
     SQ_ALLOC(h->lzb.slab_n, sizeof(int) * nst * g.nslab);
     SQ_ALLOC(h->lzb.slab_map, sizeof(int) * nst * g.nslab * g.r_cap);
   }
@@ -762,6 +817,10 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out) {
   *out = h;
   return SQ_OK;
 }
+
+}  // namespace sq
+
+extern "C" {
 
 int sq_moments(sq_handle* h) {
   if (!h) return SQ_ERR_INVALID_ARG;

@@ -15,6 +15,7 @@
 //     4x4x4 brick of U the entries meeting the brick (used by the per-point nonlocal apply).
 #pragma once
 
+#include <algorithm>
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -36,8 +37,20 @@ constexpr int kThreads = 256;    // block size of the tile kernels
 constexpr int kMaxU = 2 * 64 + 8; // largest union-window extent (m <= 64, b = 2, x padded to 4)
 constexpr int kMaxLanczos = 128;         // most Lanczos steps
 constexpr int kLzChunkTiles = 8 * 152;   // most (chunk, tile) blocks of a Lanczos wave split into chunks
-// doubles of their partial products: two sets of up to k + 1 products of 8 nodes, and the norms
-inline size_t lz_dots_len(int k) { return size_t(kLzChunkTiles) * 8 * (2 * size_t(k + 1) + 1); }
+// chunks per tile of a Lanczos wave: about eight blocks per SM, of at least 64 points, at most 32 (every block of a
+// tile adds the chunks' products for its coefficients)
+inline int lz_chunks(int ntiles, int Upts) {
+  return std::max(1, std::min({kLzChunkTiles / std::max(1, ntiles), 32, (Upts + 63) / 64}));
+}
+// doubles of the partial products of that many (chunk, tile) blocks: two sets of up to k + 1 products of 8 nodes,
+// and the norms
+inline size_t lz_dots_len(int k, int blocks = kLzChunkTiles) { return size_t(blocks) * 8 * (2 * size_t(k + 1) + 1); }
+// of the sample tiles of a handle (any number up to lz_cap)
+inline int lz_sample_blocks(int lz_cap, int Upts) {
+  int most = 1;
+  for (int n = 1; n <= lz_cap; ++n) most = std::max(most, n * lz_chunks(n, Upts));
+  return most;
+}
 
 struct AtomTab {
   int lo[3];        // support box corner (absolute lattice coordinates of the base image)
@@ -109,14 +122,13 @@ struct WaveBufs {
   int* brick_list = nullptr;      // [wt][nbricks][br_cap]
   int* brick_n = nullptr;         // [wt][nbricks]
   int4* brick_rec = nullptr;      // [wt][nbricks][br_cap][2] per-brick image records
-  float4* brick_d0 = nullptr;     // [wt][nbricks][br_cap] x - R of the record's brick corner (FP32 W table)
-  int4* brick_tma = nullptr;      // [wt][nbricks][br_cap] (atom, box-local x, y, z of the brick corner)
+  float4* brick_d0 = nullptr;     // [wt][nbricks][br_cap] x - R of the record's brick corner (FP32 W table; may lie in T[1])
+  int4* brick_tma = nullptr;      // [wt][nbricks][br_cap] (atom, box-local x, y, z of the brick corner), staged step
   int* slab_n = nullptr;          // [wt][nslab] projector rows meeting each slab (y-row of bricks)
   int* slab_map = nullptr;        // [wt][nslab][r_cap] slab row -> tile row
   void* T[3] = {nullptr, nullptr, nullptr};   // Real [wt][Upts][B]
   void* W = nullptr;              // FP32: W_b [wt][3][Upts][B]; FP64: G_ab = -grad_a W_b [wt][9][Upts][B]
   void* A = nullptr;              // Real [wt][r_cap][B]  chi_row(x_q)
-  void* P = nullptr;              // Real [wt][r_cap][B]  gamma |dOmega| chi^T t (Lanczos apply)
   void* Pg[2] = {nullptr, nullptr};   // double [wt][r_cap][B]  gamma |dOmega| chi^T t^j, ping-pong
   double* Spart = nullptr;        // [wt][slabs, their bricks or stencil row chunks][B][9]
   // the split mixed step (sq_step_mixed.cu)
@@ -145,7 +157,7 @@ struct Dev {
   double* rcmax = nullptr;        // per atom: largest projector radius
   float* gdv32 = nullptr;
   float2* gdvp = nullptr;         // gamma * dV per channel as a pair of floats
-  double* chi64 = nullptr;        // projector tables
+  double* chi64 = nullptr;        // projector tables (FP64 sweeps)
   float* chi32 = nullptr;
   float* chi32s = nullptr;        // mixed: each FP32 table value as a TF32 (hi, lo) pair
   double* mom = nullptr;          // [N_d][n_pl+1][17]
@@ -158,9 +170,9 @@ struct Dev {
   double* part = nullptr;         // contraction partials
   double* rho = nullptr;          // [N_d]
   int* status = nullptr;          // device status words
-  double* lzV = nullptr;          // Lanczos basis [(k+1)][nst][Upts][B]
-  double* lzW = nullptr;          // Lanczos work vector [nst][Upts][B]
-  double* lzP = nullptr;          // projections of the Lanczos vector [nst][r_cap][B]
+  void* lzV = nullptr;            // Real: Lanczos basis [(k+1)][nst][Upts][B]
+  void* lzW = nullptr;            // Real: Lanczos work vector [nst][Upts][B]
+  void* lzP = nullptr;            // Real: projections of the Lanczos vector [nst][r_cap][B]
   double* lzC = nullptr;          // Gram-Schmidt coefficients / alpha, beta [cols][...]
   int* lz_tiles = nullptr;        // sample tile ids [nst]
   double* lzdot = nullptr;        // chunk partials of the Lanczos products [lz_dots_len(lanczos_k)]
@@ -306,6 +318,10 @@ void dev_free(sq_handle* h, void* p, size_t bytes);
 int time_step_launch(sq_handle* h, int reps, double* ms_out);
 
 // error helpers
+// sq_footprint_bytes and sq_setup of a plan that takes its tiles in as small waves as limit bytes ask for (0: no
+// limit; more than limit when the smallest does not fit)
+size_t footprint_within(const sq_instance_desc* desc, size_t limit);
+int setup_within(const sq_instance_desc* desc, size_t limit, sq_handle** out);
 int fail(sq_handle* h, int code, const std::string& msg);
 #define SQ_CUDA_TRY(h, call)                                                              \
   do {                                                                                    \

@@ -463,12 +463,11 @@ int lanczos_columns(sq_handle* h, const Wave& w, int start, int k, Real* V, Real
   const int ncols = nst * g.B;
   const int ld = k + 1;
   const size_t vstride = (size_t)nst * g.Upts * g.B;
-  // chunks per tile: about eight blocks per SM, of at least 64 points, at most 32 (every block of a
-  // tile adds the chunks' products for its coefficients). dots holds the partial products of two passes
-  // and the norms; a wave of more tiles than it holds has one chunk per tile, in C.
-  const int nch = std::max(1, std::min({kLzChunkTiles / std::max(1, nst), 32, (g.Upts + 63) / 64}));
+  // dots holds the partial products of two passes and the norms; a wave of more tiles than it holds has
+  // one chunk per tile, in C.
+  const int nch = lz_chunks(nst, g.Upts);
   const bool small = nch * nst <= kLzChunkTiles;
-  const size_t set = (size_t)(small ? kLzChunkTiles : nst) * ld * kTileLz;
+  const size_t set = (size_t)nch * nst * ld * kTileLz;
   double* cA = small ? dots : C;
   double* cB = cA + set;
   double* nrm = cB + set;

@@ -4,9 +4,9 @@
 // admits requests in submission order as soon as the device bytes they need
 // (sq_footprint_bytes) fit under the budget next to the requests in flight and a worker slot
 // is free; admitted requests run their pipeline on their own worker thread and CUDA stream, so
-// requests that arrive while others are on the GPU overlap with them. A request larger than
-// the whole budget is answered with SQ_ERR_OOM without touching the device. Results are
-// collected with sq_server_poll; each carries its latency from submit to completion.
+// requests that arrive while others are on the GPU overlap with them. A request whose usual plan
+// is larger than the whole budget runs in smaller waves; one that does not fit in the smallest is
+// answered with SQ_ERR_OOM without touching the device. Results are collected with sq_server_poll; each carries its latency from submit to completion.
 //
 // Trajectories (sq_server_submit_traj): the requests of one trajectory are successive
 // snapshots of one cell. Its first request sets up a handle that stays resident on the device
@@ -38,6 +38,7 @@ struct Request {
   std::vector<int> species, proj_offset;
   std::vector<sq_proj> proj;
   size_t bytes = 0;
+  size_t limit = 0;   // bytes its plan is held to (0: its usual plan)
   Clock::time_point t_submit;
 };
 
@@ -118,7 +119,7 @@ void run_request(sq_server* s, Request* rq) {
   sq_handle* h = nullptr;
   if (rc == SQ_OK) {
     rq->desc.stream = st;
-    rc = sq_setup(&rq->desc, &h);
+    rc = sq::setup_within(&rq->desc, rq->limit, &h);
   }
   if (h) evaluate(h, res, rc);
   else {
@@ -151,7 +152,7 @@ void run_traj(sq_server* s, Request* rq, Resident* r, bool fresh) {
     }
     if (rc == SQ_OK) {
       rq->desc.stream = r->st;
-      rc = sq_setup(&rq->desc, &r->h);
+      rc = sq::setup_within(&rq->desc, rq->limit, &r->h);
     }
   } else {
     rc = sq_update_atoms(r->h, rq->pos.empty() ? nullptr : rq->pos.data(), rq->v.data());
@@ -278,8 +279,12 @@ void dispatch_loop(sq_server* s) {
 
 int submit(sq_server* s, const sq_instance_desc* d, long long tag, long long traj) {
   if (!s || !d) return SQ_ERR_INVALID_ARG;
-  const size_t bytes = sq_footprint_bytes(d);
+  size_t bytes = sq_footprint_bytes(d), limit = 0;
   if (bytes == 0) return SQ_ERR_INVALID_ARG;   // the descriptor does not validate
+  if (bytes > s->budget) {
+    limit = s->budget;
+    bytes = sq::footprint_within(d, limit);
+  }
   Request* rq = new Request();
   rq->tag = tag;
   rq->traj = traj;
@@ -299,6 +304,7 @@ int submit(sq_server* s, const sq_instance_desc* d, long long tag, long long tra
   }
   rq->desc.stream = nullptr;
   rq->bytes = bytes;
+  rq->limit = limit;
   rq->t_submit = Clock::now();
   {
     std::lock_guard<std::mutex> lk(s->mu);

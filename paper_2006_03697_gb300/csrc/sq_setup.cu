@@ -231,11 +231,11 @@ __global__ void k_brick_lists(Geo g, Wave w, int whole, const AtomTab* __restric
         r[1] = make_int4(ats.dim[0], ats.dim[1], int(lo32), int(hi32));
         // x - R of the brick corner for this image, (lo + l0) h - R, formed in FP64 and rounded once
         // (once per record: the per-point work adds only the in-brick offset)
-        d0[((size_t)tl * g.nbricks + br) * g.br_cap + pos_s] =
+        if (d0) d0[((size_t)tl * g.nbricks + br) * g.br_cap + pos_s] =
             make_float4(float((ats.lo[0] + l0[0]) * g.h[0] - ats.R[0]), float((ats.lo[1] + l0[1]) * g.h[1] - ats.R[1]),
                         float((ats.lo[2] + l0[2]) * g.h[2] - ats.R[2]), 0.f);
         // the brick's box in the atom's table slot (coordinates of the TMA-staged step)
-        tma[((size_t)tl * g.nbricks + br) * g.br_cap + pos_s] = make_int4(tes.atom, l0[0], l0[1], l0[2]);
+        if (tma) tma[((size_t)tl * g.nbricks + br) * g.br_cap + pos_s] = make_int4(tes.atom, l0[0], l0[1], l0[2]);
       }
     }
     cnt += __popc(mask);
@@ -498,9 +498,10 @@ int build_wave_entries(sq_handle* h, const Wave& w, WaveBufs* b) {
 
 int build_tables(sq_handle* h) {
   if (h->geo.n_atoms == 0 || h->table_len == 0) return SQ_OK;
-  k_chi_tables<double><<<dim3(h->geo.n_atoms, 32), 256, 0, h->stream>>>(h->geo, h->d.atoms, h->d.gdv, h->d.chi64);
-  SQ_LAUNCH_CHECK(h);
-  if (h->precision == SQ_MIXED) {
+  if (h->precision == SQ_FP64) {
+    k_chi_tables<double><<<dim3(h->geo.n_atoms, 32), 256, 0, h->stream>>>(h->geo, h->d.atoms, h->d.gdv, h->d.chi64);
+    SQ_LAUNCH_CHECK(h);
+  } else {
     k_chi_tables<float><<<dim3(h->geo.n_atoms, 32), 256, 0, h->stream>>>(h->geo, h->d.atoms, h->d.gdv, h->d.chi32);
     SQ_LAUNCH_CHECK(h);
     k_split_tf32<<<1024, 256, 0, h->stream>>>(h->d.chi32, h->table_len, h->d.chi32s);
