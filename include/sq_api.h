@@ -143,11 +143,11 @@ int sq_setup(const sq_instance_desc* desc, sq_handle** out);
  * Asynchronous on the handle's stream. Errors: SQ_ERR_CUDA, SQ_ERR_OOM. */
 int sq_moments(sq_handle* h);
 
-/* Fermi level: FP64 root of N(mu) = N_e, N(mu) = 2 sum'_j c^j(mu) R^j, R^j = sum_q rho_q^j, on
- * [lambda_lo - 40 kT, lambda_hi + 40 kT], by Newton steps on ln N inside a shrinking bracket
- * (bisection where a step fails) until the bracket is < 1e-13 max(1, |mu|) or 200 evaluations;
- * runs on the device and synchronises the stream. Errors: SQ_ERR_STATE (no moments),
- * SQ_ERR_NO_BRACKET, SQ_ERR_CUDA. */
+/* Fermi level by FP64 bisection on N(mu) = 2 sum'_j c^j(mu) R^j, R^j = sum_q rho_q^j, on
+ * [lambda_lo - 40 kT, lambda_hi + 40 kT] until the bracket is < 1e-13 max(1, |mu|) or 200
+ * steps (steps within a bracket on which N(mu) is known to rise are replaced by a Newton search
+ * with the same result); runs on the device and synchronises the stream. Errors: SQ_ERR_STATE
+ * (no moments), SQ_ERR_NO_BRACKET, SQ_ERR_CUDA. */
 int sq_fermi_level(sq_handle* h, double* mu_out);
 
 /* Resident state for a trajectory (successive quantum-MD snapshots of one cell): gives the
@@ -177,7 +177,7 @@ int sq_keep_lists(sq_handle* h, int enable);
  * Sec. 4, and the parts add up to the whole cell. The Fermi level needs the whole-cell sums:
  *   sq_node_sums        R_out [n_pl + 1] (host) = sum over this part's nodes of rho_q^j
  *                       (fixed order); synchronises. Errors: SQ_ERR_STATE (no moments).
- *   sq_fermi_level_sums the root search of sq_fermi_level on the caller's R_host [n_pl + 1]
+ *   sq_fermi_level_sums the bisection of sq_fermi_level on the caller's R_host [n_pl + 1]
  *                       (the sum of every part's sq_node_sums, e.g. one allreduce of n_pl + 1
  *                       doubles); synchronises. Errors: SQ_ERR_STATE, SQ_ERR_INVALID_ARG
  *                       (NULL or non-finite R_host), SQ_ERR_NO_BRACKET.
@@ -278,7 +278,7 @@ int sq_kernel_timing_read(const sq_handle* h, int kid, long long* launches, doub
 /* Fermi level without any device allocation. The paper has no counterpart: this is a
  * service for callers that cannot call cudaMalloc (an allocator that is locked or at its
  * budget, a plug-in that must leave the process's device heap alone). It runs the same
- * root search as sq_fermi_level on a moment table the caller owns:
+ * bisection as sq_fermi_level on a moment table the caller owns:
  *   mom_dev      device, [n_nodes][n_pl + 1][SQ_N_MOMENTS] FP64 (the sq_moments_copy layout;
  *                only slot 0, rho^j, is read)
  *   lambda_lo/hi the spectral bounds the table was computed with (sq_get_bounds)
@@ -381,7 +381,7 @@ void sq_server_destroy(sq_server* s);
  * FP32 vectors in SQ_MIXED), the eigenvalues theta_qi and squared first eigenvector components
  * w_qi of its tridiagonal (k-point Gauss quadrature of e_q's spectral measure, exact for
  * polynomials of degree <= 2k - 1); rho_q = (2/|dOmega|) sum_i w_qi g(theta_qi) with the Fermi
- * level from 2 sum_q sum_i w_qi g(theta_qi) = N_e (the root search of sq_fermi_level) and
+ * level from 2 sum_q sum_i w_qi g(theta_qi) = N_e (the bisection rule of sq_fermi_level) and
  * E_band = 2 sum_q sum_i w_qi theta_qi g(theta_qi). Independent of sq_moments (it neither needs
  * nor changes the Chebyshev moments; it rebuilds the per-wave lists). k in 1..128 (capped at
  * the region dimension). Host outputs: mu_out, rho_out [N_d] (x fastest), e_band_out, each may

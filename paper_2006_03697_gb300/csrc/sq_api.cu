@@ -465,7 +465,7 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why, size_t limit
     return d->bounds_mode == SQ_BOUNDS_PER_NODE ? std::max<size_t>(1, std::min<size_t>((size_t(8) << 30) / lz_tile, size_t(wc))) : size_t(0);
   };
   if (d->bounds_mode == SQ_BOUNDS_PER_NODE)
-    P.fixed_bytes += size_t(Nd) * (4 + M + 20) * sizeof(double) + 1024 * sizeof(double);
+    P.fixed_bytes += size_t(Nd) * (4 + M + 20) * sizeof(double) + sq::kNodeParts * sizeof(double);
   if (P.split_able) P.fixed_bytes += size_t(ch) * sizeof(float2);
   wc = std::max<long long>((ntl + nwaves - 1) / nwaves, P.lz_cap);
   auto total = [&](long long wc) { return P.fixed_bytes + wave_bytes(wc) + nlz_wave(wc) * lz_tile; };
@@ -735,7 +735,7 @@ int setup_within(const sq_instance_desc* desc, size_t limit, sq_handle** out) {
     SQ_ALLOC(h->d.ncoef, sizeof(double) * 2 * size_t(Nd));
     SQ_ALLOC(h->d.nF, sizeof(double) * size_t(Nd) * h->M);
     SQ_ALLOC(h->d.nrow, sizeof(double) * size_t(Nd) * 20);
-    SQ_ALLOC(h->d.npart, sizeof(double) * 1024);
+    SQ_ALLOC(h->d.npart, sizeof(double) * sq::kNodeParts);
     SQ_ALLOC(h->d.nV, real * size_t(k + 1) * nw * g.Upts * g.B);
     SQ_ALLOC(h->d.nW, real * nw * g.Upts * g.B);
     SQ_ALLOC(h->d.nP, real * nw * size_t(g.r_cap) * g.B);

@@ -5,7 +5,7 @@
 // implicit QL with Wilkinson shifts, rotating only the first row of the eigenvector matrix);
 // then [f(H_q)]_qq ~ sum_i w_qi f(theta_qi), exact for polynomials of degree <= 2k - 1.
 // rho_q = (2 / |dOmega|) sum_i w_qi g(theta_qi), the Fermi level solves
-// 2 sum_q sum_i w_qi g(theta_qi) = N_e (the root search of the Clenshaw-Curtis path) and
+// 2 sum_q sum_i w_qi g(theta_qi) = N_e (the bisection rule of the Clenshaw-Curtis path) and
 // E_band = 2 sum_q sum_i w_qi theta_qi g(theta_qi).
 #include <algorithm>
 #include <cmath>
@@ -275,7 +275,7 @@ static int gauss_t(sq_handle* h, int k, double* mu_out, double* rho_host, double
                                                                  h->d.status);
     if (cudaGetLastError() != cudaSuccess) rc = fail(h, SQ_ERR_CUDA, "k_gauss_eig launch failed");
   }
-  // Fermi level: the Clenshaw-Curtis path's root finder; the bracket from the extreme
+  // Fermi level: the Clenshaw-Curtis path's rule; the bracket from the extreme
   // weighted Gauss nodes (device reduction, two doubles to the host)
   double tmin = 0.0, tmax = 0.0;
   if (rc == SQ_OK) {
@@ -313,13 +313,13 @@ static int gauss_t(sq_handle* h, int k, double* mu_out, double* rho_host, double
       rc = fail(h, SQ_ERR_NO_BRACKET, "N(mu) - N_e has no sign change on the bisection bracket");
     } else {
       FermiRoot r;
-      r.init(lo, hi, h->n_e);
+      r.init(lo, hi, h->n_e, h->kT, true);   // (the weights are positive: N rises everywhere)
       do {
         if (count(r.mu, nm) != SQ_OK) {
           rc = fail(h, SQ_ERR_CUDA, "electron count failed");
           break;
         }
-      } while (!r.update(nm[0], nm[1]));
+      } while (!r.update(nm[0], nm[1], nm[1]));
       mu = r.mu;
     }
   }

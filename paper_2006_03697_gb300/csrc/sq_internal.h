@@ -35,6 +35,7 @@ constexpr int kBrick = 4;        // brick side in points
 constexpr int kMaxCh = 8;        // projector channels per atom
 constexpr int kThreads = 256;    // block size of the tile kernels
 constexpr int kMaxU = 2 * 64 + 8; // largest union-window extent (m <= 64, b = 2, x padded to 4)
+constexpr int kNodeParts = 1536;         // doubles of d.npart
 constexpr int kMaxLanczos = 128;         // most Lanczos steps
 constexpr int kLzChunkTiles = 8 * 152;   // most (chunk, tile) blocks of a Lanczos wave split into chunks
 // chunks per tile of a Lanczos wave: about eight blocks per SM, of at least 64 points, at most 32 (every block of a
@@ -181,7 +182,7 @@ struct Dev {
   double* ncoef = nullptr;        // [N_d][2] step coefficients (ca = 2 / zeta_q, cd = ca lap0 - 2 chi_q / zeta_q)
   double* nF = nullptr;           // [N_d][M] sum'_j cos(j theta_k) rho_q^j
   double* nrow = nullptr;         // [N_d][20] contraction terms per node
-  double* npart = nullptr;        // [1024] partial electron counts
+  double* npart = nullptr;        // [kNodeParts] partial electron counts
   void* nV = nullptr;             // Lanczos wave buffers of the per-node bounds
   void* nW = nullptr;
   void* nP = nullptr;

@@ -4,7 +4,7 @@
 //   F_k      = sum'_j cos(j theta_k) R^j,  theta_k = pi (k + 1/2) / M
 //   N(mu)    = 2 sum'_j c^j(mu) R^j = (4/M) sum_k g((chi + zeta cos theta_k - mu)/kT) F_k
 // because c^j = (2/M) sum_k g(cos theta_k) cos(j theta_k) is the M-point Chebyshev-Gauss
-// rule for the Clenshaw-Curtis coefficient integral of Sec. 4; safeguarded root of N(mu) = N_e.
+// rule for the Clenshaw-Curtis coefficient integral of Sec. 4; bisection on N(mu) = N_e (FermiRoot).
 // The contraction evaluates c^j, d^j (coefficients of r g(r), App. A) and s^j (entropy
 // function) at mu and forms rho_q, E_band, E_s, E_nl and sigma (Sec. 4 stress sums).
 #include <algorithm>
@@ -344,13 +344,13 @@ __global__ void __launch_bounds__(256) k_cosF_nodes(const double* __restrict__ m
   F[(size_t)q * M + M - 1 - k] = s[0] - s[1];   // k = M - 1 - k: the odd part is zero there
 }
 
-// part[2 block], part[2 block + 1] = N and dN/dmu of the block's nodes:
-// (4/M) sum_q sum_k g((chi_q + zeta_q cos theta_k - mu)/kT) F_q(k), and g (1 - g) / kT in place of g
+// part[3 block ..] = N, dN/dmu and D (FermiRoot) of the block's nodes: (4/M) sum_q sum_k
+// g((chi_q + zeta_q cos theta_k - mu)/kT) F_q(k), g (1 - g) / kT in place of g, and that with |F_q(k)|
 __global__ void __launch_bounds__(256) k_count_nodes(const double* __restrict__ F, const double* __restrict__ nbnd, int Nd,
                                                      int M, const double* __restrict__ tab, double kT, double mu,
                                                      double* __restrict__ part) {
   __shared__ double sh[256];
-  double a0 = 0.0, a1 = 0.0;
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
   for (int q = blockIdx.x; q < Nd; q += gridDim.x) {
     const double lo = nbnd[2 * q], hi = nbnd[2 * q + 1];
     const double chi_q = 0.5 * (hi + lo), zeta_q = 0.5 * (hi - lo);
@@ -358,32 +358,48 @@ __global__ void __launch_bounds__(256) k_count_nodes(const double* __restrict__ 
     for (int k = threadIdx.x; k < M; k += blockDim.x) {
       const double g = fermi_occ((chi_q + zeta_q * tab[2 * k + 1] - mu) / kT), gf = g * Fq[k];
       a0 += gf;
-      a1 += gf * (1.0 - g);
+      const double d = gf * (1.0 - g);
+      a1 += d;
+      a2 += fabs(d);
     }
   }
   a0 = block_sum_d(a0, sh);
   a1 = block_sum_d(a1, sh);
+  a2 = block_sum_d(a2, sh);
   if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = 4.0 / M * a0;
-    part[2 * blockIdx.x + 1] = 4.0 / M / kT * a1;
+    part[3 * blockIdx.x] = 4.0 / M * a0;
+    part[3 * blockIdx.x + 1] = 4.0 / M / kT * a1;
+    part[3 * blockIdx.x + 2] = 4.0 / M / kT * a2;
   }
 }
 
-// out[0], out[1] = sums of the (N, dN/dmu) pairs, fixed order; with nbnd: out[2] = min lo_q,
-// out[3] = max hi_q. One block of 256.
-__global__ void __launch_bounds__(256) k_sum_parts(const double* __restrict__ part, int n, const double* __restrict__ nbnd,
-                                                   int Nd, double* __restrict__ out) {
-  __shared__ double sh[256], slo[256], shi[256];
+// part[3 block], part[3 block + 1] = the block's shares of (4/M) sum F and (4/M) sum |F| over all nodes and points
+__global__ void __launch_bounds__(256) k_F_sums(const double* __restrict__ F, size_t n, int M, double* __restrict__ part) {
+  __shared__ double sh[256];
   double a0 = 0.0, a1 = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    a0 += part[2 * i];
-    a1 += part[2 * i + 1];
+  for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) {
+    a0 += F[i];
+    a1 += fabs(F[i]);
   }
   a0 = block_sum_d(a0, sh);
   a1 = block_sum_d(a1, sh);
   if (threadIdx.x == 0) {
-    out[0] = a0;
-    out[1] = a1;
+    part[3 * blockIdx.x] = 4.0 / M * a0;
+    part[3 * blockIdx.x + 1] = 4.0 / M * a1;
+    part[3 * blockIdx.x + 2] = 0.0;
+  }
+}
+
+// out[0 .. 2] = sums of the (N, dN/dmu, D) triples, fixed order; with nbnd: out[3] = min lo_q,
+// out[4] = max hi_q. One block of 256.
+__global__ void __launch_bounds__(256) k_sum_parts(const double* __restrict__ part, int n, const double* __restrict__ nbnd,
+                                                   int Nd, double* __restrict__ out) {
+  __shared__ double sh[256], slo[256], shi[256];
+  for (int c = 0; c < 3; ++c) {
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) s += part[3 * i + c];
+    s = block_sum_d(s, sh);
+    if (threadIdx.x == 0) out[c] = s;
   }
   if (!nbnd) return;
   double lo = INFINITY, hi = -INFINITY;
@@ -402,14 +418,15 @@ __global__ void __launch_bounds__(256) k_sum_parts(const double* __restrict__ pa
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    out[2] = slo[0];
-    out[3] = shi[0];
+    out[3] = slo[0];
+    out[4] = shi[0];
   }
 }
 
 // Blocks of k_count_nodes, three per SM: it is bound by the SMs' FP64 units, and 512 blocks left some SMs a third
-// more of them than others (1728 nodes: 332 -> 285 us). d.npart holds 1024 doubles: a pair per block.
+// more of them than others (1728 nodes: 332 -> 285 us). d.npart holds a triple per block.
 constexpr int kCountBlocks = 3 * 152;
+static_assert(3 * kCountBlocks <= kNodeParts, "d.npart");
 
 int run_fermi_nodes(sq_handle* h, double* mu_out) {
   const Geo& g = h->geo;
@@ -417,32 +434,40 @@ int run_fermi_nodes(sq_handle* h, double* mu_out) {
   const int M = h->M;
   k_cosF_nodes<<<dim3(((M + 1) / 2 + 255) / 256, h->Nd), 256, 0, s>>>(h->d.mom, h->Nd, g.n_pl, M, h->d.costab, h->d.nF);
   SQ_LAUNCH_CHECK(h);
-  double* out = h->d.scal + 40;   // [N, dN/dmu, min lo, max hi]
-  // ext: only the interval of all nodes (an evaluation is bound by its N_d M FP64 exponentials: 0.33 ms at 12^3)
+  double* out = h->d.scal + 40;   // [N, dN/dmu, D, min lo, max hi]
+  // ext: (4/M) sum F and sum |F| and the interval of all nodes (an evaluation is bound by its N_d M FP64
+  // exponentials: 0.28 ms at 12^3)
   auto count = [&](double mu, double* res, bool ext) -> int {
-    if (!ext) {
-      k_count_nodes<<<kCountBlocks, 256, 0, s>>>(h->d.nF, h->d.nbnd, h->Nd, M, h->d.costab, h->kT, mu, h->d.npart);
-      SQ_LAUNCH_CHECK(h);
-    }
-    k_sum_parts<<<1, 256, 0, s>>>(h->d.npart, ext ? 0 : kCountBlocks, ext ? h->d.nbnd : nullptr, h->Nd, out);
+    if (ext) k_F_sums<<<kCountBlocks, 256, 0, s>>>(h->d.nF, (size_t)h->Nd * M, M, h->d.npart);
+    else k_count_nodes<<<kCountBlocks, 256, 0, s>>>(h->d.nF, h->d.nbnd, h->Nd, M, h->d.costab, h->kT, mu, h->d.npart);
     SQ_LAUNCH_CHECK(h);
-    SQ_CUDA_TRY(h, cudaMemcpyAsync(res, out, (ext ? 4 : 2) * sizeof(double), cudaMemcpyDeviceToHost, s));
+    k_sum_parts<<<1, 256, 0, s>>>(h->d.npart, kCountBlocks, ext ? h->d.nbnd : nullptr, h->Nd, out);
+    SQ_LAUNCH_CHECK(h);
+    SQ_CUDA_TRY(h, cudaMemcpyAsync(res, out, (ext ? 5 : 3) * sizeof(double), cudaMemcpyDeviceToHost, s));
     SQ_CUDA_TRY(h, cudaStreamSynchronize(s));
     return SQ_OK;
   };
   // the shared mode's rule on [min lo_q - 40 kT, max hi_q + 40 kT]
-  double e[4], nlo[2], nhi[2];
+  double e[5], nlo[3], nhi[3];
   int rc = count(0.0, e, true);
   if (rc != SQ_OK) return rc;
-  const double lo = e[2] - 40.0 * h->kT, hi = e[3] + 40.0 * h->kT;
-  if ((rc = count(lo, nlo, false)) != SQ_OK || (rc = count(hi, nhi, false)) != SQ_OK) return rc;
+  const double lo = e[3] - 40.0 * h->kT, hi = e[4] + 40.0 * h->kT;
+  // 40 kT outside every interval g is below 5e-18 or that close to one: the sums of F and |F| tell which side of N_e
+  // the ends lie on, unless they come that close to it
+  const double tail = 5e-18 * e[1];
+  if (tail < 0.5 * h->n_e && e[0] - tail > h->n_e * (1.0 + 1e-10)) {
+    nlo[0] = 0.0;
+    nhi[0] = e[0];
+  } else if ((rc = count(lo, nlo, false)) != SQ_OK || (rc = count(hi, nhi, false)) != SQ_OK) {
+    return rc;
+  }
   if (!(nlo[0] < h->n_e && h->n_e < nhi[0]))
     return fail(h, SQ_ERR_NO_BRACKET, "N(mu) - N_e has no sign change on the bisection bracket");
   FermiRoot r;
-  r.init(lo, hi, h->n_e);
+  r.init(lo, hi, h->n_e, h->kT);
   do {
     if ((rc = count(r.mu, e, false)) != SQ_OK) return rc;
-  } while (!r.update(e[0], e[1]));
+  } while (!r.update(e[0], e[1], e[2]));
   if (mu_out) *mu_out = r.mu;
   return SQ_OK;
 }
