@@ -235,7 +235,7 @@ long long sq_kernel_launches(const sq_handle* h);
  *   counts[0]  the split mixed step (SQ_MIXED, at most 4 channels per atom): projector apply and
  *              projections on tensor cores and the stencil, each a kernel of its own
  *   counts[1]  one kernel, projections of the block's atom images staged in shared memory, scalar
- *              projector phases (SQ_FP64, > 4 channels, or bricks fuller than the split step's tables)
+ *              projector phases (SQ_FP64, > 4 channels, or no memory for the split step's tables)
  *   counts[2]  projections read and accumulated in global memory (a block meets more
  *              projector rows than shared memory holds: dense atoms, large R_cut)
  *   counts[3]  the TMA-staged step (SQ_MIXED, at most 4 channels per atom, one projector
@@ -248,8 +248,9 @@ long long sq_kernel_launches(const sq_handle* h);
  * the atom images per stage. Errors: SQ_ERR_INVALID_ARG. */
 int sq_step_launch_counts(const sq_handle* h, long long* counts);
 
-/* Autotuning hook of the step kernel: n_warps warps per step block (1..8; 0 = the default,
- * the count that leaves the fewest idle warps over a slab's bricks) and at most wave_tiles tiles
+/* Autotuning hook of the step: n_warps warps per block of the one-kernel steps (1..8; 0 = the default,
+ * the count that leaves the fewest idle warps over a slab's bricks; the split step has block sizes of
+ * its own and the count changes nothing) and at most wave_tiles tiles
  * per launch (0 = as many as the buffers sized at sq_setup hold; waves are spread evenly over the
  * handle's tiles). The settings stay with the handle. With reps > 0 and ms_per_tile non-NULL,
  * also times reps recurrence-step launches of the first wave with CUDA events on the handle's

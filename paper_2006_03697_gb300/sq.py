@@ -376,16 +376,16 @@ def sq_keep_lists(h, enable: bool = True):
 
 
 def sq_step_launch_counts(h):
-    """Step-kernel launches by variant: (shared memory + tensor cores, shared memory + scalar,
-    global-memory projections, TMA-staged step)."""
+    """Recurrence steps by variant: (split mixed step, one kernel with projections in shared memory,
+    the same with projections in global memory, TMA-staged step)."""
     c = (C.c_longlong * 4)()
     _check(lib().sq_step_launch_counts(h, c), h)
     return tuple(int(x) for x in c)
 
 
 def sq_tune_step(h, n_warps: int = 0, wave_tiles: int = 0, reps: int = 0):
-    """Sets the step kernel's warps per block and tiles per wave; with reps > 0 returns the
-    timed milliseconds per tile and step, else None."""
+    """Sets the tiles per wave and the warps per block of the one-kernel steps (the split mixed step has
+    block sizes of its own); with reps > 0 returns the timed milliseconds per tile and step, else None."""
     ms = C.c_double(0.0)
     _check(lib().sq_tune_step(h, int(n_warps), int(wave_tiles), int(reps), C.byref(ms) if reps > 0 else None), h)
     return ms.value if reps > 0 else None
@@ -394,12 +394,23 @@ def sq_tune_step(h, n_warps: int = 0, wave_tiles: int = 0, reps: int = 0):
 TUNE_CACHE = Path(__file__).resolve().parent / "_lib" / "step_tune.json"
 
 
+def _step_sources_id() -> str:
+    """Identifies the step kernels' text: a choice timed with other kernels is not taken."""
+    import hashlib
+    src = Path(__file__).resolve().parent / "csrc"
+    h = hashlib.sha1()
+    for name in ("sq_sweep.cu", "sq_step_mixed.cu", "sq_step_tma.cu", "sq_device.cuh", "sq_internal.h"):
+        h.update((src / name).read_bytes())
+    return h.hexdigest()[:10]
+
+
 def autotune_step(h, inst: dict, precision, candidates_warps=(4, 5, 6, 7, 8), wave_fractions=(1, 2, 4),
                   reps: int = 3, cache: Path | None = TUNE_CACHE, partition=None):
-    """Chooses warps per step block and tiles per wave for this handle's geometry by timing the
-    candidates (sq_tune_step) and keeps the fastest; the choice is cached per geometry key
-    (precision, n_o, region half-widths m, tiles) in a JSON file beside the built library, so the
-    next handle of the same shape takes it without timing. Returns (key, choice, timings)."""
+    """Chooses tiles per wave, and for the one-kernel steps warps per block, for this handle's geometry
+    by timing the candidates (sq_tune_step) and keeps the fastest; the choice is cached per key
+    (precision, n_o, region half-widths m, tiles, atoms, channels, step kernel text) in a JSON file beside
+    the built library, so the next handle of the same shape takes it without timing. Returns (key,
+    choice, timings)."""
     import json
     n = np.asarray(inst["n"], dtype=np.int64)
     h_ = np.asarray(inst["L"], dtype=np.float64) / n
@@ -408,7 +419,9 @@ def autotune_step(h, inst: dict, precision, candidates_warps=(4, 5, 6, 7, 8), wa
     if partition is not None:                                # this part's tile range only
         r, c = int(partition[0]), int(partition[1])
         tiles = tiles * (r + 1) // c - tiles * r // c
-    key = f"p{int(precision)}_no{int(inst['n_o'])}_m{'x'.join(str(x) for x in m)}_t{tiles}"
+    channels = [sum(2 * int(pj["l"]) + 1 for pj in sp) for sp in inst["proj"]]
+    key = (f"p{int(precision)}_no{int(inst['n_o'])}_m{'x'.join(str(x) for x in m)}_t{tiles}"
+           f"_a{len(inst['pos'])}_c{max(channels, default=0)}_{_step_sources_id()}")
     table = {}
     if cache is not None and cache.exists():
         try:
@@ -420,11 +433,16 @@ def autotune_step(h, inst: dict, precision, candidates_warps=(4, 5, 6, 7, 8), wa
         sq_tune_step(h, w, wt, 0)
         return key, table[key], None
     times = {}
+    split = sq_step_launch_counts(h)[0]
     base = sq_tune_step(h, 0, 0, reps)                       # the default settings first
     times[(0, 0)] = base
+    if sq_step_launch_counts(h)[0] > split:                  # the split step ran: warps are not its choice
+        candidates_warps = (0,)
     for frac in wave_fractions:
         wt = 0 if frac == 1 else max(1, tiles // frac)
         for w in candidates_warps:
+            if (w, wt) in times:
+                continue
             times[(w, wt)] = sq_tune_step(h, w, wt, reps)
     (w, wt), best = min(times.items(), key=lambda kv: kv[1])
     sq_tune_step(h, w, wt, 0)
