@@ -57,6 +57,15 @@ __device__ __forceinline__ void mma_tf32(float d[4], const uint32_t a[4], const 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
+// d = a * b, the same fragments. Sums longer than a product add these in FP32: the tensor core truncates where it
+// adds to an accumulator, and 24 products into one accumulator came 10 times as far from 64 bits.
+__device__ __forceinline__ void mma_tf32_set(float d[4], const uint32_t a[4], const uint32_t b[2]) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%10, %10, %10, %10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(0.f));
+}
+
 // Linear index of an absolute lattice point inside an atom image's support box, or -1.
 __device__ __forceinline__ int box_index(const AtomTab& at, const int s[3], const int n[3],
                                          int ax, int ay, int az) {
@@ -285,8 +294,8 @@ __device__ __forceinline__ bool fermi_cluster_search(const double* __restrict__ 
   return ok;
 }
 
-// ---- cross-thread sums with FP64's accuracy: doubles for FP64 vectors, pairs of floats (two-sum) for FP32
-// ones; FP64 adds issue at 1.7 lanes per clock and SM and cost more than the products they sum.
+// ---- cross-thread sums: doubles for FP64 vectors, pairs of floats (two-sum, about 2^-47 relative, on terms rounded
+// to 2^-24) for FP32 ones; FP64 adds issue at 1.7 lanes per clock and SM and cost more than the products they sum.
 struct FloatPair { float h, l; };
 
 __device__ __forceinline__ FloatPair lz_add(FloatPair a, FloatPair b) {   // Knuth's two-sum, tails added

@@ -359,7 +359,10 @@ __device__ __forceinline__ void nl_apply_pass(const Geo& g, NlShared& sh, float*
         const uint32_t bl[2] = {__float_as_uint(bt[kPlane + 64 * ks]), __float_as_uint(bt[kPlane + 64 * ks + 32])};
         mma_tf32(dl, al[ks], bh);   // small terms in their own sum (a third one cost more moves than it hid)
         mma_tf32(dl, ah[ks], bl);
-        mma_tf32(dh, ah[ks], bh);
+        float d[4];
+        mma_tf32_set(d, ah[ks], bh);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dh[i] += d[i];
       }
       if (s0) *reinterpret_cast<float2*>(y0) = make_float2(dh[0] + dl[0], dh[1] + dl[1]);
       if (s1) *reinterpret_cast<float2*>(y1) = make_float2(dh[2] + dl[2], dh[3] + dl[3]);
@@ -496,7 +499,10 @@ k_nl_project(Geo g, Wave w, NlGrid grid, int c0, int cn, const float* __restrict
             const uint32_t bl[2] = {__float_as_uint(bt[512 + 64 * ks]), __float_as_uint(bt[512 + 64 * ks + 32])};
             mma_tf32(dl, al[ks], bh);
             mma_tf32(dl, ah[ks], bl);
-            mma_tf32(dh, ah[ks], bh);
+            float d[4];
+            mma_tf32_set(d, ah[ks], bh);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) dh[i] += d[i];
           }
           float* o = po + (size_t)cur.y * 8;
           if (r < nrows) *reinterpret_cast<float2*>(o) = make_float2(dh[0] + dl[0], dh[1] + dl[1]);
@@ -591,8 +597,8 @@ k_nl_index(Geo g, Wave w, NlGrid grid, const AtomTab* __restrict__ atoms, const 
 }
 
 // P[row][q] = gamma |dOmega| times the sum of the row's partial projections over its bricks, as pairs of floats
-// (two-sum; FP64 adds issue at 1.7 lanes per clock), in a fixed order: rounded once and split to TF32 planes (hi, lo) for the apply in P, the pair
-// in Pp. One warp per image: its 8 nch values are 2 nch groups of four, so 16 / nch bricks are read at once
+// (two-sum; FP64 adds issue at 1.7 lanes per clock), in a fixed order: rounded once and split to TF32 planes
+// (hi, lo) for the apply in P, the pair in Pp. One warp per image: its 8 nch values are 2 nch groups of four, so 16 / nch bricks are read at once
 // (one brick at a time left too few loads in flight), then added over the lanes that share a group.
 __device__ __forceinline__ void pair_add(float& h, float& l, float vh, float vl) {
   const float s = __fadd_rn(h, vh), z = __fsub_rn(s, h);
@@ -890,8 +896,8 @@ k_stencil(Geo g, Wave w, const float* __restrict__ Tc, const float* __restrict__
 }
 
 // ------------------------------------------------------------------------------ host
-// Rows per stencil block: at most 448 threads, so two blocks share an SM (the rows evenly spread over the
-// blocks); windows wider than 112 points take one row and up to 544 threads.
+// Rows per stencil block: at most 448 threads (the rows evenly spread over the blocks; 127 registers and 142 KB at
+// 28 points, one block per SM); windows wider than 112 points take one row and up to 544 threads.
 int stencil_rows(const Geo& g) {
   const int most = std::max(1, 448 / (4 * g.U[0]));
   const int chunks = (g.U[1] + most - 1) / most;
