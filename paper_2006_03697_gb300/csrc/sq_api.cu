@@ -272,12 +272,18 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why, size_t limit
       }
       g.grd2[a][dd] = sum;
     }
-  g.lap0f = float(g.lap0);
   for (int a = 0; a < 3; ++a)
     for (int p = 0; p <= sq::kMaxNo; ++p) {
       g.lapf[a][p] = float(g.lap[a][p]);
       g.grdf[a][p] = float(g.grd[a][p]);
     }
+  int max_nch = 1;
+  for (int J = 0; J < d->n_atoms; ++J) {
+    int nch = 0;
+    for (int i = d->proj_offset[d->species[J]]; i < d->proj_offset[d->species[J] + 1]; ++i) nch += 2 * d->proj[i].l + 1;
+    max_nch = std::max(max_nch, nch);
+  }
+  P.split_able = d->precision == SQ_MIXED && max_nch <= 4;   // (its lists hold whole bricks)
   // atoms: base image wrapped into the cell, support box of the largest projector radius
   P.atoms.clear();
   long long off = 0;
@@ -321,7 +327,7 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why, size_t limit
     // capacity bounds: images of this atom that can meet a window of extent W on axis a
     long long nimg_u = 1, nimg_b = 1;
     for (int a = 0; a < 3; ++a) {
-      nimg_u *= floor_div(sq::kBrick * g.nbr[a] + dmax[a] - 2, g.n[a]) + 1;   // whole bricks of the window
+      nimg_u *= floor_div((P.split_able ? sq::kBrick * g.nbr[a] : g.U[a]) + dmax[a] - 2, g.n[a]) + 1;
       nimg_b *= floor_div(sq::kBrick + dmax[a] - 2, g.n[a]) + 1;
     }
     if (at.nch == 0) { nimg_u = nimg_b = 0; }
@@ -350,9 +356,6 @@ int make_plan(const sq_instance_desc* d, Plan& P, std::string& why, size_t limit
                      size_t(g.nslab) * (size_t(g.r_cap) + 1) * sizeof(int);   // slab row maps
   if (d->precision == SQ_MIXED && !d0_in_ring(g)) P.per_tile_bytes += size_t(g.nbricks) * g.br_cap * sizeof(float4);
   if (d->precision == SQ_MIXED && staged_requested()) P.per_tile_bytes += size_t(g.nbricks) * g.br_cap * sizeof(int4);
-  int max_nch = 1;
-  for (const sq::AtomTab& at : P.atoms) max_nch = std::max(max_nch, at.nch);
-  P.split_able = d->precision == SQ_MIXED && max_nch <= 4;
   // its image -> brick index and the bricks' rows (nl_*: what each atom's images bring, bricks_met)
   double nl_tile_rows = 0.0, nl_tile_imgs = 0.0;
   std::vector<double> met(P.atoms.size(), 0.0);

@@ -99,8 +99,7 @@ struct Geo {
   double lap[3][kMaxNo + 1];      // -1/2 w_p / h_a^2
   double grd[3][kMaxNo + 1];      // g_p / h_a
   double grd2[3][2 * kMaxNo + 1]; // [grad_a grad_a]_{c, c + d} at a window's centre c, d = 0 .. 2 n_o (both factors restricted)
-  float lap0f;                    // float copies used by the FP32 sweep (constant-bank operands)
-  float lapf[3][kMaxNo + 1];
+  float lapf[3][kMaxNo + 1];      // float copies used by the FP32 sweep (constant-bank operands)
   float grdf[3][kMaxNo + 1];
   int e_cap;                      // entries per tile (capacity)
   int r_cap;                      // projector rows per tile (capacity)
@@ -130,7 +129,8 @@ struct WaveBufs {
   void* T[3] = {nullptr, nullptr, nullptr};   // Real [wt][Upts][B]
   void* W = nullptr;              // FP32: W_b [wt][3][Upts][B]; FP64: G_ab = -grad_a W_b [wt][9][Upts][B]
   void* A = nullptr;              // Real [wt][r_cap][B]  chi_row(x_q)
-  void* Pg[2] = {nullptr, nullptr};   // double [wt][r_cap][B]  gamma |dOmega| chi^T t^j, ping-pong
+  void* Pg[2] = {nullptr, nullptr};   // [wt][r_cap][B] gamma |dOmega| chi^T t^j: doubles, ping-pong; the split mixed step
+                                      // keeps float pairs in the first, TF32 hi and lo planes in the second
   double* Spart = nullptr;        // [wt][slabs, their bricks or stencil row chunks][B][9]
   // the split mixed step (sq_step_mixed.cu)
   int* proj_start = nullptr;      // [wt][e_cap + 1] an image's entries of proj_idx

@@ -60,7 +60,7 @@ __global__ void k_split_tf32(const float* __restrict__ in, long long n, float* _
 
 // One block per tile of the wave: list the atom images (atom, shift s) whose support box
 // meets the tile's union window, atom-major then s (x fastest); assign projector rows.
-__global__ void k_tile_entries(Geo g, Wave w, const AtomTab* __restrict__ atoms, TileEntry* __restrict__ entries,
+__global__ void k_tile_entries(Geo g, Wave w, int whole, const AtomTab* __restrict__ atoms, TileEntry* __restrict__ entries,
                                int* __restrict__ n_entries, int* __restrict__ n_rows, int* __restrict__ status) {
   const int tl = blockIdx.x, t = wave_tile(w, tl);
   int o[3];
@@ -68,7 +68,8 @@ __global__ void k_tile_entries(Geo g, Wave w, const AtomTab* __restrict__ atoms,
   int ulo[3], uhi[3];
   for (int a = 0; a < 3; ++a) {
     ulo[a] = o[a] - g.m[a];
-    uhi[a] = ulo[a] + kBrick * g.nbr[a] - 1;   // whole bricks: tiles that share a brick list the same images
+    // whole bricks for the split mixed step: tiles that share a brick list the same images
+    uhi[a] = ulo[a] + (whole ? kBrick * g.nbr[a] : g.U[a]) - 1;
   }
   TileEntry* out = entries + (size_t)tl * g.e_cap;
   int base_e = 0, base_r = 0;
@@ -160,7 +161,8 @@ __global__ void k_brick_lists(Geo g, Wave w, int whole, const AtomTab* __restric
   for (int a = 0; a < 3; ++a) bhi[a] = whole ? bl[a] + kBrick - 1 : min(bl[a] + kBrick, o[a] - g.m[a] + g.U[a]) - 1;
   // the slab: all of U in x and z, the brick's planes in y
   const int sl[3] = {o[0] - g.m[0], bl[1], o[2] - g.m[2]};
-  const int shi[3] = {sl[0] + kBrick * g.nbr[0] - 1, bhi[1], sl[2] + kBrick * g.nbr[2] - 1};
+  const int shi[3] = {sl[0] + (whole ? kBrick * g.nbr[0] : g.U[0]) - 1, bhi[1],
+                      sl[2] + (whole ? kBrick * g.nbr[2] : g.U[2]) - 1};
   const bool slab_writer = (bx == 0 && bz == 0);
   int* smap = slab_map + ((size_t)tl * g.nslab + by) * g.r_cap;
   const int ne = n_entries[tl];
@@ -487,10 +489,11 @@ int build_wave_entries(sq_handle* h, const Wave& w, WaveBufs* b) {
   cudaStream_t s = h->stream;
   if (!b) b = &h->wb;
   if (b == &h->wb) h->lists_key = {w.tile0, w.ntiles, w.ids, h->atoms_epoch, false};
-  k_tile_entries<<<w.ntiles, 256, 0, s>>>(g, w, h->d.atoms, b->entries, b->n_entries, b->n_rows, h->d.status);
+  const int whole = h->split_able ? 1 : 0;
+  k_tile_entries<<<w.ntiles, 256, 0, s>>>(g, w, whole, h->d.atoms, b->entries, b->n_entries, b->n_rows, h->d.status);
   SQ_LAUNCH_CHECK(h);
-  k_brick_lists<<<dim3(g.nbricks, w.ntiles), 32, 0, s>>>(g, w, h->split_able ? 1 : 0, h->d.atoms, h->d.rcmax, b->entries, b->n_entries,
-                                                          b->brick_list, b->brick_n, b->brick_rec, b->brick_d0,
+  k_brick_lists<<<dim3(g.nbricks, w.ntiles), 32, 0, s>>>(g, w, whole, h->d.atoms, h->d.rcmax, b->entries, b->n_entries, b->brick_list,
+                                                          b->brick_n, b->brick_rec, b->brick_d0,
                                                           b->brick_tma, b->slab_n, b->slab_map, h->d.status);
   SQ_LAUNCH_CHECK(h);
   return SQ_OK;

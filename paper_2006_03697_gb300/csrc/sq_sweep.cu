@@ -21,6 +21,7 @@
 //               row; then (k_step) clears Pg^j, which accumulates the projections of step j + 1.
 //   k_apply_h / k_project   plain H_q v for the Lanczos bounds (sweep precision).
 #include <algorithm>
+#include <type_traits>
 
 #include "sq_device.cuh"
 
@@ -217,12 +218,10 @@ k_apply_h(Geo g, Wave w, const Real* __restrict__ Tc, Real* __restrict__ Tn, con
 // stencil weights of the sweep's precision, read straight from the kernel parameters
 template <typename Real> struct Coef;
 template <> struct Coef<float> {
-  static __device__ __forceinline__ float lap0(const Geo& g) { return g.lap0f; }
   static __device__ __forceinline__ float lap(const Geo& g, int a, int p) { return g.lapf[a][p]; }
   static __device__ __forceinline__ float grd(const Geo& g, int a, int p) { return g.grdf[a][p]; }
 };
 template <> struct Coef<double> {
-  static __device__ __forceinline__ double lap0(const Geo& g) { return g.lap0; }
   static __device__ __forceinline__ double lap(const Geo& g, int a, int p) { return g.lap[a][p]; }
   static __device__ __forceinline__ double grd(const Geo& g, int a, int p) { return g.grd[a][p]; }
 };
@@ -261,8 +260,9 @@ int step_parts(const Geo& g, int ntiles, bool fp64) {
   return fp64 && (long long)bricks * g.nslab * ntiles <= kStepFill ? bricks : 1;
 }
 
-// NCH: every atom has one channel (1: a table value per point in place of a padded group of four) or any number (4)
-template <typename Real, int NO, bool kSmemP, int NCH>
+// NCH: every atom has one channel (1: a table value per point in place of a padded group of four) or any number (4).
+// kParts: a block per brick, a warp per z-plane of it (step_parts)
+template <typename Real, int NO, bool kSmemP, int NCH, bool kParts>
 __global__ void __launch_bounds__(kStepThreads, sizeof(Real) == 4 ? 4 : 2)
 k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, Real* __restrict__ Tn,
        const double* __restrict__ Pg, double* __restrict__ Pg_next, const Real* __restrict__ Wt,
@@ -350,9 +350,9 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
   // a warp's units of work: whole bricks, or one z-plane of a brick (step_parts); FP64 takes a plane's four
   // points per lane at a time, FP32 two planes'
   constexpr int kGrp = kG ? 1 : 2;   // planes per group
-  const int bps = nbx * nbz, sub = gridDim.z > 1 ? 4 : 1;
-  for (int un = blockIdx.z + gridDim.z * warp; un < bps * sub; un += gridDim.z * nw) {
-    const int bi = un % bps, pl0 = un / bps, pl1 = sub > 1 ? pl0 + 1 : 4;   // planes [pl0, pl1)
+  const int bps = nbx * nbz, step = kParts ? gridDim.z * nw : nw;
+  for (int un = kParts ? blockIdx.z + gridDim.z * warp : warp; un < (kParts ? 4 * bps : bps); un += step) {
+    const int bi = kParts ? un % bps : un, pl0 = kParts ? un / bps : 0, pl1 = kParts ? pl0 + 1 : 4;   // planes [pl0, pl1)
     const int bx = bi % nbx, bz = bi / nbx, by = slab;
     const int br = (bz * nby + by) * nbx + bx;
     const int4* rb = brec + ((size_t)tl * g.nbricks + br) * g.br_cap * 2;
@@ -413,16 +413,20 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
         Real tn = Real(0);
         if (inwin) {
           // loads that do not depend on the stencil, issued first
-          Real wv[kG ? 9 : 3];
+          const Real w0 = Wq[e], w1 = Wq[wstr + e], w2 = Wq[2 * wstr + e];
+          Real wv[kG ? 6 : 1];
+          if constexpr (kG) {
 #pragma unroll
-          for (int k = 0; k < (kG ? 9 : 3); ++k) wv[k] = Wq[k * wstr + e];
+            for (int k = 0; k < 6; ++k) wv[k] = Wq[(3 + k) * wstr + e];
+          }
           const Real tp = (mode == 1) ? Tp[tbase + e] : Real(0);
           const Real tc = T[e];
           Real y = Real(0);                           // off-diagonal part of H t^j
-          Real gr[3] = {Real(0), Real(0), Real(0)};
+          Real gr[3];
           const int u[3] = {ux, uy, uz};
 #pragma unroll
           for (int a = 0; a < 3; ++a) {
+            gr[a] = Real(0);
 #pragma unroll
             for (int pp = 1; pp <= NO; ++pp) {
               const Real fp = (u[a] + pp < Ua[a]) ? T[e + (size_t)pp * st[a]] : Real(0);
@@ -437,10 +441,19 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
             tn = caA * y + (cdA + caA * vloc) * tc - cc * tp;
             Tn[tbase + e] = tn;
           }
+          if constexpr (kG) {
+            sacc[0] += w0 * tc;
+            sacc[1] += w1 * tc;
+            sacc[2] += w2 * tc;
 #pragma unroll
-          for (int a = 0; a < 3; ++a) {
+            for (int k = 0; k < 6; ++k) sacc[3 + k] += wv[k] * tc;
+          } else {
 #pragma unroll
-            for (int b = 0; b < 3; ++b) sacc[3 * a + b] += kG ? wv[kG ? 3 * a + b : 0] * tc : gr[a] * wv[b];
+            for (int a = 0; a < 3; ++a) {
+              sacc[3 * a + 0] += gr[a] * w0;
+              sacc[3 * a + 1] += gr[a] * w1;
+              sacc[3 * a + 2] += gr[a] * w2;
+            }
           }
         } else if (inU && mode != 2) {
           Tn[tbase + e] = Real(0);
@@ -461,7 +474,7 @@ k_step(Geo g, Wave w, const Real* __restrict__ Tc, const Real* __restrict__ Tp, 
           const int nch = r0.w & 0xff, nchp = (r0.w >> 8) & 0xff;
           const int prow = kSmemP ? (int(unsigned(r0.w) >> 16)) : r0.y;
           const unsigned mlo = unsigned(r1.z) >> pa, mhi = unsigned(r1.w) >> pa;
-          if (sub > 1 && !((unsigned(pl0 < 2 ? r1.z : r1.w) >> (16 * (pl0 & 1))) & 0xffffu)) continue;
+          if (kParts && !((unsigned(pl0 < 2 ? r1.z : r1.w) >> (16 * (pl0 & 1))) & 0xffffu)) continue;
           if constexpr (NCH == 1) {
             Real acc = Real(0);
 #pragma unroll 8
@@ -578,7 +591,7 @@ k_moments(Geo g, Wave w, int j, const Real* __restrict__ Tj, const Real* __restr
       val[pr] = s;
     }
     // N^j = w_q^T V_nl,q t^j = sum_rows chi_row(x_q) (gamma |dOmega| chi_row^T t^j)
-    if constexpr (kPair) {   // float pairs: products and sums with their rounding errors (FP64's accuracy at FP32 rates)
+    if constexpr (kPair) {   // float pairs: products and sums with their rounding errors (about 2^-47 relative)
       float nh = 0.f, nl = 0.f;
       for (int r = lane; r < nr; r += 32) {
         const size_t k = (size_t)r * B + q;
@@ -655,10 +668,19 @@ static int launch_step(sq_handle* h, const Wave& w, dim3 grid, size_t smem, cons
                                              h->d.status);
     return SQ_OK;
   };
-  int rc;
-  if (staged) rc = one ? go(k_step<Real, NO, true, 1>, smem + smem_warps, rows_smem)
-                       : go(k_step<Real, NO, true, 4>, smem + smem_warps, rows_smem);
-  else rc = one ? go(k_step<Real, NO, false, 1>, smem_warps, 0) : go(k_step<Real, NO, false, 4>, smem_warps, 0);
+  int rc = SQ_OK;
+  auto pick = [&](auto parts) {
+    constexpr bool kP = decltype(parts)::value;
+    if (staged) rc = one ? go(k_step<Real, NO, true, 1, kP>, smem + smem_warps, rows_smem)
+                         : go(k_step<Real, NO, true, 4, kP>, smem + smem_warps, rows_smem);
+    else rc = one ? go(k_step<Real, NO, false, 1, kP>, smem_warps, 0) : go(k_step<Real, NO, false, 4, kP>, smem_warps, 0);
+  };
+  if constexpr (sizeof(Real) == 8) {
+    if (grid.z > 1) pick(std::true_type{});
+    else pick(std::false_type{});
+  } else {
+    pick(std::false_type{});
+  }
   if (rc != SQ_OK) return rc;
   SQ_LAUNCH_CHECK(h);
   return SQ_OK;
@@ -759,8 +781,8 @@ static int sweep_t(sq_handle* h, const Real* chi, const Real* v, const Real* gdv
       timing_end(h, ev);
       ev = capturing ? nullptr : timing_begin(h, SQ_K_MOMENTS, 0.0);
       if (split)
-        k_moments<Real, true><<<w.ntiles, kThreads, 0, s>>>(g, w, j, Tc, A, Pg[0], h->wb.n_rows, h->wb.Spart,
-                                                            stencil_chunks(g), h->d.mom);
+        k_moments<float, true><<<w.ntiles, kThreads, 0, s>>>(g, w, j, (const float*)Tc, (const float*)A, Pg[0],
+                                                             h->wb.n_rows, h->wb.Spart, stencil_chunks(g), h->d.mom);
       else
         k_moments<Real, false><<<w.ntiles, kThreads, 0, s>>>(g, w, j, Tc, A, Pg[j % 2], h->wb.n_rows, h->wb.Spart,
                                                              g.nslab * parts, h->d.mom);
