@@ -64,8 +64,11 @@ extern "C" {
 #define SQ_FP64 0    /* FP64 recurrence, projectors and moments                          */
 #define SQ_MIXED 1   /* FP32 recurrence and moment products, projector products on TF32
                         tensor cores with a hi/lo split (about 2^-21 relative), FP32
-                        Lanczos vectors for the bounds; FP64 node and cross-thread sums,
-                        Gram-Schmidt coefficients, Fermi search and contraction          */
+                        Lanczos vectors for the bounds; their sums (over a brick's
+                        projections, a tile's rows, a Krylov product) as pairs of floats
+                        (about 2^-47), the stencil's nonlocal stress as FP32 per warp;
+                        FP64 K^j, node sums, Gram-Schmidt coefficients, Fermi search and
+                        contraction                                                      */
 
 /* spectral bound modes (the paper takes chi, zeta from the extreme eigenvalues of H_q) */
 #define SQ_BOUNDS_LANCZOS 0   /* k-step Lanczos on sample regions, widened (default)   */

@@ -72,7 +72,7 @@ __global__ void k_lz_init_unit(Geo g, Wave w, Real* __restrict__ V0) {
 // share out the vectors V_i, each taking all groups of its vectors, so x is read from memory once, a
 // V chunk read by the update is still in cache for the products, and no product crosses warps. The
 // four products of a lane are added over the warp by a reduce-scatter (5 exchanges in place of 16).
-// Cross-thread sums keep FP64's accuracy: FP64 vectors add doubles, FP32 vectors add pairs of floats
+// Cross-thread sums: FP64 vectors add doubles, FP32 vectors add pairs of floats
 // (two-sum; FP64 adds issue at 1.7 lanes per clock here and cost more than the products).
 constexpr int kLzThreads = 256, kLzWarps = kLzThreads / 32;
 
